@@ -184,7 +184,7 @@ DIROTQ_API dirotq_status_t dirotq_int_gemm_debug(const int8_t* act_codes, int M,
  * between the other two; 512: the NVFP4 kernel in pairs of CTAs (clusters of two, tcgen05.mma.cta_group::2, 256 token
  * rows x 256 columns per pair, each CTA loading its own rows and one half of the weight tile), forced; 0 takes it
  * where its schedule is the shortest (a pair does two wide tiles' work in about 0.9 of a wide tile's time: every FLUX
- * shape at M = 4608).  A value that names a plan of
+ * shape at M = 4608); for W4A8 128 is single CTAs, 256 and 512 are CTA pairs with 128 and 256 columns.  A value that names a plan of
  * one kernel leaves the other formats' kernels choosing for themselves.  Process-wide; results do not depend on it (each
  * output element is accumulated in the same order).  Other values: DIROTQ_ERR_INVALID_ARG. */
 DIROTQ_API dirotq_status_t dirotq_set_gemm_tile(int columns);

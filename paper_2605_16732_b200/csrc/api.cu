@@ -504,18 +504,14 @@ dirotq_status_t dirotq_prepare_layer_w4a8(const void* W, int w_dtype, int w_layo
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_qt64, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L->blob + lay.off_qt, (uint64_t)K, (uint64_t)K,
                             (uint64_t)K * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
-    if (st == DIROTQ_OK)
-        st = encode_tmap_2d(&L->tmap_wpacked, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, L->blob + lay.off_wpacked,
-                            (uint64_t)g.K_lp / 2, (uint64_t)N, (uint64_t)g.K_lp / 2, 64, kGemmBN, CU_TENSOR_MAP_SWIZZLE_NONE);
-    if (st == DIROTQ_OK)
-        st = encode_tmap_2d(&L->tmap_wh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L->blob + lay.off_wh, (uint64_t)g.r_pad,
-                            (uint64_t)N, (uint64_t)g.r_pad * 2, 64, kGemmBN, CU_TENSOR_MAP_SWIZZLE_128B);
-    if (st == DIROTQ_OK)
-        st = encode_tmap_2d(&L->tmap_wpacked128, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, L->blob + lay.off_wpacked,
-                            (uint64_t)g.K_lp / 2, (uint64_t)N, (uint64_t)g.K_lp / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
-    if (st == DIROTQ_OK)
-        st = encode_tmap_2d(&L->tmap_wh128, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L->blob + lay.off_wh, (uint64_t)g.r_pad,
-                            (uint64_t)N, (uint64_t)g.r_pad * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
+    for (const int rows : {64, 128}) {  // a CTA's weight rows in the second kernel's plans
+        if (st != DIROTQ_OK) break;
+        st = encode_tmap_2d(rows == 64 ? &L->tmap_wpacked64 : &L->tmap_wpacked128, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, L->blob + lay.off_wpacked,
+                            (uint64_t)g.K_lp / 2, (uint64_t)N, (uint64_t)g.K_lp / 2, 64, rows, CU_TENSOR_MAP_SWIZZLE_NONE);
+        if (st == DIROTQ_OK)
+            st = encode_tmap_2d(rows == 64 ? &L->tmap_wh64 : &L->tmap_wh128, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L->blob + lay.off_wh,
+                                (uint64_t)g.r_pad, (uint64_t)N, (uint64_t)g.r_pad * 2, 64, rows, CU_TENSOR_MAP_SWIZZLE_128B);
+    }
     if (st == DIROTQ_OK)
         st = launch_prepare_w4a8(L, W, w_dtype, w_layout, Q, q_dtype, bias, static_cast<double*>(scratch),
                                  static_cast<cudaStream_t>(stream));
@@ -656,7 +652,7 @@ dirotq_status_t dirotq_set_gemm_tile(int columns) {
     const bool int4_only = columns == 64 || columns == 66 || columns == 192;  // 66: 64 columns with the reduction split over a cluster
     dirotq_status_t st = set_w4a4_tile_columns(columns == 512 ? 0 : columns);
     if (st == DIROTQ_OK) st = set_nvfp4_tile_columns(int4_only ? 0 : columns);
-    return st != DIROTQ_OK ? st : set_w4a8_tile_columns(int4_only || columns == 512 ? 0 : columns);
+    return st != DIROTQ_OK ? st : set_w4a8_tile_columns(int4_only ? 0 : columns);
 }
 
 dirotq_status_t dirotq_rotate_quantize(const void* x, int M, const dirotq_layer_t* layer, void* workspace,

@@ -451,6 +451,7 @@ dirotq_status_t launch_workspace_export(const dirotq_layer* L, int M, const char
 dirotq_status_t launch_workspace_export_asym(const dirotq_layer* L, int M, const char* workspace, uint16_t* xh,
                                              uint8_t* codes, uint16_t* scales, uint16_t* zeros, cudaStream_t stream);
 dirotq_status_t launch_zero_term_export(const dirotq_layer* L, float* d, cudaStream_t stream);
+dirotq_status_t launch_w4a8_pair(const dirotq_layer* L, int columns, const A8GemmArgs& a, cudaStream_t stream);  // (not for partials)
 dirotq_status_t launch_w4a8_gemm(const dirotq_layer* L, const A8GemmArgs& a, cudaStream_t stream);
 dirotq_status_t launch_a8_quantize(const dirotq_layer* L, int M, const float* xtilde, const unsigned int* rowmax, int8_t* codes,
                                    float* xscale, cudaStream_t stream);

@@ -10,11 +10,11 @@
 // the operand buffer and four unpack warps expand them in place, turning every nibble into the byte 16 q (shift the nibble into the high half, flip
 // bit 7: 16 (q + 8) - 128), so the accumulator holds 16 P and the epilogue shifts it back.
 //
-// Roles (448 threads): warp 0 TMA producer, warp 1 MMA issuer + TMEM owner, warps 2..5 unpack,
-// warps 6..13 epilogue (one token row per thread, two warps per lane quadrant).  TMEM: columns 0..255 the int32 tile, 256..511 the
-// fp32 tile of the bf16 rank-r branch (kind::f16 cannot accumulate into the integer tile); with 256-column tiles that
-// pair fills tensor memory and a tile's epilogue (one pass) is not overlapped with the next tile's MMAs; with 128-column
-// tiles two pairs alternate and it is.
+// This kernel computes 128 x 128 tiles on single CTAs, for calls of at most 128 token rows and where the CTA pairs of w4a8_pair.cu would
+// need as many turns (and for the export of the integer sums).  448 threads: warp 0 TMA producer, warp 1 MMA issuer + TMEM
+// owner, warps 2..5 unpack, warps 6..13 epilogue (one token row per thread, two warps per lane quadrant).  Two accumulator
+// sets alternate in tensor memory, so a tile's epilogue runs under the next tile's MMAs; a set is the int32 tile and the
+// fp32 tile of the bf16 rank-r branch (kind::f16 cannot accumulate into the integer tile).
 #include "common.h"
 #include "ptx.cuh"
 
@@ -32,24 +32,21 @@ constexpr int NUM_THREADS = 448;
 constexpr int NUM_UNPACK_WARPS = 4;
 constexpr int NUM_EPI_WARPS = 8;  // two per TMEM lane quadrant, half of the tile's columns each
 
-// Shared-memory plan for tiles of BN output columns (256, or 128 where wide tiles would leave SMs idle).
-template <int BN>
-struct Plan {
-    static constexpr int STAGES = BN == 256 ? 4 : 6;
-    static constexpr int BU_BYTES = BN * BKC;      // unpacked weight codes / bf16 W~_h chunk (32 KB at BN = 256)
-    static constexpr int BP_BYTES = BN * BKC / 2;  // packed weight codes: TMA puts them into the UPPER HALF of the
-    static constexpr int BP_OFFSET = A_BYTES + BU_BYTES - BP_BYTES;  // operand buffer and the unpack expands them in place
-    static constexpr int STAGE_BYTES = A_BYTES + BU_BYTES;           // 48 KB x 4 or 32 KB x 6
-    static constexpr int BAR_OFFSET = STAGES * STAGE_BYTES;
-    static constexpr int SCALE_OFFSET = BAR_OFFSET + 256;  // two buffers of {weight scales, bias} for a tile's columns
-    static constexpr int SCALE_BYTES = 2 * 2 * BN * 4;
-    // one 32-row x 64-byte staging tile per epilogue warp (64-byte swizzle), from which the outputs leave as TMA stores
-    static constexpr int STORE_OFFSET = (SCALE_OFFSET + SCALE_BYTES + 1023) / 1024 * 1024;
-    static constexpr int SMEM_BYTES = STORE_OFFSET + NUM_EPI_WARPS * 2048 + 1024;
-    static constexpr int NACC = 512 / (2 * BN);  // {int32 tile, fp32 tile} pairs in tensor memory: 1 (wide) or 2 (narrow tiles)
-    static_assert(8 * (3 * STAGES + 4) <= 192, "barriers must end below the two words at +192");
-    static_assert(SMEM_BYTES <= 232448 && STAGE_BYTES % 1024 == 0, "shared memory plan");
-};
+constexpr int BN = 128;      // output columns of a tile
+constexpr int STAGES = 6;
+constexpr int BU_BYTES = BN * BKC;      // unpacked weight codes / bf16 W~_h chunk
+constexpr int BP_BYTES = BN * BKC / 2;  // packed weight codes: TMA puts them into the UPPER HALF of the
+constexpr int BP_OFFSET = A_BYTES + BU_BYTES - BP_BYTES;  // operand buffer and the unpack expands them in place
+constexpr int STAGE_BYTES = A_BYTES + BU_BYTES;           // 32 KB
+constexpr int BAR_OFFSET = STAGES * STAGE_BYTES;
+constexpr int SCALE_OFFSET = BAR_OFFSET + 256;  // two buffers of {weight scales, bias} for a tile's columns
+constexpr int SCALE_BYTES = 2 * 2 * BN * 4;
+// one 32-row x 64-byte staging tile per epilogue warp (64-byte swizzle), from which the outputs leave as TMA stores
+constexpr int STORE_OFFSET = (SCALE_OFFSET + SCALE_BYTES + 1023) / 1024 * 1024;
+constexpr int SMEM_BYTES = STORE_OFFSET + NUM_EPI_WARPS * 2048 + 1024;
+constexpr int NACC = 512 / (2 * BN);  // {int32 tile, fp32 tile} pairs in tensor memory
+static_assert(8 * (3 * STAGES + 4) <= 192, "barriers must end below the two words at +192");
+static_assert(SMEM_BYTES <= 232448 && STAGE_BYTES % 1024 == 0, "shared memory plan");
 
 struct A8KernelParams {
     int M, N, num_kb, lr_chunks;
@@ -74,14 +71,11 @@ __device__ __forceinline__ void tmem_ld_fence32(uint32_t (&v)[32]) {
                  :: "memory");
 }
 
-template <bool kPartials, int BN>
+template <bool kPartials>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_constant__ CUtensorMap tmap_wpacked,
                  const __grid_constant__ CUtensorMap tmap_xh, const __grid_constant__ CUtensorMap tmap_wh,
                  const __grid_constant__ CUtensorMap tmap_y, const A8KernelParams p) {
-    using P = Plan<BN>;
-    constexpr int STAGES = P::STAGES, BU_BYTES = P::BU_BYTES, BP_BYTES = P::BP_BYTES, BP_OFFSET = P::BP_OFFSET;
-    constexpr int STAGE_BYTES = P::STAGE_BYTES, BAR_OFFSET = P::BAR_OFFSET, SCALE_OFFSET = P::SCALE_OFFSET;
     constexpr int PIECES = BN * 4 / (NUM_UNPACK_WARPS * 32);  // 16-byte pieces of the packed tile per unpack thread
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -90,7 +84,6 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
     auto unp_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
     auto empty_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + s); };
-    constexpr int NACC = P::NACC;
     auto tfull_bar = [&](uint32_t a) { return bar_base + 8u * (3 * STAGES + a); };
     auto tempty_bar = [&](uint32_t a) { return bar_base + 8u * (3 * STAGES + 2 + a); };
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + BAR_OFFSET + 192);
@@ -347,7 +340,7 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     // cycles per tile and slowing the operand loads).  The warp converts 32 columns of its 32 rows into its
                     // staging tile (64-byte swizzle: a quarter-warp's pieces fall into different banks) and one lane hands
                     // it to a TMA store, which writes whole sectors and clips at M and N.
-                    const uint32_t sbuf = smem_base + P::STORE_OFFSET + static_cast<uint32_t>(warp - (2 + NUM_UNPACK_WARPS)) * 2048u;
+                    const uint32_t sbuf = smem_base + STORE_OFFSET + static_cast<uint32_t>(warp - (2 + NUM_UNPACK_WARPS)) * 2048u;
                     // the chunk is converted first; only then does the warp wait for the copy engine to have read the staging
                     // tile's previous contents (this epilogue is exposed: nothing else hides that read)
                     uint32_t packed[16];
@@ -404,8 +397,7 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     }
 }
 
-template <int BN>
-static dirotq_status_t launch_w4a8_gemm_bn(const dirotq_layer* L, const A8GemmArgs& a, cudaStream_t stream) {
+static dirotq_status_t launch_single(const dirotq_layer* L, const A8GemmArgs& a, cudaStream_t stream) {
     const Geometry& g = L->geo;
     CUtensorMap tmap_codes, tmap_xh;
     dirotq_status_t st;
@@ -426,10 +418,9 @@ static dirotq_status_t launch_w4a8_gemm_bn(const dirotq_layer* L, const A8GemmAr
     const int num_tiles = ((a.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
     const int grid = num_tiles < sm_count(L->device) ? num_tiles : sm_count(L->device);
     const bool dbg = a.partials != nullptr;
-    auto kern = dbg ? w4a8_gemm_kernel<true, BN> : w4a8_gemm_kernel<false, BN>;
+    auto kern = dbg ? w4a8_gemm_kernel<true> : w4a8_gemm_kernel<false>;
     static SmemOptIn<2> opt_in;
-    if (!opt_in.ensure(kern, dbg ? 1 : 0, L->device, Plan<BN>::SMEM_BYTES)) return DIROTQ_ERR_CUDA;
-    const bool narrow = BN == 128;
+    if (!opt_in.ensure(kern, dbg ? 1 : 0, L->device, SMEM_BYTES)) return DIROTQ_ERR_CUDA;
     // the outputs leave as TMA stores of 32 rows x 32 columns (64-byte swizzle in shared memory); the debug export of the
     // integer sums stores directly and is given the activation map in its place
     CUtensorMap tmap_y = tmap_xh;
@@ -438,33 +429,32 @@ static dirotq_status_t launch_w4a8_gemm_bn(const dirotq_layer* L, const A8GemmAr
                             CU_TENSOR_MAP_SWIZZLE_64B);
         if (st != DIROTQ_OK) return st;
     }
-    const cudaError_t err = launch_kernel(kern, grid, NUM_THREADS, Plan<BN>::SMEM_BYTES, stream, true, tmap_codes,
-                                          narrow ? L->tmap_wpacked128 : L->tmap_wpacked, tmap_xh,
-                                          narrow ? L->tmap_wh128 : L->tmap_wh, tmap_y, p);
+    const cudaError_t err = launch_kernel(kern, grid, NUM_THREADS, SMEM_BYTES, stream, true, tmap_codes,
+                                          L->tmap_wpacked128, tmap_xh, L->tmap_wh128, tmap_y, p);
     return err == cudaSuccess ? DIROTQ_OK : DIROTQ_ERR_CUDA;
 }
 
-static std::atomic<int> g_a8_tile_columns{0};  // 0: chosen per call; 128 / 256: forced
+static std::atomic<int> g_a8_tile_columns{0};  // 0: chosen per call; 128: single CTAs; 256 / 512: CTA pairs, 128 / 256 columns
 
 }  // namespace
 
 dirotq_status_t set_w4a8_tile_columns(int columns) {
-    if (columns != 0 && columns != 128 && columns != 256) return DIROTQ_ERR_INVALID_ARG;
+    if (columns != 0 && columns != 128 && columns != 256 && columns != 512) return DIROTQ_ERR_INVALID_ARG;
     g_a8_tile_columns.store(columns);
     return DIROTQ_OK;
 }
 
 dirotq_status_t launch_w4a8_gemm(const dirotq_layer* L, const A8GemmArgs& a, cudaStream_t stream) {
-    // narrow tiles only where the wide ones leave SMs idle: a 128-column tile costs about NARROW_COST of a 256-column one
-    constexpr double NARROW_COST = 0.68;  // measured: 0.220 against 0.162 ms with twice as many tiles (4608 x 3072 -> 9216)
+    // A CTA pair takes 256 token rows at once, so calls of at most 128 rows keep single CTAs.  Otherwise the wide pair plan runs
+    // wherever it does not need clearly more turns: per turn the narrow one costs 0.85 of it (31 against 34 us for 4096 x 4608
+    // -> 1152 with two turns each, 160 against 100 us for 4608 x 3072 -> 9216 with 18 and 9), single CTAs 0.95.
     const int forced = g_a8_tile_columns.load();
-    const int sms = sm_count(L->device);
-    const long m_blocks = (a.M + BM - 1) / BM;
-    const long t_wide = m_blocks * ((L->geo.N + 255) / 256), t_narrow = m_blocks * ((L->geo.N + 127) / 128);
-    const bool narrow_pays =
-        NARROW_COST * static_cast<double>((t_narrow + sms - 1) / sms) < 0.98 * static_cast<double>((t_wide + sms - 1) / sms);
-    const bool narrow = forced ? forced == 128 : narrow_pays;
-    return narrow ? launch_w4a8_gemm_bn<128>(L, a, stream) : launch_w4a8_gemm_bn<256>(L, a, stream);
+    const int pairs = sm_count(L->device) / 2;
+    const long m_blocks = (a.M + 2 * BM - 1) / (2 * BM);
+    const long turns128 = (m_blocks * ((L->geo.N + 127) / 128) + pairs - 1) / pairs, turns256 = (m_blocks * ((L->geo.N + 255) / 256) + pairs - 1) / pairs;
+    const int plan = forced ? forced : a.M <= BM ? 128 : 0.85 * static_cast<double>(turns128) < static_cast<double>(turns256) ? 256 : 512;
+    if (a.partials != nullptr || plan == 128) return launch_single(L, a, stream);
+    return launch_w4a8_pair(L, plan / 2, a, stream);
 }
 
 }  // namespace dirotq
