@@ -171,10 +171,9 @@ DIROTQ_API dirotq_status_t dirotq_int_gemm_debug(const int8_t* act_codes, int M,
                                       dirotq_stream_t stream);
 
 /* Tuning knob of the second kernels (all four formats): output columns per tile.
- * 0 (default): chosen per call from M, N and the number of SMs (INT4: 256 columns unless 128-column tiles fill the
- * SMs so much better that they win although a narrow tile costs about 0.73 of a wide one, and 64 columns when even
- * 128-column tiles would keep under half of the SMs busy, i.e. for calls with few token rows; NVFP4 likewise with 0.6
- * and no 64-column plan);
+ * 0 (default): chosen per call from M, N and the number of SMs (grouped INT4: the shortest schedule of 256-, 128- and
+ * 64-column tiles, which cost 1 : 0.6 : 0.34 with groups of 64 and 1 : 0.64 : 0.4 with groups of 128; NVFP4: 256 columns
+ * unless 128-column tiles, at 0.6 of a wide one, shorten the schedule);
  * 128 or 256: forced; 64: the grouped INT4 kernel's plan for few token rows, forced, one CTA per tile; 66: the same
  * tiles with the K-groups of a tile cut over a cluster of up to four CTAs (partial tiles added in one of them through
  * distributed shared memory) wherever every tile's cluster is resident at once and every CTA keeps two k-blocks; never

@@ -309,6 +309,7 @@ dirotq_status_t encode_tmap_2d(CUtensorMap* out, CUtensorMapDataType dt, size_t 
 
 // launchers (each returns after enqueueing on `stream`)
 dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& a, cudaStream_t stream);
+dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, bool may_split, cudaStream_t stream);  // (not for partials)
 dirotq_status_t launch_w4a4_gemm(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream);
 dirotq_status_t set_w4a4_tile_columns(int columns);
 // Launches `kern`; with `dependent` (and unless switched off process-wide) as a programmatic dependent launch: the

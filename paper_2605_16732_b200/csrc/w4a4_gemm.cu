@@ -29,25 +29,18 @@
 // bf16 rank-r branch is issued as one more "group" (kind::f16 into the same ping-pong tile) and added
 // unscaled.
 //
+// Tiles of 256, 128 or (on request) 192 columns here; w4a4_narrow.cu has the same computation in 64-column tiles.
+//
 // Roles (384 threads = 3 warpgroups):
 //   warpgroup 0: warp 0 TMA producer, warp 1 MMA issuer + TMEM owner, warps 2-3 nibble -> byte unpack
 //   warpgroups 1-2: epilogue; warp%4 selects the TMEM lane quadrant (token rows), the warpgroup
 //                   selects the half of the tile's columns.
-#include "common.h"
-#include "ptx.cuh"
-
-#include <cuda_bf16.h>
+#include "w4a4.cuh"
 
 #include <atomic>
 
 namespace dirotq {
 namespace {
-
-constexpr int BM = 128;
-constexpr int BKC = 128;  // one-byte codes per k-block (128-byte rows)
-constexpr int A_BYTES = BM * BKC;          // 16 KB  activation codes / bf16 x~_h chunk
-constexpr uint32_t kSignMag = 0x87878787u;  // sign and 3-bit magnitude of four one-byte codes
-constexpr float kAccUnit = kI8Path ? 1.0f : kWScaleFold;  // integer group sum = accumulator value x this
 
 // Plan for tiles of BN output columns.
 //   256: two epilogue warpgroups, 128 columns (128 fp32 accumulators) per thread; an accumulator tile can only be read in
@@ -56,26 +49,15 @@ constexpr float kAccUnit = kI8Path ? 1.0f : kWScaleFold;  // integer group sum =
 //        buffers, so the tile goes back to the tensor core after the first quarter of a group, and three warps per scheduler
 //        hide each other's waits.  16 warps: 152 registers for the epilogue threads, 56 for the others.
 //   128: two warpgroups, 64 columns per thread, four accumulator tiles; for layers whose wider tiles would leave SMs idle.
-//    64: one warpgroup, 64 columns per thread, four accumulator tiles, seven stages; for calls with so few token rows that
-//        even 128-column tiles occupy a fraction of the SMs: there a tile's K-groups are a chain of hand-overs between the
-//        tensor core and the epilogue, whose length does not depend on the tile's width, so more, narrower tiles on more SMs
-//        shorten the call.  256 threads, no register re-partitioning (every thread may use 255).
-//    64 + SPLITK: clusters of up to four CTAs cut the K-groups of one 128 x 64 tile into contiguous ranges; each CTA rescales its
-//        range into its own fp32 accumulators, the others store theirs into the last CTA's shared memory (distributed shared
-//        memory, one cluster-scope barrier), and that CTA adds them in rank order, adds the rank-r branch and the bias, and
-//        stores.  For calls so small that the chain of K-groups per tile, not the number of tiles, sets the time.
-constexpr int SPLIT_MAX = 4;          // CTAs per cluster of the split plan
-constexpr int RED_BYTES = 128 * 64 * 4;  // one CTA's partial tile: 128 rows x 64 columns fp32
-template <int BN, bool SPLITK = false>
+template <int BN>
 struct Plan {
-    static constexpr int EPI_WG = BN == 192 ? 3 : BN == 64 ? 1 : 2;  // epilogue warpgroups
+    static constexpr int EPI_WG = BN == 192 ? 3 : 2;  // epilogue warpgroups
     static constexpr int EPI_WARPS = 4 * EPI_WG;
     static constexpr int THREADS = 128 + 128 * EPI_WG;
-    static constexpr bool REPARTITION = EPI_WG > 1;            // setmaxnreg after the role split
     static constexpr int EPI_REGS = EPI_WG == 3 ? 152 : 216;  // setmaxnreg budgets: 128 * AUX + 128 * EPI_WG * EPI <= 65536
     static constexpr int AUX_REGS = EPI_WG == 3 ? 56 : 64;
     static constexpr int SC_SLOTS = BN == 192 ? 6 : 8;
-    static constexpr int STAGES = BN == 256 ? 3 : BN == 192 ? 4 : BN == 128 ? 5 : SPLITK ? 3 : 7;
+    static constexpr int STAGES = BN == 256 ? 3 : BN == 192 ? 4 : 5;
     static constexpr int BU_BYTES = BN * BKC;         // unpacked weight codes / bf16 W~_h chunk (32 KB at BN = 256)
     static constexpr int BP_BYTES = BN * BKC / 2;     // packed weight codes (TMA staging)
     static constexpr int STAGE_BYTES = A_BYTES + BU_BYTES + BP_BYTES;  // 64 KB / 40 KB
@@ -83,98 +65,21 @@ struct Plan {
     static constexpr int SC_SX_BYTES = 2 * BM * 4;    // activation scales of up to two groups
     static constexpr int SC_BYTES = SC_SW_BYTES + SC_SX_BYTES;  // 3 KB / 2 KB
     static constexpr int BAR_OFFSET = STAGES * STAGE_BYTES + SC_SLOTS * SC_BYTES;
-    static constexpr int RED_OFFSET = BAR_OFFSET + 512;  // split plan: the other CTAs' partial tiles land here (last CTA)
-    static constexpr int SMEM_BYTES = BAR_OFFSET + 512 + 1024 + (SPLITK ? (SPLIT_MAX - 1) * RED_BYTES : 0);
-    static_assert(!SPLITK || BN == 64, "the split plan has 64-column tiles");
+    static constexpr int SMEM_BYTES = BAR_OFFSET + 512 + 1024;
 };
-static_assert(Plan<64, true>::SMEM_BYTES <= 232448, "shared memory plan too large");
 static_assert(Plan<256>::SMEM_BYTES <= 232448 && Plan<192>::SMEM_BYTES <= 232448 && Plan<128>::SMEM_BYTES <= 232448, "shared memory plan too large");
 static_assert(Plan<128>::STAGE_BYTES % 1024 == 0 && Plan<128>::SC_BYTES % 128 == 0, "tile alignment");
 static_assert(Plan<192>::STAGE_BYTES % 1024 == 0 && Plan<192>::SC_BYTES % 128 == 0, "tile alignment");
-static_assert(Plan<64>::SMEM_BYTES <= 232448 && Plan<64>::STAGE_BYTES % 1024 == 0 && Plan<64>::SC_BYTES % 128 == 0, "tile alignment");
-static_assert(8 * (3 * Plan<128>::STAGES + 2 * 8 + 9) <= 400 && 8 * (3 * Plan<192>::STAGES + 2 * 6 + 9) <= 400 &&
-              8 * (3 * Plan<64>::STAGES + 2 * 8 + 9) <= 400, "barriers end below the words at +400");
+static_assert(8 * (3 * Plan<128>::STAGES + 2 * 8 + 9) <= 400 && 8 * (3 * Plan<192>::STAGES + 2 * 6 + 9) <= 400,
+              "barriers end below the words at +400");
 
-struct GemmKernelParams {
-    int M, N, n_g, num_kb, lr_chunks;
-    const float* bias;
-    uint16_t* y;
-    int32_t* partials;
-    int* status;
-};
-
-// Wait accounting (diagnostics): cycles a role spends blocked on each kind of barrier are summed into
-// 64-bit counters that follow the status word in the workspace (8-byte slots 1..8, see WaitSlot).
-enum WaitSlot : int { WS_PROD_EMPTY = 1, WS_MMA_OPERANDS = 2, WS_MMA_TEMPTY = 3, WS_UNPACK_FULL = 4, WS_EPI_TFULL = 5,
-                      WS_EPI_SCALES = 6, WS_EPI_TOTAL = 7, WS_KERNEL = 8 };
-
-__device__ __forceinline__ bool timed_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int code,
-                                           long long& acc) {
-    if (mbar_try_wait(bar, parity)) return true;  // the common case costs no clock reads
-    const long long t0 = clock64();
-    const bool ok = mbar_wait(bar, parity, abort_flag, status, code);
-    acc += clock64() - t0;
-    return ok;
-}
-
-__device__ __forceinline__ void flush_wait(int* status, int slot, long long cycles) {
-    atomicAdd(reinterpret_cast<unsigned long long*>(status) + slot, static_cast<unsigned long long>(cycles));
-}
-
-// Two fp32 values in one 64-bit register pair (sm_100 has packed fp32 arithmetic on such pairs).
-__device__ __forceinline__ uint64_t pack_u32x2(uint32_t lo, uint32_t hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-    return r;
-}
-__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) { return pack_u32x2(__float_as_uint(lo), __float_as_uint(hi)); }
-__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi) {
-    uint32_t a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
-    lo = __uint_as_float(a);
-    hi = __uint_as_float(b);
-}
-__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {  // round to nearest even, per element
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
-// Four weight codes as the bytes the MMA reads: the sign-magnitude bytes themselves (E4M3 path) or, in the integer-path
-// build, their two's complement (per byte: (m ^ s) - s with s = 0xFF where the sign bit is set).
-__device__ __forceinline__ uint32_t code_bytes(uint32_t v) {
-    if constexpr (!kI8Path) {
-        return v;
-    } else {
-        const uint32_t sg = ((v >> 7) & 0x01010101u) * 0xFFu;
-        return __vsub4((v & 0x07070707u) ^ sg, sg);
-    }
-}
-
-__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {  // round to nearest even, per element
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-    __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<uint32_t*>(&v);
-}
-
-template <int G, bool kPartials, int BN, bool SPLITK = false>
+template <int G, bool kPartials, int BN>
 __global__ void __launch_bounds__(Plan<BN>::THREADS, 1)
 w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_constant__ CUtensorMap tmap_wpacked,
                  const __grid_constant__ CUtensorMap tmap_wscale, const __grid_constant__ CUtensorMap tmap_xscale,
                  const __grid_constant__ CUtensorMap tmap_xh, const __grid_constant__ CUtensorMap tmap_wh,
                  const GemmKernelParams p) {
-    using P = Plan<BN, SPLITK>;
-    static_assert(!SPLITK || !kPartials, "the debug export runs unsplit");
+    using P = Plan<BN>;
     constexpr int STAGES = P::STAGES, STAGE_BYTES = P::STAGE_BYTES, BU_BYTES = P::BU_BYTES, BP_BYTES = P::BP_BYTES;
     constexpr int SC_SW_BYTES = P::SC_SW_BYTES, SC_BYTES = P::SC_BYTES, BAR_OFFSET = P::BAR_OFFSET;
     constexpr int SC_SLOTS = P::SC_SLOTS, NUM_EPI_WARPS = P::EPI_WARPS;
@@ -182,7 +87,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     constexpr int CHUNKS = HB / 32;    // 32-column chunks per epilogue warp and accumulator tile
     constexpr int GPK = BKC / G;       // groups per k-block: 2 (G = 64) or 1 (G = 128)
     constexpr int MMA_PER_G = G / 32;  // 8-bit MMA instructions (K = 32) per group
-    constexpr int NBUF = BN == 64 ? 4 : 512 / BN;  // accumulator tiles in tensor memory: 2 of 256 columns, 4 of 128 or of 64 (the barrier map has four slots)
+    constexpr int NBUF = 512 / BN;     // accumulator tiles in tensor memory: 2 of 256 columns, 4 of 128 (the barrier map has four slots)
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -211,22 +116,6 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     const int num_m_blocks = (p.M + BM - 1) / BM;
     const int num_n_blocks = (p.N + BN - 1) / BN;
     const int num_tiles = num_m_blocks * num_n_blocks;
-    // Split plan: this CTA's range of k-blocks [kb0, kb1) and of K-groups [g0, g1) of the cluster's tile (the first ranks take
-    // one k-block more when the division leaves a rest); the LAST rank gathers the partial tiles and has the rank-r branch.
-    // (Without the split every one of these is the constant or the parameter it stands for.)
-    const uint32_t csize = SPLITK ? cluster_nctarank() : 1u, crank = SPLITK ? cluster_ctarank() : 0u;
-    const bool gathers = !SPLITK || crank == csize - 1;
-    const int split_base = SPLITK ? p.num_kb / static_cast<int>(csize) : 0, split_rest = SPLITK ? p.num_kb % static_cast<int>(csize) : 0;
-    const int kb0 = SPLITK ? static_cast<int>(crank) * split_base + min(static_cast<int>(crank), split_rest) : 0;
-    const int kb1 = SPLITK ? kb0 + split_base + (static_cast<int>(crank) < split_rest ? 1 : 0) : p.num_kb;
-    const int g0 = SPLITK ? kb0 * GPK : 0, g1 = SPLITK ? min(kb1 * GPK, p.n_g) : p.n_g;
-    const int lr_here = gathers ? p.lr_chunks : 0;
-    // (tile loops read these where they are needed, like blockIdx.x and gridDim.x themselves: held in registers across the
-    // roles' loops they cost the 256-column plan spills)
-    auto first_tile = [&]() { return SPLITK ? static_cast<int>(blockIdx.x / csize) : static_cast<int>(blockIdx.x); };
-    auto tile_stride = [&]() { return SPLITK ? static_cast<int>(gridDim.x / csize) : static_cast<int>(gridDim.x); };
-    const uint32_t red_bar = bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 9);  // split plan: "partial tiles landed" (last CTA)
-
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(full_bar(s), 1);
@@ -242,11 +131,6 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             mbar_init(tempty_bar(a), NUM_EPI_WARPS * 32);
         }
         mbar_init(bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 8), 1);  // spare: see umma_drain
-        if constexpr (SPLITK) {
-            mbar_init(red_bar, 1);  // counts the bytes of the other CTAs' partial tiles
-            mbar_init(red_bar + 8u, 128);  // this CTA's partial tile is in its shared memory (every epilogue thread arrives)
-            if (gathers) mbar_arrive_expect_tx(red_bar, (csize - 1) * RED_BYTES);
-        }
         *abort_flag = 0;
         fence_mbar_init();
         tma_prefetch_desc(&tmap_codes);
@@ -262,7 +146,6 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     }
     tc_fence_before_sync();
     __syncthreads();
-    if constexpr (SPLITK) cluster_sync_all();  // the gathering CTA's barrier is initialised before anything arrives on it
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
     // everything above touched only this CTA's own shared and tensor memory; what follows reads the first kernel's output
@@ -273,7 +156,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     grid_launch_dependents();
 
     if (warp < 4) {
-        if constexpr (P::REPARTITION) reg_dealloc<P::AUX_REGS>();
+        reg_dealloc<P::AUX_REGS>();
 
         if (warp == 0) {
             // -------------------------------------------------------- TMA producer
@@ -283,10 +166,10 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 uint32_t it = 0, sc_it = 0;
                 long long w_empty = 0;
                 bool ok = true;
-                for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
+                for (int tile = static_cast<int>(blockIdx.x); ok && tile < num_tiles; tile += static_cast<int>(gridDim.x)) {
                     const int m0 = (tile % num_m_blocks) * BM;
                     const int n0 = (tile / num_m_blocks) * BN;
-                    for (int kb = kb0; kb < kb1; ++kb, ++it, ++sc_it) {
+                    for (int kb = 0; kb < p.num_kb; ++kb, ++it, ++sc_it) {
                         const int s = it % STAGES;
                         if (!timed_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER, w_empty)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
@@ -306,7 +189,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         }
                     }
                     if (!ok) break;
-                    for (int lr = 0; lr < lr_here; ++lr, ++it) {
+                    for (int lr = 0; lr < p.lr_chunks; ++lr, ++it) {
                         const int s = it % STAGES;
                         if (!mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
@@ -353,13 +236,13 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 long long w_ops = 0, w_tempty = 0;
                 const long long t_kernel = clock64();
                 bool ok = true;
-                for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
-                    int groups_left = g1 - g0;
-                    for (int kb = kb0; ok && kb < kb1; ++kb) {
+                for (int tile = static_cast<int>(blockIdx.x); ok && tile < num_tiles; tile += static_cast<int>(gridDim.x)) {
+                    int groups_left = p.n_g;
+                    for (int kb = 0; ok && kb < p.num_kb; ++kb) {
                         // the unpack warps arrive after they have seen the stage's loads land (one barrier for both operands), so
                         // their barrier covers the activation codes as well
                         if (!timed_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_ops)) { ok = false; break; }
-                        if (lane == 0) { if (kb == kb0) TRACE_CLK(p.status, 16); if (kb == 4) TRACE_CLK(p.status, 17); if (kb == kb1 - 1) TRACE_CLK(p.status, 18); }
+                        if (lane == 0) { if (kb == 0) TRACE_CLK(p.status, 16); if (kb == 4) TRACE_CLK(p.status, 17); if (kb == p.num_kb - 1) TRACE_CLK(p.status, 18); }
                         tc_fence_after_sync();
                         const uint32_t a_lo = desc_lo0 + s * (STAGE_BYTES >> 4), b_lo = a_lo + (A_BYTES >> 4);
 #pragma unroll
@@ -387,11 +270,10 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         if (++s == STAGES) { s = 0; ph ^= 1; }
                     }
                     if (!ok) break;
-                    if (SPLITK && lr_here == 0) continue;  // split plan: only the gathering CTA has the rank-r branch
                     // rank-r bf16 branch: one more accumulator tile, fp32
                     if (!mbar_wait(tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                     tc_fence_after_sync();
-                    for (int lr = 0; lr < lr_here; ++lr) {
+                    for (int lr = 0; lr < p.lr_chunks; ++lr) {
                         if (!mbar_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                         tc_fence_after_sync();
                         const uint32_t a_lo = desc_lo0 + s * (STAGE_BYTES >> 4), b_lo = a_lo + (A_BYTES >> 4);
@@ -420,14 +302,14 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             uint32_t it = 0;
             long long w_full = 0;
             bool ok = true;
-            for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
-                const int items = (kb1 - kb0) + lr_here;
+            for (int tile = static_cast<int>(blockIdx.x); ok && tile < num_tiles; tile += static_cast<int>(gridDim.x)) {
+                const int items = p.num_kb + p.lr_chunks;
                 for (int i = 0; i < items; ++i, ++it) {
                     const int s = it % STAGES;
                     ok = timed_wait(full_bar(s), (it / STAGES) & 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK, w_full);
                     if (!ok) break;
                     if (it == 0 && u == 0) TRACE_CLK(p.status, 14);
-                    if (i < kb1 - kb0) {
+                    if (i < p.num_kb) {
                         // 16-byte piece idx = u + 64 j of the packed tile: row = idx/4 = u/4 + 16 j, piece c = u%4.
                         // The swizzle phase row%8 = (u/4)%8 and the piece do not depend on j, so every address is
                         // a per-thread base plus a compile-time offset.
@@ -469,7 +351,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             if (u == 0) flush_wait(p.status, WS_UNPACK_FULL, w_full);
         }
     } else {
-        if constexpr (P::REPARTITION) reg_alloc<P::EPI_REGS>();
+        reg_alloc<P::EPI_REGS>();
         // ------------------------------------------------------------ epilogue (warps 4..11)
         // A warp owns 32 token rows (its TMEM lane quadrant) x BN/2 columns.  The accumulators are read with the
         // 16x256b shape: a thread then holds 4 rows (l/4 + 8 i) x the column pairs 2 (l%4) + {0, 1} of every block
@@ -505,7 +387,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             tc_fence_before_sync();
             mbar_arrive(tempty_bar(buf));  // all lanes arrive (see the unpack warps' note on the cost of electing one)
         };
-        for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
+        for (int tile = static_cast<int>(blockIdx.x); ok && tile < num_tiles; tile += static_cast<int>(gridDim.x)) {
             const int m0 = (tile % num_m_blocks) * BM;
             const int n0 = (tile / num_m_blocks) * BN;
             const int rbase = m0 + q * 32 + lr4;  // this thread's rows: rbase + 8 i, i = 0..3
@@ -514,18 +396,15 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
 #pragma unroll
             for (int j = 0; j < HB / 2; ++j) acc2[j] = 0ull;
 
-            // first scales and first accumulator tile of this output tile (split plan: of this CTA's range, which may be
-            // empty, and only the gathering CTA has a rank-r tile)
-            if (!SPLITK || g1 > g0) ok = timed_wait(scfull_bar(slot), sph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_sc);
-            if (!SPLITK || g1 > g0 || lr_here > 0) {
-                ok = ok && timed_wait(tfull_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
-                if (!ok) break;
-                if (warp == 4 && lane == 0) TRACE_CLK(p.status, 20);
-                tc_fence_after_sync();
-                request_chunk(b, 0, raw[0]);
-            }
+            // first scales and first accumulator tile of this output tile
+            ok = timed_wait(scfull_bar(slot), sph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_sc) &&
+                 timed_wait(tfull_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
+            if (!ok) break;
+            if (warp == 4 && lane == 0) TRACE_CLK(p.status, 20);
+            tc_fence_after_sync();
+            request_chunk(b, 0, raw[0]);
 
-            for (int g = g0; g < g1; ++g) {
+            for (int g = 0; g < p.n_g; ++g) {
                 if (warp == 4 && lane == 0 && g == 8) TRACE_CLK(p.status, 21);
                 const int gi = g & (GPK - 1);
                 const bool last_of_kb = gi == GPK - 1 || g == p.n_g - 1;
@@ -542,8 +421,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 // what comes after this tile: the next group's, or the rank-r tile
                 const uint32_t nb = b + 1 == NBUF ? 0 : b + 1, nbph = b + 1 == NBUF ? bph ^ 1 : bph;
                 const uint32_t nslot = slot + 1 == SC_SLOTS ? 0 : slot + 1, nsph = slot + 1 == SC_SLOTS ? sph ^ 1 : sph;
-                const bool new_scales = last_of_kb && g + 1 < g1;
-                const bool more = !SPLITK || g + 1 < g1 || lr_here > 0;  // another accumulator tile follows (always, unless split)
+                const bool new_scales = last_of_kb && g + 1 < p.n_g;
                 bool ahead = false;
 #pragma unroll
                 for (int c = 0; c < CHUNKS; ++c) {
@@ -566,7 +444,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     } else {
                         // the whole tile is in registers: hand it back to the MMA warp, and look at the next one
                         release_tile(b);
-                        ahead = more && mbar_test_wait(tfull_bar(nb), nbph) && (!new_scales || mbar_test_wait(scfull_bar(nslot), nsph));
+                        ahead = mbar_test_wait(tfull_bar(nb), nbph) && (!new_scales || mbar_test_wait(scfull_bar(nslot), nsph));
                         if (ahead) {
                             tc_fence_after_sync();
                             request_chunk(nb, 0, raw[0]);  // CHUNKS is even: the last chunk sits in raw[1]
@@ -612,7 +490,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 }
                 b = nb;
                 bph = nbph;
-                if (!ahead && more) {
+                if (!ahead) {
                     if (new_scales) ok = timed_wait(scfull_bar(slot), sph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_sc);
                     ok = ok && timed_wait(tfull_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
                     if (!ok) break;
@@ -623,51 +501,24 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             if (!ok) break;
             if (warp == 4 && lane == 0) TRACE_CLK(p.status, 22);
             // rank-r branch: an fp32 tile whose first chunk is already on its way
-            if (!SPLITK || lr_here > 0) {
 #pragma unroll
-                for (int c = 0; c < CHUNKS; ++c) {
-                    uint32_t (&cur)[32] = raw[c & 1];
-                    tmem_ld_wait();
-                    tmem_ld_fence(cur);
-                    if (c < CHUNKS - 1) request_chunk(b, c + 1, raw[(c + 1) & 1]);
-                    else release_tile(b);
+            for (int c = 0; c < CHUNKS; ++c) {
+                uint32_t (&cur)[32] = raw[c & 1];
+                tmem_ld_wait();
+                tmem_ld_fence(cur);
+                if (c < CHUNKS - 1) request_chunk(b, c + 1, raw[(c + 1) & 1]);
+                else release_tile(b);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < 4; ++i)
 #pragma unroll
-                        for (int cb = 0; cb < 4; ++cb) {
-                            const int pidx = 16 * (i >> 1) + 4 * cb + 2 * (i & 1);
-                            const int a = (c * 4 + cb) * 4 + i;
-                            acc2[a] = add_f32x2(acc2[a], pack_u32x2(cur[pidx], cur[pidx + 1]));
-                        }
-                }
-                if (++b == NBUF) { b = 0; bph ^= 1; }
+                    for (int cb = 0; cb < 4; ++cb) {
+                        const int pidx = 16 * (i >> 1) + 4 * cb + 2 * (i & 1);
+                        const int a = (c * 4 + cb) * 4 + i;
+                        acc2[a] = add_f32x2(acc2[a], pack_u32x2(cur[pidx], cur[pidx + 1]));
+                    }
             }
+            if (++b == NBUF) { b = 0; bph ^= 1; }
             if (warp == 4 && lane == 0) TRACE_CLK(p.status, 23);
-            if constexpr (SPLITK) {
-                // The partial tiles meet in the last CTA of the cluster.  Every other CTA's epilogue threads put their 32
-                // register pairs into their own shared memory (the operand ring, idle by now: every MMA of this CTA has
-                // completed), word j of thread t at [j][t]; one thread then sends the 32 KB to the gathering CTA with a bulk
-                // copy that counts its bytes on that CTA's barrier.  The gathering thread t holds the same rows and columns
-                // in every CTA and adds the partial tiles in rank order.
-                const uint32_t et = threadIdx.x - 128u;
-                const uint32_t red_base = smem_base + P::RED_OFFSET;
-                if (!gathers) {
-#pragma unroll
-                    for (int j = 0; j < HB / 2; ++j) st_shared_u64(smem_base + j * 1024u + et * 8u, acc2[j]);
-                    fence_proxy_async_smem();       // these writes -> visible to the copy engine
-                    mbar_arrive(red_bar + 8u);
-                    if (et == 0 && mbar_wait(red_bar + 8u, 0, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE))  // a bounded wait, like all
-                        bulk_copy_to_cluster(map_to_cta(red_base + crank * RED_BYTES, csize - 1), smem_base, RED_BYTES,
-                                             map_to_cta(red_bar, csize - 1));
-                    continue;  // one tile per cluster: nothing else to do (the cluster meets once more before anyone leaves)
-                }
-                if (!mbar_wait(red_bar, 0, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE)) { ok = false; break; }
-                for (uint32_t r = 0; r + 1 < csize; ++r) {
-#pragma unroll
-                    for (int j = 0; j < HB / 2; ++j)
-                        acc2[j] = add_f32x2(acc2[j], ld_shared_u64(red_base + r * RED_BYTES + j * 1024u + et * 8u));
-                }
-            }
             if constexpr (!kPartials) {
                 // A lane holds 2 of the 8 columns of every block; four blocks are transposed inside the quad of lanes
                 // (two exchange steps) so that each lane ends up with all 8 columns = 16 bytes of one block and the
@@ -718,28 +569,14 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     if (warp == 1 && lane == 0 && *abort_flag != 0) umma_drain(bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 8));  // a wait gave up: let issued MMAs finish first
     tc_fence_before_sync();
     __syncthreads();
-    if constexpr (SPLITK) cluster_sync_all();  // no CTA of the cluster leaves while another may still write into it or signal it
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem_base, 512);
     }
 }
 
-// A 128-column tile takes 0.70-0.76 of the time of a 256-column one (measured: the activation tile, the rank-r
-// branch, the pipeline fill and the per-group hand-over are paid per tile whatever its width), so narrow tiles are
-// chosen only when they shorten the schedule by more than that: when the wide tiles' last wave would be nearly
-// empty (PixArt-sized layers, N = 1152: 160 wide tiles on 148 SMs) or when there are fewer wide tiles than SMs.
-static bool narrow_tiles_pay(int M, int N, int sms) {
-    const long m_blocks = (M + BM - 1) / BM;
-    const long wide = m_blocks * ((N + 255) / 256), narrow = m_blocks * ((N + 127) / 128);
-    const double cost_wide = static_cast<double>((wide + sms - 1) / sms);
-    const double cost_narrow = 0.73 * static_cast<double>((narrow + sms - 1) / sms);
-    return cost_narrow < 0.98 * cost_wide;
-}
-
-// split: 0 = one CTA per tile; 2..SPLIT_MAX = the split plan with clusters of that many CTAs (BN = 64, no debug export)
 template <int BN>
-static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream, int split = 0) {
+static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream) {
     const Geometry& g = L->geo;
     CUtensorMap tmap_codes, tmap_xscale, tmap_xh;
     dirotq_status_t st;
@@ -770,23 +607,12 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
     else           kern = dbg ? w4a4_gemm_kernel<128, true, BN> : w4a4_gemm_kernel<128, false, BN>;
     static SmemOptIn<4> opt_in;  // one per instantiation of this launcher, i.e. per tile width
     const int vi = (g.G == 64 ? 0 : 2) + (dbg ? 1 : 0);
-    if constexpr (BN == 64) {
-        if (split >= 2 && !dbg) {
-            const KernelFn ks = g.G == 64 ? w4a4_gemm_kernel<64, false, 64, true> : w4a4_gemm_kernel<128, false, 64, true>;
-            static SmemOptIn<2> opt_in_split;
-            if (!opt_in_split.ensure(ks, g.G == 64 ? 0 : 1, L->device, Plan<64, true>::SMEM_BYTES)) return DIROTQ_ERR_CUDA;
-            const cudaError_t es = launch_kernel_clusters(ks, num_tiles * split, split, Plan<64>::THREADS, Plan<64, true>::SMEM_BYTES,
-                                                          stream, true, tmap_codes, L->tmap_wpacked64, L->tmap_wscale64, tmap_xscale,
-                                                          tmap_xh, L->tmap_wh64, p);
-            return es == cudaSuccess ? DIROTQ_OK : DIROTQ_ERR_CUDA;
-        }
-    }
     if (!opt_in.ensure(kern, vi, L->device, Plan<BN>::SMEM_BYTES)) return DIROTQ_ERR_CUDA;
     const cudaError_t err = launch_kernel(kern, grid, Plan<BN>::THREADS, Plan<BN>::SMEM_BYTES, stream, true, tmap_codes,
-                                          BN == 64 ? L->tmap_wpacked64 : BN == 128 ? L->tmap_wpacked128 : BN == 192 ? L->tmap_wpacked192 : L->tmap_wpacked,
-                                          BN == 64 ? L->tmap_wscale64 : BN == 128 ? L->tmap_wscale128 : BN == 192 ? L->tmap_wscale192 : L->tmap_wscale,
+                                          BN == 128 ? L->tmap_wpacked128 : BN == 192 ? L->tmap_wpacked192 : L->tmap_wpacked,
+                                          BN == 128 ? L->tmap_wscale128 : BN == 192 ? L->tmap_wscale192 : L->tmap_wscale,
                                           tmap_xscale, tmap_xh,
-                                          BN == 64 ? L->tmap_wh64 : BN == 128 ? L->tmap_wh128 : BN == 192 ? L->tmap_wh192 : L->tmap_wh, p);
+                                          BN == 128 ? L->tmap_wh128 : BN == 192 ? L->tmap_wh192 : L->tmap_wh, p);
     return err == cudaSuccess ? DIROTQ_OK : DIROTQ_ERR_CUDA;
 }
 
@@ -801,43 +627,17 @@ dirotq_status_t set_w4a4_tile_columns(int columns) {
 }
 
 dirotq_status_t launch_w4a4_gemm(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream) {
-    const int forced = g_tile_columns.load();
-    if (forced == 192) return launch_w4a4_gemm_bn<192>(L, a, stream);
-    // few token rows: when even 128-column tiles would keep fewer than half of the SMs busy, 64-column tiles on twice as many
-    const int sms = sm_count(L->device);
-    const long t128 = static_cast<long>((a.M + BM - 1) / BM) * ((L->geo.N + 127) / 128);
-    if (forced == 64 || forced == 66 || (forced == 0 && 2 * t128 <= sms)) {
-        // The split plan: the largest cluster (4, 3 or 2 CTAs over the k-blocks of a tile) that leaves every CTA at least two
-        // k-blocks and whose clusters, one per tile, are all resident at once (asked of the runtime once per device and size).
-        // Only on request (knob value 66): the partial tiles are added in another order than one CTA adds the groups, and by
-        // default a token's output bits do not depend on how many other tokens the call has.  Measured on the 1152 -> 1152 layer
-        // at M = 256: 14.5 against 15.1 us per layer in graph replay.
-        int split = 0;
-        if (forced == 66 && a.partials == nullptr) {
-            const long t64 = static_cast<long>((a.M + BM - 1) / BM) * ((L->geo.N + 63) / 64);
-            const int num_kb = (L->geo.K_lp + BKC - 1) / BKC;
-            static std::atomic<int> resident[64][SPLIT_MAX + 1];  // 0: not asked yet; else clusters resident at once + 1
-            for (int c = SPLIT_MAX; c >= 2 && split == 0; --c) {
-                if (num_kb / c < 2) continue;
-                const int dev = L->device;
-                int have = dev >= 0 && dev < 64 ? resident[dev][c].load() : 0;
-                if (have == 0) {
-                    // (the question needs the kernel's shared-memory limit raised first; both group sizes have the same footprint)
-                    if (cudaFuncSetAttribute(w4a4_gemm_kernel<64, false, 64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             Plan<64, true>::SMEM_BYTES) != cudaSuccess) {
-                        cudaGetLastError();
-                        break;
-                    }
-                    have = 1 + max_active_clusters(w4a4_gemm_kernel<64, false, 64, true>, c, Plan<64>::THREADS, Plan<64, true>::SMEM_BYTES);
-                    if (dev >= 0 && dev < 64) resident[dev][c].store(have);
-                }
-                if (t64 <= have - 1) split = c;
-            }
-        }
-        return launch_w4a4_gemm_bn<64>(L, a, stream, split);
-    }
-    const bool narrow = forced ? forced == 128 : narrow_tiles_pay(a.M, L->geo.N, sm_count(L->device));
-    return narrow ? launch_w4a4_gemm_bn<128>(L, a, stream) : launch_w4a4_gemm_bn<256>(L, a, stream);
+    // The plan with the shortest schedule: turns of the SMs x what one tile of the plan costs.  Costs relative to a 256-column tile, from
+    // the cycles per 128 codes of a tile: 2360, 1390 and 780 with groups of 64, 1600, 990 and 620 with groups of 128 (the
+    // activation tile, the rank-r branch, the pipeline fill and the hand-overs are paid per tile whatever its width).
+    const int forced = g_tile_columns.load(), sms = sm_count(L->device);
+    const long m_blocks = (a.M + BM - 1) / BM;
+    auto turns = [&](int columns) { return static_cast<double>((m_blocks * ((L->geo.N + columns - 1) / columns) + sms - 1) / sms); };
+    const double c256 = turns(256), c128 = (L->geo.G == 64 ? 0.60 : 0.64) * turns(128), c64 = (L->geo.G == 64 ? 0.34 : 0.40) * turns(64);
+    const int plan = forced ? forced : c64 <= c128 && c64 <= c256 ? 64 : c128 < c256 ? 128 : 256;
+    if (a.partials == nullptr && (plan == 64 || plan == 66)) return launch_w4a4_narrow(L, a, plan == 66, stream);
+    if (plan == 192) return launch_w4a4_gemm_bn<192>(L, a, stream);
+    return plan == 256 ? launch_w4a4_gemm_bn<256>(L, a, stream) : launch_w4a4_gemm_bn<128>(L, a, stream);
 }
 
 }  // namespace dirotq
