@@ -43,36 +43,64 @@ __device__ __forceinline__ double load_w(const void* W, int w_dtype, int w_layou
                                        : bf16_to_f64(static_cast<const uint16_t*>(W)[i]);
 }
 
-// Wt[i][n] = sum_k Q[k][i] * W[k][n]     (64 x 64 output tile, 4 x 4 per thread, fp64)
-__global__ void __launch_bounds__(256) fold_kernel(const void* Q, int q_dtype, const void* W, int w_dtype, int w_layout,
-                                                   double* Wt, int K, int N) {
-    __shared__ double sq[16][64 + 1];
-    __shared__ double sw[16][64 + 1];
+// Wt[i][n] = sum_k Q[k][i] * W[k][n] in fp64, k ascending: 128 x 64 output tile, 8 x 4 per thread.
+// Bound by the fp64 multiply-adds (16 lanes per scheduler: a warp's 32 of one k take 64 cycles), which needs few shared-memory
+// loads per multiply-add (six 16-byte loads per 32; with 4 x 4 per thread and scalar loads, eight per 16, the loads set the time)
+// and the next tile's global loads, 12 per thread, in flight under them.  1152 -> 4608: 1463 us with the 4 x 4 tile.
+constexpr int FOLD_I = 128, FOLD_N = 64, FOLD_K = 16;
+__global__ void __launch_bounds__(256, 2) fold_kernel(const void* Q, int q_dtype, const void* W, int w_dtype, int w_layout,
+                                                      double* Wt, int K, int N) {
+    __shared__ __align__(16) double sq[FOLD_K][FOLD_I + 2];
+    __shared__ __align__(16) double sw[FOLD_K][FOLD_N + 2];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int i0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    double acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-            const int kk = e >> 6, c = e & 63;
-            sq[kk][c] = (i0 + c < K) ? load_q(Q, q_dtype, K, k0 + kk, i0 + c) : 0.0;
-            sw[kk][c] = (n0 + c < N) ? load_w(W, w_dtype, w_layout, K, N, k0 + kk, n0 + c) : 0.0;
+    const int i0 = blockIdx.y * FOLD_I, n0 = blockIdx.x * FOLD_N;
+    // this thread's elements of the two input tiles: along the contiguous index of each
+    const int qc = threadIdx.x & 127, qk = threadIdx.x >> 7;  // Q: k = qk + 2 u
+    const bool kn = w_layout == DIROTQ_LAYOUT_KN;
+    const int wc = kn ? threadIdx.x & 63 : threadIdx.x >> 4, wk = kn ? threadIdx.x >> 6 : threadIdx.x & 15;  // W: k = wk + 4 u, or n = wc + 16 u
+    double rq[8], rw[4];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) rq[u] = i0 + qc < K ? load_q(Q, q_dtype, K, k0 + qk + 2 * u, i0 + qc) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int n = n0 + wc + (kn ? 0 : 16 * u), k = k0 + wk + (kn ? 4 * u : 0);
+            rw[u] = n < N ? load_w(W, w_dtype, w_layout, K, N, k, n) : 0.0;
         }
+    };
+    double acc[8][4] = {};
+    fetch(0);
+    for (int k0 = 0; k0 < K; k0 += FOLD_K) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) sq[qk + 2 * u][qc] = rq[u];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) sw[wk + (kn ? 4 * u : 0)][wc + (kn ? 0 : 16 * u)] = rw[u];
         __syncthreads();
+        if (k0 + FOLD_K < K) fetch(k0 + FOLD_K);
+#pragma unroll 4
+        for (int kk = 0; kk < FOLD_K; ++kk) {
+            double2 a[4], b[2];
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            double a[4], b[4];
+            for (int u = 0; u < 4; ++u) a[u] = *reinterpret_cast<const double2*>(&sq[kk][ty * 8 + 2 * u]);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) { a[u] = sq[kk][ty * 4 + u]; b[u] = sw[kk][tx * 4 + u]; }
+            for (int v = 0; v < 2; ++v) b[v] = *reinterpret_cast<const double2*>(&sw[kk][tx * 2 + 32 * v]);
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
+                for (int v = 0; v < 2; ++v) {
+                    acc[2 * u][2 * v] = fma(a[u].x, b[v].x, acc[2 * u][2 * v]);
+                    acc[2 * u][2 * v + 1] = fma(a[u].x, b[v].y, acc[2 * u][2 * v + 1]);
+                    acc[2 * u + 1][2 * v] = fma(a[u].y, b[v].x, acc[2 * u + 1][2 * v]);
+                    acc[2 * u + 1][2 * v + 1] = fma(a[u].y, b[v].y, acc[2 * u + 1][2 * v + 1]);
+                }
         }
         __syncthreads();
     }
-    for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const int i = i0 + ty * 4 + u, n = n0 + tx * 4 + v;
+            const int i = i0 + ty * 8 + u, n = n0 + tx * 2 + 32 * (v >> 1) + (v & 1);
             if (i < K && n < N) Wt[static_cast<size_t>(i) * N + n] = acc[u][v];
         }
 }
@@ -81,7 +109,6 @@ __host__ __device__ __forceinline__ int packed_byte_index(int k) {  // byte of c
     const int w = k & 31;
     return (k >> 5) * 16 + (w >> 3) * 4 + (w & 3);
 }
-__host__ __device__ __forceinline__ int packed_is_high(int k) { return (k >> 2) & 1; }
 
 // One thread per (group, output column): Eq. 1 with z = 0, s = bf16(max|w|/7), ties to even.
 __global__ void quantize_weights_kernel(const double* Wt, uint8_t* wpacked, float* wscale, uint16_t* wh, Geometry g) {
@@ -162,12 +189,16 @@ __global__ void pack_codes_kernel(const int8_t* codes, const uint16_t* scales, u
     }
 }
 
-// wh[n][i] = bf16(Wt[i][n]) for i < r, zero up to r_pad.
+// wh[n][i] = bf16(Wt[i][n]) for i < r, zero up to r_pad: eight rows i per thread, one 16-byte store (one thread per column, all
+// rows in sequence, took 25 us for 32 rows of 4608 columns).
 __global__ void high_rows_kernel(const double* Wt, uint16_t* wh, Geometry g) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    const int n = blockIdx.x * blockDim.x + threadIdx.x, i0 = blockIdx.y * 8;
     if (n >= g.N) return;
-    for (int i = 0; i < g.r_pad; ++i)
-        wh[static_cast<size_t>(n) * g.r_pad + i] = i < g.r ? f64_to_bf16(Wt[static_cast<size_t>(i) * g.N + n]) : 0;
+    uint32_t w[4] = {};
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        if (i0 + u < g.r) w[u >> 1] |= static_cast<uint32_t>(f64_to_bf16(Wt[static_cast<size_t>(i0 + u) * g.N + n])) << (16 * (u & 1));
+    *reinterpret_cast<uint4*>(wh + static_cast<size_t>(n) * g.r_pad + i0) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 // qt[c'][k] = bf16(Q[k][col(c')]) with the low-precision columns first (tiled transpose).
@@ -195,18 +226,18 @@ __global__ void bias_kernel(const uint16_t* bias, float* out, int N) {
 
 // ---------------------------------------------------------------- exports (parity checks)
 
+// One thread per column and 32-bit word of eight codes.
 __global__ void export_wcodes_kernel(const uint8_t* wpacked, int8_t* wcodes, Geometry g) {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    if (n >= g.N || j >= g.K_l) return;
-    const uint8_t* row = wpacked + static_cast<size_t>(n) * (g.K_lp / 2);
-    if (g.fmt == 3) {  // W4A8: nibble = q + 8
-        const uint8_t byte = row[packed_byte_index(j)];
-        const int nib = packed_is_high(j) ? (byte >> 4) : (byte & 0xF);
-        wcodes[static_cast<size_t>(j) * g.N + n] = static_cast<int8_t>(nib - 8);
-    } else {           // grouped formats: sign + magnitude, see signmag_nibble_bits
-        const uint32_t word = *reinterpret_cast<const uint32_t*>(row + packed_byte_index(j & ~7));
-        wcodes[static_cast<size_t>(j) * g.N + n] = static_cast<int8_t>(signmag_nibble_decode(word, j & 7));
+    const int j0 = blockIdx.y * 8;
+    if (n >= g.N) return;
+    const uint32_t word = *reinterpret_cast<const uint32_t*>(wpacked + static_cast<size_t>(n) * (g.K_lp / 2) + packed_byte_index(j0));
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        if (j0 + t >= g.K_l) break;
+        // W4A8: nibble = q + 8; grouped formats: sign + magnitude, see signmag_nibble_bits
+        const int q = g.fmt == 3 ? static_cast<int>((word >> (8 * (t & 3) + 4 * (t >> 2))) & 0xFu) - 8 : signmag_nibble_decode(word, t);
+        wcodes[static_cast<size_t>(j0 + t) * g.N + n] = static_cast<int8_t>(q);
     }
 }
 
@@ -305,19 +336,24 @@ __global__ void debug_codes_kernel(const int8_t* in, uint8_t* out, float* xscale
 
 // ================================================================ W4A8 (paper Sec. 5.1: per-channel 4-bit weights, per-token 8-bit activations)
 
-// One thread per output column: Eq. 1 with z = 0 over the whole column (one scale per channel), codes packed like
-// the grouped format (nibble = q + 8).
-__global__ void w4a8_quantize_weights_kernel(const double* Wt, uint8_t* wpacked, float* wscale, Geometry g) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= g.N) return;
+// Eq. 1 with z = 0 over the whole column (one scale per channel), codes packed like the grouped format (nibble = q + 8).  A block
+// takes 32 columns, its 16 warps share the rows (one thread per column was a chain of 2 K loads: 1.9 ms for 3072 -> 9216).
+__global__ void __launch_bounds__(512) w4a8_quantize_weights_kernel(const double* Wt, uint8_t* wpacked, float* wscale, Geometry g) {
+    __shared__ double part[16][33];
+    const int n = blockIdx.x * 32 + threadIdx.x, y = threadIdx.y;
     const double* col = Wt + static_cast<size_t>(g.r) * g.N + n;
     double a = 0.0;
-    for (int j = 0; j < g.K_l; ++j) a = fmax(a, fabs(col[static_cast<size_t>(j) * g.N]));
+    if (n < g.N)
+        for (int j = y; j < g.K_l; j += 16) a = fmax(a, fabs(col[static_cast<size_t>(j) * g.N]));
+    part[y][threadIdx.x] = a;
+    __syncthreads();
+    for (int i = 0; i < 16; ++i) a = fmax(a, part[i][threadIdx.x]);
+    if (n >= g.N) return;
     const uint16_t sb = (a == 0.0) ? 0 : f64_to_bf16(a / 7.0);
     const double s = bf16_to_f64(sb);
-    wscale[n] = static_cast<float>(s);
+    if (y == 0) wscale[n] = static_cast<float>(s);
     uint8_t* row = wpacked + static_cast<size_t>(n) * (g.K_lp / 2);
-    for (int jb = 0; jb < g.K_lp; jb += 8) {
+    for (int jb = 8 * y; jb < g.K_lp; jb += 128) {
         uint32_t word = 0;
         for (int t = 0; t < 8; ++t) {
             const int j = jb + t;
@@ -552,14 +588,14 @@ dirotq_status_t launch_prepare(const dirotq_layer* L, const void* W, int w_dtype
                                cudaStream_t stream) {
     const Geometry& g = L->geo;
     char* blob = L->blob;
-    fold_kernel<<<dim3((g.N + 63) / 64, (g.K + 63) / 64), 256, 0, stream>>>(Q, q_dtype, W, w_dtype, w_layout, scratch,
+    fold_kernel<<<dim3((g.N + FOLD_N - 1) / FOLD_N, (g.K + FOLD_I - 1) / FOLD_I), 256, 0, stream>>>(Q, q_dtype, W, w_dtype, w_layout, scratch,
                                                                           g.K, g.N);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     // zero the packed codes first: slots of a ragged last group stay zero
     if (cudaMemsetAsync(blob + L->lay.off_wpacked, 0, static_cast<size_t>(g.N) * (g.K_lp / 2), stream) != cudaSuccess)
         return DIROTQ_ERR_CUDA;
     // the rank-r rows first (zero padded to r_pad), then the quantizer, which for fmt 2 fills its extra columns
-    high_rows_kernel<<<(g.N + 127) / 128, 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
+    high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     if (wcodes)
         pack_codes_kernel<<<dim3((g.N + 127) / 128, g.n_g), 128, 0, stream>>>(
@@ -712,7 +748,7 @@ dirotq_status_t launch_prepare_ph(const dirotq_layer* L, const void* W, int w_dt
     if (cudaMemsetAsync(blob + L->lay.off_wpacked, 0, static_cast<size_t>(g.N) * (g.K_lp / 2), stream) != cudaSuccess)
         return DIROTQ_ERR_CUDA;
     // scratch now holds [r + K][N]: the same shape the INT4 pipeline quantizes (rows < r in 16 bits, the rest in groups)
-    high_rows_kernel<<<(g.N + 127) / 128, 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
+    high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     quantize_weights_kernel<<<dim3((g.N + 127) / 128, g.n_g), 128, 0, stream>>>(
         scratch, reinterpret_cast<uint8_t*>(blob + L->lay.off_wpacked), reinterpret_cast<float*>(blob + L->lay.off_wscale),
@@ -735,7 +771,7 @@ dirotq_status_t launch_layer_export(const dirotq_layer* L, int8_t* wcodes, uint1
     const Geometry& g = L->geo;
     const char* blob = L->blob;
     if (wcodes) {
-        export_wcodes_kernel<<<dim3((g.N + 127) / 128, g.K_l), 128, 0, stream>>>(
+        export_wcodes_kernel<<<dim3((g.N + 127) / 128, (g.K_l + 7) / 8), 128, 0, stream>>>(
             reinterpret_cast<const uint8_t*>(blob + L->lay.off_wpacked), wcodes, g);
         if (!launch_ok()) return DIROTQ_ERR_CUDA;
     }
@@ -762,12 +798,12 @@ dirotq_status_t launch_prepare_w4a8(const dirotq_layer* L, const void* W, int w_
                                     int q_dtype, const void* bias, double* scratch, cudaStream_t stream) {
     const Geometry& g = L->geo;
     char* blob = L->blob;
-    fold_kernel<<<dim3((g.N + 63) / 64, (g.K + 63) / 64), 256, 0, stream>>>(Q, q_dtype, W, w_dtype, w_layout, scratch,
+    fold_kernel<<<dim3((g.N + FOLD_N - 1) / FOLD_N, (g.K + FOLD_I - 1) / FOLD_I), 256, 0, stream>>>(Q, q_dtype, W, w_dtype, w_layout, scratch,
                                                                           g.K, g.N);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
-    high_rows_kernel<<<(g.N + 127) / 128, 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
+    high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
-    w4a8_quantize_weights_kernel<<<(g.N + 127) / 128, 128, 0, stream>>>(
+    w4a8_quantize_weights_kernel<<<(g.N + 31) / 32, dim3(32, 16), 0, stream>>>(
         scratch, reinterpret_cast<uint8_t*>(blob + L->lay.off_wpacked), reinterpret_cast<float*>(blob + L->lay.off_wscale), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     rotation_kernel<<<dim3((g.K + 31) / 32, (g.K + 31) / 32), dim3(32, 8), 0, stream>>>(
@@ -840,7 +876,7 @@ dirotq_status_t launch_prepare_nvfp4(const dirotq_layer* L, const void* W, int w
     const Geometry& g = L->geo;
     char* blob = L->blob;
     Nvfp4Meta* meta = reinterpret_cast<Nvfp4Meta*>(blob + L->lay.off_meta);
-    fold_kernel<<<dim3((g.N + 63) / 64, (g.K + 63) / 64), 256, 0, stream>>>(Q, q_dtype, W, w_dtype, w_layout, scratch,
+    fold_kernel<<<dim3((g.N + FOLD_N - 1) / FOLD_N, (g.K + FOLD_I - 1) / FOLD_I), 256, 0, stream>>>(Q, q_dtype, W, w_dtype, w_layout, scratch,
                                                                           g.K, g.N);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     if (cudaMemsetAsync(meta, 0, 64, stream) != cudaSuccess) return DIROTQ_ERR_CUDA;
