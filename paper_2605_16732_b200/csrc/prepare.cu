@@ -47,34 +47,40 @@ __device__ __forceinline__ double load_w(const void* W, int w_dtype, int w_layou
 // Bound by the fp64 multiply-adds (16 lanes per scheduler: a warp's 32 of one k take 64 cycles), which needs few shared-memory
 // loads per multiply-add (six 16-byte loads per 32; with 4 x 4 per thread and scalar loads, eight per 16, the loads set the time)
 // and the next tile's global loads, 12 per thread, in flight under them.  1152 -> 4608: 1463 us with the 4 x 4 tile.
-constexpr int FOLD_I = 128, FOLD_N = 64, FOLD_K = 16;
-__global__ void __launch_bounds__(256, 2) fold_kernel(const void* Q, int q_dtype, const void* W, int w_dtype, int w_layout,
-                                                      double* Wt, int K, int N) {
+// The loads in flight are held as they come: converted at once, every tile waited for them (779 us).
+constexpr int FOLD_I = 128, FOLD_N = 64;
+__device__ __forceinline__ double to_f64(double v) { return v; }
+__device__ __forceinline__ double to_f64(float v) { return static_cast<double>(v); }
+__device__ __forceinline__ double to_f64(uint16_t v) { return bf16_to_f64(v); }
+template <typename TQ, typename TW, bool kn>
+__global__ void __launch_bounds__(256, 2) fold_kernel(const TQ* Q, const TW* W, double* Wt, int K, int N) {
+    constexpr int FOLD_K = sizeof(TQ) == 8 ? 8 : 16;  // (as many as the registers for a tile in flight allow)
     __shared__ __align__(16) double sq[FOLD_K][FOLD_I + 2];
     __shared__ __align__(16) double sw[FOLD_K][FOLD_N + 2];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int i0 = blockIdx.y * FOLD_I, n0 = blockIdx.x * FOLD_N;
     // this thread's elements of the two input tiles: along the contiguous index of each
     const int qc = threadIdx.x & 127, qk = threadIdx.x >> 7;  // Q: k = qk + 2 u
-    const bool kn = w_layout == DIROTQ_LAYOUT_KN;
-    const int wc = kn ? threadIdx.x & 63 : threadIdx.x >> 4, wk = kn ? threadIdx.x >> 6 : threadIdx.x & 15;  // W: k = wk + 4 u, or n = wc + 16 u
-    double rq[8], rw[4];
+    constexpr int WN = 256 / FOLD_K;
+    const int wc = kn ? threadIdx.x & 63 : threadIdx.x / FOLD_K, wk = kn ? threadIdx.x >> 6 : threadIdx.x % FOLD_K;  // W: k = wk + 4 u, or n = wc + WN u
+    TQ rq[FOLD_K / 2];
+    TW rw[FOLD_K / 4];
     auto fetch = [&](int k0) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) rq[u] = i0 + qc < K ? load_q(Q, q_dtype, K, k0 + qk + 2 * u, i0 + qc) : 0.0;
+        for (int u = 0; u < FOLD_K / 2; ++u) rq[u] = i0 + qc < K ? Q[static_cast<size_t>(k0 + qk + 2 * u) * K + i0 + qc] : TQ(0);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int n = n0 + wc + (kn ? 0 : 16 * u), k = k0 + wk + (kn ? 4 * u : 0);
-            rw[u] = n < N ? load_w(W, w_dtype, w_layout, K, N, k, n) : 0.0;
+        for (int u = 0; u < FOLD_K / 4; ++u) {
+            const int n = n0 + wc + (kn ? 0 : WN * u), k = k0 + wk + (kn ? 4 * u : 0);
+            rw[u] = n < N ? W[kn ? static_cast<size_t>(k) * N + n : static_cast<size_t>(n) * K + k] : TW(0);
         }
     };
     double acc[8][4] = {};
     fetch(0);
     for (int k0 = 0; k0 < K; k0 += FOLD_K) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) sq[qk + 2 * u][qc] = rq[u];
+        for (int u = 0; u < FOLD_K / 2; ++u) sq[qk + 2 * u][qc] = to_f64(rq[u]);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) sw[wk + (kn ? 4 * u : 0)][wc + (kn ? 0 : 16 * u)] = rw[u];
+        for (int u = 0; u < FOLD_K / 4; ++u) sw[wk + (kn ? 4 * u : 0)][wc + (kn ? 0 : WN * u)] = to_f64(rw[u]);
         __syncthreads();
         if (k0 + FOLD_K < K) fetch(k0 + FOLD_K);
 #pragma unroll 4
@@ -103,6 +109,26 @@ __global__ void __launch_bounds__(256, 2) fold_kernel(const void* Q, int q_dtype
             const int i = i0 + ty * 8 + u, n = n0 + tx * 2 + 32 * (v >> 1) + (v & 1);
             if (i < K && n < N) Wt[static_cast<size_t>(i) * N + n] = acc[u][v];
         }
+}
+
+template <typename TQ>
+bool launch_fold_q(const TQ* Q, const void* W, int w_dtype, int w_layout, double* Wt, int K, int N, cudaStream_t stream) {
+    const dim3 grid((N + FOLD_N - 1) / FOLD_N, (K + FOLD_I - 1) / FOLD_I);
+    const float* wf = static_cast<const float*>(W);
+    const uint16_t* wb = static_cast<const uint16_t*>(W);
+    const bool f32 = w_dtype == DIROTQ_DTYPE_F32;
+    if (w_layout == DIROTQ_LAYOUT_KN) {
+        if (f32) fold_kernel<TQ, float, true><<<grid, 256, 0, stream>>>(Q, wf, Wt, K, N);
+        else fold_kernel<TQ, uint16_t, true><<<grid, 256, 0, stream>>>(Q, wb, Wt, K, N);
+    } else {
+        if (f32) fold_kernel<TQ, float, false><<<grid, 256, 0, stream>>>(Q, wf, Wt, K, N);
+        else fold_kernel<TQ, uint16_t, false><<<grid, 256, 0, stream>>>(Q, wb, Wt, K, N);
+    }
+    return cudaGetLastError() == cudaSuccess;
+}
+bool launch_fold(const void* Q, int q_dtype, const void* W, int w_dtype, int w_layout, double* Wt, int K, int N, cudaStream_t stream) {
+    return q_dtype == DIROTQ_DTYPE_F64 ? launch_fold_q(static_cast<const double*>(Q), W, w_dtype, w_layout, Wt, K, N, stream)
+                                       : launch_fold_q(static_cast<const float*>(Q), W, w_dtype, w_layout, Wt, K, N, stream);
 }
 
 __host__ __device__ __forceinline__ int packed_byte_index(int k) {  // byte of code k inside its row
@@ -588,9 +614,7 @@ dirotq_status_t launch_prepare(const dirotq_layer* L, const void* W, int w_dtype
                                cudaStream_t stream) {
     const Geometry& g = L->geo;
     char* blob = L->blob;
-    fold_kernel<<<dim3((g.N + FOLD_N - 1) / FOLD_N, (g.K + FOLD_I - 1) / FOLD_I), 256, 0, stream>>>(Q, q_dtype, W, w_dtype, w_layout, scratch,
-                                                                          g.K, g.N);
-    if (!launch_ok()) return DIROTQ_ERR_CUDA;
+    if (!launch_fold(Q, q_dtype, W, w_dtype, w_layout, scratch, g.K, g.N, stream)) return DIROTQ_ERR_CUDA;
     // zero the packed codes first: slots of a ragged last group stay zero
     if (cudaMemsetAsync(blob + L->lay.off_wpacked, 0, static_cast<size_t>(g.N) * (g.K_lp / 2), stream) != cudaSuccess)
         return DIROTQ_ERR_CUDA;
@@ -798,9 +822,7 @@ dirotq_status_t launch_prepare_w4a8(const dirotq_layer* L, const void* W, int w_
                                     int q_dtype, const void* bias, double* scratch, cudaStream_t stream) {
     const Geometry& g = L->geo;
     char* blob = L->blob;
-    fold_kernel<<<dim3((g.N + FOLD_N - 1) / FOLD_N, (g.K + FOLD_I - 1) / FOLD_I), 256, 0, stream>>>(Q, q_dtype, W, w_dtype, w_layout, scratch,
-                                                                          g.K, g.N);
-    if (!launch_ok()) return DIROTQ_ERR_CUDA;
+    if (!launch_fold(Q, q_dtype, W, w_dtype, w_layout, scratch, g.K, g.N, stream)) return DIROTQ_ERR_CUDA;
     high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     w4a8_quantize_weights_kernel<<<(g.N + 31) / 32, dim3(32, 16), 0, stream>>>(
@@ -876,9 +898,7 @@ dirotq_status_t launch_prepare_nvfp4(const dirotq_layer* L, const void* W, int w
     const Geometry& g = L->geo;
     char* blob = L->blob;
     Nvfp4Meta* meta = reinterpret_cast<Nvfp4Meta*>(blob + L->lay.off_meta);
-    fold_kernel<<<dim3((g.N + FOLD_N - 1) / FOLD_N, (g.K + FOLD_I - 1) / FOLD_I), 256, 0, stream>>>(Q, q_dtype, W, w_dtype, w_layout, scratch,
-                                                                          g.K, g.N);
-    if (!launch_ok()) return DIROTQ_ERR_CUDA;
+    if (!launch_fold(Q, q_dtype, W, w_dtype, w_layout, scratch, g.K, g.N, stream)) return DIROTQ_ERR_CUDA;
     if (cudaMemsetAsync(meta, 0, 64, stream) != cudaSuccess) return DIROTQ_ERR_CUDA;
     if (cudaMemsetAsync(blob + L->lay.off_wscale, 0, wsf_bytes(g.N, g.nkb64p), stream) !=
         cudaSuccess)
