@@ -1,6 +1,8 @@
 // C ABI of libdirotq: argument validation, tensor-map construction, launch sequencing.
 #include "common.h"
 
+#include <algorithm>
+
 #include <atomic>
 
 #include <mutex>
@@ -692,7 +694,7 @@ namespace {
 struct HostPipe {
     bool ready = false;
     cudaStream_t h2d = nullptr, d2h = nullptr;
-    static constexpr int kMaxChunks = 8;
+    static constexpr int kMaxChunks = 32;
     cudaEvent_t start = nullptr, done = nullptr, copied[kMaxChunks] = {}, computed[kMaxChunks] = {};
 };
 std::mutex g_pipe_mutex;
@@ -730,9 +732,15 @@ dirotq_status_t dirotq_linear_host(const void* x_host, int M, const dirotq_layer
     // Token rows are independent: the call is cut into row chunks whose host-to-device copy, computation and
     // device-to-host copy overlap (copy engines in both directions + SMs).  The chunks' kernels run one after another on
     // `stream`, so they can share the workspace.
-    int chunks = M / 1024;
-    if (chunks > HostPipe::kMaxChunks) chunks = HostPipe::kMaxChunks;
-    if (chunks <= 1) {
+    // A chunk is about 8 MB of the larger side (smaller ones pay more for starting copies, about 15 us each, and, with few rows, more per
+    // row for the kernels), but a good quarter of a short call, and at least 256 rows.  The first one and the last ones are
+    // shorter: the first copy in, and the last rows' computation and copy out, overlap with nothing.  4608 x 3072 -> 3072: 915 us
+    // in four equal chunks, 850 tapered; 1024 x 3072 -> 3072 311 us in one piece, 236 in chunks.
+    constexpr size_t CHUNK_BYTES = 8u << 20;
+    auto rows128 = [](long rows) { return (rows + 127) / 128 * 128; };
+    long base = static_cast<long>(CHUNK_BYTES / (xrow > yrow ? xrow : yrow));
+    base = rows128(std::max(std::min(base, M * 10L / 37), std::max(256L, M / 24L)));  // (at most kMaxChunks in all)
+    if (M < 512) {
         cudaError_t e = cudaMemcpyAsync(x_dev, x_host, xrow * M, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) { set_error("cudaMemcpyAsync(H2D)", e); return DIROTQ_ERR_CUDA; }
         st = dirotq_linear(x_dev, M, layer, y_dev, workspace, workspace_bytes, stream);
@@ -745,13 +753,13 @@ dirotq_status_t dirotq_linear_host(const void* x_host, int M, const dirotq_layer
     HostPipe* p = nullptr;
     st = host_pipe(layer->device, &p);
     if (st != DIROTQ_OK) return st;
-    const int rows_per_chunk = ((M + chunks - 1) / chunks + 127) / 128 * 128;
     cudaError_t e = cudaEventRecord(p->start, s);  // the staging buffers may still be in use by earlier work on `stream`
     if (e == cudaSuccess) e = cudaStreamWaitEvent(p->h2d, p->start, 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(p->d2h, p->start, 0);
     int c = 0;
-    for (int m0 = 0; m0 < M && e == cudaSuccess; m0 += rows_per_chunk, ++c) {
-        const int mc = M - m0 < rows_per_chunk ? M - m0 : rows_per_chunk;
+    for (int m0 = 0, mc = 0; m0 < M && e == cudaSuccess; m0 += mc, ++c) {
+        const long left = M - m0;
+        mc = static_cast<int>(left <= std::max(384L, 2 * base / 5) ? left : std::max(256L, std::min(rows128(3 * left / 5), m0 ? base : rows128(3 * base / 5))));
         char* xd = static_cast<char*>(x_dev) + xrow * m0;
         char* yd = static_cast<char*>(y_dev) + yrow * m0;
         e = cudaMemcpyAsync(xd, static_cast<const char*>(x_host) + xrow * m0, xrow * mc, cudaMemcpyHostToDevice, p->h2d);
