@@ -650,17 +650,19 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 } else if constexpr (FMT == 2) {
                     if (nlow > 0) {
                         // asymmetric: z = bf16(min), s = bf16((max - min) / 15) over the group's real elements
-                        float lo = v[0], hi = v[0];
+                        // (two chains each instead of one of G dependent instructions)
+                        float lo2[2] = {v[0], v[1]}, hi2[2] = {v[0], v[1]};
 #pragma unroll
                         for (int b = 0; b < G / 16; ++b) {
                             if (16 * b < nlow) {
 #pragma unroll
                                 for (int j = 0; j < 16; ++j) {
-                                    lo = fminf(lo, v[16 * b + j]);
-                                    hi = fmaxf(hi, v[16 * b + j]);
+                                    lo2[j & 1] = fminf(lo2[j & 1], v[16 * b + j]);
+                                    hi2[j & 1] = fmaxf(hi2[j & 1], v[16 * b + j]);
                                 }
                             }
                         }
+                        const float lo = fminf(lo2[0], lo2[1]), hi = fmaxf(hi2[0], hi2[1]);
                         const __nv_bfloat16 zb = __float2bfloat16_rn(lo);
                         const float z = __bfloat162float(zb);
                         const float s = hi > lo ? __bfloat162float(__float2bfloat16_rn(__fdiv_rn(hi - lo, 15.0f))) : 0.f;
@@ -783,7 +785,11 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 for (int c = p.r; c < p.r_pad0; c += 8)
                     *reinterpret_cast<uint4*>(p.xh + static_cast<size_t>(row) * p.r_pad + c) = make_uint4(0, 0, 0, 0);
                 if constexpr (FMT == 2) {  // behind the 3 n_g zero-point columns
-                    for (int c = p.r_pad0 + 3 * p.n_g; c < p.r_pad; ++c) p.xh[static_cast<size_t>(row) * p.r_pad + c] = 0;
+                    // (16 bytes at a time: with two, this tail kept one CTA busy for 17 thousand cycles after all others had left)
+                    uint16_t* xrow = p.xh + static_cast<size_t>(row) * p.r_pad;
+                    int c = p.r_pad0 + 3 * p.n_g;
+                    for (; (c & 7) != 0; ++c) xrow[c] = 0;
+                    for (; c < p.r_pad; c += 8) *reinterpret_cast<uint4*>(xrow + c) = make_uint4(0, 0, 0, 0);
                 }
             }
         }
