@@ -588,7 +588,6 @@ static RotateArgs rotate_args(const dirotq_layer_t* layer, const void* x, int M,
         a.xrot = xrot;
         a.status = reinterpret_cast<int*>(ws + w.off_status);
         a.xtilde = reinterpret_cast<float*>(ws + w.off_xtilde);
-        a.rowmax = reinterpret_cast<unsigned int*>(ws + w.off_rowmax);
         return a;
     }
     const bool nv = layer->geo.fmt == 1;
@@ -606,14 +605,13 @@ static RotateArgs rotate_args(const dirotq_layer_t* layer, const void* x, int M,
 }
 
 // First kernel(s): rotation + split + quantization.  W4A8 needs the token's whole row before it can quantize: the rotation
-// kernel writes fp32 coefficients and the row maxima, a second small kernel quantizes.
+// kernel writes fp32 coefficients, a second small kernel quantizes.
 static dirotq_status_t first_kernel(const dirotq_layer_t* layer, const RotateArgs& ra, int M, cudaStream_t s) {
     if (layer->geo.ph) return launch_project_quantize(layer, ra, s);
     if (layer->geo.fmt == 3) {
-        if (cudaMemsetAsync(ra.rowmax, 0, static_cast<size_t>(M) * 4, s) != cudaSuccess) return DIROTQ_ERR_CUDA;
         dirotq_status_t st = launch_rotate_quantize(layer, ra, s);
         if (st != DIROTQ_OK) return st;
-        return launch_a8_quantize(layer, M, ra.xtilde, ra.rowmax, ra.codes, ra.xscale, s);
+        return launch_a8_quantize(layer, M, ra.xtilde, ra.codes, ra.xscale, s);
     }
     return launch_rotate_quantize(layer, ra, s);
 }

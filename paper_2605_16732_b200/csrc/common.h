@@ -208,9 +208,9 @@ inline WorkspaceLayout make_workspace_layout(const Geometry& g, int M) {
 }
 
 // W4A8 (fmt 3): off_codes = int8 [M][K_lp]; off_xscale = f32 [M] token scales; off_xtilde = f32 [M][K_lp] rotated
-// low-precision coefficients (first pass); off_rowmax = u32 [M] bit patterns of the tokens' max |x~| (atomic max).
+// low-precision coefficients (first pass).
 struct WorkspaceLayoutA8 {
-    size_t off_status, off_codes, off_xscale, off_rowmax, off_xh, off_xtilde, total;
+    size_t off_status, off_codes, off_xscale, off_xh, off_xtilde, total;
 };
 inline WorkspaceLayoutA8 make_workspace_layout_w4a8(const Geometry& g, int M) {
     WorkspaceLayoutA8 w;
@@ -218,7 +218,6 @@ inline WorkspaceLayoutA8 make_workspace_layout_w4a8(const Geometry& g, int M) {
     w.off_status = o;  o = align_up(o + 256);
     w.off_codes = o;   o = align_up(o + (size_t)M * g.K_lp);
     w.off_xscale = o;  o = align_up(o + (size_t)M * 4);
-    w.off_rowmax = o;  o = align_up(o + (size_t)M * 4);
     w.off_xh = o;      o = align_up(o + (size_t)M * g.r_pad * 2);
     w.off_xtilde = o;  o = align_up(o + (size_t)M * g.K_lp * 4);
     w.total = o;
@@ -278,7 +277,6 @@ struct RotateArgs {
     int* status;
     uint8_t* xsf = nullptr;  // NVFP4 variant: scale-factor atoms (codes then holds packed E2M1)
     float* xtilde = nullptr;       // W4A8: fp32 [M][K_lp] rotated low-precision coefficients
-    unsigned int* rowmax = nullptr;  // W4A8: bit patterns of the tokens' max |x~| (zeroed before the launch)
 };
 
 struct A8GemmArgs {
@@ -454,8 +452,7 @@ dirotq_status_t launch_workspace_export_asym(const dirotq_layer* L, int M, const
 dirotq_status_t launch_zero_term_export(const dirotq_layer* L, float* d, cudaStream_t stream);
 dirotq_status_t launch_w4a8_pair(const dirotq_layer* L, int columns, const A8GemmArgs& a, cudaStream_t stream);  // (not for partials)
 dirotq_status_t launch_w4a8_gemm(const dirotq_layer* L, const A8GemmArgs& a, cudaStream_t stream);
-dirotq_status_t launch_a8_quantize(const dirotq_layer* L, int M, const float* xtilde, const unsigned int* rowmax, int8_t* codes,
-                                   float* xscale, cudaStream_t stream);
+dirotq_status_t launch_a8_quantize(const dirotq_layer* L, int M, const float* xtilde, int8_t* codes, float* xscale, cudaStream_t stream);
 dirotq_status_t launch_prepare_w4a8(const dirotq_layer* L, const void* W, int w_dtype, int w_layout, const void* Q,
                                     int q_dtype, const void* bias, double* scratch, cudaStream_t stream);
 dirotq_status_t launch_workspace_export_w4a8(const dirotq_layer* L, int M, const char* workspace, uint16_t* xh, int8_t* codes,

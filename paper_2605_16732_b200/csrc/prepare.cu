@@ -11,6 +11,7 @@
 // w4a4_gemm.cu).  The W4A8 format keeps the nibble u = q + 8 (code 8j + b in the low, 8j + 4 + b in the high nibble
 // of byte 4j + b), which its own kernel turns into the int8 value 16 q.
 #include "common.h"
+#include "ptx.cuh"
 
 #include <cuda_bf16.h>
 
@@ -395,46 +396,53 @@ __global__ void __launch_bounds__(512) w4a8_quantize_weights_kernel(const double
     }
 }
 
-// Second pass of the W4A8 activation side, one warp per token: s = bf16(max|x~| / 127), q = clip(rint(x~ / s), -127, 127).
-__global__ void a8_quantize_kernel(const float* xtilde, const unsigned int* rowmax, int8_t* codes, float* xscale, int M,
-                                   Geometry g) {
-    const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (m >= M) return;
-    const float amax = __uint_as_float(rowmax[m]);
+// Second pass of the W4A8 activation side: s = bf16(max|x~| / 127), q = clip(rint(x~ / s), -127, 127).  THREADS threads per token
+// hold its row in registers (4 V values each, requested at once), find the maximum and quantize: the row is read once and the
+// rotation kernel in front has no maxima to gather (it used to, with atomics on words that a memset had to clear first; the memset
+// kept all three launches from overlapping).  Rows longer than 16384 are read a second time past the registers.
+template <int THREADS, int V>
+__global__ void __launch_bounds__(THREADS) a8_quantize_kernel(const float* xtilde, int8_t* codes, float* xscale, int M, int K_l, int K_lp) {
+    __shared__ float part[THREADS / 32];
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const int m = blockIdx.x, t = threadIdx.x;
+    const float* xr = xtilde + static_cast<size_t>(m) * K_lp;
+    int8_t* cr = codes + static_cast<size_t>(m) * K_lp;
+    float4 v[V];
+    // K_l is a multiple of 16: four values are all real or all padding
+    auto load = [&](int j) { return j < K_l ? __ldcs(reinterpret_cast<const float4*>(xr + j)) : make_float4(0.f, 0.f, 0.f, 0.f); };
+    auto max4 = [](float4 f) { return fmaxf(fmaxf(fabsf(f.x), fabsf(f.y)), fmaxf(fabsf(f.z), fabsf(f.w))); };
+#pragma unroll
+    for (int u = 0; u < V; ++u) v[u] = load(4 * (t + THREADS * u));
+    float amax = 0.f;
+#pragma unroll
+    for (int u = 0; u < V; ++u) amax = fmaxf(amax, max4(v[u]));
+    for (int j = 4 * (t + THREADS * V); j < K_l; j += 4 * THREADS) amax = fmaxf(amax, max4(load(j)));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    if ((t & 31) == 0) part[t >> 5] = amax;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < THREADS / 32; ++w) amax = fmaxf(amax, part[w]);
     const float s = amax > 0.f ? __bfloat162float(__float2bfloat16_rn(__fdiv_rn(amax, 127.0f))) : 0.f;
     const bool slow = !(s >= 1e-30f);
     const float inv = slow ? 0.f : __frcp_rn(s);
-    if (lane == 0) xscale[m] = s;
-    const float* xr = xtilde + static_cast<size_t>(m) * g.K_lp;
-    int8_t* cr = codes + static_cast<size_t>(m) * g.K_lp;
-    // four independent 16-byte loads in flight per thread (a warp covers 2 KB of its row per step): with one load per
-    // step the pass ran at the latency of a load, not at the rate of the memory
-    constexpr int UNROLL = 4;
-    for (int j0 = lane * 4; j0 < g.K_lp; j0 += 128 * UNROLL) {
-        float4 v[UNROLL];
+    if (t == 0) xscale[m] = s;
+    auto store = [&](int j, float4 f) {
+        const float vv[4] = {f.x, f.y, f.z, f.w};
+        uint32_t word = 0;
 #pragma unroll
-        for (int u = 0; u < UNROLL; ++u) {
-            const int j = j0 + 128 * u;
-            v[u] = j < g.K_l ? __ldcs(reinterpret_cast<const float4*>(xr + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int e = 0; e < 4; ++e) {
+            float q = slow ? (s != 0.f ? vv[e] / s : 0.f) : vv[e] * inv;
+            q = fminf(fmaxf(q, -127.0f), 127.0f);
+            word |= (static_cast<uint32_t>(__float2int_rn(q)) & 0xFFu) << (8 * e);
         }
+        *reinterpret_cast<uint32_t*>(cr + j) = word;
+    };
 #pragma unroll
-        for (int u = 0; u < UNROLL; ++u) {
-            const int j = j0 + 128 * u;
-            if (j >= g.K_lp) break;
-            uint32_t word = 0;
-            if (j < g.K_l) {  // K_l is a multiple of 16: the four values are all real or all padding
-                const float vv[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    float q = slow ? (s != 0.f ? vv[t] / s : 0.f) : vv[t] * inv;
-                    q = fminf(fmaxf(q, -127.0f), 127.0f);
-                    word |= (static_cast<uint32_t>(__float2int_rn(q)) & 0xFFu) << (8 * t);
-                }
-            }
-            *reinterpret_cast<uint32_t*>(cr + j) = word;
-        }
-    }
+    for (int u = 0; u < V; ++u)
+        if (4 * (t + THREADS * u) < K_lp) store(4 * (t + THREADS * u), v[u]);
+    for (int j = 4 * (t + THREADS * V); j < K_lp; j += 4 * THREADS) store(j, load(j));
 }
 
 __global__ void export_workspace_w4a8_kernel(const int8_t* codes, const float* xscale, const uint16_t* xh_pad, int M, Geometry g,
@@ -836,10 +844,16 @@ dirotq_status_t launch_prepare_w4a8(const dirotq_layer* L, const void* W, int w_
     return launch_ok() ? DIROTQ_OK : DIROTQ_ERR_CUDA;
 }
 
-dirotq_status_t launch_a8_quantize(const dirotq_layer* L, int M, const float* xtilde, const unsigned int* rowmax, int8_t* codes,
-                                   float* xscale, cudaStream_t stream) {
-    a8_quantize_kernel<<<(M + 7) / 8, 256, 0, stream>>>(xtilde, rowmax, codes, xscale, M, L->geo);
-    return launch_ok() ? DIROTQ_OK : DIROTQ_ERR_CUDA;
+dirotq_status_t launch_a8_quantize(const dirotq_layer* L, int M, const float* xtilde, int8_t* codes, float* xscale, cudaStream_t stream) {
+    const int K_l = L->geo.K_l, K_lp = L->geo.K_lp;
+    // as few threads per row as hold it with four 16-byte loads in flight each: more rows are then under way per SM
+    auto go = [&](auto kern, int threads) {
+        return launch_kernel(kern, M, threads, 0, stream, true, xtilde, codes, xscale, M, K_l, K_lp) == cudaSuccess ? DIROTQ_OK : DIROTQ_ERR_CUDA;
+    };
+    if (K_lp <= 2048) return go(a8_quantize_kernel<128, 4>, 128);
+    if (K_lp <= 4096) return go(a8_quantize_kernel<256, 4>, 256);
+    if (K_lp <= 8192) return go(a8_quantize_kernel<512, 4>, 512);
+    return go(a8_quantize_kernel<512, 8>, 512);
 }
 
 dirotq_status_t launch_workspace_export_w4a8(const dirotq_layer* L, int M, const char* workspace, uint16_t* xh, int8_t* codes,

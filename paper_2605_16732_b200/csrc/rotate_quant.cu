@@ -58,7 +58,6 @@ struct RotKernelParams {
     int ex;           // exponent of the activations' per-tensor power-of-two scale
     // W4A8 variant: first pass only (the token's scale needs its whole row)
     float* xtilde;          // fp32 [M][K_lp]
-    unsigned int* rowmax;   // per-token max |x~_l| as a bit pattern, atomic max (zeroed by the host before the launch)
     // Split reduction (first step of the projection form with few row tiles): the k-blocks are cut into `ksplit` ranges,
     // one tile each, and every range's fp32 accumulators go to partial[range][M][n_out]; nothing else is written.
     int ksplit = 1;
@@ -514,7 +513,6 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             tc_fence_after_sync();
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + (BM == 256 ? half * 256 : acc * BN);
 
-            float tile_amax = 0.f;  // W4A8: this thread's row, this tile's columns
 #pragma unroll 1
             for (int chunk = (BM == 256 ? 0 : half * CPH); chunk < min(CHUNKS, (BM == 256 ? 1 : half + 1) * CPH); ++chunk) {
                 const int col0 = n0 + chunk * G;  // permuted column of v[0]
@@ -607,17 +605,9 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                       }
                     }
                 } else if constexpr (FMT == 3) {
-                    // W4A8, first pass: the rotated low-precision coefficients go out as fp32 and the token's maximum is
-                    // gathered with an atomic max (non-negative floats order like their bit patterns).  Columns of the chunk
+                    // W4A8, first pass: the rotated low-precision coefficients go out as fp32.  Columns of the chunk
                     // past K_l are written too where the chunk is staged (the quantizer pass reads none of them).
                     if (nlow > 0) {
-#pragma unroll
-                        for (int b = 0; b < G / 16; ++b) {
-                            if (16 * b < nlow) {
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) tile_amax = fmaxf(tile_amax, fabsf(v[16 * b + j]));
-                            }
-                        }
                         if constexpr (STAGED) {
 #pragma unroll
                             for (int h = 0; h < G / 32; ++h) {  // 32 floats = 128 bytes per row at a time
@@ -772,9 +762,6 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     }
                 }
             }
-            if constexpr (FMT == 3) {
-                if (row_ok && tile_amax > 0.f) atomicMax(p.rowmax + row, __float_as_uint(tile_amax));
-            }
             // release the accumulator: every tcgen05.ld of this warp has completed
             tc_fence_before_sync();
             // every lane arrives for itself: a warp barrier followed by one elected lane's arrival costs about a hundred cycles more
@@ -876,7 +863,7 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
     p.M = a.M; p.K = g.K; p.K_l = g.K_l; p.K_lp = g.K_lp; p.r = g.r; p.r_pad = g.r_pad; p.r_pad0 = g.r_pad0; p.ldm = a.ldm; p.n_g = g.n_g;
     p.codes = a.codes; p.xscale = a.xscale; p.xh = a.xh; p.xrot = a.xrot; p.status = a.status;
     p.xsf = a.xsf; p.K4 = g.K4; p.nkb64p = g.nkb64p; p.ex = L->act_scale_log2;
-    p.xtilde = a.xtilde; p.rowmax = a.rowmax;
+    p.xtilde = a.xtilde;
     // Tile plan.  128 x 256 is the default.  128 x 128 when the wide tiles would not give every SM about two of them
     // (few, large tiles leave a nearly empty last wave: 160 tiles on 148 SMs take as long as 296).  256 x 256 (a third
     // fewer operand bytes per flop, but the epilogue, about 11 k-blocks' worth, is not overlapped) for long main
@@ -929,7 +916,7 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
         CUtensorMap tmap_out;
         stp = encode_out_map(&tmap_out, g, a, tmap_xp);
         if (stp != DIROTQ_OK) return stp;
-        return launch_kernel_pairs(pair_table[vi], 2 * pairs, NUM_THREADS, SMEM_BYTES, stream, g.fmt != 3, tmap_xp, L->tmap_qt128,
+        return launch_kernel_pairs(pair_table[vi], 2 * pairs, NUM_THREADS, SMEM_BYTES, stream, true, tmap_xp, L->tmap_qt128,
                                    tmap_xp, L->tmap_qt128, tmap_out, p) == cudaSuccess
                    ? DIROTQ_OK
                    : DIROTQ_ERR_CUDA;
@@ -950,7 +937,7 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
         CUtensorMap tmap_out5;
         st5 = encode_out_map(&tmap_out5, g, a, tmap_x5);
         if (st5 != DIROTQ_OK) return st5;
-        return launch_kernel(table5[vi5], static_cast<int>(tiles5 < sms ? tiles5 : sms), NUM_THREADS, SMEM_BYTES, stream, g.fmt != 3,
+        return launch_kernel(table5[vi5], static_cast<int>(tiles5 < sms ? tiles5 : sms), NUM_THREADS, SMEM_BYTES, stream, true,
                              tmap_x5, L->tmap_qt64, tmap_x5, L->tmap_qt64, tmap_out5, p) == cudaSuccess
                    ? DIROTQ_OK
                    : DIROTQ_ERR_CUDA;
@@ -972,16 +959,13 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
         {rotate_quant_kernel<64, 0, 256, 256>, rotate_quant_kernel<128, 0, 256, 256>, rotate_quant_kernel<64, 1, 256, 256>,
          rotate_quant_kernel<64, 2, 256, 256>, rotate_quant_kernel<128, 2, 256, 256>, rotate_quant_kernel<64, 3, 256, 256>}};
     const KernelFn kern = table[plan - 1][vi];
-    // the W4A8 path puts a memset in front of this kernel; programmatic serialization only relaxes the wait for a
-    // preceding KERNEL, so nothing would be gained there and the launch is a plain one
-    const bool dependent = g.fmt != 3;
     static SmemOptIn<18> opt_in;
     if (!opt_in.ensure(kern, (plan - 1) * 6 + vi, L->device, SMEM_BYTES)) return DIROTQ_ERR_CUDA;
     const CUtensorMap& tmap_q = plan == 1 ? L->tmap_qt128 : L->tmap_qt;
     CUtensorMap tmap_out;
     st = encode_out_map(&tmap_out, g, a, tmap_x);
     if (st != DIROTQ_OK) return st;
-    return launch_kernel(kern, grid, NUM_THREADS, SMEM_BYTES, stream, dependent, tmap_x, tmap_q, tmap_x, tmap_q, tmap_out, p) == cudaSuccess
+    return launch_kernel(kern, grid, NUM_THREADS, SMEM_BYTES, stream, true, tmap_x, tmap_q, tmap_x, tmap_q, tmap_out, p) == cudaSuccess
                ? DIROTQ_OK
                : DIROTQ_ERR_CUDA;
 }
@@ -996,7 +980,7 @@ dirotq_status_t launch_project_quantize(const dirotq_layer* L, const RotateArgs&
     RotKernelParams p;
     p.M = a.M; p.K = g.K; p.K_lp = g.K_lp; p.r_pad = g.r_pad; p.r_pad0 = g.r_pad0; p.ldm = a.ldm; p.n_g = g.n_g;
     p.codes = a.codes; p.xscale = a.xscale; p.xh = a.xh; p.xrot = nullptr; p.status = a.status;
-    p.xsf = nullptr; p.K4 = 0; p.nkb64p = 0; p.ex = 0; p.xtilde = nullptr; p.rowmax = nullptr;
+    p.xsf = nullptr; p.K4 = 0; p.nkb64p = 0; p.ex = 0; p.xtilde = nullptr;
     dirotq_status_t st;
     CUtensorMap tmap_x;
     st = encode_tmap_2d(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)g.K, (uint64_t)a.M, (uint64_t)g.K * 2, BK,
