@@ -197,7 +197,8 @@ __device__ __forceinline__ uint32_t nvfp4_block16(const float* v, float pre, flo
 // 87 against 79 us for the whole first stage at M = 4608, K = 12288.)
 // EPI_WARPS: 8, or 16 for the PH mode with groups of 64 (four warps per lane quadrant, one 64-column chunk each): that
 // mode has no long main loop to hide the epilogue under, and its epilogue is a chain of dependent instructions per
-// thread that only more warps per scheduler speed up.
+// thread (3.4 thousand cycles per chunk) that more warps per scheduler hide.  Whole first stage, 4608 x 12288 NVFP4: 62.7 -> 55.4 us;
+// the staging tiles of 16 warps fit where those of 8 did, a chunk's codes being at most 2 KB.
 // PAIR: launched as clusters of two CTAs that share every MMA (tcgen05.mma.cta_group::2, M = 256): a pair owns 256
 // token rows x BN columns, each CTA loads its own 128 rows of x and HALF of the rotation tile (BN / 2 rows of Q^T), so a
 // third fewer operand bytes travel from L2 per flop than with 128 x 256 tiles, and both accumulator buffers stay free
@@ -493,8 +494,8 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             // W4A8 path's fp32 coefficients (128 bytes per row at a time) go into the warp's staging tile instead, swizzled
             // so that a quarter-warp's pieces fall into different banks, and one lane hands the tile to a TMA store
             // (tmap_out), which writes whole sectors and clips at M and at the row's width.
-            constexpr bool STAGED = EPI_WARPS == 8;
-            const uint32_t sbuf = smem_base + STORE_OFFSET + static_cast<uint32_t>(warp - 2) * 4096u;
+            constexpr bool STAGED = true;
+            const uint32_t sbuf = smem_base + STORE_OFFSET + static_cast<uint32_t>(warp - 2) * (EPI_WARPS == 16 ? 2048u : 4096u);
             const int row0w = row - lane;  // the warp's first row
             auto stage_piece128 = [&](int piece, uint4 val) {  // rows of 128 bytes, 128-byte swizzle
                 const uint32_t dst = sbuf + static_cast<uint32_t>(lane) * 128u + (static_cast<uint32_t>(piece ^ (lane & 7)) << 4);
@@ -1026,9 +1027,9 @@ dirotq_status_t launch_project_quantize(const dirotq_layer* L, const RotateArgs&
         RotKernelParams p2 = p;
         p2.n_out = g.K; p2.k_red = g.r_pad; p2.K_l = g.K; p2.r = g.r;
         const int vi = g.fmt == 1 ? 2 : (g.G == 64 ? 0 : 1);
-        static const KernelFn k2s[3] = {rotate_quant_kernel<64, 4, 256, 128, true, 8>, rotate_quant_kernel<128, 4, 256, 128>,
-                                        rotate_quant_kernel<64, 1, 256, 128, true, 8>};
-        const int threads2 = NUM_THREADS;
+        static const KernelFn k2s[3] = {rotate_quant_kernel<64, 4, 256, 128, true, 16>, rotate_quant_kernel<128, 4, 256, 128>,
+                                        rotate_quant_kernel<64, 1, 256, 128, true, 16>};
+        const int threads2 = vi == 1 ? NUM_THREADS : 64 + 32 * 16;
         const KernelFn k2 = k2s[vi];
         if (g.fmt == 1) { p2.xsf = a.xsf; p2.K4 = g.K4; p2.nkb64p = g.nkb64p; p2.ex = L->act_scale_log2; }
         static SmemOptIn<3> opt_in2;
