@@ -189,7 +189,8 @@ DIROTQ_API dirotq_status_t dirotq_int_gemm_debug(const int8_t* act_codes, int M,
 DIROTQ_API dirotq_status_t dirotq_set_gemm_tile(int columns);
 
 /* Tuning knob of the first kernel (rotation): tile plan.  0 (default): chosen per call from M, K and the number of
- * SMs; 1: 128 tokens x 128 rotated columns; 2: 128 x 256; 3: 256 x 256 (two MMAs share one tile of the rotation: a
+ * SMs; 1: 128 tokens x 128 rotated columns (in CTA pairs sharing
+ * a tile of the rotation above 128 tokens where that takes no more turns); 2: 128 x 256; 3: 256 x 256 (two MMAs share one tile of the rotation: a
  * third fewer operand bytes per flop, no overlap of the epilogue; pays where a layer has many tiles per SM, e.g.
  * K = 12288 at M = 4608); 4: 256 x 256 per PAIR of CTAs (clusters of two: tcgen05.mma.cta_group::2, each CTA loads its
  * own 128 rows of x and half of the rotation tile; the epilogue stays overlapped); 5: 128 x 64 (groups of 64 only, else

@@ -219,7 +219,7 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // where a tile's main loop is long and there are many tiles per SM.
     static_assert(BM == 128 || (BM == 256 && BN == 256), "256-row tiles are 256 columns wide");
     constexpr int A_BYTES = BM * BK * 2;
-    static_assert(!PAIR || (BM == 128 && BN == 256 && !PH), "pairs: 128 rows per CTA, 256 columns per pair");
+    static_assert(!PAIR || (BM == 128 && BN >= 128 && !PH), "pairs: 128 rows per CTA, 256 or 128 columns per pair");
     constexpr int B_ROWS = PAIR ? BN / 2 : BN;  // rows of the rotation tile this CTA holds
     static_assert(BN >= G, "a tile holds whole groups");
     // 64-column tiles (few token rows) put TWO k-blocks into a stage: there the kernel is paced by the producer's and the MMA
@@ -227,7 +227,7 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // stages shorten it (the split reduction of the projection form's first step never runs with this plan)
     constexpr int KSUB = BN == 64 ? 2 : 1;
     constexpr int SUB_BYTES = A_BYTES + B_ROWS * BK * 2;  // one k-block's operands: [x tile | rotation tile]
-    constexpr int STAGES = BM == 256 ? 3 : (B_ROWS == 256 ? STAGES_WIDE : B_ROWS == 128 ? 6 : 4);
+    constexpr int STAGES = BM == 256 ? 3 : (B_ROWS == 256 ? STAGES_WIDE : B_ROWS == 128 ? 6 : 8 / KSUB);
     constexpr int STAGE_BYTES = KSUB * SUB_BYTES;
     constexpr int ACC_BUFS = BM == 256 ? 1 : 2;
     static_assert(STAGES * STAGE_BYTES == STAGES_WIDE * STAGE_BYTES_WIDE && STAGE_BYTES % 1024 == 0, "ring layout");
@@ -871,12 +871,16 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
     // loops only: measured 0.99 -> 0.92 ms at M = 4608, K = 12288 and 1.54 -> 1.48 ms at K = 15360, but 0.125 ->
     // 0.141 ms at M = 9216, K = 3072.
     const int sms = sm_count(L->device);
-    const long mb128 = (a.M + 127) / 128, mb256 = (a.M + 255) / 256, nb256 = (g.K + 255) / 256;
+    const long mb128 = (a.M + 127) / 128, mb256 = (a.M + 255) / 256, nb128 = (g.K + 127) / 128, nb256 = (g.K + 255) / 256;
+    // 128 x 128 tiles (plan 1) are computed in CTA pairs, 256 x 128 per pair, wherever that does not take more turns (not for up to
+    // 128 rows): a single CTA's 32 KB per k-block come in at 72 bytes a cycle, 445 cycles where the MMAs need 256; a CTA of a
+    // pair loads 24 KB.  Whole NVFP4 layers, 3072 -> 3072: 23.7 -> 21.8 us at 512 tokens, 54.9 -> 48.9 at 2048.
+    const long turns_single = (mb128 * nb128 + sms - 1) / sms, turns_pair = (mb256 * nb128 + sms / 2 - 1) / (sms / 2);
+    const bool pairs_narrow = a.M > 128 && turns_pair <= turns_single;
     int plan = g_rotation_plan.load();
     if (plan == 0) {
-        const long nb128 = (g.K + 127) / 128;
         const long waves128 = (mb128 * nb256 + sms - 1) / sms, waves256 = (mb256 * nb256 + sms - 1) / sms;
-        const long waves_narrow = (mb128 * nb128 + sms - 1) / sms;
+        const long waves_narrow = pairs_narrow ? turns_pair : turns_single;
         const double kb = static_cast<double>(g.K / BK);
         // a 256-row tile in units of a 128-row tile; once x no longer fits the L2 beside the rotation the 128-row plan
         // re-reads it from HBM and the ratio falls to 1.9 (measured at M = 18432, K = 3072: 0.304 -> 0.288 ms)
@@ -891,6 +895,9 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
         // one SM's port to L2, so the time of a call this small falls with the bytes per CTA
         if (2 * mb128 * nb128 <= sms && g.G == 64) plan = 5;
         else if (0.62 * static_cast<double>(waves_narrow) < static_cast<double>(waves128)) plan = 1;
+        // long main loops, all pairs resident at once: the rotation streams from HBM, and plan 2 reads it once per 128 rows (M = 256,
+        // K = 12288: 101 -> 87 us)
+        else if (g.K >= 8192 && a.M > 128 && mb256 * nb256 <= sms / 2) plan = 4;
         else if ((g.K >= 8192 || x_exceeds_l2) && cost256 * static_cast<double>(waves256) < 0.98 * static_cast<double>(waves128)) plan = 3;
         // CTA pairs where there are a few waves of tiles and the main loop is not long enough for the operand traffic
         // to hide behind the MMAs anyway (measured against 128 x 256 tiles: M = 4608, K = 3072 68.4 -> 67.3 us; M = 9216,
@@ -898,31 +905,36 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
         else if (mb128 * nb256 >= 5 * sms / 2 && g.K < 8192) plan = 4;
         else plan = 2;
     }
-    if (plan == 4) {
-        // CTA pairs: 256 rows x 256 columns per pair, 128 rows of x and half of the rotation tile per CTA
+    if (plan == 5 && g.G != 64) plan = 1;  // a tile holds whole groups
+    if (plan == 4 || (plan == 1 && pairs_narrow)) {
+        // CTA pairs: 256 rows x 256 (plan 1: 128) columns per pair, 128 rows of x and half of the rotation tile per CTA
+        const bool wide = plan == 4;
         CUtensorMap tmap_xp;
         dirotq_status_t stp = encode_tmap_2d(&tmap_xp, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)g.K, (uint64_t)a.M,
                                              (uint64_t)g.K * 2, BK, 128, CU_TENSOR_MAP_SWIZZLE_128B);
         if (stp != DIROTQ_OK) return stp;
-        const long pair_tiles = ((a.M + 255) / 256) * nb256;
+        const long pair_tiles = mb256 * (wide ? nb256 : nb128);
         const int pairs = static_cast<int>(pair_tiles < sms / 2 ? pair_tiles : sms / 2);
         const int vi = g.fmt == 1 ? 2 : g.fmt == 3 ? 5 : (g.fmt == 2 ? (g.G == 64 ? 3 : 4) : (g.G == 64 ? 0 : 1));
         using PairFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const RotKernelParams);
-        static const PairFn pair_table[6] = {
-            rotate_quant_kernel<64, 0, 256, 128, false, 8, true>, rotate_quant_kernel<128, 0, 256, 128, false, 8, true>,
-            rotate_quant_kernel<64, 1, 256, 128, false, 8, true>, rotate_quant_kernel<64, 2, 256, 128, false, 8, true>,
-            rotate_quant_kernel<128, 2, 256, 128, false, 8, true>, rotate_quant_kernel<64, 3, 256, 128, false, 8, true>};
-        static SmemOptIn<6> opt_in_pair;
-        if (!opt_in_pair.ensure(pair_table[vi], vi, L->device, SMEM_BYTES)) return DIROTQ_ERR_CUDA;
+        static const PairFn pair_table[2][6] = {
+            {rotate_quant_kernel<64, 0, 128, 128, false, 8, true>, rotate_quant_kernel<128, 0, 128, 128, false, 8, true>,
+             rotate_quant_kernel<64, 1, 128, 128, false, 8, true>, rotate_quant_kernel<64, 2, 128, 128, false, 8, true>,
+             rotate_quant_kernel<128, 2, 128, 128, false, 8, true>, rotate_quant_kernel<64, 3, 128, 128, false, 8, true>},
+            {rotate_quant_kernel<64, 0, 256, 128, false, 8, true>, rotate_quant_kernel<128, 0, 256, 128, false, 8, true>,
+             rotate_quant_kernel<64, 1, 256, 128, false, 8, true>, rotate_quant_kernel<64, 2, 256, 128, false, 8, true>,
+             rotate_quant_kernel<128, 2, 256, 128, false, 8, true>, rotate_quant_kernel<64, 3, 256, 128, false, 8, true>}};
+        const PairFn kern = pair_table[wide][vi];
+        const CUtensorMap& tmap_q = wide ? L->tmap_qt128 : L->tmap_qt64;
+        static SmemOptIn<12> opt_in_pair;
+        if (!opt_in_pair.ensure(kern, 6 * wide + vi, L->device, SMEM_BYTES)) return DIROTQ_ERR_CUDA;
         CUtensorMap tmap_out;
         stp = encode_out_map(&tmap_out, g, a, tmap_xp);
         if (stp != DIROTQ_OK) return stp;
-        return launch_kernel_pairs(pair_table[vi], 2 * pairs, NUM_THREADS, SMEM_BYTES, stream, true, tmap_xp, L->tmap_qt128,
-                                   tmap_xp, L->tmap_qt128, tmap_out, p) == cudaSuccess
+        return launch_kernel_pairs(kern, 2 * pairs, NUM_THREADS, SMEM_BYTES, stream, true, tmap_xp, tmap_q, tmap_xp, tmap_q, tmap_out, p) == cudaSuccess
                    ? DIROTQ_OK
                    : DIROTQ_ERR_CUDA;
     }
-    if (plan == 5 && g.G != 64) plan = 1;  // a tile holds whole groups
     if (plan == 5) {
         CUtensorMap tmap_x5;
         dirotq_status_t st5 = encode_tmap_2d(&tmap_x5, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)g.K, (uint64_t)a.M,

@@ -380,8 +380,11 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         bool ok = true;
         uint32_t raw[2][32];  // [0..15]: TMEM lanes 0..15 of the quadrant (rows i = 0, 1), [16..31]: lanes 16..31
         auto request_chunk = [&](uint32_t buf, int c, uint32_t* dst) {
-            tmem_ld_16x256b_x4(taddr0 + buf * BN + c * 32, dst);
-            tmem_ld_16x256b_x4(taddr0 + buf * BN + (16u << 16) + c * 32, dst + 16);
+            const uint32_t t = taddr0 + buf * BN + c * 32;
+            tmem_ld_16x256b_x2(t, dst);
+            tmem_ld_16x256b_x2(t + 16, dst + 8);
+            tmem_ld_16x256b_x2(t + (16u << 16), dst + 16);
+            tmem_ld_16x256b_x2(t + (16u << 16) + 16, dst + 24);
         };
         auto release_tile = [&](uint32_t buf) {  // every tcgen05.ld of this thread on the tile has completed
             tc_fence_before_sync();

@@ -377,8 +377,10 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
         auto request_unit = [&](uint32_t buf, int u, uint32_t (&dst)[UC]) {
             const uint32_t t = taddr0 + buf * BUF_COLS + u / UPG * BN + u % UPG * UC;
             if constexpr (UC == 32) {
-                tmem_ld_16x256b_x4(t, dst);
-                tmem_ld_16x256b_x4(t + (16u << 16), dst + 16);
+                tmem_ld_16x256b_x2(t, dst);
+                tmem_ld_16x256b_x2(t + 16, dst + 8);
+                tmem_ld_16x256b_x2(t + (16u << 16), dst + 16);
+                tmem_ld_16x256b_x2(t + (16u << 16) + 16, dst + 24);
             } else {
                 tmem_ld_16x256b_x2(t, dst);
                 tmem_ld_16x256b_x2(t + (16u << 16), dst + 8);
