@@ -44,44 +44,47 @@ __device__ __forceinline__ double load_w(const void* W, int w_dtype, int w_layou
                                        : bf16_to_f64(static_cast<const uint16_t*>(W)[i]);
 }
 
-// Wt[i][n] = sum_k Q[k][i] * W[k][n] in fp64, k ascending: 128 x 64 output tile, 8 x 4 per thread.
+// Wt[i][n] = sum_k Q[k][i] * W[k][n] in fp64, k ascending: 64 x 64 output tile, 8 x 4 per thread,
+// four blocks per SM (small tiles spread the last ones over the SMs).
 // Bound by the fp64 multiply-adds (16 lanes per scheduler: a warp's 32 of one k take 64 cycles), which needs few shared-memory
 // loads per multiply-add (six 16-byte loads per 32; with 4 x 4 per thread and scalar loads, eight per 16, the loads set the time)
 // and the next tile's global loads, 12 per thread, in flight under them.  1152 -> 4608: 1463 us with the 4 x 4 tile.
 // The loads in flight are held as they come: converted at once, every tile waited for them (779 us).
-constexpr int FOLD_I = 128, FOLD_N = 64;
+constexpr int FOLD_I = 64, FOLD_N = 64, FOLD_THREADS = 128;
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return static_cast<double>(v); }
 __device__ __forceinline__ double to_f64(uint16_t v) { return bf16_to_f64(v); }
 template <typename TQ, typename TW, bool kn>
-__global__ void __launch_bounds__(256, 2) fold_kernel(const TQ* Q, const TW* W, double* Wt, int K, int N) {
-    constexpr int FOLD_K = sizeof(TQ) == 8 ? 8 : 16;  // (as many as the registers for a tile in flight allow)
-    __shared__ __align__(16) double sq[FOLD_K][FOLD_I + 2];
-    __shared__ __align__(16) double sw[FOLD_K][FOLD_N + 2];
+__global__ void __launch_bounds__(FOLD_THREADS, 4) fold_kernel(const TQ* Q, const TW* W, double* Wt, int K, int N) {
+    constexpr int FOLD_K = 8;  // (as many as the registers for a tile in flight allow)
+    __shared__ __align__(16) double sqs[2][FOLD_K][FOLD_I + 2];  // (two: one barrier per tile)
+    __shared__ __align__(16) double sws[2][FOLD_K][FOLD_N + 2];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int i0 = blockIdx.y * FOLD_I, n0 = blockIdx.x * FOLD_N;
     // this thread's elements of the two input tiles: along the contiguous index of each
-    const int qc = threadIdx.x & 127, qk = threadIdx.x >> 7;  // Q: k = qk + 2 u
-    constexpr int WN = 256 / FOLD_K;
-    const int wc = kn ? threadIdx.x & 63 : threadIdx.x / FOLD_K, wk = kn ? threadIdx.x >> 6 : threadIdx.x % FOLD_K;  // W: k = wk + 4 u, or n = wc + WN u
+    const int qc = threadIdx.x & 63, qk = threadIdx.x >> 6;  // Q: k = qk + 2 u
+    constexpr int WN = FOLD_THREADS / FOLD_K;
+    const int wc = kn ? threadIdx.x & 63 : threadIdx.x / FOLD_K, wk = kn ? threadIdx.x >> 6 : threadIdx.x % FOLD_K;  // W: k = wk + 2 u, or n = wc + WN u
     TQ rq[FOLD_K / 2];
-    TW rw[FOLD_K / 4];
+    TW rw[FOLD_K / 2];
     auto fetch = [&](int k0) {
 #pragma unroll
         for (int u = 0; u < FOLD_K / 2; ++u) rq[u] = i0 + qc < K ? Q[static_cast<size_t>(k0 + qk + 2 * u) * K + i0 + qc] : TQ(0);
 #pragma unroll
-        for (int u = 0; u < FOLD_K / 4; ++u) {
-            const int n = n0 + wc + (kn ? 0 : WN * u), k = k0 + wk + (kn ? 4 * u : 0);
+        for (int u = 0; u < FOLD_K / 2; ++u) {
+            const int n = n0 + wc + (kn ? 0 : WN * u), k = k0 + wk + (kn ? 2 * u : 0);
             rw[u] = n < N ? W[kn ? static_cast<size_t>(k) * N + n : static_cast<size_t>(n) * K + k] : TW(0);
         }
     };
     double acc[8][4] = {};
     fetch(0);
     for (int k0 = 0; k0 < K; k0 += FOLD_K) {
+        double(&sq)[FOLD_K][FOLD_I + 2] = sqs[(k0 / FOLD_K) & 1];
+        double(&sw)[FOLD_K][FOLD_N + 2] = sws[(k0 / FOLD_K) & 1];
 #pragma unroll
         for (int u = 0; u < FOLD_K / 2; ++u) sq[qk + 2 * u][qc] = to_f64(rq[u]);
 #pragma unroll
-        for (int u = 0; u < FOLD_K / 4; ++u) sw[wk + (kn ? 4 * u : 0)][wc + (kn ? 0 : WN * u)] = to_f64(rw[u]);
+        for (int u = 0; u < FOLD_K / 2; ++u) sw[wk + (kn ? 2 * u : 0)][wc + (kn ? 0 : WN * u)] = to_f64(rw[u]);
         __syncthreads();
         if (k0 + FOLD_K < K) fetch(k0 + FOLD_K);
 #pragma unroll 4
@@ -101,7 +104,6 @@ __global__ void __launch_bounds__(256, 2) fold_kernel(const TQ* Q, const TW* W, 
                     acc[2 * u + 1][2 * v + 1] = fma(a[u].y, b[v].y, acc[2 * u + 1][2 * v + 1]);
                 }
         }
-        __syncthreads();
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u)
@@ -119,11 +121,11 @@ bool launch_fold_q(const TQ* Q, const void* W, int w_dtype, int w_layout, double
     const uint16_t* wb = static_cast<const uint16_t*>(W);
     const bool f32 = w_dtype == DIROTQ_DTYPE_F32;
     if (w_layout == DIROTQ_LAYOUT_KN) {
-        if (f32) fold_kernel<TQ, float, true><<<grid, 256, 0, stream>>>(Q, wf, Wt, K, N);
-        else fold_kernel<TQ, uint16_t, true><<<grid, 256, 0, stream>>>(Q, wb, Wt, K, N);
+        if (f32) fold_kernel<TQ, float, true><<<grid, FOLD_THREADS, 0, stream>>>(Q, wf, Wt, K, N);
+        else fold_kernel<TQ, uint16_t, true><<<grid, FOLD_THREADS, 0, stream>>>(Q, wb, Wt, K, N);
     } else {
-        if (f32) fold_kernel<TQ, float, false><<<grid, 256, 0, stream>>>(Q, wf, Wt, K, N);
-        else fold_kernel<TQ, uint16_t, false><<<grid, 256, 0, stream>>>(Q, wb, Wt, K, N);
+        if (f32) fold_kernel<TQ, float, false><<<grid, FOLD_THREADS, 0, stream>>>(Q, wf, Wt, K, N);
+        else fold_kernel<TQ, uint16_t, false><<<grid, FOLD_THREADS, 0, stream>>>(Q, wb, Wt, K, N);
     }
     return cudaGetLastError() == cudaSuccess;
 }
