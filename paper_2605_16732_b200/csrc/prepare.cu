@@ -44,22 +44,23 @@ __device__ __forceinline__ double load_w(const void* W, int w_dtype, int w_layou
                                        : bf16_to_f64(static_cast<const uint16_t*>(W)[i]);
 }
 
-// Wt[i][n] = sum_k Q[k][i] * W[k][n] in fp64, k ascending: 64 x 64 output tile, 8 x 4 per thread,
-// four blocks per SM (small tiles spread the last ones over the SMs).
-// Bound by the fp64 multiply-adds (16 lanes per scheduler: a warp's 32 of one k take 64 cycles), which needs few shared-memory
-// loads per multiply-add (six 16-byte loads per 32; with 4 x 4 per thread and scalar loads, eight per 16, the loads set the time)
-// and the next tile's global loads, 12 per thread, in flight under them.  1152 -> 4608: 1463 us with the 4 x 4 tile.
-// The loads in flight are held as they come: converted at once, every tile waited for them (779 us).
+// Wt[i][n] = sum_k Q[k][i] * W[k][n] in fp64 on the double-precision matrix instruction (8 x 8 x 4 per warp): 64 x 64 output
+// tile, a warp 32 x 32, four blocks per SM (small tiles spread the last ones over the SMs).  A fragment's element is row lane / 4 of k
+// lane % 4; rows of FOLD_I + 4 doubles put a half-warp's 16 elements into different banks.
+// Bound by fp64 arithmetic: 28 TFLOP/s at 3072^3.  Eight 8-byte loads per lane feed 16 instructions of 256 multiply-adds; with
+// scalar multiply-adds (8 x 4 per thread) their register operands held the pipe at 55 %.  The next tile's loads are in flight
+// under the arithmetic and are held in their own type (converted at once, every tile waited for them).  Preparation and export,
+// 1152 -> 4608: 1595 us with a scalar 4 x 4 per thread, 682 with 8 x 4, 524 now.
 constexpr int FOLD_I = 64, FOLD_N = 64, FOLD_THREADS = 128;
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return static_cast<double>(v); }
 __device__ __forceinline__ double to_f64(uint16_t v) { return bf16_to_f64(v); }
 template <typename TQ, typename TW, bool kn>
 __global__ void __launch_bounds__(FOLD_THREADS, 4) fold_kernel(const TQ* Q, const TW* W, double* Wt, int K, int N) {
-    constexpr int FOLD_K = 8;  // (as many as the registers for a tile in flight allow)
-    __shared__ __align__(16) double sqs[2][FOLD_K][FOLD_I + 2];  // (two: one barrier per tile)
-    __shared__ __align__(16) double sws[2][FOLD_K][FOLD_N + 2];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    constexpr int FOLD_K = 8;
+    __shared__ __align__(16) double sqs[2][FOLD_K][FOLD_I + 4];  // (two: one barrier per tile)
+    __shared__ __align__(16) double sws[2][FOLD_K][FOLD_N + 4];
+    const int lane = threadIdx.x & 31, wi = (threadIdx.x >> 5 & 1) * 32, wn = (threadIdx.x >> 6) * 32;  // the warp's 32 x 32
     const int i0 = blockIdx.y * FOLD_I, n0 = blockIdx.x * FOLD_N;
     // this thread's elements of the two input tiles: along the contiguous index of each
     const int qc = threadIdx.x & 63, qk = threadIdx.x >> 6;  // Q: k = qk + 2 u
@@ -76,41 +77,38 @@ __global__ void __launch_bounds__(FOLD_THREADS, 4) fold_kernel(const TQ* Q, cons
             rw[u] = n < N ? W[kn ? static_cast<size_t>(k) * N + n : static_cast<size_t>(n) * K + k] : TW(0);
         }
     };
-    double acc[8][4] = {};
+    double acc[4][4][2] = {};
     fetch(0);
     for (int k0 = 0; k0 < K; k0 += FOLD_K) {
-        double(&sq)[FOLD_K][FOLD_I + 2] = sqs[(k0 / FOLD_K) & 1];
-        double(&sw)[FOLD_K][FOLD_N + 2] = sws[(k0 / FOLD_K) & 1];
+        double(&sq)[FOLD_K][FOLD_I + 4] = sqs[(k0 / FOLD_K) & 1];
+        double(&sw)[FOLD_K][FOLD_N + 4] = sws[(k0 / FOLD_K) & 1];
 #pragma unroll
         for (int u = 0; u < FOLD_K / 2; ++u) sq[qk + 2 * u][qc] = to_f64(rq[u]);
 #pragma unroll
         for (int u = 0; u < FOLD_K / 2; ++u) sw[wk + (kn ? 2 * u : 0)][wc + (kn ? 0 : WN * u)] = to_f64(rw[u]);
         __syncthreads();
         if (k0 + FOLD_K < K) fetch(k0 + FOLD_K);
-#pragma unroll 4
-        for (int kk = 0; kk < FOLD_K; ++kk) {
-            double2 a[4], b[2];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) a[u] = *reinterpret_cast<const double2*>(&sq[kk][ty * 8 + 2 * u]);
+        for (int kk = 0; kk < FOLD_K; kk += 4) {
+            double a[4], b[4];
 #pragma unroll
-            for (int v = 0; v < 2; ++v) b[v] = *reinterpret_cast<const double2*>(&sw[kk][tx * 2 + 32 * v]);
+            for (int u = 0; u < 4; ++u) a[u] = sq[kk + (lane & 3)][wi + 8 * u + (lane >> 2)];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) b[v] = sw[kk + (lane & 3)][wn + 8 * v + (lane >> 2)];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int v = 0; v < 2; ++v) {
-                    acc[2 * u][2 * v] = fma(a[u].x, b[v].x, acc[2 * u][2 * v]);
-                    acc[2 * u][2 * v + 1] = fma(a[u].x, b[v].y, acc[2 * u][2 * v + 1]);
-                    acc[2 * u + 1][2 * v] = fma(a[u].y, b[v].x, acc[2 * u + 1][2 * v]);
-                    acc[2 * u + 1][2 * v + 1] = fma(a[u].y, b[v].y, acc[2 * u + 1][2 * v + 1]);
-                }
+                for (int v = 0; v < 4; ++v)
+                    asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                        : "+d"(acc[u][v][0]), "+d"(acc[u][v][1]) : "d"(a[u]), "d"(b[v]));
         }
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const int i = i0 + ty * 8 + u, n = n0 + tx * 2 + 32 * (v >> 1) + (v & 1);
-            if (i < K && n < N) Wt[static_cast<size_t>(i) * N + n] = acc[u][v];
+            const int i = i0 + wi + 8 * u + (lane >> 2), n = n0 + wn + 8 * v + 2 * (lane & 3);
+            if (i < K && n < N) *reinterpret_cast<double2*>(Wt + static_cast<size_t>(i) * N + n) = make_double2(acc[u][v][0], acc[u][v][1]);
         }
 }
 
