@@ -5,8 +5,6 @@
 
 #include <atomic>
 
-#include <mutex>
-
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -15,12 +13,14 @@
 
 namespace dirotq {
 namespace {
-
 thread_local char g_last_error[256] = "";
+}  // namespace
 
 void set_error(const char* what, cudaError_t e) {
     snprintf(g_last_error, sizeof g_last_error, "%s: %s", what, cudaGetErrorString(e));
 }
+
+namespace {
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -563,8 +563,9 @@ dirotq_status_t dirotq_layer_info(const dirotq_layer_t* layer, int* K, int* N, i
     return DIROTQ_OK;
 }
 
-static dirotq_status_t check_call(const dirotq_layer_t* layer, int M, const void* workspace, size_t workspace_bytes,
-                                  bool rotates = true) {
+}  // extern "C"
+
+dirotq_status_t dirotq::check_call(const dirotq_layer_t* layer, int M, const void* workspace, size_t workspace_bytes, bool rotates) {
     if (!valid_layer(layer) || !workspace || M < 1) return DIROTQ_ERR_INVALID_ARG;
     if (rotates && layer->geo.no_rot) return DIROTQ_ERR_INVALID_ARG;  // a sibling layer holds no rotation
     if ((reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) != 0) return DIROTQ_ERR_INVALID_ARG;
@@ -575,6 +576,8 @@ static dirotq_status_t check_call(const dirotq_layer_t* layer, int M, const void
     if (dev != layer->device) return DIROTQ_ERR_INVALID_ARG;
     return DIROTQ_OK;
 }
+
+extern "C" {
 
 static RotateArgs rotate_args(const dirotq_layer_t* layer, const void* x, int M, char* ws, float* xrot) {
     if (layer->geo.fmt == 3) {
@@ -684,97 +687,6 @@ dirotq_status_t dirotq_w4a4_gemm(int M, const dirotq_layer_t* layer, const void*
     char* ws = const_cast<char*>(static_cast<const char*>(workspace));
     const RotateArgs ra = rotate_args(layer, nullptr, M, ws, nullptr);
     return second_kernel(layer, ra, M, y, static_cast<cudaStream_t>(stream));
-}
-
-namespace {
-
-// Copy streams and events of dirotq_linear_host, created once per device (no device memory involved).
-struct HostPipe {
-    bool ready = false;
-    cudaStream_t h2d = nullptr, d2h = nullptr;
-    static constexpr int kMaxChunks = 32;
-    cudaEvent_t start = nullptr, done = nullptr, copied[kMaxChunks] = {}, computed[kMaxChunks] = {};
-};
-std::mutex g_pipe_mutex;
-HostPipe g_pipe[64];
-
-// Caller holds g_pipe_mutex (also while it enqueues on the pipe: its events are shared by all calls on the device).
-dirotq_status_t host_pipe(int dev, HostPipe** out) {
-    if (dev < 0 || dev >= 64) return DIROTQ_ERR_INVALID_ARG;
-    HostPipe& p = g_pipe[dev];
-    if (!p.ready) {
-        cudaError_t e = cudaStreamCreateWithFlags(&p.h2d, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p.d2h, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p.start, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p.done, cudaEventDisableTiming);
-        for (int i = 0; i < HostPipe::kMaxChunks && e == cudaSuccess; ++i) {
-            e = cudaEventCreateWithFlags(&p.copied[i], cudaEventDisableTiming);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p.computed[i], cudaEventDisableTiming);
-        }
-        if (e != cudaSuccess) { set_error("host pipeline set-up", e); return DIROTQ_ERR_CUDA; }
-        p.ready = true;
-    }
-    *out = &p;
-    return DIROTQ_OK;
-}
-
-}  // namespace
-
-dirotq_status_t dirotq_linear_host(const void* x_host, int M, const dirotq_layer_t* layer, void* y_host, void* x_dev,
-                                   void* y_dev, void* workspace, size_t workspace_bytes, dirotq_stream_t stream) {
-    dirotq_status_t st = check_call(layer, M, workspace, workspace_bytes);
-    if (st != DIROTQ_OK) return st;
-    if (!x_host || !y_host || !x_dev || !y_dev) return DIROTQ_ERR_INVALID_ARG;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const size_t xrow = static_cast<size_t>(layer->geo.K) * 2, yrow = static_cast<size_t>(layer->geo.N) * 2;
-    // Token rows are independent: the call is cut into row chunks whose host-to-device copy, computation and
-    // device-to-host copy overlap (copy engines in both directions + SMs).  The chunks' kernels run one after another on
-    // `stream`, so they can share the workspace.
-    // A chunk is about 8 MB of the larger side (smaller ones pay more for starting copies, about 15 us each, and, with few rows, more per
-    // row for the kernels), but a good quarter of a short call, and at least 256 rows.  The first one and the last ones are
-    // shorter: the first copy in, and the last rows' computation and copy out, overlap with nothing.  4608 x 3072 -> 3072: 915 us
-    // in four equal chunks, 850 tapered; 1024 x 3072 -> 3072 311 us in one piece, 236 in chunks.
-    constexpr size_t CHUNK_BYTES = 8u << 20;
-    auto rows128 = [](long rows) { return (rows + 127) / 128 * 128; };
-    long base = static_cast<long>(CHUNK_BYTES / (xrow > yrow ? xrow : yrow));
-    base = rows128(std::max(std::min(base, M * 10L / 37), std::max(256L, M / 24L)));  // (at most kMaxChunks in all)
-    if (M < 512) {
-        cudaError_t e = cudaMemcpyAsync(x_dev, x_host, xrow * M, cudaMemcpyHostToDevice, s);
-        if (e != cudaSuccess) { set_error("cudaMemcpyAsync(H2D)", e); return DIROTQ_ERR_CUDA; }
-        st = dirotq_linear(x_dev, M, layer, y_dev, workspace, workspace_bytes, stream);
-        if (st != DIROTQ_OK) return st;
-        e = cudaMemcpyAsync(y_host, y_dev, yrow * M, cudaMemcpyDeviceToHost, s);
-        if (e != cudaSuccess) { set_error("cudaMemcpyAsync(D2H)", e); return DIROTQ_ERR_CUDA; }
-        return DIROTQ_OK;
-    }
-    std::lock_guard<std::mutex> lock(g_pipe_mutex);
-    HostPipe* p = nullptr;
-    st = host_pipe(layer->device, &p);
-    if (st != DIROTQ_OK) return st;
-    cudaError_t e = cudaEventRecord(p->start, s);  // the staging buffers may still be in use by earlier work on `stream`
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(p->h2d, p->start, 0);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(p->d2h, p->start, 0);
-    int c = 0;
-    for (int m0 = 0, mc = 0; m0 < M && e == cudaSuccess; m0 += mc, ++c) {
-        const long left = M - m0;
-        mc = static_cast<int>(left <= std::max(384L, 2 * base / 5) ? left : std::max(256L, std::min(rows128(3 * left / 5), m0 ? base : rows128(3 * base / 5))));
-        char* xd = static_cast<char*>(x_dev) + xrow * m0;
-        char* yd = static_cast<char*>(y_dev) + yrow * m0;
-        e = cudaMemcpyAsync(xd, static_cast<const char*>(x_host) + xrow * m0, xrow * mc, cudaMemcpyHostToDevice, p->h2d);
-        if (e == cudaSuccess) e = cudaEventRecord(p->copied[c], p->h2d);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->copied[c], 0);
-        if (e != cudaSuccess) break;
-        st = dirotq_linear(xd, mc, layer, yd, workspace, workspace_bytes, stream);
-        if (st != DIROTQ_OK) return st;
-        e = cudaEventRecord(p->computed[c], s);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(p->d2h, p->computed[c], 0);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(static_cast<char*>(y_host) + yrow * m0, yd, yrow * mc, cudaMemcpyDeviceToHost, p->d2h);
-    }
-    if (e == cudaSuccess) e = cudaEventRecord(p->done, p->d2h);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->done, 0);  // later work on `stream` (and its synchronisation) sees y_host
-    if (e != cudaSuccess) { set_error("host pipeline", e); return DIROTQ_ERR_CUDA; }
-    return DIROTQ_OK;
 }
 
 dirotq_status_t dirotq_workspace_status(const void* workspace, dirotq_stream_t stream, int* device_code) {

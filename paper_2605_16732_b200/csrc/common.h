@@ -305,6 +305,11 @@ dirotq_status_t encode_tmap_2d(CUtensorMap* out, CUtensorMapDataType dt, size_t 
                                uint64_t dim0, uint64_t dim1, uint64_t stride1_bytes, uint32_t box0, uint32_t box1,
                                CUtensorMapSwizzle swz);
 
+// Records the text dirotq_last_error returns on this thread (api.cu).
+void set_error(const char* what, cudaError_t e);
+// What every call on a prepared layer checks of its layer, its workspace and the current device (api.cu).
+dirotq_status_t check_call(const dirotq_layer_t* layer, int M, const void* workspace, size_t workspace_bytes, bool rotates = true);
+
 // launchers (each returns after enqueueing on `stream`)
 dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& a, cudaStream_t stream);
 dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, bool may_split, cudaStream_t stream);  // (not for partials)
