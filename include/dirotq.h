@@ -119,11 +119,15 @@ DIROTQ_API dirotq_status_t dirotq_linear(const void* x, int M, const dirotq_laye
 
 /* Same computation with HOST input and output (pinned memory, or the copies do not overlap):
  * copies x into x_dev, runs dirotq_linear, copies y_dev into y_host; x_dev [M,K] and y_dev [M,N]
- * are device staging buffers of the caller.  For M >= 2048 the call is cut into up to 8 row chunks
- * (token rows are independent) whose two copies run on two copy streams the library creates once
- * per device, overlapping each other and the kernels on `stream`; everything is ordered after the
- * work already on `stream`, and later work on `stream` (or a synchronisation of it) is ordered
- * after the last copy into y_host.  Not for use during stream capture. */
+ * are device staging buffers of the caller.  From 512 rows on the call is cut into up to 32 row chunks
+ * (token rows are independent) whose two copies run on two copy streams that the library creates once
+ * per device, overlapping each other and the kernels on `stream`; everything is ordered after the work
+ * already on `stream`, and later work on `stream` (or a synchronisation of it) is ordered after the
+ * last copy into y_host, also where the call fails.  Calls of 2048 rows and more share their copy
+ * streams, so one queues behind those made before it on other streams; shorter calls wait for no
+ * call on another stream: while one is under way on the short calls' copy streams, another runs in one
+ * piece on its own stream, as calls of fewer than 512 rows and calls on a stream that is being
+ * captured do. */
 DIROTQ_API dirotq_status_t dirotq_linear_host(const void* x_host, int M, const dirotq_layer_t* layer, void* y_host,
                                    void* x_dev, void* y_dev, void* workspace, size_t workspace_bytes,
                                    dirotq_stream_t stream);

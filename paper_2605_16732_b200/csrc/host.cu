@@ -7,33 +7,61 @@
 namespace dirotq {
 namespace {
 
-// Copy streams and events of dirotq_linear_host, created once per device (no device memory involved).
+// Copy streams and events, created when first needed and kept for the device (no device memory involved).
 struct HostPipe {
+    std::mutex mutex;  // held while a call is enqueued: its calls share the events
     bool ready = false;
+    unsigned long long user = 0;  // id of the caller's stream of the last call
     cudaStream_t h2d = nullptr, d2h = nullptr;
     cudaEvent_t start = nullptr, done = nullptr, copied[kMaxHostChunks] = {}, computed[kMaxHostChunks] = {};
 };
-std::mutex g_pipe_mutex;
-HostPipe g_pipe[64];
+// Two pipes per device.  Long calls share one, in the order they are made: their copies fill the link in either direction, and more
+// copy streams would have to share the device's eight queues with the callers' own (the four FLUX layers on four streams: 5.5 ms
+// with one pipe, 5.5 to 6.4 with four).  Short calls wait for nobody: one takes the other pipe if no call of another stream is
+// under way on it, and otherwise stays on its own stream, in one piece.
+constexpr int kLongCallRows = 2048;
+struct DevicePipes {
+    HostPipe long_calls, short_calls;
+} g_device[64];
 
-// Caller holds g_pipe_mutex (also while it enqueues on the pipe: its events are shared by all calls on the device).
-dirotq_status_t host_pipe(int dev, HostPipe** out) {
-    if (dev < 0 || dev >= 64) return DIROTQ_ERR_INVALID_ARG;
-    HostPipe& p = g_pipe[dev];
-    if (!p.ready) {
-        cudaError_t e = cudaStreamCreateWithFlags(&p.h2d, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p.d2h, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p.start, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p.done, cudaEventDisableTiming);
-        for (int i = 0; i < kMaxHostChunks && e == cudaSuccess; ++i) {
-            e = cudaEventCreateWithFlags(&p.copied[i], cudaEventDisableTiming);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p.computed[i], cudaEventDisableTiming);
-        }
-        if (e != cudaSuccess) { set_error("host pipeline set-up", e); return DIROTQ_ERR_CUDA; }
-        p.ready = true;
+// Looking at an event and making streams and events must not disturb a capture that some other thread has under way.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+bool create(HostPipe& p) {
+    auto event = [](cudaEvent_t& e) { return e != nullptr || cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess; };
+    auto streams = [](cudaStream_t& s) { return s != nullptr || cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess; };
+    bool ok = streams(p.h2d) && streams(p.d2h) && event(p.start) && event(p.done);
+    for (int i = 0; i < kMaxHostChunks && ok; ++i) ok = event(p.copied[i]) && event(p.computed[i]);
+    return p.ready = ok;  // (what a failed attempt has made is there for the next one)
+}
+
+// Locks the pipe that a call of M rows on `stream` runs on; an empty lock: the call stays in one piece on its own stream.
+HostPipe* take_pipe(int device, int M, cudaStream_t stream, std::unique_lock<std::mutex>& lock) {
+    if (M < kMinPipelinedRows || device < 0 || device >= 64) return nullptr;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    // (a call that is being captured: the copy streams would be part of the capture until it ends)
+    if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone || cudaStreamGetId(stream, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
     }
-    *out = &p;
-    return DIROTQ_OK;
+    RelaxedCapture relaxed;
+    const bool shares = M >= kLongCallRows;
+    HostPipe& p = shares ? g_device[device].long_calls : g_device[device].short_calls;
+    lock = shares ? std::unique_lock<std::mutex>(p.mutex) : std::unique_lock<std::mutex>(p.mutex, std::try_to_lock);
+    bool ok = lock.owns_lock() && (p.ready || create(p));
+    if (ok && !shares && p.user != id) ok = cudaEventQuery(p.done) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();  // neither a call still under way nor a missing pipe is an error of this call
+        if (lock.owns_lock()) lock.unlock();
+        return nullptr;
+    }
+    p.user = id;
+    return &p;
 }
 
 // The steps of run_host_chunks on a pipe.  The chunks' kernels run one after another on `stream`, so they share the workspace.
@@ -91,7 +119,9 @@ extern "C" dirotq_status_t dirotq_linear_host(const void* x_host, int M, const d
     const size_t xrow = static_cast<size_t>(layer->geo.K) * 2, yrow = static_cast<size_t>(layer->geo.N) * 2;
     // Token rows are independent: the call is cut into row chunks whose host-to-device copy, computation and
     // device-to-host copy overlap (copy engines in both directions + SMs).
-    if (M < kMinPipelinedRows) {
+    std::unique_lock<std::mutex> lock;
+    HostPipe* p = take_pipe(layer->device, M, s, lock);
+    if (!p) {
         cudaError_t e = cudaMemcpyAsync(x_dev, x_host, xrow * M, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) { set_error("cudaMemcpyAsync(H2D)", e); return DIROTQ_ERR_CUDA; }
         st = dirotq_linear(x_dev, M, layer, y_dev, workspace, workspace_bytes, stream);
@@ -100,10 +130,6 @@ extern "C" dirotq_status_t dirotq_linear_host(const void* x_host, int M, const d
         if (e != cudaSuccess) { set_error("cudaMemcpyAsync(D2H)", e); return DIROTQ_ERR_CUDA; }
         return DIROTQ_OK;
     }
-    std::lock_guard<std::mutex> lock(g_pipe_mutex);
-    HostPipe* p = nullptr;
-    st = host_pipe(layer->device, &p);
-    if (st != DIROTQ_OK) return st;
     int rows[kMaxHostChunks];
     const int n = plan_host_chunks(M, xrow, yrow, rows);
     PipeOps ops = {*p, s, layer, static_cast<const char*>(x_host), static_cast<char*>(y_host), static_cast<char*>(x_dev), static_cast<char*>(y_dev),
