@@ -127,10 +127,18 @@ def _check(st: int, where: str):
         raise DirotqError(st, where, lib().dirotq_last_error().decode())
 
 
+# torch's own way to the current stream's handle without a Stream object, which takes 3 of a small call's 10 us to build.  Not
+# part of its public interface: a torch that has no such functions gets the object.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream=None) -> int:
-    if stream is None:  # the handle alone: building a torch.cuda.Stream object first took 3 of a small call's 10 us
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
-    return stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _current_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 def _ptr(t):
