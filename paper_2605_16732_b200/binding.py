@@ -141,6 +141,25 @@ def _stream(stream=None) -> int:
     return _raw_stream(_current_device())
 
 
+class _PrepareStream:
+    """Around a prepare call that runs on `stream` with buffers that were allocated, and some of them cleared, on the current
+    stream: `stream` comes after them, and has finished when the scratch goes back to the current stream's allocator."""
+
+    def __init__(self, stream):
+        self.stream = stream
+
+    def __enter__(self):
+        if self.stream is not None:
+            self.stream.wait_stream(torch.cuda.current_stream())
+
+    def __exit__(self, exc_type, *_):
+        try:
+            (torch.cuda.current_stream() if self.stream is None else self.stream).synchronize()
+        except RuntimeError:
+            if exc_type is None:  # (else the call's own error is the one to report)
+                raise
+
+
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
@@ -200,11 +219,11 @@ def dirotq_prepare_layer(W: torch.Tensor, Q: torch.Tensor, r: int, group: int, b
     scratch_bytes = dirotq_prepare_scratch_bytes(K, N)
     scratch = _alloc_bytes(scratch_bytes, W.device)
     handle = ctypes.c_void_p(0)
-    st = lib().dirotq_prepare_layer(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), K, N, r, group,
-                                    blob.data_ptr(), blob.numel(), scratch.data_ptr(), scratch_bytes, _stream(stream),
-                                    ctypes.byref(handle))
-    _check(st, "dirotq_prepare_layer")
-    torch.cuda.current_stream().synchronize()  # scratch is released when this function returns
+    with _PrepareStream(stream):
+        st = lib().dirotq_prepare_layer(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), K, N, r, group,
+                                        blob.data_ptr(), blob.numel(), scratch.data_ptr(), scratch_bytes, _stream(stream),
+                                        ctypes.byref(handle))
+        _check(st, "dirotq_prepare_layer")
     return Layer(handle.value, blob, K, N, r, group)
 
 
@@ -308,7 +327,7 @@ def dirotq_mma_rate_probe(kind: int, iters: int = 20000, stream=None) -> float:
 def dirotq_act_scale_log2_from_rotated(xrot: torch.Tensor, r: int, stream=None) -> int:
     """Exponent of the NVFP4 activations' power-of-two scale from fp32 rotated calibration activations [M, K]."""
     assert xrot.is_cuda and xrot.is_contiguous() and xrot.dtype == torch.float32
-    word = torch.zeros(1, dtype=torch.int32, device=xrot.device)
+    word = torch.empty(1, dtype=torch.int32, device=xrot.device)  # (the call clears it, on its own stream)
     out = ctypes.c_int(0)
     _check(lib().dirotq_act_scale_log2_from_rotated(xrot.data_ptr(), xrot.shape[0], xrot.shape[1], int(r), word.data_ptr(),
                                                     ctypes.byref(out), _stream(stream)), "dirotq_act_scale_log2_from_rotated")
@@ -361,11 +380,11 @@ def dirotq_prepare_layer_nvfp4(W: torch.Tensor, Q: torch.Tensor, r: int, act_sca
     scratch_bytes = dirotq_prepare_scratch_bytes(K, N)
     scratch = _alloc_bytes(scratch_bytes, W.device)
     handle = ctypes.c_void_p(0)
-    st = lib().dirotq_prepare_layer_nvfp4(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), K, N, r,
-                                          int(act_scale_log2), blob.data_ptr(), blob.numel(), scratch.data_ptr(),
-                                          scratch_bytes, _stream(stream), ctypes.byref(handle))
-    _check(st, "dirotq_prepare_layer_nvfp4")
-    torch.cuda.current_stream().synchronize()
+    with _PrepareStream(stream):
+        st = lib().dirotq_prepare_layer_nvfp4(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), K, N, r,
+                                              int(act_scale_log2), blob.data_ptr(), blob.numel(), scratch.data_ptr(),
+                                              scratch_bytes, _stream(stream), ctypes.byref(handle))
+        _check(st, "dirotq_prepare_layer_nvfp4")
     return Layer(handle.value, blob, K, N, r, 16, fmt="nvfp4")
 
 
@@ -416,11 +435,11 @@ def dirotq_prepare_layer_asym(W: torch.Tensor, Q: torch.Tensor, r: int, group: i
     scratch_bytes = dirotq_prepare_scratch_bytes(K, N)
     scratch = _alloc_bytes(scratch_bytes, W.device)
     handle = ctypes.c_void_p(0)
-    st = lib().dirotq_prepare_layer_asym(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), K, N, r, group,
-                                         blob.data_ptr(), blob.numel(), scratch.data_ptr(), scratch_bytes, _stream(stream),
-                                         ctypes.byref(handle))
-    _check(st, "dirotq_prepare_layer_asym")
-    torch.cuda.current_stream().synchronize()
+    with _PrepareStream(stream):
+        st = lib().dirotq_prepare_layer_asym(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), K, N, r, group,
+                                             blob.data_ptr(), blob.numel(), scratch.data_ptr(), scratch_bytes, _stream(stream),
+                                             ctypes.byref(handle))
+        _check(st, "dirotq_prepare_layer_asym")
     return Layer(handle.value, blob, K, N, r, group, fmt="int4_asym")
 
 
@@ -442,11 +461,11 @@ def dirotq_prepare_layer_sibling(W: torch.Tensor, Q: torch.Tensor, r: int, group
     scratch_bytes = dirotq_prepare_scratch_bytes(K, N)
     scratch = _alloc_bytes(scratch_bytes, W.device)
     handle = ctypes.c_void_p(0)
-    st = lib().dirotq_prepare_layer_sibling(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), int(asym), K, N, r, group,
-                                            blob.data_ptr(), blob.numel(), scratch.data_ptr(), scratch_bytes, _stream(stream),
-                                            ctypes.byref(handle))
-    _check(st, "dirotq_prepare_layer_sibling")
-    torch.cuda.current_stream().synchronize()
+    with _PrepareStream(stream):
+        st = lib().dirotq_prepare_layer_sibling(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), int(asym), K, N, r, group,
+                                                blob.data_ptr(), blob.numel(), scratch.data_ptr(), scratch_bytes, _stream(stream),
+                                                ctypes.byref(handle))
+        _check(st, "dirotq_prepare_layer_sibling")
     return Layer(handle.value, blob, K, N, r, group, fmt="int4_asym" if asym else "int4")
 
 
@@ -464,11 +483,11 @@ def dirotq_prepare_layer_ph(W: torch.Tensor, Uh: torch.Tensor, group: int, bias:
     blob = _alloc_bytes(nb.value, W.device)
     scratch = _alloc_bytes(ns.value, W.device)
     handle = ctypes.c_void_p(0)
-    st = lib().dirotq_prepare_layer_ph(_ptr(W), w_dtype, w_layout, _ptr(Uh), uh_dtype, _ptr(bias), K, N, r, group,
-                                       blob.data_ptr(), blob.numel(), scratch.data_ptr(), ns.value, _stream(stream),
-                                       ctypes.byref(handle))
-    _check(st, "dirotq_prepare_layer_ph")
-    torch.cuda.current_stream().synchronize()
+    with _PrepareStream(stream):
+        st = lib().dirotq_prepare_layer_ph(_ptr(W), w_dtype, w_layout, _ptr(Uh), uh_dtype, _ptr(bias), K, N, r, group,
+                                           blob.data_ptr(), blob.numel(), scratch.data_ptr(), ns.value, _stream(stream),
+                                           ctypes.byref(handle))
+        _check(st, "dirotq_prepare_layer_ph")
     return Layer(handle.value, blob, K, N, r, group, fmt="int4_ph")
 
 
@@ -486,11 +505,11 @@ def dirotq_prepare_layer_nvfp4_ph(W: torch.Tensor, Uh: torch.Tensor, act_scale_l
     blob = _alloc_bytes(nb.value, W.device)
     scratch = _alloc_bytes(ns.value, W.device)
     handle = ctypes.c_void_p(0)
-    st = lib().dirotq_prepare_layer_nvfp4_ph(_ptr(W), w_dtype, w_layout, _ptr(Uh), uh_dtype, _ptr(bias), K, N, r,
-                                             int(act_scale_log2), blob.data_ptr(), blob.numel(), scratch.data_ptr(), ns.value,
-                                             _stream(stream), ctypes.byref(handle))
-    _check(st, "dirotq_prepare_layer_nvfp4_ph")
-    torch.cuda.current_stream().synchronize()
+    with _PrepareStream(stream):
+        st = lib().dirotq_prepare_layer_nvfp4_ph(_ptr(W), w_dtype, w_layout, _ptr(Uh), uh_dtype, _ptr(bias), K, N, r,
+                                                 int(act_scale_log2), blob.data_ptr(), blob.numel(), scratch.data_ptr(), ns.value,
+                                                 _stream(stream), ctypes.byref(handle))
+        _check(st, "dirotq_prepare_layer_nvfp4_ph")
     return Layer(handle.value, blob, K, N, r, 16, fmt="nvfp4_ph")
 
 
@@ -545,11 +564,11 @@ def dirotq_prepare_layer_codes(W: torch.Tensor, Q: torch.Tensor, wcodes: torch.T
     scratch_bytes = dirotq_prepare_scratch_bytes(K, N)
     scratch = _alloc_bytes(scratch_bytes, W.device)
     handle = ctypes.c_void_p(0)
-    st = lib().dirotq_prepare_layer_codes(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), wcodes.data_ptr(),
-                                          wscales.data_ptr(), int(asym), K, N, r, group, blob.data_ptr(), blob.numel(),
-                                          scratch.data_ptr(), scratch_bytes, _stream(stream), ctypes.byref(handle))
-    _check(st, "dirotq_prepare_layer_codes")
-    torch.cuda.current_stream().synchronize()
+    with _PrepareStream(stream):
+        st = lib().dirotq_prepare_layer_codes(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), wcodes.data_ptr(),
+                                              wscales.data_ptr(), int(asym), K, N, r, group, blob.data_ptr(), blob.numel(),
+                                              scratch.data_ptr(), scratch_bytes, _stream(stream), ctypes.byref(handle))
+        _check(st, "dirotq_prepare_layer_codes")
     return Layer(handle.value, blob, K, N, r, group, fmt="int4_asym" if asym else "int4")
 
 
@@ -569,11 +588,11 @@ def dirotq_prepare_layer_gptq(W: torch.Tensor, Q: torch.Tensor, calib_x: torch.T
     _check(lib().dirotq_prepare_scratch_bytes_gptq(K, N, r, calib_x.shape[0], ctypes.byref(need)), "dirotq_prepare_scratch_bytes_gptq")
     scratch = _alloc_bytes(need.value, W.device)
     handle = ctypes.c_void_p(0)
-    st = lib().dirotq_prepare_layer_gptq(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), calib_x.data_ptr(),
-                                         calib_x.shape[0], float(damp), int(block), int(asym), K, N, r, group, blob.data_ptr(),
-                                         blob.numel(), scratch.data_ptr(), need.value, _stream(stream), ctypes.byref(handle))
-    _check(st, "dirotq_prepare_layer_gptq")
-    torch.cuda.current_stream().synchronize()
+    with _PrepareStream(stream):
+        st = lib().dirotq_prepare_layer_gptq(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), calib_x.data_ptr(),
+                                             calib_x.shape[0], float(damp), int(block), int(asym), K, N, r, group, blob.data_ptr(),
+                                             blob.numel(), scratch.data_ptr(), need.value, _stream(stream), ctypes.byref(handle))
+        _check(st, "dirotq_prepare_layer_gptq")
     return Layer(handle.value, blob, K, N, r, group, fmt="int4_asym" if asym else "int4")
 
 
@@ -615,11 +634,11 @@ def dirotq_prepare_layer_w4a8(W: torch.Tensor, Q: torch.Tensor, r: int, bias: to
     scratch_bytes = dirotq_prepare_scratch_bytes(K, N)
     scratch = _alloc_bytes(scratch_bytes, W.device)
     handle = ctypes.c_void_p(0)
-    st = lib().dirotq_prepare_layer_w4a8(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), K, N, r, blob.data_ptr(),
-                                         blob.numel(), scratch.data_ptr(), scratch_bytes, _stream(stream),
-                                         ctypes.byref(handle))
-    _check(st, "dirotq_prepare_layer_w4a8")
-    torch.cuda.current_stream().synchronize()
+    with _PrepareStream(stream):
+        st = lib().dirotq_prepare_layer_w4a8(_ptr(W), w_dtype, w_layout, _ptr(Q), q_dtype, _ptr(bias), K, N, r, blob.data_ptr(),
+                                             blob.numel(), scratch.data_ptr(), scratch_bytes, _stream(stream),
+                                             ctypes.byref(handle))
+        _check(st, "dirotq_prepare_layer_w4a8")
     return Layer(handle.value, blob, K, N, r, 128, fmt="w4a8")
 
 

@@ -127,3 +127,32 @@ def test_threads_on_their_own_streams_and_layers_that_come_and_go():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+def test_prepare_on_another_stream():
+    """The call's scratch, and a blob that starts cleared, come from the current stream: neither is touched from there while a busy stream
+    still prepares the layer."""
+    g = torch.Generator(device="cuda").manual_seed(8)
+    Q = torch.linalg.qr(torch.randn(K, K, generator=g, device="cuda", dtype=torch.float64))[0].contiguous()
+    W = 0.02 * torch.randn(K, N, generator=g, device="cuda")
+    side = torch.cuda.Stream()
+
+    def busy(s):
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(int(4e7))  # about 20 ms
+
+    for prepare, export in ((lambda **kw: dq.dirotq_prepare_layer(W, Q, R, 64, **kw), dq.dirotq_layer_export),
+                            (lambda **kw: dq.dirotq_prepare_layer_nvfp4(W, Q, R, 0, **kw), dq.dirotq_layer_export_nvfp4)):
+        plain = prepare()
+        want = [t.clone() for t in export(plain) if isinstance(t, torch.Tensor)]
+        torch.cuda.synchronize()
+        for late in (side, torch.cuda.current_stream()):  # the preparing stream is behind, then the current one
+            busy(late)
+            layer = prepare(stream=side)
+            junk = [torch.full((K * N,), float("nan"), dtype=torch.float64, device="cuda") for _ in range(3)]  # where the scratch was
+            torch.cuda.synchronize()
+            got = [t for t in export(layer) if isinstance(t, torch.Tensor)]
+            assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(got, want))
+            layer.close()
+            del junk
+        plain.close()
