@@ -28,18 +28,21 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 // The driver entry point is looked up at run time so that the library loads on machines
 // without a driver (build hosts); any call that needs it fails with DIROTQ_ERR_CUDA there.
-EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+// (A function-local static: threads that come here together all wait for the one look-up.  A failed one is not repeated.)
+struct EncodeLookup {
+    EncodeTiledFn fn = nullptr;
+    cudaError_t error = cudaSuccess;
+    EncodeLookup() {
         void* p = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres);
-        if (e == cudaSuccess && qres == cudaDriverEntryPointSuccess) fn = reinterpret_cast<EncodeTiledFn>(p);
-        else set_error("cudaGetDriverEntryPoint(cuTensorMapEncodeTiled)", e);
+        cudaDriverEntryPointQueryResult found;
+        error = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &found);
+        if (error == cudaSuccess && found == cudaDriverEntryPointSuccess) fn = reinterpret_cast<EncodeTiledFn>(p);
     }
-    return fn;
+};
+EncodeTiledFn encode_fn() {
+    static const EncodeLookup lookup;
+    if (!lookup.fn) set_error("cudaGetDriverEntryPoint(cuTensorMapEncodeTiled)", lookup.error);
+    return lookup.fn;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -69,14 +72,14 @@ dirotq_status_t check_device(int* device_out) {
 }  // namespace
 
 int sm_count(int device) {
-    static int cached[64] = {0};
+    static std::atomic<int> cached[64];
     if (device < 0 || device >= 64) return 148;
-    if (cached[device] == 0) {
-        int n = 0;
+    int n = cached[device].load(std::memory_order_relaxed);
+    if (n == 0) {
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || n <= 0) n = 148;
-        cached[device] = n;
+        cached[device].store(n, std::memory_order_relaxed);
     }
-    return cached[device];
+    return n;
 }
 
 dirotq_status_t encode_tmap_2d(CUtensorMap* out, CUtensorMapDataType dt, size_t elem_bytes, const void* base,
