@@ -357,8 +357,8 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         // 16x256b shape: a thread then holds 4 rows (l/4 + 8 i) x the column pairs 2 (l%4) + {0, 1} of every block
         // of 8 columns, so one load of weight scales serves four rows (with the 32x32b shape, one row per thread,
         // every thread would need all 128 column scales of every group and the shared-memory pipe, not the FMA
-        // pipe, would bound the kernel).  A chunk is 32 columns: two .x4 loads (TMEM lanes 0..15 and 16..31 of the
-        // quadrant), 32 values per thread, and the 8 weight scales of the thread's columns, which the layer stores
+        // pipe, would bound the kernel).  A chunk is 32 columns: TMEM lanes 0..15 and 16..31 of the quadrant, 32 values
+        // per thread (see request_chunk), and the 8 weight scales of the thread's columns, which the layer stores
         // side by side (see wscale_index in common.h), in two 16-byte loads.
         //
         // The accumulator tiles of an output tile (one per K-group, then the rank-r one) are one stream: while the
@@ -380,12 +380,13 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         bool ok = true;
         uint32_t raw[2][32];  // [0..15]: TMEM lanes 0..15 of the quadrant (rows i = 0, 1), [16..31]: lanes 16..31
         auto request_chunk = [&](uint32_t buf, int c, uint32_t* dst) {
-            // 32 columns move in 32 cycles as two .x2 loads and in 64 as one .x4; where a single tile's hand-overs set the time (128
-            // columns) fewer instructions are worth more (32.3 against 32.8 us for 27 tokens of 7424 -> 11600)
+            // 32 columns move in 32 cycles as two .x2 loads and in 64 as one .x4, which is half the instructions.  Measured on 18 layers, .x2 is
+            // ahead by up to 4 %, except in 128-column tiles with groups of 128, where .x4 is by 1 to 2 %.  .x2 / .x4 in us, 4608 -> 1152
+            // at 4096 tokens: 256 columns 91.5 / 92.4 (groups of 64), 64.2 / 65.3 (of 128); 128 columns 55.7 / 55.9, 39.7 / 39.0.
             const uint32_t t = taddr0 + buf * BN + c * 32;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                if constexpr (BN == 128) {
+                if constexpr (BN == 128 && G == 128) {
                     tmem_ld_16x256b_x4(t + (static_cast<uint32_t>(h) << 20), dst + 16 * h);
                 } else {
                     tmem_ld_16x256b_x2(t + (static_cast<uint32_t>(h) << 20), dst + 16 * h);
