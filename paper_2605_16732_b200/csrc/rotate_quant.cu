@@ -657,8 +657,8 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         const __nv_bfloat16 zb = __float2bfloat16_rn(lo);
                         const float z = __bfloat162float(zb);
                         const float s = hi > lo ? __bfloat162float(__float2bfloat16_rn(__fdiv_rn(hi - lo, 15.0f))) : 0.f;
-                        const bool slow = !(s >= 1e-30f);
-                        const float inv = slow ? 0.f : __frcp_rn(s);
+                        const bool tiny = !(s >= 1e-30f), slow = tiny && row_ok;  // (as for symmetric codes)
+                        const float inv = tiny ? 0.f : __frcp_rn(s);
                         int8_t* crow = p.codes + static_cast<size_t>(row) * p.K_lp + col0;
                         if constexpr (STAGED) {
                             if (lane == 0) bulk_wait_group_read_all();
@@ -712,8 +712,10 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     }
                     const float amax = fmaxf(fmaxf(am[0], am[1]), fmaxf(am[2], am[3])) * kPre;
                     const float s = __bfloat162float(__float2bfloat16_rn(__fdiv_rn(amax, 7.0f)));
-                    const bool slow = !(s >= 1e-30f);  // zero or tiny scale: divide instead of multiplying
-                    const float inv = slow ? 0.f : __frcp_rn(s) * kPre;
+                    // zero or tiny scale: divide instead of multiplying (not for rows past M: their zeros are not stored, and a tile's
+                    // epilogue takes twice as long with the divisions)
+                    const bool tiny = !(s >= 1e-30f), slow = tiny && row_ok;
+                    const float inv = tiny ? 0.f : __frcp_rn(s) * kPre;
                     int8_t* crow = p.codes + static_cast<size_t>(row) * p.K_lp + col0;
                     if constexpr (STAGED) {
                         if (lane == 0) bulk_wait_group_read_all();  // the staging tile's previous contents have been read
