@@ -867,11 +867,8 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
     p.codes = a.codes; p.xscale = a.xscale; p.xh = a.xh; p.xrot = a.xrot; p.status = a.status;
     p.xsf = a.xsf; p.K4 = g.K4; p.nkb64p = g.nkb64p; p.ex = L->act_scale_log2;
     p.xtilde = a.xtilde;
-    // Tile plan.  128 x 256 is the default.  128 x 128 when the wide tiles would not give every SM about two of them
-    // (few, large tiles leave a nearly empty last wave: 160 tiles on 148 SMs take as long as 296).  256 x 256 (a third
-    // fewer operand bytes per flop, but the epilogue, about 11 k-blocks' worth, is not overlapped) for long main
-    // loops only: measured 0.99 -> 0.92 ms at M = 4608, K = 12288 and 1.54 -> 1.48 ms at K = 15360, but 0.125 ->
-    // 0.141 ms at M = 9216, K = 3072.
+    // Tile plan: the one with the shortest schedule, turns of the SMs (or pairs of SMs) x what a tile costs.  Times below are of this kernel
+    // on symmetric INT4 codes, each plan forced, bursts of 2 ms unless stated.
     const int sms = sm_count(L->device);
     const long mb128 = (a.M + 127) / 128, mb256 = (a.M + 255) / 256, nb128 = (g.K + 127) / 128, nb256 = (g.K + 255) / 256;
     // 128 x 128 tiles (plan 1) are computed in CTA pairs, 256 x 128 per pair, wherever that does not take more turns (not for up to
@@ -882,29 +879,32 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
     int plan = g_rotation_plan.load();
     if (plan == 0) {
         const long waves128 = (mb128 * nb256 + sms - 1) / sms, waves256 = (mb256 * nb256 + sms - 1) / sms;
+        const long turns_pair_wide = (mb256 * nb256 + sms / 2 - 1) / (sms / 2);
         const long waves_narrow = pairs_narrow ? turns_pair : turns_single;
         const double kb = static_cast<double>(g.K / BK);
         // a 256-row tile in units of a 128-row tile; once x no longer fits the L2 beside the rotation the 128-row plan
         // re-reads it from HBM and the ratio falls to 1.9 (measured at M = 18432, K = 3072: 0.304 -> 0.288 ms)
         const bool x_exceeds_l2 = static_cast<double>(a.M) * g.K * 2.0 > 96e6;
         const double cost256 = x_exceeds_l2 ? 1.9 : 1.86 + 11.0 / kb;
-        // a 128-column tile costs about 0.62 of a 256-column one: narrow tiles when that shortens the schedule (few
-        // tiles: M = 256, K = 1152 runs on 18 instead of 10 SMs; M = 4096, K = 1152: 288 tiles in two waves instead of
-        // 160 in two), not otherwise (M = 1024, K = 3072: 96 wide tiles in one wave, 30 us, against 192 narrow ones in
-        // two, 45 us)
         // few token rows: when even the 128-column tiles would keep fewer than half of the SMs busy, 64-column tiles (eight
         // 24 KB stages) on twice as many: every CTA streams all of x's row block and its own columns of the rotation through
         // one SM's port to L2, so the time of a call this small falls with the bytes per CTA
         if (2 * mb128 * nb128 <= sms && g.G == 64) plan = 5;
+        // a turn of 128 x 128 tiles costs 0.57 to 0.60 of one of 128 x 256 tiles where there are several (4096 tokens, K = 3072, 4608 and
+        // 12288) and 0.73 to 0.82 where there is one; 0.62 takes them at equal turns (K = 3072, 512 tokens: 14.1 against 18.5 us) and up
+        // to 1.6 times as many (2048 tokens: 3 against 2 turns, 35.3 against 37.3), not at 2 against 1 (1000 tokens: 23.0 against 20.2)
         else if (0.62 * static_cast<double>(waves_narrow) < static_cast<double>(waves128)) plan = 1;
-        // long main loops, all pairs resident at once: the rotation streams from HBM, and plan 2 reads it once per 128 rows (M = 256,
-        // K = 12288: 101 -> 87 us)
-        else if (g.K >= 8192 && a.M > 128 && mb256 * nb256 <= sms / 2) plan = 4;
+        // 256 x 256: a third fewer operand bytes per flop, but the epilogue, about 11 k-blocks' worth, is not overlapped: for long main
+        // loops, and at the power cap.  K = 12288, 4608 tokens, against 128 x 256 tiles and CTA pairs: 1070, 1107, 1032 us in bursts,
+        // 1041, 1131, 1070 over 150 ms; 9216 tokens over 150 ms 2319, 2573, 2449
         else if ((g.K >= 8192 || x_exceeds_l2) && cost256 * static_cast<double>(waves256) < 0.98 * static_cast<double>(waves128)) plan = 3;
-        // CTA pairs where there are a few waves of tiles and the main loop is not long enough for the operand traffic
-        // to hide behind the MMAs anyway (measured against 128 x 256 tiles: M = 4608, K = 3072 68.4 -> 67.3 us; M = 9216,
-        // K = 3072 122 -> 114; M = 4096, K = 4608 124 -> 111; at K = 12288 and 15360 the 256-row plan stays ahead)
-        else if (mb128 * nb256 >= 5 * sms / 2 && g.K < 8192) plan = 4;
+        // CTA pairs (256 x 256 per pair): the rotation is read once per 256 rows, 32 instead of 48 KB per CTA and k-block, and a turn costs
+        // 0.84 to 0.93 of one of 128 x 256 tiles.  From K = 6144 on at any number of turns (against 128 x 256 tiles: K = 6144, 512 tokens
+        // 40.0 -> 36.0 us; K = 8192, 1536 tokens 165 -> 147, 4096 399 -> 361; K = 12288, 1000 tokens 277 -> 249, 4096 992 -> 924), below
+        // where there are a few turns (K = 3072: 3 turns 65.1 -> 61.1, 1 turn 20.2 -> 20.7; K = 4608: 4 turns 128 -> 117, 1 turn 29.9 either
+        // way).  A pair covers 256 rows, so odd row counts can cost it a turn (K = 3072, 4736 tokens: 4 against 3, 64.8 against 61.0)
+        else if (a.M > 128 && 0.88 * static_cast<double>(turns_pair_wide) <= static_cast<double>(waves128) && (g.K >= 6144 || mb128 * nb256 >= 5 * sms / 2))
+            plan = 4;
         else plan = 2;
     }
     if (plan == 5 && g.G != 64) plan = 1;  // a tile holds whole groups
