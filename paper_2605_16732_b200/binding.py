@@ -527,13 +527,15 @@ def dirotq_layer_export_v(layer: Layer, stream=None) -> torch.Tensor:
 
 
 def dirotq_set_gemm_tile(columns: int) -> None:
-    """Output columns per tile of the INT4 and NVFP4 second kernels: 0 automatic, 128 or 256 forced (process-wide)."""
+    """Tile plan of the second kernels (process-wide): 0 automatic; 128 or 256 columns per tile; 64, 66 (the reduction split over a
+    cluster) and 192: plans of the INT4 kernels only; 512: CTA pairs with 256 columns, of the NVFP4 and W4A8 kernels (for W4A8 128 is
+    single CTAs, 256 CTA pairs with 128 columns)."""
     _check(lib().dirotq_set_gemm_tile(int(columns)), "dirotq_set_gemm_tile")
 
 
 def dirotq_set_rotation_tile(plan: int) -> None:
-    """Tile plan of the rotation kernel: 0 automatic, 1 = 128x128, 2 = 128x256, 3 = 256x256, 4 = 256x256 per pair of CTAs sharing
-    every MMA (process-wide)."""
+    """Tile plan of the rotation kernel (process-wide): 0 automatic, 1 = 128x128 (above 128 tokens in CTA pairs where that takes no
+    more turns), 2 = 128x256, 3 = 256x256, 4 = 256x256 per pair of CTAs sharing every MMA, 5 = 128x64 (groups of 64 only)."""
     _check(lib().dirotq_set_rotation_tile(int(plan)), "dirotq_set_rotation_tile")
 
 

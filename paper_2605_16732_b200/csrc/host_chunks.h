@@ -9,10 +9,15 @@ namespace dirotq {
 constexpr int kMaxHostChunks = 32;
 constexpr int kMinPipelinedRows = 512;  // shorter calls stay in one piece
 
-// A full chunk is about 8 MB of the larger side (smaller ones pay more for starting copies, about 15 us each, and, with few rows, more per
-// row for the kernels), but a good quarter of a short call, and at least 256 rows.  The first one and the last ones are
-// shorter: the first copy in, and the last rows' computation and copy out, overlap with nothing.  4608 x 3072 -> 3072: 915 us
-// in four equal chunks, 850 tapered; 1024 x 3072 -> 3072 311 us in one piece, 236 in chunks.
+// What a chunk costs beside its bytes is about 15 us for starting its copies and, with few rows, more per row for the kernels (at
+// least 256 rows); what it saves is overlap, of which the first copy in and the last rows' computation and copy out have none.  So a full
+// chunk is about 8 MB of the larger side, of a short call a little over a quarter (10 / 37: 4608 rows of 3072 are 768 + 1280 + 1280 + 768 +
+// 512, where an exact quarter leaves a sixth chunk of 128), of a long one at least M / 24 rows (the event tables hold 32 chunks), the first one
+// three fifths of that, and the end is cut in fifths 3 : 2 while it is longer than 384 rows or two fifths of a chunk.
+// Measured from pinned memory, us, before (one piece below 2048 rows, up to eight equal chunks above) / after: 3072 -> 3072 at 1024,
+// 4608 and 9216 rows 386 / 258, 889 / 829, 1662 / 1578; 1152 -> 4608 at 1024 258 / 237; 12288 -> 12288 at 4608 3401 / 2872; the widest
+// layers' many chunks each read their rotation again and still gain up to some 5000 rows: 12288 -> 3072 at 1024, 4608 and 9216
+// 936 / 694, 2593 / 2504, 4700 / 4841.  Chunks that grow with the root of the call's bytes come out the same on average.
 // `xrow`, `yrow`: bytes of a token row in and out.  Returns the number of chunks, whose sizes it writes to `rows`.
 inline int plan_host_chunks(int M, size_t xrow, size_t yrow, int rows[kMaxHostChunks]) {
     constexpr size_t CHUNK_BYTES = 8u << 20;

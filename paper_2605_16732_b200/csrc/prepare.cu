@@ -50,7 +50,7 @@ __device__ __forceinline__ double load_w(const void* W, int w_dtype, int w_layou
 // Bound by fp64 arithmetic: 28 TFLOP/s at 3072^3.  Eight 8-byte loads per lane feed 16 instructions of 256 multiply-adds; with
 // scalar multiply-adds (8 x 4 per thread) their register operands held the pipe at 55 %.  The next tile's loads are in flight
 // under the arithmetic and are held in their own type (converted at once, every tile waited for them).  Preparation and export,
-// 1152 -> 4608: 1595 us with a scalar 4 x 4 per thread, 682 with 8 x 4, 524 now.
+// 1152 -> 4608: 1595 us with a scalar 4 x 4 per thread, 682 with 8 x 4, 508 now.
 constexpr int FOLD_I = 64, FOLD_N = 64, FOLD_THREADS = 128;
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return static_cast<double>(v); }

@@ -101,8 +101,8 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
     const int kb1 = SPLITK ? kb0 + split_base + (static_cast<int>(crank) < split_rest ? 1 : 0) : p.num_kb;
     const int g0 = SPLITK ? kb0 * GPK : 0, g1 = SPLITK ? min(kb1 * GPK, p.n_g) : p.n_g;
     const int lr_here = gathers ? p.lr_chunks : 0;
-    // (tile loops read these where they are needed, like blockIdx.x and gridDim.x themselves: held in registers across the
-    // roles' loops they cost the 256-column plan spills)
+    // (tile loops read these where they are needed, like blockIdx.x and gridDim.x themselves, not held in registers across the
+    // roles' loops)
     auto first_tile = [&]() { return SPLITK ? static_cast<int>(blockIdx.x / csize) : static_cast<int>(blockIdx.x); };
     auto tile_stride = [&]() { return SPLITK ? static_cast<int>(gridDim.x / csize) : static_cast<int>(gridDim.x); };
     const uint32_t red_bar = bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 9);  // split plan: "partial tiles landed" (last CTA)
