@@ -5,8 +5,8 @@
 // long as the chain: more, narrower tiles on more SMs, and a short chain.  A tensor-memory buffer holds the accumulator tiles
 // of ALL groups of a k-block of 128 codes, so there is one hand-over per k-block where w4a4_gemm.cu has one per group; the
 // two unpack warps take k-blocks in turn (half of a turn is waiting); the epilogue asks for a unit's scales with the unit.
-// With groups of 64 a k-block takes 780 cycles, with one hand-over per group it took 1060: 1152 -> 1152 at
-// 256 tokens 12.7 -> 8.9 thousand cycles, 3072 -> 9216 at 16 tokens 18.0 -> 15.5 us.
+// With groups of 64 a k-block takes 760 to 780 cycles, with one hand-over per group it took 1060: 1152 -> 1152 at
+// 256 tokens (replayed from a graph) 8.6 -> 6.9 us, 3072 -> 9216 at 16 tokens 18.0 -> 15.5.
 //
 // Roles (384 threads = 3 warpgroups):
 //   warpgroup 0: warp 0 TMA producer, warp 1 MMA issuer + TMEM owner, warps 2-3 nibble -> byte unpack (k-blocks in turn)

@@ -10,8 +10,8 @@
 // the operand buffer and four unpack warps expand them in place, turning every nibble into the byte 16 q (shift the nibble into the high half, flip
 // bit 7: 16 (q + 8) - 128), so the accumulator holds 16 P and the epilogue shifts it back.
 //
-// This kernel computes 128 x 128 tiles on single CTAs, for calls of at most 128 token rows and where the CTA pairs of w4a8_pair.cu would
-// need as many turns (and for the export of the integer sums).  448 threads: warp 0 TMA producer, warp 1 MMA issuer + TMEM
+// This kernel computes 128 x 128 tiles on single CTAs, for calls of at most 128 token rows (above that the CTA pairs of w4a8_pair.cu
+// run) and for the export of the integer sums.  448 threads: warp 0 TMA producer, warp 1 MMA issuer + TMEM
 // owner, warps 2..5 unpack, warps 6..13 epilogue (one token row per thread, two warps per lane quadrant).  Two accumulator
 // sets alternate in tensor memory, so a tile's epilogue runs under the next tile's MMAs; a set is the int32 tile and the
 // fp32 tile of the bf16 rank-r branch (kind::f16 cannot accumulate into the integer tile).
@@ -446,8 +446,10 @@ dirotq_status_t set_w4a8_tile_columns(int columns) {
 
 dirotq_status_t launch_w4a8_gemm(const dirotq_layer* L, const A8GemmArgs& a, cudaStream_t stream) {
     // A CTA pair takes 256 token rows at once, so calls of at most 128 rows keep single CTAs.  Otherwise the wide pair plan runs
-    // wherever it does not need clearly more turns: per turn the narrow one costs 0.85 of it (31 against 34 us for 4096 x 4608
-    // -> 1152 with two turns each, 160 against 100 us for 4608 x 3072 -> 9216 with 18 and 9), single CTAs 0.95.
+    // wherever it does not need clearly more turns: per turn the narrow one costs 0.85 to 0.9 of it (30 against 34 us for 4096 x 4608
+    // -> 1152 with two turns each, 161 against 101 us for 4608 x 3072 -> 9216 with 18 and 9).  Single CTAs above 128 rows take 14.4 us
+    // where pairs take 13.6 (256 x 3072 -> 9216), 188 against 101 (4608), and are ahead on the smallest layers alone (512 x 512 ->
+    // 512: 5.9 against 6.6).
     const int forced = g_a8_tile_columns.load();
     const int pairs = sm_count(L->device) / 2;
     const long m_blocks = (a.M + 2 * BM - 1) / (2 * BM);

@@ -10,7 +10,7 @@
 // arriving, 8 + 16 for the expansion and 32 for the tensor core per CTA, on three rings with depths of their own (codes, packed
 // weights, expanded weights), the expansion done by three teams of two warps that take k-blocks in turn (one team's turn is
 // mostly waiting).  A k-block takes 650 cycles, of which the MMAs 512.  Second kernel, before -> after: 4608 x 3072 -> 9216 165 ->
-// 100 us (2.6 POP/s), 1024 x 3072 -> 3072 17.7 -> 15.9, 2048 x 1152 -> 4608 16.9 -> 15.4.
+// 100 us (2.6 POP/s), 1024 x 3072 -> 3072 17.7 -> 16.4, 2048 x 1152 -> 4608 16.9 -> 15.4.
 // An output tile is two accumulator passes, the int32 one over K and the fp32 one of the rank-r branch, in two tensor-memory
 // buffers; the epilogue warps take the first into registers while the second runs, so the next tile's MMAs start at once.
 #include "common.h"
