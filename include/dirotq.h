@@ -184,9 +184,9 @@ DIROTQ_API dirotq_status_t dirotq_int_gemm_debug(const int8_t* act_codes, int M,
  * chosen automatically, because its outputs differ from the other plans' in fp32 summation order (a bf16 step on a few
  * values), and with 0 a token's output bits do not depend on how many tokens a call has; 192: the grouped INT4 kernel's plan
  * with three epilogue warpgroups (64 columns per thread), never chosen automatically: on the FLUX shapes at 4608 tokens
- * it measured between the other two; 512: the NVFP4 kernel in pairs of CTAs (clusters of two, tcgen05.mma.cta_group::2, 256 token
+ * it measured between the other two; 512: the grouped INT4 and NVFP4 kernels in pairs of CTAs (clusters of two, tcgen05.mma.cta_group::2, 256 token
  * rows x 256 columns per pair, each CTA loading its own rows and one half of the weight tile), forced; 0 takes it
- * where its schedule is the shortest (a pair does two wide tiles' work in about 0.9 of a wide tile's time: every FLUX
+ * where its schedule is the shortest (a pair does two wide tiles' work in 0.86 to 0.96 of a wide tile's time: every FLUX
  * shape at M = 4608); for W4A8 128 is single CTAs, 256 and 512 are CTA pairs with 128 and 256 columns.  A value that names a plan of
  * one kernel leaves the other formats' kernels choosing for themselves.  Process-wide; results do not depend on it, 66
  * apart (each output element is accumulated in the same order).  Other values: DIROTQ_ERR_INVALID_ARG. */

@@ -246,15 +246,6 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// Error path only.  After a bounded wait gave up, MMAs that were already issued may still be running: the issuing
-// thread waits (again with a limit) for them on a spare barrier (count 1, never used otherwise) before the tensor
-// memory they write into is freed.
-__device__ __forceinline__ void umma_drain(uint32_t spare_bar) {
-    umma_commit(spare_bar);
-    const unsigned long long t0 = globaltimer_ns();
-    while (!mbar_try_wait(spare_bar, 0) && globaltimer_ns() - t0 < 100000000ull) {}
-}
-
 // ---------------------------------------------------------------- CTA pairs (cta_group::2)
 // Two CTAs of a cluster of two share one MMA: the even CTA (rank 0, the leader) issues tcgen05.mma.cta_group::2 with
 // M = 256; each CTA supplies the 128 rows of A and half of the B tile's N rows from its own shared memory (same offsets
@@ -345,12 +336,45 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, 
         : "memory");
 }
 
+// The 8-bit kinds over the pair (see umma_f8f6f4, umma_i8).
+__device__ __forceinline__ void umma_f8f6f4_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, {%5, %5, %5, %5, %5, %5, %5, %5}, p;\n\t"
+        "}\n" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(0u)
+        : "memory");
+}
+__device__ __forceinline__ void umma_i8_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, {%5, %5, %5, %5, %5, %5, %5, %5}, p;\n\t"
+        "}\n" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(0u)
+        : "memory");
+}
+
 // Arrival, on completion of all MMAs issued so far by this thread, on the barrier at `bar`'s offset in the shared memory
 // of every CTA named in cta_mask (bit 0: rank 0, bit 1: rank 1).  A barrier arrival, not a data transfer.
 __device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t cta_mask) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
                  "h"(cta_mask)
                  : "memory");
+}
+
+// Error path only.  After a bounded wait gave up, MMAs that were already issued may still be running: the issuing
+// thread waits (again with a limit) for them on a spare barrier (count 1, never used otherwise) before the tensor
+// memory they write into is freed.
+template <bool PAIR = false>
+__device__ __forceinline__ void umma_drain(uint32_t spare_bar) {
+    if constexpr (PAIR) umma_commit_pair(spare_bar, 1);
+    else umma_commit(spare_bar);
+    const unsigned long long t0 = globaltimer_ns();
+    while (!mbar_try_wait(spare_bar, 0) && globaltimer_ns() - t0 < 100000000ull) {}
 }
 
 // ---------------------------------------------------------------- programmatic dependent launch

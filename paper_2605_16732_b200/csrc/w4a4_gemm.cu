@@ -31,6 +31,12 @@
 //
 // Tiles of 256, 128 or (on request) 192 columns here; w4a4_narrow.cu has the same computation in 64-column tiles.
 //
+// CTA pairs (PAIR; 256 token rows x 256 columns per cluster of two, tcgen05.mma.cta_group::2): each CTA loads its own activation codes and
+// loads AND expands half of the tile's weights.  A K-group of a 128 x 256 tile keeps the schedulers of an SM busy for most of its time (the
+// rescale's packed multiply and multiply-add take two issue cycles each: 660 of 1125 cycles), so what a pair saves is
+// what the expansion takes from them and from shared memory: half.  4608 x 3072 -> 9216, us alone: groups of 64 278 -> 266, of 128 190 -> 164
+// (there the two expanding warps had no time left: 1430 of 1509 cycles per k-block).
+//
 // Roles (384 threads = 3 warpgroups):
 //   warpgroup 0: warp 0 TMA producer, warp 1 MMA issuer + TMEM owner, warps 2-3 nibble -> byte unpack
 //   warpgroups 1-2: epilogue; warp%4 selects the TMEM lane quadrant (token rows), the warpgroup
@@ -49,7 +55,7 @@ namespace {
 //        buffers, so the tile goes back to the tensor core after the first quarter of a group, and three warps per scheduler
 //        hide each other's waits.  16 warps: 152 registers for the epilogue threads, 56 for the others.
 //   128: two warpgroups, 64 columns per thread, four accumulator tiles; for layers whose wider tiles would leave SMs idle.
-template <int BN>
+template <int BN, bool PAIR = false>
 struct Plan {
     static constexpr int EPI_WG = BN == 192 ? 3 : 2;  // epilogue warpgroups
     static constexpr int EPI_WARPS = 4 * EPI_WG;
@@ -57,9 +63,10 @@ struct Plan {
     static constexpr int EPI_REGS = EPI_WG == 3 ? 152 : 216;  // setmaxnreg budgets: 128 * AUX + 128 * EPI_WG * EPI <= 65536
     static constexpr int AUX_REGS = EPI_WG == 3 ? 56 : 64;
     static constexpr int SC_SLOTS = BN == 192 ? 6 : 8;
-    static constexpr int STAGES = BN == 256 ? 3 : BN == 192 ? 4 : 5;
-    static constexpr int BU_BYTES = BN * BKC;         // unpacked weight codes / bf16 W~_h chunk (32 KB at BN = 256)
-    static constexpr int BP_BYTES = BN * BKC / 2;     // packed weight codes (TMA staging)
+    static constexpr int STAGES = PAIR ? 5 : BN == 256 ? 3 : BN == 192 ? 4 : 5;
+    static constexpr int WROWS = PAIR ? BN / 2 : BN;  // weight rows this CTA loads and expands
+    static constexpr int BU_BYTES = WROWS * BKC;      // unpacked weight codes / bf16 W~_h chunk (32 KB at BN = 256)
+    static constexpr int BP_BYTES = WROWS * BKC / 2;  // packed weight codes (TMA staging)
     static constexpr int STAGE_BYTES = A_BYTES + BU_BYTES + BP_BYTES;  // 64 KB / 40 KB
     static constexpr int SC_SW_BYTES = 2 * BN * 4;    // up to two groups per k-block
     static constexpr int SC_SX_BYTES = 2 * BM * 4;    // activation scales of up to two groups
@@ -67,19 +74,19 @@ struct Plan {
     static constexpr int BAR_OFFSET = STAGES * STAGE_BYTES + SC_SLOTS * SC_BYTES;
     static constexpr int SMEM_BYTES = BAR_OFFSET + 512 + 1024;
 };
-static_assert(Plan<256>::SMEM_BYTES <= 232448 && Plan<192>::SMEM_BYTES <= 232448 && Plan<128>::SMEM_BYTES <= 232448, "shared memory plan too large");
+static_assert(Plan<256>::SMEM_BYTES <= 232448 && Plan<256, true>::SMEM_BYTES <= 232448 && Plan<192>::SMEM_BYTES <= 232448 && Plan<128>::SMEM_BYTES <= 232448, "shared memory plan too large");
 static_assert(Plan<128>::STAGE_BYTES % 1024 == 0 && Plan<128>::SC_BYTES % 128 == 0, "tile alignment");
 static_assert(Plan<192>::STAGE_BYTES % 1024 == 0 && Plan<192>::SC_BYTES % 128 == 0, "tile alignment");
-static_assert(8 * (3 * Plan<128>::STAGES + 2 * 8 + 9) <= 400 && 8 * (3 * Plan<192>::STAGES + 2 * 6 + 9) <= 400,
+static_assert(8 * (3 * Plan<256, true>::STAGES + 2 * 8 + 11) <= 400 && 8 * (3 * Plan<128>::STAGES + 2 * 8 + 9) <= 400 && 8 * (3 * Plan<192>::STAGES + 2 * 6 + 9) <= 400,
               "barriers end below the words at +400");
 
-template <int G, bool kPartials, int BN>
-__global__ void __launch_bounds__(Plan<BN>::THREADS, 1)
+template <int G, bool kPartials, int BN, bool PAIR>
+__global__ void __launch_bounds__(Plan<BN, PAIR>::THREADS, 1)
 w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_constant__ CUtensorMap tmap_wpacked,
                  const __grid_constant__ CUtensorMap tmap_wscale, const __grid_constant__ CUtensorMap tmap_xscale,
                  const __grid_constant__ CUtensorMap tmap_xh, const __grid_constant__ CUtensorMap tmap_wh,
                  const GemmKernelParams p) {
-    using P = Plan<BN>;
+    using P = Plan<BN, PAIR>;
     constexpr int STAGES = P::STAGES, STAGE_BYTES = P::STAGE_BYTES, BU_BYTES = P::BU_BYTES, BP_BYTES = P::BP_BYTES;
     constexpr int SC_SW_BYTES = P::SC_SW_BYTES, SC_BYTES = P::SC_BYTES, BAR_OFFSET = P::BAR_OFFSET;
     constexpr int SC_SLOTS = P::SC_SLOTS, NUM_EPI_WARPS = P::EPI_WARPS;
@@ -102,6 +109,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     auto scempty_bar = [&](int s) { return bar_base + 8u * (3 * STAGES + SC_SLOTS + s); };
     auto tfull_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + a); };
     auto tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 4 + a); };
+    auto peer_tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 9 + a); };  // pairs: in the leader, the other CTA's
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + BAR_OFFSET + 400);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + BAR_OFFSET + 404);
 
@@ -113,13 +121,20 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     // folded in the last group, 23 the rank-r tile, 24 has stored its last outputs.
     if (threadIdx.x == 0) TRACE_CLK(p.status, 9);
 
-    const int num_m_blocks = (p.M + BM - 1) / BM;
+    // a tile is BM token rows of one CTA, or of each CTA of a pair
+    const uint32_t crank = PAIR ? cluster_ctarank() : 0u;
+    constexpr int TILE_ROWS = PAIR ? 2 * BM : BM;
+    const int num_m_blocks = (p.M + TILE_ROWS - 1) / TILE_ROWS;
     const int num_n_blocks = (p.N + BN - 1) / BN;
+    auto first_tile = [&]() { return static_cast<int>(PAIR ? blockIdx.x >> 1 : blockIdx.x); };
+    auto tile_stride = [&]() { return static_cast<int>(PAIR ? gridDim.x >> 1 : gridDim.x); };
+    auto tile_row = [&](int tile) { return (tile % num_m_blocks) * TILE_ROWS + static_cast<int>(crank) * BM; };  // this CTA's first row
     const int num_tiles = num_m_blocks * num_n_blocks;
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(full_bar(s), 1);
-            mbar_init(unp_bar(s), 64);  // every thread of the two unpack warps arrives for itself
+            // every thread of the two unpack warps arrives for itself; of a pair's four, one lane each, on the leader's barrier
+            mbar_init(unp_bar(s), PAIR ? 4 : 64);
             mbar_init(empty_bar(s), 1);
         }
         for (int s = 0; s < SC_SLOTS; ++s) {
@@ -129,6 +144,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         for (int a = 0; a < NBUF; ++a) {
             mbar_init(tfull_bar(a), 1);
             mbar_init(tempty_bar(a), NUM_EPI_WARPS * 32);
+            if (PAIR) mbar_init(peer_tempty_bar(a), 1);
         }
         mbar_init(bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 8), 1);  // spare: see umma_drain
         *abort_flag = 0;
@@ -141,11 +157,17 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         tma_prefetch_desc(&tmap_wh);
     }
     if (warp == 1) {
-        tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
-        tmem_relinquish();
+        if constexpr (PAIR) {
+            tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+            tmem_relinquish();
+        }
     }
     tc_fence_before_sync();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();  // the other CTA's barriers are initialised before anything arrives on them
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
     // everything above touched only this CTA's own shared and tensor memory; what follows reads the first kernel's output
@@ -166,9 +188,9 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 uint32_t it = 0, sc_it = 0;
                 long long w_empty = 0;
                 bool ok = true;
-                for (int tile = static_cast<int>(blockIdx.x); ok && tile < num_tiles; tile += static_cast<int>(gridDim.x)) {
-                    const int m0 = (tile % num_m_blocks) * BM;
-                    const int n0 = (tile / num_m_blocks) * BN;
+                for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
+                    const int m0 = tile_row(tile);
+                    const int n0 = (tile / num_m_blocks) * BN, w0 = n0 + static_cast<int>(crank) * P::WROWS;
                     for (int kb = 0; kb < p.num_kb; ++kb, ++it, ++sc_it) {
                         const int s = it % STAGES;
                         if (!timed_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER, w_empty)) { ok = false; break; }
@@ -176,7 +198,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         if (elect_one()) {
                             mbar_arrive_expect_tx(full_bar(s), A_BYTES + BP_BYTES);
                             tma_load_2d(st, &tmap_codes, full_bar(s), kb * BKC, m0);
-                            tma_load_2d(st + A_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), n0);
+                            tma_load_2d(st + A_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), w0);
                         }
                         const int slot = sc_it % SC_SLOTS;
                         if (!mbar_wait(scempty_bar(slot), ((sc_it / SC_SLOTS) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
@@ -196,7 +218,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         if (elect_one()) {
                             mbar_arrive_expect_tx(full_bar(s), A_BYTES + BU_BYTES);
                             tma_load_2d(st, &tmap_xh, full_bar(s), lr * 64, m0);
-                            tma_load_2d(st + A_BYTES, &tmap_wh, full_bar(s), lr * 64, n0);
+                            tma_load_2d(st + A_BYTES, &tmap_wh, full_bar(s), lr * 64, w0);
                         }
                     }
                 }
@@ -217,6 +239,19 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     }
                 }
             }
+        } else if (PAIR && warp == 1 && crank != 0) {
+            // -------------------------------------------------------- pairs: "accumulator tile drained", passed on to the leader
+            // (one arrival over the cluster for the 256 of this CTA's epilogue threads, which do not wait for it)
+            uint32_t b = 0, bph = 0;
+            bool ok = true;
+            for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
+                for (int g = 0; g <= p.n_g; ++g) {
+                    ok = mbar_wait(tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA);
+                    if (!ok) break;
+                    if (elect_one()) mbar_arrive_cluster(map_to_cta(peer_tempty_bar(b), 0));
+                    if (++b == NBUF) { b = 0; bph ^= 1; }
+                }
+            }
         } else if (warp == 1) {
             // -------------------------------------------------------- MMA issuer
             // One thread, and every instruction it executes waits its turn behind the two epilogue warps of its
@@ -225,18 +260,22 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             // word, which cannot overflow: shared-memory addresses have 18 bits, the field holds address / 16).
             // (whole warp in the loops, one elected lane issues, as in the producer)
             {
-                constexpr uint32_t idesc_f8 = umma_idesc(1 /*f32*/, 0 /*E4M3*/, BM, BN);
-                constexpr uint32_t idesc_i8 = umma_idesc(2 /*s32*/, 1 /*s8*/, BM, BN);  // integer-path build only
-                constexpr uint32_t idesc_bf = umma_idesc(1 /*f32*/, 1 /*bf16*/, BM, BN);
+                constexpr uint32_t idesc_f8 = umma_idesc(1 /*f32*/, 0 /*E4M3*/, TILE_ROWS, BN);
+                constexpr uint32_t idesc_i8 = umma_idesc(2 /*s32*/, 1 /*s8*/, TILE_ROWS, BN);  // integer-path build only
+                constexpr uint32_t idesc_bf = umma_idesc(1 /*f32*/, 1 /*bf16*/, TILE_ROWS, BN);
                 const uint64_t desc0 = umma_desc_sw128(smem_base);
                 const uint32_t desc_hi = static_cast<uint32_t>(desc0 >> 32), desc_lo0 = static_cast<uint32_t>(desc0);
                 auto desc = [&](uint32_t lo) { return (static_cast<uint64_t>(desc_hi) << 32) | lo; };
+                auto commit = [&](uint32_t bar) {
+                    if constexpr (PAIR) umma_commit_pair(bar, 3);  // the same barrier of both CTAs
+                    else umma_commit(bar);
+                };
                 uint32_t s = 0, ph = 0;        // stage of the operand ring and its parity
                 uint32_t b = 0, bph = 1;       // accumulator tile and the parity its "empty" barrier is waited with
                 long long w_ops = 0, w_tempty = 0;
                 const long long t_kernel = clock64();
                 bool ok = true;
-                for (int tile = static_cast<int>(blockIdx.x); ok && tile < num_tiles; tile += static_cast<int>(gridDim.x)) {
+                for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
                     int groups_left = p.n_g;
                     for (int kb = 0; ok && kb < p.num_kb; ++kb) {
                         // the unpack warps arrive after they have seen the stage's loads land (one barrier for both operands), so
@@ -248,30 +287,36 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
 #pragma unroll
                         for (int gi = 0; gi < GPK; ++gi) {
                             if (gi < groups_left) {
-                                if (!timed_wait(tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_tempty)) { ok = false; break; }
+                                if (!timed_wait(tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_tempty) ||
+                                    (PAIR && !timed_wait(peer_tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_tempty))) { ok = false; break; }
                                 tc_fence_after_sync();
                                 if (elect_one()) {
 #pragma unroll
                                     for (int k = 0; k < MMA_PER_G; ++k) {
                                         const int kk = gi * MMA_PER_G + k;  // 32-byte step inside the 128-byte row
-                                        if constexpr (kI8Path)
+                                        if constexpr (PAIR && kI8Path)
+                                            umma_i8_pair(tmem_base + b * BN, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), idesc_i8, k != 0);
+                                        else if constexpr (PAIR)
+                                            umma_f8f6f4_pair(tmem_base + b * BN, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), idesc_f8, k != 0);
+                                        else if constexpr (kI8Path)
                                             umma_i8(tmem_base + b * BN, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), idesc_i8, k != 0);
                                         else
                                             umma_f8f6f4(tmem_base + b * BN, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), idesc_f8, k != 0);
                                     }
-                                    umma_commit(tfull_bar(b));
+                                    commit(tfull_bar(b));
                                 }
                                 if (++b == NBUF) { b = 0; bph ^= 1; }
                             }
                         }
                         if (!ok) break;
                         groups_left -= GPK;
-                        if (elect_one()) umma_commit(empty_bar(s));
+                        if (elect_one()) commit(empty_bar(s));
                         if (++s == STAGES) { s = 0; ph ^= 1; }
                     }
                     if (!ok) break;
                     // rank-r bf16 branch: one more accumulator tile, fp32
-                    if (!mbar_wait(tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
+                    if (!mbar_wait(tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA) ||
+                        (PAIR && !mbar_wait(peer_tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA))) { ok = false; break; }
                     tc_fence_after_sync();
                     for (int lr = 0; lr < p.lr_chunks; ++lr) {
                         if (!mbar_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
@@ -279,14 +324,16 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         const uint32_t a_lo = desc_lo0 + s * (STAGE_BYTES >> 4), b_lo = a_lo + (A_BYTES >> 4);
                         if (elect_one()) {
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                umma_bf16(tmem_base + b * BN, desc(a_lo + 2 * k), desc(b_lo + 2 * k), idesc_bf, (lr | k) != 0);
-                            umma_commit(empty_bar(s));
+                            for (int k = 0; k < 4; ++k) {
+                                if constexpr (PAIR) umma_bf16_pair(tmem_base + b * BN, desc(a_lo + 2 * k), desc(b_lo + 2 * k), idesc_bf, (lr | k) != 0);
+                                else umma_bf16(tmem_base + b * BN, desc(a_lo + 2 * k), desc(b_lo + 2 * k), idesc_bf, (lr | k) != 0);
+                            }
+                            commit(empty_bar(s));
                         }
                         if (++s == STAGES) { s = 0; ph ^= 1; }
                     }
                     if (!ok) break;
-                    if (elect_one()) umma_commit(tfull_bar(b));
+                    if (elect_one()) commit(tfull_bar(b));
                     if (lane == 0) TRACE_CLK(p.status, 19);
                     if (++b == NBUF) { b = 0; bph ^= 1; }
                 }
@@ -302,7 +349,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             uint32_t it = 0;
             long long w_full = 0;
             bool ok = true;
-            for (int tile = static_cast<int>(blockIdx.x); ok && tile < num_tiles; tile += static_cast<int>(gridDim.x)) {
+            for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
                 const int items = p.num_kb + p.lr_chunks;
                 for (int i = 0; i < items; ++i, ++it) {
                     const int s = it % STAGES;
@@ -321,7 +368,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         // The loads of a batch are issued before any of its stores: the compiler cannot prove that the
                         // staging buffer and the operand tile do not overlap, so a load written after a store would wait
                         // for it and the whole unpack would run as one dependent chain.
-                        constexpr int PIECES = (BN * 4) / 64, BATCH = PIECES % 8 == 0 ? 8 : 4;
+                        constexpr int PIECES = (P::WROWS * 4) / 64, BATCH = PIECES % 8 == 0 ? 8 : 4;
 #pragma unroll
                         for (int jb = 0; jb < PIECES; jb += BATCH) {
                             uint4 pk[BATCH];
@@ -344,7 +391,12 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     }
                     // each thread signs off its own writes (a warp-wide barrier followed by one lane's arrival costs about
                     // a hundred cycles more on this part than 32 arrivals)
-                    mbar_arrive(unp_bar(s));
+                    if constexpr (PAIR) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_cluster(map_to_cta(unp_bar(s), 0));
+                    } else {
+                        mbar_arrive(unp_bar(s));
+                    }
                     if (it == 0 && u == 0) TRACE_CLK(p.status, 15);
                 }
             }
@@ -398,8 +450,8 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             tc_fence_before_sync();
             mbar_arrive(tempty_bar(buf));  // all lanes arrive (see the unpack warps' note on the cost of electing one)
         };
-        for (int tile = static_cast<int>(blockIdx.x); ok && tile < num_tiles; tile += static_cast<int>(gridDim.x)) {
-            const int m0 = (tile % num_m_blocks) * BM;
+        for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
+            const int m0 = tile_row(tile);
             const int n0 = (tile / num_m_blocks) * BN;
             const int rbase = m0 + q * 32 + lr4;  // this thread's rows: rbase + 8 i, i = 0..3
             const int colbase = n0 + half * HB;
@@ -577,16 +629,18 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     }
 
     // ---------------------------------------------------------------- teardown
-    if (warp == 1 && lane == 0 && *abort_flag != 0) umma_drain(bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 8));  // a wait gave up: let issued MMAs finish first
+    if (warp == 1 && lane == 0 && crank == 0 && *abort_flag != 0) umma_drain<PAIR>(bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 8));  // a wait gave up: let issued MMAs finish first
     tc_fence_before_sync();
-    __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();  // neither CTA leaves while the other may still read its operands or signal its barriers
+    else __syncthreads();
     if (warp == 1) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, 512);
+        if constexpr (PAIR) tmem_dealloc_pair(tmem_base, 512);
+        else tmem_dealloc(tmem_base, 512);
     }
 }
 
-template <int BN>
+template <int BN, bool PAIR = false>
 static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream) {
     const Geometry& g = L->geo;
     CUtensorMap tmap_codes, tmap_xscale, tmap_xh;
@@ -608,22 +662,30 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
     p.bias = reinterpret_cast<const float*>(L->blob + L->lay.off_bias);
     p.y = a.y; p.partials = a.partials; p.status = a.status;
 
-    const int num_tiles = ((a.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
-    const int grid = num_tiles < sm_count(L->device) ? num_tiles : sm_count(L->device);
+    using P = Plan<BN, PAIR>;
+    constexpr int TILE_ROWS = PAIR ? 2 * BM : BM, CTAS = PAIR ? 2 : 1;
+    const int num_tiles = ((a.M + TILE_ROWS - 1) / TILE_ROWS) * ((g.N + BN - 1) / BN), slots = sm_count(L->device) / CTAS;
+    const int grid = CTAS * (num_tiles < slots ? num_tiles : slots);
     using KernelFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                               const CUtensorMap, const CUtensorMap, const GemmKernelParams);
     KernelFn kern;
     const bool dbg = a.partials != nullptr;
-    if (g.G == 64) kern = dbg ? w4a4_gemm_kernel<64, true, BN> : w4a4_gemm_kernel<64, false, BN>;
-    else           kern = dbg ? w4a4_gemm_kernel<128, true, BN> : w4a4_gemm_kernel<128, false, BN>;
+    if constexpr (PAIR) {  // (the debug entry's group sums come from single CTAs)
+        kern = g.G == 64 ? w4a4_gemm_kernel<64, false, BN, true> : w4a4_gemm_kernel<128, false, BN, true>;
+    } else {
+        if (g.G == 64) kern = dbg ? w4a4_gemm_kernel<64, true, BN, false> : w4a4_gemm_kernel<64, false, BN, false>;
+        else           kern = dbg ? w4a4_gemm_kernel<128, true, BN, false> : w4a4_gemm_kernel<128, false, BN, false>;
+    }
     static SmemOptIn<4> opt_in;  // one per instantiation of this launcher, i.e. per tile width
     const int vi = (g.G == 64 ? 0 : 2) + (dbg ? 1 : 0);
-    if (!opt_in.ensure(kern, vi, L->device, Plan<BN>::SMEM_BYTES)) return DIROTQ_ERR_CUDA;
-    const cudaError_t err = launch_kernel(kern, grid, Plan<BN>::THREADS, Plan<BN>::SMEM_BYTES, stream, true, tmap_codes,
-                                          BN == 128 ? L->tmap_wpacked128 : BN == 192 ? L->tmap_wpacked192 : L->tmap_wpacked,
-                                          BN == 128 ? L->tmap_wscale128 : BN == 192 ? L->tmap_wscale192 : L->tmap_wscale,
-                                          tmap_xscale, tmap_xh,
-                                          BN == 128 ? L->tmap_wh128 : BN == 192 ? L->tmap_wh192 : L->tmap_wh, p);
+    if (!opt_in.ensure(kern, vi, L->device, P::SMEM_BYTES)) return DIROTQ_ERR_CUDA;
+    auto launch = [&](const auto&... args) {
+        return PAIR ? launch_kernel_pairs(kern, grid, P::THREADS, P::SMEM_BYTES, stream, true, args...)
+                    : launch_kernel(kern, grid, P::THREADS, P::SMEM_BYTES, stream, true, args...);
+    };
+    const cudaError_t err = launch(tmap_codes, P::WROWS == 128 ? L->tmap_wpacked128 : P::WROWS == 192 ? L->tmap_wpacked192 : L->tmap_wpacked,
+                                   BN == 128 ? L->tmap_wscale128 : BN == 192 ? L->tmap_wscale192 : L->tmap_wscale, tmap_xscale, tmap_xh,
+                                   P::WROWS == 128 ? L->tmap_wh128 : P::WROWS == 192 ? L->tmap_wh192 : L->tmap_wh, p);
     return err == cudaSuccess ? DIROTQ_OK : DIROTQ_ERR_CUDA;
 }
 
@@ -632,7 +694,7 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
 static std::atomic<int> g_tile_columns{0};  // 0: chosen per call; 64 / 128 / 192 / 256: forced; 66: 64 columns, split plan where it applies
 
 dirotq_status_t set_w4a4_tile_columns(int columns) {
-    if (columns != 0 && columns != 64 && columns != 66 && columns != 128 && columns != 192 && columns != 256) return DIROTQ_ERR_INVALID_ARG;
+    if (columns != 0 && columns != 64 && columns != 66 && columns != 128 && columns != 192 && columns != 256 && columns != 512) return DIROTQ_ERR_INVALID_ARG;
     g_tile_columns.store(columns);
     return DIROTQ_OK;
 }
@@ -641,14 +703,18 @@ dirotq_status_t launch_w4a4_gemm(const dirotq_layer* L, const GemmArgs& a, cudaS
     // The plan with the shortest schedule: turns of the SMs x what one tile of the plan costs.  Costs relative to a 256-column tile, from
     // the cycles per 128 codes of a tile: 2360, 1390 and 780 with groups of 64, 1600, 990 and 620 with groups of 128 (the
     // activation tile, the rank-r branch, the pipeline fill and the hand-overs are paid per tile whatever its width).
+    // A turn of pair tiles takes 0.957 of a turn of 256-column tiles with groups of 64, 0.86 with groups of 128; a pair covers two row blocks, which can
+    // cost it a turn (4173 x 3072 -> 12288: 12 turns against 11, 349 us against 339).
     const int forced = g_tile_columns.load(), sms = sm_count(L->device);
     const long m_blocks = (a.M + BM - 1) / BM;
     auto turns = [&](int columns) { return static_cast<double>((m_blocks * ((L->geo.N + columns - 1) / columns) + sms - 1) / sms); };
     const double c256 = turns(256), c128 = (L->geo.G == 64 ? 0.60 : 0.64) * turns(128), c64 = (L->geo.G == 64 ? 0.34 : 0.40) * turns(64);
-    const int plan = forced ? forced : c64 <= c128 && c64 <= c256 ? 64 : c128 < c256 ? 128 : 256;
+    const double c512 = (L->geo.G == 64 ? 0.957 : 0.86) * static_cast<double>(((m_blocks + 1) / 2 * ((L->geo.N + 255) / 256) + sms / 2 - 1) / (sms / 2));
+    const int plan = forced ? forced : c512 < c256 && c512 <= c128 && c512 <= c64 ? 512 : c64 <= c128 && c64 <= c256 ? 64 : c128 < c256 ? 128 : 256;
     if (a.partials == nullptr && (plan == 64 || plan == 66)) return launch_w4a4_narrow(L, a, plan == 66, stream);
+    if (plan == 512 && a.partials == nullptr) return launch_w4a4_gemm_bn<256, true>(L, a, stream);
     if (plan == 192) return launch_w4a4_gemm_bn<192>(L, a, stream);
-    return plan == 256 ? launch_w4a4_gemm_bn<256>(L, a, stream) : launch_w4a4_gemm_bn<128>(L, a, stream);
+    return plan >= 256 ? launch_w4a4_gemm_bn<256>(L, a, stream) : launch_w4a4_gemm_bn<128>(L, a, stream);
 }
 
 }  // namespace dirotq
