@@ -175,18 +175,17 @@ DIROTQ_API dirotq_status_t dirotq_int_gemm_debug(const int8_t* act_codes, int M,
                                       dirotq_stream_t stream);
 
 /* Tuning knob of the second kernels (all four formats): output columns per tile.
- * 0 (default): chosen per call from M, N and the number of SMs (grouped INT4: the shortest schedule of 256-, 128- and
- * 64-column tiles, which cost 1 : 0.6 : 0.34 with groups of 64 and 1 : 0.64 : 0.4 with groups of 128; NVFP4: 256 columns
- * unless 128-column tiles, at 0.6 of a wide one, shorten the schedule);
+ * 0 (default): chosen per call from M, N and the number of SMs, the shortest schedule of the plans below, 66 apart (NVFP4: 256
+ * columns unless 128-column tiles, at 0.6 of a wide one, shorten the schedule);
  * 128 or 256: forced; 64: the grouped INT4 kernel's plan for few token rows, forced, one CTA per tile; 66: the same
  * tiles with the K-groups of a tile cut over a cluster of up to four CTAs (partial tiles added in one of them through
  * distributed shared memory) wherever every tile's cluster is resident at once and every CTA keeps two k-blocks; never
  * chosen automatically, because its outputs differ from the other plans' in fp32 summation order (a bf16 step on a few
- * values), and with 0 a token's output bits do not depend on how many tokens a call has; 192: the grouped INT4 kernel's plan
- * with three epilogue warpgroups (64 columns per thread), never chosen automatically: on the FLUX shapes at 4608 tokens
- * it measured between the other two; 512: the grouped INT4 and NVFP4 kernels in pairs of CTAs (clusters of two, tcgen05.mma.cta_group::2, 256 token
- * rows x 256 columns per pair, each CTA loading its own rows and one half of the weight tile), forced; 0 takes it
- * where its schedule is the shortest (a pair does two wide tiles' work in 0.86 to 0.96 of a wide tile's time: every FLUX
+ * values), and with 0 a token's output bits do not depend on how many tokens a call has; 130: the grouped INT4 kernel with 256 token
+ * rows x 128 columns per CTA; 192: the grouped INT4 kernel's plan
+ * with three epilogue warpgroups (64 columns per thread); 512: the grouped INT4 and NVFP4 kernels in pairs of CTAs (clusters of two,
+ * tcgen05.mma.cta_group::2, 256 token rows x 256 columns per pair, each CTA loading its own rows and one half of the weight tile), forced;
+ * 0 takes it where its schedule is the shortest (every FLUX
  * shape at M = 4608); for W4A8 128 is single CTAs, 256 and 512 are CTA pairs with 128 and 256 columns.  A value that names a plan of
  * one kernel leaves the other formats' kernels choosing for themselves.  Process-wide; results do not depend on it, 66
  * apart (each output element is accumulated in the same order).  Other values: DIROTQ_ERR_INVALID_ARG. */

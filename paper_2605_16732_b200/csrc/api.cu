@@ -183,7 +183,7 @@ static dirotq_status_t encode_tmaps_192(dirotq_layer* L, int N, int group) {
                                         (uint64_t)g.K_lp / 2, (uint64_t)N, (uint64_t)g.K_lp / 2, 64, 192, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wscale192, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, L->blob + lay.off_wscale,
-                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, 192, 128 / group,
+                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, 192, 1,
                             CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wh192, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L->blob + lay.off_wh, (uint64_t)g.r_pad,
@@ -253,7 +253,7 @@ static dirotq_status_t prepare_int4(bool asym, bool sibling, const void* W, int 
                             (uint64_t)g.K_lp / 2, (uint64_t)N, (uint64_t)g.K_lp / 2, 64, kGemmBN, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wscale, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, L->blob + lay.off_wscale,
-                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, kGemmBN, 128 / group,
+                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, kGemmBN, 1,
                             CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L->blob + lay.off_wh, (uint64_t)g.r_pad,
@@ -263,7 +263,7 @@ static dirotq_status_t prepare_int4(bool asym, bool sibling, const void* W, int 
                             (uint64_t)g.K_lp / 2, (uint64_t)N, (uint64_t)g.K_lp / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wscale128, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, L->blob + lay.off_wscale,
-                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, 128, 128 / group,
+                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, 128, 1,
                             CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wh128, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L->blob + lay.off_wh, (uint64_t)g.r_pad,
@@ -427,7 +427,7 @@ dirotq_status_t dirotq_prepare_layer_ph(const void* W, int w_dtype, int w_layout
                             (uint64_t)g.K_lp / 2, (uint64_t)N, (uint64_t)g.K_lp / 2, 64, kGemmBN, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wscale, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, L->blob + lay.off_wscale,
-                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, kGemmBN, 128 / group,
+                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, kGemmBN, 1,
                             CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L->blob + lay.off_wh, (uint64_t)g.r_pad,
@@ -437,7 +437,7 @@ dirotq_status_t dirotq_prepare_layer_ph(const void* W, int w_dtype, int w_layout
                             (uint64_t)g.K_lp / 2, (uint64_t)N, (uint64_t)g.K_lp / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wscale128, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, L->blob + lay.off_wscale,
-                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, 128, 128 / group,
+                            (uint64_t)wscale_row_len(N), (uint64_t)g.n_g, (uint64_t)wscale_row_len(N) * 4, 128, 1,
                             CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st == DIROTQ_OK)
         st = encode_tmap_2d(&L->tmap_wh128, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L->blob + lay.off_wh, (uint64_t)g.r_pad,
@@ -654,8 +654,8 @@ dirotq_status_t dirotq_set_dependent_launch(int enabled) {
 }
 
 dirotq_status_t dirotq_set_gemm_tile(int columns) {
-    // 64, 66 and 192: plans of the grouped INT4 second kernel only
-    const bool int4_only = columns == 64 || columns == 66 || columns == 192;  // 66: 64 columns with the reduction split over a cluster
+    // 64, 66, 130 and 192: plans of the grouped INT4 second kernel only
+    const bool int4_only = columns == 64 || columns == 66 || columns == 130 || columns == 192;  // 66: 64 columns with the reduction split over a cluster
     dirotq_status_t st = set_w4a4_tile_columns(columns);
     if (st == DIROTQ_OK) st = set_nvfp4_tile_columns(int4_only ? 0 : columns);
     return st != DIROTQ_OK ? st : set_w4a8_tile_columns(int4_only ? 0 : columns);

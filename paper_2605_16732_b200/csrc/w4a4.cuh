@@ -23,6 +23,17 @@ struct GemmKernelParams {
     int* status;
 };
 
+// Compile-time loop: f(Int<0>{}), ..., f(Int<N - 1>{}).
+template <int V>
+struct Int { static constexpr int value = V; };
+template <int N, int I = 0, class F>
+__device__ __forceinline__ void static_for(F&& f) {
+    if constexpr (I < N) {
+        f(Int<I>{});
+        static_for<N, I + 1>(f);
+    }
+}
+
 // Wait accounting (diagnostics): cycles a role spends blocked on each kind of barrier are summed into
 // 64-bit counters that follow the status word in the workspace (8-byte slots 1..8, see WaitSlot).
 enum WaitSlot : int { WS_PROD_EMPTY = 1, WS_MMA_OPERANDS = 2, WS_MMA_TEMPTY = 3, WS_UNPACK_FULL = 4, WS_EPI_TFULL = 5,

@@ -29,13 +29,21 @@
 // bf16 rank-r branch is issued as one more "group" (kind::f16 into the same ping-pong tile) and added
 // unscaled.
 //
-// Tiles of 256, 128 or (on request) 192 columns here; w4a4_narrow.cu has the same computation in 64-column tiles.
+// Tiles of 256, 192 or 128 columns here; w4a4_narrow.cu has the same computation in 64-column tiles.
 //
-// CTA pairs (PAIR; 256 token rows x 256 columns per cluster of two, tcgen05.mma.cta_group::2): each CTA loads its own activation codes and
-// loads AND expands half of the tile's weights.  A K-group of a 128 x 256 tile keeps the schedulers of an SM busy for most of its time (the
-// rescale's packed multiply and multiply-add take two issue cycles each: 660 of 1125 cycles), so what a pair saves is
-// what the expansion takes from them and from shared memory: half.  4608 x 3072 -> 9216, us alone: groups of 64 278 -> 266, of 128 190 -> 164
-// (there the two expanding warps had no time left: 1430 of 1509 cycles per k-block).
+// What bounds it: the issue slots of the schedulers.  The rescale's packed multiply and multiply-add hold a scheduler's issue port for two
+// cycles each and nothing issues beside them: of the 1125 cycles a K-group of a 128 x 256 tile took, 660 were these, and everything else that
+// is issued on the same schedulers (the epilogue's own loads, barriers and counters, the weight expansion, the MMA warp) came on top, in no
+// pipe's peak but in the sum.  So what helps is fewer instructions per group:
+//   * CTA pairs (PAIRED): each CTA loads its own activation codes and loads AND expands half of the tile's weights, half the expansion.  With groups of
+//     128 the two expanding warps had set the pace (1430 of 1509 cycles per k-block busy).  One tile of 256 rows in one CTA (TALL) halves it too.
+//   * a group's scales in a record of their own that lands with the operands: no barriers, tests and arrivals for scales, one offset to step on;
+//   * the next tile's first chunk requested after a plain wait, at one place (the tile is practically always there);
+//   * warp numbers known to be uniform, so that addresses and barriers are worked out on the uniform path;
+//   * row and column numbers worked out at the end of a tile, not held: with 128 accumulators and 64 values in flight a thread
+//     has 30 registers left, and every one too many turned into moves on the port that is the bound.
+// 4608 x 3072 -> 9216, us alone, groups of 64 / 128: 256 columns 278 -> 252 / 190 -> 185, pairs 236 / 153 (266 / 164 before the others), tall
+// 241 / 157, 192 columns 311 -> 267 / 211 -> 200, 128 columns 328 -> 290 / 222 -> 224.
 //
 // Roles (384 threads = 3 warpgroups):
 //   warpgroup 0: warp 0 TMA producer, warp 1 MMA issuer + TMEM owner, warps 2-3 nibble -> byte unpack
@@ -55,65 +63,77 @@ namespace {
 //        buffers, so the tile goes back to the tensor core after the first quarter of a group, and three warps per scheduler
 //        hide each other's waits.  16 warps: 152 registers for the epilogue threads, 56 for the others.
 //   128: two warpgroups, 64 columns per thread, four accumulator tiles; for layers whose wider tiles would leave SMs idle.
-template <int BN, bool PAIR = false>
+// and of how many token rows:
+//   ONE:  128.
+//   PAIR: 128 in each of two CTAs that share every MMA (tcgen05.mma.cta_group::2, 256 columns): each loads its own activation codes and loads and
+//         expands half of the tile's weights.
+//   TALL: 256 in one CTA, a warpgroup for each half (128 columns): a warp's share is that of the 256-column tile, the weights to expand are half.
+enum Rows : int { ONE, PAIRED, TALL };
+template <int BN, Rows ROWS = ONE>
 struct Plan {
     static constexpr int EPI_WG = BN == 192 ? 3 : 2;  // epilogue warpgroups
     static constexpr int EPI_WARPS = 4 * EPI_WG;
     static constexpr int THREADS = 128 + 128 * EPI_WG;
-    static constexpr int EPI_REGS = EPI_WG == 3 ? 152 : 216;  // setmaxnreg budgets: 128 * AUX + 128 * EPI_WG * EPI <= 65536
-    static constexpr int AUX_REGS = EPI_WG == 3 ? 56 : 64;
-    static constexpr int SC_SLOTS = BN == 192 ? 6 : 8;
-    static constexpr int STAGES = PAIR ? 5 : BN == 256 ? 3 : BN == 192 ? 4 : 5;
-    static constexpr int WROWS = PAIR ? BN / 2 : BN;  // weight rows this CTA loads and expands
+    // setmaxnreg budgets: 128 * AUX + 128 * EPI_WG * EPI at most what the block is launched with
+    static constexpr int HB = ROWS == TALL ? BN : BN / EPI_WG;  // columns per epilogue warp
+    static constexpr int EPI_REGS = EPI_WG == 3 ? 152 : HB == 128 ? 224 : 216;
+    static constexpr int AUX_REGS = EPI_WG == 3 ? 56 : HB == 128 ? 56 : 64;
+    static constexpr int SC_SLOTS = BN == 192 ? 13 : BN == 128 && ROWS == ONE ? 18 : 14;  // scale records, one per group
+    static constexpr int STAGES = ROWS == PAIRED ? 5 : ROWS == TALL ? 3 : BN == 256 ? 3 : BN == 192 ? 4 : 5;
+    static constexpr int CTA_ROWS = ROWS == TALL ? 2 * BM : BM;   // token rows of a CTA
+    static constexpr int TILE_ROWS = ROWS == ONE ? BM : 2 * BM;   // ... of a tile
+    static constexpr int BUF_COLS = ROWS == TALL ? 2 * BN : BN;   // tensor-memory columns of an accumulator tile
+    static constexpr int WROWS = ROWS == PAIRED ? BN / 2 : BN;    // weight rows this CTA loads and expands
+    static constexpr int AC_BYTES = CTA_ROWS * BKC;   // activation codes / bf16 x~_h chunk
     static constexpr int BU_BYTES = WROWS * BKC;      // unpacked weight codes / bf16 W~_h chunk (32 KB at BN = 256)
     static constexpr int BP_BYTES = WROWS * BKC / 2;  // packed weight codes (TMA staging)
-    static constexpr int STAGE_BYTES = A_BYTES + BU_BYTES + BP_BYTES;  // 64 KB / 40 KB
-    static constexpr int SC_SW_BYTES = 2 * BN * 4;    // up to two groups per k-block
-    static constexpr int SC_SX_BYTES = 2 * BM * 4;    // activation scales of up to two groups
-    static constexpr int SC_BYTES = SC_SW_BYTES + SC_SX_BYTES;  // 3 KB / 2 KB
+    static constexpr int STAGE_BYTES = AC_BYTES + BU_BYTES + BP_BYTES;  // 64 KB / 40 KB
+    static constexpr int SC_SW_BYTES = BN * 4, SC_BYTES = SC_SW_BYTES + CTA_ROWS * 4;  // weight scales, activation scales
     static constexpr int BAR_OFFSET = STAGES * STAGE_BYTES + SC_SLOTS * SC_BYTES;
     static constexpr int SMEM_BYTES = BAR_OFFSET + 512 + 1024;
+    static_assert(SMEM_BYTES <= 232448, "shared memory plan too large");
+    static_assert(STAGE_BYTES % 1024 == 0 && SC_BYTES % 128 == 0, "tile alignment");
+    static_assert(8 * (3 * STAGES + 11) <= 400, "barriers end below the words at +400");
 };
-static_assert(Plan<256>::SMEM_BYTES <= 232448 && Plan<256, true>::SMEM_BYTES <= 232448 && Plan<192>::SMEM_BYTES <= 232448 && Plan<128>::SMEM_BYTES <= 232448, "shared memory plan too large");
-static_assert(Plan<128>::STAGE_BYTES % 1024 == 0 && Plan<128>::SC_BYTES % 128 == 0, "tile alignment");
-static_assert(Plan<192>::STAGE_BYTES % 1024 == 0 && Plan<192>::SC_BYTES % 128 == 0, "tile alignment");
-static_assert(8 * (3 * Plan<256, true>::STAGES + 2 * 8 + 11) <= 400 && 8 * (3 * Plan<128>::STAGES + 2 * 8 + 9) <= 400 && 8 * (3 * Plan<192>::STAGES + 2 * 6 + 9) <= 400,
-              "barriers end below the words at +400");
 
-template <int G, bool kPartials, int BN, bool PAIR>
-__global__ void __launch_bounds__(Plan<BN, PAIR>::THREADS, 1)
+template <int G, bool kPartials, int BN, Rows ROWS>
+__global__ void __launch_bounds__(Plan<BN, ROWS>::THREADS, 1)
 w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_constant__ CUtensorMap tmap_wpacked,
                  const __grid_constant__ CUtensorMap tmap_wscale, const __grid_constant__ CUtensorMap tmap_xscale,
                  const __grid_constant__ CUtensorMap tmap_xh, const __grid_constant__ CUtensorMap tmap_wh,
                  const GemmKernelParams p) {
-    using P = Plan<BN, PAIR>;
+    using P = Plan<BN, ROWS>;
+    constexpr bool PAIR = ROWS == PAIRED;
     constexpr int STAGES = P::STAGES, STAGE_BYTES = P::STAGE_BYTES, BU_BYTES = P::BU_BYTES, BP_BYTES = P::BP_BYTES;
     constexpr int SC_SW_BYTES = P::SC_SW_BYTES, SC_BYTES = P::SC_BYTES, BAR_OFFSET = P::BAR_OFFSET;
     constexpr int SC_SLOTS = P::SC_SLOTS, NUM_EPI_WARPS = P::EPI_WARPS;
-    constexpr int HB = BN / P::EPI_WG;  // columns per epilogue warp: the warpgroup selects the slice of the tile
+    constexpr int HB = P::HB;          // columns per epilogue warp: the warpgroup selects the slice of the tile (TALL: the half of its rows)
+    constexpr int AC_BYTES = P::AC_BYTES, BUF_COLS = P::BUF_COLS, TILE_ROWS = P::TILE_ROWS;
     constexpr int CHUNKS = HB / 32;    // 32-column chunks per epilogue warp and accumulator tile
     constexpr int GPK = BKC / G;       // groups per k-block: 2 (G = 64) or 1 (G = 128)
     constexpr int MMA_PER_G = G / 32;  // 8-bit MMA instructions (K = 32) per group
-    constexpr int NBUF = 512 / BN;     // accumulator tiles in tensor memory: 2 of 256 columns, 4 of 128 (the barrier map has four slots)
+    constexpr int NBUF = 512 / BUF_COLS;  // accumulator tiles in tensor memory: 2 of 256 columns, 4 of 128 (the barrier map has four slots)
+    // A group's scales land with its k-block's operands, on the same barrier, in a ring of records that has no "empty" barriers: the
+    // producer loads k-block j when the MMAs of j - STAGES are done, those had waited until the epilogue was through with the group
+    // NBUF accumulator tiles before their last one, so of the groups before k-block j only the last STAGES * GPK + NBUF may still be read.
+    static_assert(SC_SLOTS >= (STAGES + 1) * GPK + NBUF, "scale records");
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
     const uint32_t sc_base = smem_base + STAGES * STAGE_BYTES;
     const uint32_t bar_base = smem_base + BAR_OFFSET;
-    // barriers: full[S], unpacked[S], empty[S], sc_full[SC], sc_empty[SC], tmem_full[NBUF], tmem_empty[NBUF]
+    // barriers: full[S], unpacked[S], empty[S], tmem_full[4], tmem_empty[4], spare, the other CTA's tmem_empty[2]
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
     auto unp_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
     auto empty_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + s); };
-    auto scfull_bar = [&](int s) { return bar_base + 8u * (3 * STAGES + s); };
-    auto scempty_bar = [&](int s) { return bar_base + 8u * (3 * STAGES + SC_SLOTS + s); };
-    auto tfull_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + a); };
-    auto tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 4 + a); };
-    auto peer_tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 9 + a); };  // pairs: in the leader, the other CTA's
+    auto tfull_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + a); };
+    auto tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 4 + a); };
+    auto peer_tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 9 + a); };  // pairs: in the leader, the other CTA's
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + BAR_OFFSET + 400);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + BAR_OFFSET + 404);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
     const int lane = threadIdx.x & 31;
     // Trace build (TRACE_CLK): slot 9 entry, 10 set-up done, 11 previous grid ended, 12 / 13 producer has issued its first k-block /
     // everything, 14 / 15 first unpack warp sees / has expanded the first stage, 16 / 17 / 18 MMA warp starts the first / fifth / last
@@ -121,9 +141,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     // folded in the last group, 23 the rank-r tile, 24 has stored its last outputs.
     if (threadIdx.x == 0) TRACE_CLK(p.status, 9);
 
-    // a tile is BM token rows of one CTA, or of each CTA of a pair
-    const uint32_t crank = PAIR ? cluster_ctarank() : 0u;
-    constexpr int TILE_ROWS = PAIR ? 2 * BM : BM;
+    const uint32_t crank = PAIR ? blockIdx.x & 1u : 0u;  // (the rank in the cluster, known to be uniform)
     const int num_m_blocks = (p.M + TILE_ROWS - 1) / TILE_ROWS;
     const int num_n_blocks = (p.N + BN - 1) / BN;
     auto first_tile = [&]() { return static_cast<int>(PAIR ? blockIdx.x >> 1 : blockIdx.x); };
@@ -137,16 +155,12 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             mbar_init(unp_bar(s), PAIR ? 4 : 64);
             mbar_init(empty_bar(s), 1);
         }
-        for (int s = 0; s < SC_SLOTS; ++s) {
-            mbar_init(scfull_bar(s), 1);
-            mbar_init(scempty_bar(s), NUM_EPI_WARPS * 32);
-        }
         for (int a = 0; a < NBUF; ++a) {
             mbar_init(tfull_bar(a), 1);
             mbar_init(tempty_bar(a), NUM_EPI_WARPS * 32);
             if (PAIR) mbar_init(peer_tempty_bar(a), 1);
         }
-        mbar_init(bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 8), 1);  // spare: see umma_drain
+        mbar_init(bar_base + 8u * (3 * STAGES + 8), 1);  // spare: see umma_drain
         *abort_flag = 0;
         fence_mbar_init();
         tma_prefetch_desc(&tmap_codes);
@@ -185,29 +199,34 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             // (the whole warp walks the loops and waits, one elected lane issues: counters, addresses and coordinates stay
             // warp-uniform, which shortens the chain of instructions per stage)
             {
-                uint32_t it = 0, sc_it = 0;
+                uint32_t it = 0, slot = 0;
                 long long w_empty = 0;
                 bool ok = true;
                 for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
                     const int m0 = tile_row(tile);
                     const int n0 = (tile / num_m_blocks) * BN, w0 = n0 + static_cast<int>(crank) * P::WROWS;
-                    for (int kb = 0; kb < p.num_kb; ++kb, ++it, ++sc_it) {
+                    for (int kb = 0; kb < p.num_kb; ++kb, ++it) {
                         const int s = it % STAGES;
                         if (!timed_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER, w_empty)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
+                        const int groups = min(GPK, p.n_g - kb * GPK);  // (an odd number of groups: the last k-block has one)
                         if (elect_one()) {
-                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + BP_BYTES);
+                            mbar_arrive_expect_tx(full_bar(s), AC_BYTES + BP_BYTES + groups * SC_BYTES);
                             tma_load_2d(st, &tmap_codes, full_bar(s), kb * BKC, m0);
-                            tma_load_2d(st + A_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), w0);
+                            if (ROWS == TALL) tma_load_2d(st + A_BYTES, &tmap_codes, full_bar(s), kb * BKC, m0 + BM);
+                            tma_load_2d(st + AC_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), w0);
                         }
-                        const int slot = sc_it % SC_SLOTS;
-                        if (!mbar_wait(scempty_bar(slot), ((sc_it / SC_SLOTS) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
-                        const uint32_t sc = sc_base + slot * SC_BYTES;
-                        if (elect_one()) {
-                            mbar_arrive_expect_tx(scfull_bar(slot), GPK * (BN + BM) * 4);
-                            tma_load_2d(sc, &tmap_wscale, scfull_bar(slot), n0, kb * GPK);
-                            tma_load_2d(sc + SC_SW_BYTES, &tmap_xscale, scfull_bar(slot), m0, kb * GPK);
-                            if (it == 0) TRACE_CLK(p.status, 12);
+#pragma unroll
+                        for (int gi = 0; gi < GPK; ++gi) {
+                            if (gi < groups) {
+                                if (elect_one()) {
+                                    const uint32_t sc = sc_base + slot * SC_BYTES;
+                                    tma_load_2d(sc, &tmap_wscale, full_bar(s), n0, kb * GPK + gi);
+                                    tma_load_2d(sc + SC_SW_BYTES, &tmap_xscale, full_bar(s), m0, kb * GPK + gi);
+                                    if (it == 0) TRACE_CLK(p.status, 12);
+                                }
+                                if (++slot == SC_SLOTS) slot = 0;
+                            }
                         }
                     }
                     if (!ok) break;
@@ -216,9 +235,10 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         if (!mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         if (elect_one()) {
-                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + BU_BYTES);
+                            mbar_arrive_expect_tx(full_bar(s), AC_BYTES + BU_BYTES);
                             tma_load_2d(st, &tmap_xh, full_bar(s), lr * 64, m0);
-                            tma_load_2d(st + A_BYTES, &tmap_wh, full_bar(s), lr * 64, w0);
+                            if (ROWS == TALL) tma_load_2d(st + A_BYTES, &tmap_xh, full_bar(s), lr * 64, m0 + BM);
+                            tma_load_2d(st + AC_BYTES, &tmap_wh, full_bar(s), lr * 64, w0);
                         }
                     }
                 }
@@ -229,12 +249,6 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     for (uint32_t j = first; j < it; ++j) {
                         const unsigned long long t0 = globaltimer_ns();
                         while (!mbar_try_wait(full_bar(j % STAGES), (j / STAGES) & 1) &&
-                               globaltimer_ns() - t0 < 100000000ull) {}
-                    }
-                    const uint32_t sfirst = sc_it > SC_SLOTS ? sc_it - SC_SLOTS : 0;
-                    for (uint32_t j = sfirst; j < sc_it; ++j) {
-                        const unsigned long long t0 = globaltimer_ns();
-                        while (!mbar_try_wait(scfull_bar(j % SC_SLOTS), (j / SC_SLOTS) & 1) &&
                                globaltimer_ns() - t0 < 100000000ull) {}
                     }
                 }
@@ -260,9 +274,10 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             // word, which cannot overflow: shared-memory addresses have 18 bits, the field holds address / 16).
             // (whole warp in the loops, one elected lane issues, as in the producer)
             {
-                constexpr uint32_t idesc_f8 = umma_idesc(1 /*f32*/, 0 /*E4M3*/, TILE_ROWS, BN);
-                constexpr uint32_t idesc_i8 = umma_idesc(2 /*s32*/, 1 /*s8*/, TILE_ROWS, BN);  // integer-path build only
-                constexpr uint32_t idesc_bf = umma_idesc(1 /*f32*/, 1 /*bf16*/, TILE_ROWS, BN);
+                constexpr uint32_t MMA_ROWS = PAIR ? 2 * BM : BM;
+                constexpr uint32_t idesc_f8 = umma_idesc(1 /*f32*/, 0 /*E4M3*/, MMA_ROWS, BN);
+                constexpr uint32_t idesc_i8 = umma_idesc(2 /*s32*/, 1 /*s8*/, MMA_ROWS, BN);  // integer-path build only
+                constexpr uint32_t idesc_bf = umma_idesc(1 /*f32*/, 1 /*bf16*/, MMA_ROWS, BN);
                 const uint64_t desc0 = umma_desc_sw128(smem_base);
                 const uint32_t desc_hi = static_cast<uint32_t>(desc0 >> 32), desc_lo0 = static_cast<uint32_t>(desc0);
                 auto desc = [&](uint32_t lo) { return (static_cast<uint64_t>(desc_hi) << 32) | lo; };
@@ -283,7 +298,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         if (!timed_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_ops)) { ok = false; break; }
                         if (lane == 0) { if (kb == 0) TRACE_CLK(p.status, 16); if (kb == 4) TRACE_CLK(p.status, 17); if (kb == p.num_kb - 1) TRACE_CLK(p.status, 18); }
                         tc_fence_after_sync();
-                        const uint32_t a_lo = desc_lo0 + s * (STAGE_BYTES >> 4), b_lo = a_lo + (A_BYTES >> 4);
+                        const uint32_t a_lo = desc_lo0 + s * (STAGE_BYTES >> 4), b_lo = a_lo + (AC_BYTES >> 4);
 #pragma unroll
                         for (int gi = 0; gi < GPK; ++gi) {
                             if (gi < groups_left) {
@@ -292,16 +307,20 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                                 tc_fence_after_sync();
                                 if (elect_one()) {
 #pragma unroll
-                                    for (int k = 0; k < MMA_PER_G; ++k) {
-                                        const int kk = gi * MMA_PER_G + k;  // 32-byte step inside the 128-byte row
+                                    for (int k = 0; k < MMA_PER_G * (ROWS == TALL ? 2 : 1); ++k) {
+                                        const int kk = gi * MMA_PER_G + k % MMA_PER_G;  // 32-byte step inside the 128-byte row
+                                        const int half = k / MMA_PER_G;                 // (TALL: the second 128 token rows)
+                                        const uint32_t d = tmem_base + b * BUF_COLS + half * BN;
+                                        const uint64_t ad = desc(a_lo + half * (A_BYTES >> 4) + 2 * kk), bd = desc(b_lo + 2 * kk);
+                                        const uint32_t acc = k % MMA_PER_G != 0;
                                         if constexpr (PAIR && kI8Path)
-                                            umma_i8_pair(tmem_base + b * BN, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), idesc_i8, k != 0);
+                                            umma_i8_pair(d, ad, bd, idesc_i8, acc);
                                         else if constexpr (PAIR)
-                                            umma_f8f6f4_pair(tmem_base + b * BN, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), idesc_f8, k != 0);
+                                            umma_f8f6f4_pair(d, ad, bd, idesc_f8, acc);
                                         else if constexpr (kI8Path)
-                                            umma_i8(tmem_base + b * BN, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), idesc_i8, k != 0);
+                                            umma_i8(d, ad, bd, idesc_i8, acc);
                                         else
-                                            umma_f8f6f4(tmem_base + b * BN, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), idesc_f8, k != 0);
+                                            umma_f8f6f4(d, ad, bd, idesc_f8, acc);
                                     }
                                     commit(tfull_bar(b));
                                 }
@@ -321,12 +340,14 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     for (int lr = 0; lr < p.lr_chunks; ++lr) {
                         if (!mbar_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                         tc_fence_after_sync();
-                        const uint32_t a_lo = desc_lo0 + s * (STAGE_BYTES >> 4), b_lo = a_lo + (A_BYTES >> 4);
+                        const uint32_t a_lo = desc_lo0 + s * (STAGE_BYTES >> 4), b_lo = a_lo + (AC_BYTES >> 4);
                         if (elect_one()) {
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
-                                if constexpr (PAIR) umma_bf16_pair(tmem_base + b * BN, desc(a_lo + 2 * k), desc(b_lo + 2 * k), idesc_bf, (lr | k) != 0);
-                                else umma_bf16(tmem_base + b * BN, desc(a_lo + 2 * k), desc(b_lo + 2 * k), idesc_bf, (lr | k) != 0);
+                                const uint32_t d = tmem_base + b * BUF_COLS;
+                                if constexpr (PAIR) umma_bf16_pair(d, desc(a_lo + 2 * k), desc(b_lo + 2 * k), idesc_bf, (lr | k) != 0);
+                                else umma_bf16(d, desc(a_lo + 2 * k), desc(b_lo + 2 * k), idesc_bf, (lr | k) != 0);
+                                if (ROWS == TALL) umma_bf16(d + BN, desc(a_lo + (A_BYTES >> 4) + 2 * k), desc(b_lo + 2 * k), idesc_bf, (lr | k) != 0);
                             }
                             commit(empty_bar(s));
                         }
@@ -361,10 +382,10 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         // The swizzle phase row%8 = (u/4)%8 and the piece do not depend on j, so every address is
                         // a per-thread base plus a compile-time offset.
                         uint8_t* st = smem_gen + s * STAGE_BYTES;
-                        const uint4* src = reinterpret_cast<const uint4*>(st + A_BYTES + BU_BYTES) + u;
+                        const uint4* src = reinterpret_cast<const uint4*>(st + AC_BYTES + BU_BYTES) + u;
                         const int c = u & 3, sw = (u >> 2) & 7;
-                        uint8_t* d0 = st + A_BYTES + (u >> 2) * 128 + (((2 * c) ^ sw) << 4);
-                        uint8_t* d1 = st + A_BYTES + (u >> 2) * 128 + (((2 * c + 1) ^ sw) << 4);
+                        uint8_t* d0 = st + AC_BYTES + (u >> 2) * 128 + (((2 * c) ^ sw) << 4);
+                        uint8_t* d1 = st + AC_BYTES + (u >> 2) * 128 + (((2 * c + 1) ^ sw) << 4);
                         // The loads of a batch are issued before any of its stores: the compiler cannot prove that the
                         // staging buffer and the operand tile do not overlap, so a load written after a store would wait
                         // for it and the whole unpack would run as one dependent chain.
@@ -413,29 +434,46 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         // per thread (see request_chunk), and the 8 weight scales of the thread's columns, which the layer stores
         // side by side (see wscale_index in common.h), in two 16-byte loads.
         //
-        // The accumulator tiles of an output tile (one per K-group, then the rank-r one) are one stream: while the
-        // last chunk of a tile is folded in, the next tile's barrier is tested (not waited for) and, if it has
-        // completed, its first chunk is requested, so that in the steady state neither the hand-over nor the first
-        // tensor-memory round trip is paid between groups.
+        // The accumulator tiles of an output tile (one per K-group, then the rank-r one) are one stream: before the last chunk
+        // of a tile is folded in, the next tile is waited for (it is there in the steady state: the MMAs of a group take a third
+        // of the rescale) and its first chunk requested, so that neither the hand-over nor the first tensor-memory round trip is
+        // paid between groups.
         const int q = warp & 3;
         const int half = (warp - 4) >> 2;
         const int lr4 = lane >> 2;        // row inside a group of 8
         const int lc2 = (lane & 3) * 2;   // first of this thread's two columns inside a block of 8
-        uint32_t b = 0, bph = 0;          // accumulator tile read next, parity its "full" barrier is waited with
-        uint32_t slot = 0, sph = 0;       // scale slot of the current k-block, parity of its "full" barrier
-        long long w_tfull = 0, w_sc = 0;
+        uint32_t sc_off = 0;              // the current group's scale record
+        long long w_tfull = 0;
         const long long t_epi = clock64();
+        const int cta_row = (ROWS == TALL ? half * BM : 0) + q * 32 + lr4, tile_col = ROWS == TALL ? 0 : half * HB;  // this thread's first row, warp's first column
         const uint32_t taddr0 = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + half * HB;
-        const float* sc0 = reinterpret_cast<const float*>(smem_gen + STAGES * STAGE_BYTES);
+        // The accumulator tile read next (its tensor-memory address and its "full" barrier, the "empty" one lies a fixed distance behind it),
+        // that barrier's parity and the next tile's.
+        uint32_t tcur = taddr0, bcur = tfull_bar(0), pcur = 0, pnxt = 0;
+        auto tnext = [&]() { return NBUF == 2 ? 2 * taddr0 + BUF_COLS - tcur : tcur == taddr0 + (NBUF - 1) * BUF_COLS ? taddr0 : tcur + BUF_COLS; };
+        auto bnext = [&]() { return NBUF == 2 ? 2 * tfull_bar(0) + 8u - bcur : bcur == tfull_bar(NBUF - 1) ? tfull_bar(0) : bcur + 8u; };
+        auto advance = [&](uint32_t t, uint32_t b) {
+            tcur = t;
+            bcur = b;
+            const uint32_t p1 = pcur;
+            pcur = pnxt;
+            // the tile after the next one: two tiles, the one just left, a phase later; four, a phase later than the next one where that is the last
+            pnxt = NBUF == 2 ? p1 ^ 1 : b == tfull_bar(NBUF - 1) ? pnxt ^ 1 : pnxt;
+        };
+        const uint8_t* sw_base = smem_gen + STAGES * STAGE_BYTES + 4 * (tile_col + 4 * lc2);
+        const uint8_t* sx_base = smem_gen + STAGES * STAGE_BYTES + SC_SW_BYTES + 4 * cta_row;
+        // (worked out where they are needed, not held in registers across the groups)
+        auto first_row = [&](int tile) { return tile_row(tile) + cta_row; };  // this thread's rows: first_row + 8 i, i = 0..3
+        auto first_col = [&](int tile) { return (tile / num_m_blocks) * BN + tile_col; };
         // No vote after a wait: the warp is converged there, so the barrier test, the abort flag and the clock are read
         // by one instruction for all lanes and every lane gets the same answer.
         bool ok = true;
         uint32_t raw[2][32];  // [0..15]: TMEM lanes 0..15 of the quadrant (rows i = 0, 1), [16..31]: lanes 16..31
-        auto request_chunk = [&](uint32_t buf, int c, uint32_t* dst) {
+        auto request_chunk = [&](uint32_t tile_addr, int c, uint32_t* dst) {
             // 32 columns move in 32 cycles as two .x2 loads and in 64 as one .x4, which is half the instructions.  Measured on 18 layers, .x2 is
             // ahead by up to 4 %, except in 128-column tiles with groups of 128, where .x4 is by 1 to 2 %.  .x2 / .x4 in us, 4608 -> 1152
             // at 4096 tokens: 256 columns 91.5 / 92.4 (groups of 64), 64.2 / 65.3 (of 128); 128 columns 55.7 / 55.9, 39.7 / 39.0.
-            const uint32_t t = taddr0 + buf * BN + c * 32;
+            const uint32_t t = tile_addr + c * 32;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if constexpr (BN == 128 && G == 128) {
@@ -446,46 +484,35 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 }
             }
         };
-        auto release_tile = [&](uint32_t buf) {  // every tcgen05.ld of this thread on the tile has completed
+        auto release_tile = [&]() {  // every tcgen05.ld of this thread on the current tile has completed
             tc_fence_before_sync();
-            mbar_arrive(tempty_bar(buf));  // all lanes arrive (see the unpack warps' note on the cost of electing one)
+            mbar_arrive(bcur + (tempty_bar(0) - tfull_bar(0)));  // all lanes arrive (see the unpack warps' note on the cost of electing one)
         };
         for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
-            const int m0 = tile_row(tile);
-            const int n0 = (tile / num_m_blocks) * BN;
-            const int rbase = m0 + q * 32 + lr4;  // this thread's rows: rbase + 8 i, i = 0..3
-            const int colbase = n0 + half * HB;
             uint64_t acc2[HB / 2];  // two adjacent columns per 64-bit register: [(block of 8 columns) * 4 + row i]
 #pragma unroll
             for (int j = 0; j < HB / 2; ++j) acc2[j] = 0ull;
 
-            // first scales and first accumulator tile of this output tile
-            ok = timed_wait(scfull_bar(slot), sph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_sc) &&
-                 timed_wait(tfull_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
+            // first accumulator tile of this output tile (its scales landed with the operands it was made from)
+            ok = timed_wait(bcur, pcur, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
             if (!ok) break;
             if (warp == 4 && lane == 0) TRACE_CLK(p.status, 20);
             tc_fence_after_sync();
-            request_chunk(b, 0, raw[0]);
+            request_chunk(tcur, 0, raw[0]);
 
             for (int g = 0; g < p.n_g; ++g) {
                 if (warp == 4 && lane == 0 && g == 8) TRACE_CLK(p.status, 21);
-                const int gi = g & (GPK - 1);
-                const bool last_of_kb = gi == GPK - 1 || g == p.n_g - 1;
-                const float* s_sw = sc0 + slot * (SC_BYTES / 4);
+                const float* s_sx = reinterpret_cast<const float*>(sx_base + sc_off);
+                const ulonglong2* swp = reinterpret_cast<const ulonglong2*>(sw_base + sc_off);
+                sc_off = sc_off == (SC_SLOTS - 1) * SC_BYTES ? 0 : sc_off + SC_BYTES;
                 // the accumulator holds S = 2^-18 P (integer-path build: P as int32, and 2^-18 goes into the token scale)
-                float sxv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    sxv[i] = s_sw[2 * BN + gi * BM + q * 32 + lr4 + 8 * i] * (kI8Path ? 1.0f / kWScaleFold : 1.0f);
                 uint64_t sx2[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) sx2[i] = pack_f32x2(sxv[i], sxv[i]);
-                const ulonglong2* swp = reinterpret_cast<const ulonglong2*>(s_sw + gi * BN + half * HB + 4 * lc2);
-                // what comes after this tile: the next group's, or the rank-r tile
-                const uint32_t nb = b + 1 == NBUF ? 0 : b + 1, nbph = b + 1 == NBUF ? bph ^ 1 : bph;
-                const uint32_t nslot = slot + 1 == SC_SLOTS ? 0 : slot + 1, nsph = slot + 1 == SC_SLOTS ? sph ^ 1 : sph;
-                const bool new_scales = last_of_kb && g + 1 < p.n_g;
-                bool ahead = false;
+                for (int i = 0; i < 4; ++i) {
+                    const float sx = s_sx[8 * i] * (kI8Path ? 1.0f / kWScaleFold : 1.0f);
+                    sx2[i] = pack_f32x2(sx, sx);
+                }
+                const uint32_t tn = tnext(), bn = bnext();  // what comes after this tile: the next group's, or the rank-r tile
 #pragma unroll
                 for (int c = 0; c < CHUNKS; ++c) {
                     uint32_t (&cur)[32] = raw[c & 1];
@@ -503,18 +530,18 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         for (int i = 0; i < 32; ++i) cur[i] = __float_as_uint(__int2float_rn(static_cast<int>(cur[i])));  // |P| < 2^24: exact
                     }
                     if (c < CHUNKS - 1) {
-                        request_chunk(b, c + 1, raw[(c + 1) & 1]);
+                        request_chunk(tcur, c + 1, raw[(c + 1) & 1]);
                     } else {
-                        // the whole tile is in registers: hand it back to the MMA warp, and look at the next one
-                        release_tile(b);
-                        ahead = mbar_test_wait(tfull_bar(nb), nbph) && (!new_scales || mbar_test_wait(scfull_bar(nslot), nsph));
-                        if (ahead) {
-                            tc_fence_after_sync();
-                            request_chunk(nb, 0, raw[0]);  // CHUNKS is even: the last chunk sits in raw[1]
-                        }
+                        // the whole tile is in registers: hand it back to the MMA warp, and request the next one's first chunk
+                        release_tile();
+                        ok = timed_wait(bn, pnxt, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
+                        if (!ok) break;
+                        tc_fence_after_sync();
+                        request_chunk(tn, 0, raw[0]);  // CHUNKS is even: the last chunk sits in raw[1]
                     }
                     if constexpr (kPartials) {
                         // unit scales here: 2^18 S = P, an integer
+                        const int rbase = first_row(tile), colbase = first_col(tile);
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -545,21 +572,8 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                             }
                     }
                 }
-                if (last_of_kb) {
-                    // this k-block's scales have all been read (the multiply-adds that consumed them were issued above)
-                    mbar_arrive(scempty_bar(slot));
-                    slot = nslot;
-                    sph = nsph;
-                }
-                b = nb;
-                bph = nbph;
-                if (!ahead) {
-                    if (new_scales) ok = timed_wait(scfull_bar(slot), sph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_sc);
-                    ok = ok && timed_wait(tfull_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
-                    if (!ok) break;
-                    tc_fence_after_sync();
-                    request_chunk(b, 0, raw[0]);
-                }
+                if (!ok) break;
+                advance(tn, bn);
             }
             if (!ok) break;
             if (warp == 4 && lane == 0) TRACE_CLK(p.status, 22);
@@ -569,8 +583,8 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 uint32_t (&cur)[32] = raw[c & 1];
                 tmem_ld_wait();
                 tmem_ld_fence(cur);
-                if (c < CHUNKS - 1) request_chunk(b, c + 1, raw[(c + 1) & 1]);
-                else release_tile(b);
+                if (c < CHUNKS - 1) request_chunk(tcur, c + 1, raw[(c + 1) & 1]);
+                else release_tile();
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -580,13 +594,14 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         acc2[a] = add_f32x2(acc2[a], pack_u32x2(cur[pidx], cur[pidx + 1]));
                     }
             }
-            if (++b == NBUF) { b = 0; bph ^= 1; }
+            advance(tnext(), bnext());
             if (warp == 4 && lane == 0) TRACE_CLK(p.status, 23);
             if constexpr (!kPartials) {
                 // A lane holds 2 of the 8 columns of every block; four blocks are transposed inside the quad of lanes
                 // (two exchange steps) so that each lane ends up with all 8 columns = 16 bytes of one block and the
                 // warp writes 64 contiguous bytes per row.
                 const int j = lane & 3;
+                const int rbase = first_row(tile), colbase = first_col(tile);
 #pragma unroll
                 for (int m = 0; m < CHUNKS; ++m) {
                     float2 bv[4];
@@ -623,13 +638,12 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         if (warp == 4 && lane == 0) TRACE_CLK(p.status, 24);
         if (warp == 4 && lane == 0) {
             flush_wait(p.status, WS_EPI_TFULL, w_tfull);
-            flush_wait(p.status, WS_EPI_SCALES, w_sc);
             flush_wait(p.status, WS_EPI_TOTAL, clock64() - t_epi);
         }
     }
 
     // ---------------------------------------------------------------- teardown
-    if (warp == 1 && lane == 0 && crank == 0 && *abort_flag != 0) umma_drain<PAIR>(bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 8));  // a wait gave up: let issued MMAs finish first
+    if (warp == 1 && lane == 0 && crank == 0 && *abort_flag != 0) umma_drain<PAIR>(bar_base + 8u * (3 * STAGES + 8));  // a wait gave up: let issued MMAs finish first
     tc_fence_before_sync();
     if constexpr (PAIR) cluster_sync_all();  // neither CTA leaves while the other may still read its operands or signal its barriers
     else __syncthreads();
@@ -640,8 +654,10 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     }
 }
 
-template <int BN, bool PAIR = false>
+template <int BN, Rows ROWS = ONE>
 static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream) {
+    using P = Plan<BN, ROWS>;
+    constexpr bool PAIR = ROWS == PAIRED;
     const Geometry& g = L->geo;
     CUtensorMap tmap_codes, tmap_xscale, tmap_xh;
     dirotq_status_t st;
@@ -649,7 +665,7 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
                         (uint64_t)g.K_lp, BKC, BM, CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
     st = encode_tmap_2d(&tmap_xscale, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.xscale, (uint64_t)a.ldm, (uint64_t)g.n_g,
-                        (uint64_t)a.ldm * 4, BM, BKC / g.G, CU_TENSOR_MAP_SWIZZLE_NONE);
+                        (uint64_t)a.ldm * 4, P::CTA_ROWS, 1, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st != DIROTQ_OK) return st;
     st = encode_tmap_2d(&tmap_xh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.xh, (uint64_t)g.r_pad, (uint64_t)a.M,
                         (uint64_t)g.r_pad * 2, 64, BM, CU_TENSOR_MAP_SWIZZLE_128B);
@@ -662,19 +678,18 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
     p.bias = reinterpret_cast<const float*>(L->blob + L->lay.off_bias);
     p.y = a.y; p.partials = a.partials; p.status = a.status;
 
-    using P = Plan<BN, PAIR>;
-    constexpr int TILE_ROWS = PAIR ? 2 * BM : BM, CTAS = PAIR ? 2 : 1;
-    const int num_tiles = ((a.M + TILE_ROWS - 1) / TILE_ROWS) * ((g.N + BN - 1) / BN), slots = sm_count(L->device) / CTAS;
+    constexpr int CTAS = PAIR ? 2 : 1;
+    const int num_tiles = ((a.M + P::TILE_ROWS - 1) / P::TILE_ROWS) * ((g.N + BN - 1) / BN), slots = sm_count(L->device) / CTAS;
     const int grid = CTAS * (num_tiles < slots ? num_tiles : slots);
     using KernelFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                               const CUtensorMap, const CUtensorMap, const GemmKernelParams);
     KernelFn kern;
     const bool dbg = a.partials != nullptr;
-    if constexpr (PAIR) {  // (the debug entry's group sums come from single CTAs)
-        kern = g.G == 64 ? w4a4_gemm_kernel<64, false, BN, true> : w4a4_gemm_kernel<128, false, BN, true>;
+    if constexpr (ROWS != ONE) {  // (the debug entry's group sums come from the other plans)
+        kern = g.G == 64 ? w4a4_gemm_kernel<64, false, BN, ROWS> : w4a4_gemm_kernel<128, false, BN, ROWS>;
     } else {
-        if (g.G == 64) kern = dbg ? w4a4_gemm_kernel<64, true, BN, false> : w4a4_gemm_kernel<64, false, BN, false>;
-        else           kern = dbg ? w4a4_gemm_kernel<128, true, BN, false> : w4a4_gemm_kernel<128, false, BN, false>;
+        if (g.G == 64) kern = dbg ? w4a4_gemm_kernel<64, true, BN, ONE> : w4a4_gemm_kernel<64, false, BN, ONE>;
+        else           kern = dbg ? w4a4_gemm_kernel<128, true, BN, ONE> : w4a4_gemm_kernel<128, false, BN, ONE>;
     }
     static SmemOptIn<4> opt_in;  // one per instantiation of this launcher, i.e. per tile width
     const int vi = (g.G == 64 ? 0 : 2) + (dbg ? 1 : 0);
@@ -694,25 +709,34 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
 static std::atomic<int> g_tile_columns{0};  // 0: chosen per call; 64 / 128 / 192 / 256: forced; 66: 64 columns, split plan where it applies
 
 dirotq_status_t set_w4a4_tile_columns(int columns) {
-    if (columns != 0 && columns != 64 && columns != 66 && columns != 128 && columns != 192 && columns != 256 && columns != 512) return DIROTQ_ERR_INVALID_ARG;
+    if (columns != 0 && columns != 64 && columns != 66 && columns != 128 && columns != 192 && columns != 256 && columns != 512 && columns != 130) return DIROTQ_ERR_INVALID_ARG;
     g_tile_columns.store(columns);
     return DIROTQ_OK;
 }
 
 dirotq_status_t launch_w4a4_gemm(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream) {
-    // The plan with the shortest schedule: turns of the SMs x what one tile of the plan costs.  Costs relative to a 256-column tile, from
-    // the cycles per 128 codes of a tile: 2360, 1390 and 780 with groups of 64, 1600, 990 and 620 with groups of 128 (the
-    // activation tile, the rank-r branch, the pipeline fill and the hand-overs are paid per tile whatever its width).
-    // A turn of pair tiles takes 0.957 of a turn of 256-column tiles with groups of 64, 0.86 with groups of 128; a pair covers two row blocks, which can
-    // cost it a turn (4173 x 3072 -> 12288: 12 turns against 11, 349 us against 339).
+    // The plan with the shortest schedule: turns of the SMs (or of the pairs of SMs) x what one tile of the plan costs.  Costs relative to a pair's tile,
+    // from 4608 x 3072 -> 9216 (a turn of pairs: 26.2 us with groups of 64, 17.0 with groups of 128).  Over 60 shapes of 16 to 12003
+    // rows, 512 to 11776 coefficients and 560 to 11184 columns what is chosen is within 3 % of the fastest plan, in the mean within 0.3 %.
     const int forced = g_tile_columns.load(), sms = sm_count(L->device);
-    const long m_blocks = (a.M + BM - 1) / BM;
-    auto turns = [&](int columns) { return static_cast<double>((m_blocks * ((L->geo.N + columns - 1) / columns) + sms - 1) / sms); };
-    const double c256 = turns(256), c128 = (L->geo.G == 64 ? 0.60 : 0.64) * turns(128), c64 = (L->geo.G == 64 ? 0.34 : 0.40) * turns(64);
-    const double c512 = (L->geo.G == 64 ? 0.957 : 0.86) * static_cast<double>(((m_blocks + 1) / 2 * ((L->geo.N + 255) / 256) + sms / 2 - 1) / (sms / 2));
-    const int plan = forced ? forced : c512 < c256 && c512 <= c128 && c512 <= c64 ? 512 : c64 <= c128 && c64 <= c256 ? 64 : c128 < c256 ? 128 : 256;
+    const bool g64 = L->geo.G == 64;
+    struct Candidate { int knob, rows, columns, ctas; double cost64, cost128; };
+    static constexpr Candidate kPlans[] = {{64, 128, 64, 1, 0.378, 0.454}, {128, 128, 128, 1, 0.615, 0.73}, {192, 128, 192, 1, 0.846, 0.957},
+                                           {130, 256, 128, 1, 1.02, 1.03}, {256, 128, 256, 1, 1.068, 1.21}, {512, 256, 256, 2, 1.0, 1.0}};
+    int plan = forced;
+    double best = 0.0;
+    for (const Candidate& c : kPlans) {
+        if (forced) break;
+        const long tiles = static_cast<long>((a.M + c.rows - 1) / c.rows) * ((L->geo.N + c.columns - 1) / c.columns), slots = sms / c.ctas;
+        const double t = static_cast<double>((tiles + slots - 1) / slots) * (g64 ? c.cost64 : c.cost128);
+        if (plan == 0 || t < best) {
+            plan = c.knob;
+            best = t;
+        }
+    }
     if (a.partials == nullptr && (plan == 64 || plan == 66)) return launch_w4a4_narrow(L, a, plan == 66, stream);
-    if (plan == 512 && a.partials == nullptr) return launch_w4a4_gemm_bn<256, true>(L, a, stream);
+    if (plan == 512 && a.partials == nullptr) return launch_w4a4_gemm_bn<256, PAIRED>(L, a, stream);
+    if (plan == 130 && a.partials == nullptr) return launch_w4a4_gemm_bn<128, TALL>(L, a, stream);
     if (plan == 192) return launch_w4a4_gemm_bn<192>(L, a, stream);
     return plan >= 256 ? launch_w4a4_gemm_bn<256>(L, a, stream) : launch_w4a4_gemm_bn<128>(L, a, stream);
 }

@@ -1,5 +1,6 @@
-"""The grouped INT4 second kernel in CTA pairs (256 token rows x 256 columns): the edges of its tiles against the oracle, and the
-same bits as single CTAs where a pair takes several tiles (each output element is accumulated in the same order)."""
+"""The grouped INT4 second kernel with tiles of 256 token rows, in CTA pairs (512: x 256 columns) and in one CTA (130: x 128 columns): the edges
+of the tiles against the oracle, and the same bits as the other plans where a CTA takes several tiles (each output element is
+accumulated in the same order)."""
 import pytest
 import torch
 
@@ -9,7 +10,7 @@ from paper_2605_16732_b200 import binding as dq
 from paper_2605_16732_b200 import synth
 
 pytestmark = pytest.mark.gpu
-PLANS = [512]
+PLANS = [512, 130]
 
 
 @pytest.fixture
