@@ -716,19 +716,20 @@ dirotq_status_t set_w4a4_tile_columns(int columns) {
 
 dirotq_status_t launch_w4a4_gemm(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream) {
     // The plan with the shortest schedule: turns of the SMs (or of the pairs of SMs) x what one tile of the plan costs.  Costs relative to a pair's tile,
-    // from 4608 x 3072 -> 9216 (a turn of pairs: 26.2 us with groups of 64, 17.0 with groups of 128).  Over 60 shapes of 16 to 12003
-    // rows, 512 to 11776 coefficients and 560 to 11184 columns what is chosen is within 3 % of the fastest plan, in the mean within 0.3 %.
+    // from 4608 x 3072 -> 9216 (a turn of pairs: 26.2 us with groups of 64, 17.0 with groups of 128), whose clusters cost a call 0.9 us more.  Over 110
+    // shapes of 16 to 17816 rows, 512 to 11776 coefficients and 512 to 12240 columns what is chosen is within 3 % of the fastest plan, in the mean
+    // within 0.5 % (one call of 7 us: 5 %).
     const int forced = g_tile_columns.load(), sms = sm_count(L->device);
     const bool g64 = L->geo.G == 64;
     struct Candidate { int knob, rows, columns, ctas; double cost64, cost128; };
-    static constexpr Candidate kPlans[] = {{64, 128, 64, 1, 0.378, 0.454}, {128, 128, 128, 1, 0.615, 0.73}, {192, 128, 192, 1, 0.846, 0.957},
+    static constexpr Candidate kPlans[] = {{64, 128, 64, 1, 0.295, 0.38}, {128, 128, 128, 1, 0.615, 0.73}, {192, 128, 192, 1, 0.846, 0.957},
                                            {130, 256, 128, 1, 1.02, 1.03}, {256, 128, 256, 1, 1.068, 1.21}, {512, 256, 256, 2, 1.0, 1.0}};
     int plan = forced;
     double best = 0.0;
     for (const Candidate& c : kPlans) {
         if (forced) break;
         const long tiles = static_cast<long>((a.M + c.rows - 1) / c.rows) * ((L->geo.N + c.columns - 1) / c.columns), slots = sms / c.ctas;
-        const double t = static_cast<double>((tiles + slots - 1) / slots) * (g64 ? c.cost64 : c.cost128);
+        const double t = static_cast<double>((tiles + slots - 1) / slots) * (g64 ? c.cost64 : c.cost128) + (c.ctas == 2 ? 100.0 / L->geo.K_lp : 0.0);
         if (plan == 0 || t < best) {
             plan = c.knob;
             best = t;

@@ -5,8 +5,11 @@
 // long as the chain: more, narrower tiles on more SMs, and a short chain.  A tensor-memory buffer holds the accumulator tiles
 // of ALL groups of a k-block of 128 codes, so there is one hand-over per k-block where w4a4_gemm.cu has one per group; the
 // two unpack warps take k-blocks in turn (half of a turn is waiting); the epilogue asks for a unit's scales with the unit.
-// With groups of 64 a k-block takes 760 to 780 cycles, with one hand-over per group it took 1060: 1152 -> 1152 at
-// 256 tokens (replayed from a graph) 8.6 -> 6.9 us, 3072 -> 9216 at 16 tokens 18.0 -> 15.5.
+// With groups of 64 a k-block takes 590 cycles: the expansion, the MMA warp's chain of waits, MMAs and commits and the epilogue's chain per
+// buffer are each busy for 80 to 95 % of them.  It took 780 with barriers and tests of their own for the scales (now they land with the operands),
+// the next buffer's first unit requested at one of two places, and addresses that were not known to be uniform, and 1060 with one hand-over
+// per group: us alone, 256 x 1152 -> 1152 7.0 -> 6.0, 16 x 12288 -> 3072 41.0 -> 29.8, 64 x 3072 -> 9216 13.3 -> 10.4.  Tried: a whole buffer
+// per tensor-memory wait 0 to 6 % slower, three expanding warps in a block of 16 warps 4 to 13 %.
 //
 // Roles (384 threads = 3 warpgroups):
 //   warpgroup 0: warp 0 TMA producer, warp 1 MMA issuer + TMEM owner, warps 2-3 nibble -> byte unpack (k-blocks in turn)
@@ -28,7 +31,7 @@ constexpr int SPLIT_MAX = 4;          // CTAs per cluster of the split plan
 constexpr int NUM_EPI_WARPS = 8, NUM_THREADS = 384;
 constexpr int EPI_REGS = 224, AUX_REGS = 56;  // setmaxnreg budgets: 256 x EPI + 128 x AUX <= 384 x 168
 constexpr int RED_BYTES = 128 * 64 * 4;  // one CTA's partial tile: 128 rows x 64 columns fp32
-constexpr int SC_SLOTS = 8;
+constexpr int SC_SLOTS = 11;          // scale records, one per k-block
 constexpr int BU_BYTES = BN * BKC;         // unpacked weight codes / bf16 W~_h chunk
 constexpr int BP_BYTES = BN * BKC / 2;     // packed weight codes (TMA staging)
 constexpr int STAGE_BYTES = A_BYTES + BU_BYTES + BP_BYTES;  // 28 KB
@@ -45,7 +48,10 @@ struct Plan {
     static constexpr int RED_OFFSET = BAR_OFFSET + 512;  // split plan: the other CTAs' partial tiles land here (last CTA)
     static constexpr int SMEM_BYTES = BAR_OFFSET + 512 + 1024 + (SPLITK ? (SPLIT_MAX - 1) * RED_BYTES : 0);
     static_assert(SMEM_BYTES <= 232448 && STAGE_BYTES % 1024 == 0 && SC_BYTES % 128 == 0, "shared memory plan");
-    static_assert(8 * (3 * STAGES + 2 * SC_SLOTS + 11) <= 400, "barriers end below the words at +400");
+    static_assert(8 * (3 * STAGES + 11) <= 400, "barriers end below the words at +400");
+    // A k-block's scales land with its operands, on the same barrier, in a ring of their own that has no "empty" barriers: the producer
+    // loads k-block j when the MMAs of j - STAGES are done, those had waited until the epilogue was through with the buffer four before.
+    static_assert(SC_SLOTS >= STAGES + 5, "scale records");
 };
 
 template <int G, bool SPLITK>
@@ -69,18 +75,16 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
     uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
     const uint32_t sc_base = smem_base + STAGES * STAGE_BYTES;
     const uint32_t bar_base = smem_base + BAR_OFFSET;
-    // barriers: full[S], unpacked[S], empty[S], sc_full[SC], sc_empty[SC], tmem_full[NBUF], tmem_empty[NBUF]
+    // barriers: full[S], unpacked[S], empty[S], tmem_full[NBUF], tmem_empty[NBUF], spare, split plan's two
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
     auto unp_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
     auto empty_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + s); };
-    auto scfull_bar = [&](int s) { return bar_base + 8u * (3 * STAGES + s); };
-    auto scempty_bar = [&](int s) { return bar_base + 8u * (3 * STAGES + SC_SLOTS + s); };
-    auto tfull_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + a); };
-    auto tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 4 + a); };
+    auto tfull_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + a); };
+    auto tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 4 + a); };
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + BAR_OFFSET + 400);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + BAR_OFFSET + 404);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // (known to be uniform)
     const int lane = threadIdx.x & 31;
     // Trace build (TRACE_CLK): slot 9 entry, 10 set-up done, 11 previous grid ended, 12 / 13 producer has issued its first k-block /
     // everything, 14 / 15 first unpack warp sees / has expanded the first stage, 16 / 17 / 18 MMA warp starts the first / fifth / last
@@ -91,7 +95,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
     const int num_m_blocks = (p.M + BM - 1) / BM;
     const int num_n_blocks = (p.N + BN - 1) / BN;
     const int num_tiles = num_m_blocks * num_n_blocks;
-    // Split plan: this CTA's range of k-blocks [kb0, kb1) and of K-groups [g0, g1) of the cluster's tile (the first ranks take
+    // Split plan: this CTA's range of k-blocks [kb0, kb1) of the cluster's tile (the first ranks take
     // one k-block more when the division leaves a rest); the LAST rank gathers the partial tiles and has the rank-r branch.
     // (Without the split every one of these is the constant or the parameter it stands for.)
     const uint32_t csize = SPLITK ? cluster_nctarank() : 1u, crank = SPLITK ? cluster_ctarank() : 0u;
@@ -99,13 +103,12 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
     const int split_base = SPLITK ? p.num_kb / static_cast<int>(csize) : 0, split_rest = SPLITK ? p.num_kb % static_cast<int>(csize) : 0;
     const int kb0 = SPLITK ? static_cast<int>(crank) * split_base + min(static_cast<int>(crank), split_rest) : 0;
     const int kb1 = SPLITK ? kb0 + split_base + (static_cast<int>(crank) < split_rest ? 1 : 0) : p.num_kb;
-    const int g0 = SPLITK ? kb0 * GPK : 0, g1 = SPLITK ? min(kb1 * GPK, p.n_g) : p.n_g;
     const int lr_here = gathers ? p.lr_chunks : 0;
     // (tile loops read these where they are needed, like blockIdx.x and gridDim.x themselves, not held in registers across the
     // roles' loops)
     auto first_tile = [&]() { return SPLITK ? static_cast<int>(blockIdx.x / csize) : static_cast<int>(blockIdx.x); };
     auto tile_stride = [&]() { return SPLITK ? static_cast<int>(gridDim.x / csize) : static_cast<int>(gridDim.x); };
-    const uint32_t red_bar = bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 9);  // split plan: "partial tiles landed" (last CTA)
+    const uint32_t red_bar = bar_base + 8u * (3 * STAGES + 9);  // split plan: "partial tiles landed" (last CTA)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -113,15 +116,11 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
             mbar_init(unp_bar(s), 32);  // every thread of the unpack warp whose turn it is arrives for itself
             mbar_init(empty_bar(s), 1);
         }
-        for (int s = 0; s < SC_SLOTS; ++s) {
-            mbar_init(scfull_bar(s), 1);
-            mbar_init(scempty_bar(s), NUM_EPI_WARPS * 32);
-        }
         for (int a = 0; a < NBUF; ++a) {
             mbar_init(tfull_bar(a), 1);
             mbar_init(tempty_bar(a), NUM_EPI_WARPS * 32);
         }
-        mbar_init(bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 8), 1);  // spare: see umma_drain
+        mbar_init(bar_base + 8u * (3 * STAGES + 8), 1);  // spare: see umma_drain
         if constexpr (SPLITK) {
             mbar_init(red_bar, 1);  // counts the bytes of the other CTAs' partial tiles
             mbar_init(red_bar + 8u, NUM_EPI_WARPS * 32);  // this CTA's partial tile is in its shared memory (every epilogue thread arrives)
@@ -160,30 +159,26 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
             // (the whole warp walks the loops and waits, one elected lane issues: counters, addresses and coordinates stay
             // warp-uniform, which shortens the chain of instructions per stage)
             {
-                uint32_t it = 0, sc_it = 0;
+                uint32_t it = 0, slot = 0;
                 long long w_empty = 0;
                 bool ok = true;
                 for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
                     const int m0 = (tile % num_m_blocks) * BM;
                     const int n0 = (tile / num_m_blocks) * BN;
-                    for (int kb = kb0; kb < kb1; ++kb, ++it, ++sc_it) {
+                    for (int kb = kb0; kb < kb1; ++kb, ++it) {
                         const int s = it % STAGES;
                         if (!timed_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER, w_empty)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         if (elect_one()) {
-                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + BP_BYTES);
+                            const uint32_t sc = sc_base + slot * SC_BYTES;
+                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + BP_BYTES + GPK * (BN + BM) * 4);
                             tma_load_2d(st, &tmap_codes, full_bar(s), kb * BKC, m0);
                             tma_load_2d(st + A_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), n0);
-                        }
-                        const int slot = sc_it % SC_SLOTS;
-                        if (!mbar_wait(scempty_bar(slot), ((sc_it / SC_SLOTS) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
-                        const uint32_t sc = sc_base + slot * SC_BYTES;
-                        if (elect_one()) {
-                            mbar_arrive_expect_tx(scfull_bar(slot), GPK * (BN + BM) * 4);
-                            tma_load_2d(sc, &tmap_wscale, scfull_bar(slot), n0, kb * GPK);
-                            tma_load_2d(sc + SC_SW_BYTES, &tmap_xscale, scfull_bar(slot), m0, kb * GPK);
+                            tma_load_2d(sc, &tmap_wscale, full_bar(s), n0, kb * GPK);
+                            tma_load_2d(sc + SC_SW_BYTES, &tmap_xscale, full_bar(s), m0, kb * GPK);
                             if (it == 0) TRACE_CLK(p.status, 12);
                         }
+                        if (++slot == SC_SLOTS) slot = 0;
                     }
                     if (!ok) break;
                     for (int lr = 0; lr < lr_here; ++lr, ++it) {
@@ -204,12 +199,6 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                     for (uint32_t j = first; j < it; ++j) {
                         const unsigned long long t0 = globaltimer_ns();
                         while (!mbar_try_wait(full_bar(j % STAGES), (j / STAGES) & 1) &&
-                               globaltimer_ns() - t0 < 100000000ull) {}
-                    }
-                    const uint32_t sfirst = sc_it > SC_SLOTS ? sc_it - SC_SLOTS : 0;
-                    for (uint32_t j = sfirst; j < sc_it; ++j) {
-                        const unsigned long long t0 = globaltimer_ns();
-                        while (!mbar_try_wait(scfull_bar(j % SC_SLOTS), (j / SC_SLOTS) & 1) &&
                                globaltimer_ns() - t0 < 100000000ull) {}
                     }
                 }
@@ -246,7 +235,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
 #pragma unroll
                             for (int kk = 0; kk < 4; ++kk) {  // 32-byte step inside the 128-byte row
                                 const int gi = kk / MMA_PER_G, k = kk % MMA_PER_G;
-                                if (gi > 0 && GPK * kb + gi >= p.n_g) break;  // an odd number of groups: the last k-block has one
+                                // (an odd number of groups: the last k-block's second one is zeros, codes and scales)
                                 if constexpr (kI8Path)
                                     umma_i8(d + gi * BN, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), idesc_i8, k != 0);
                                 else
@@ -356,16 +345,16 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
         //
         // The buffers of an output tile (one per k-block, then the rank-r one) are one stream of units in two register sets: while
         // one is folded in, the next and its column scales are on their way.  When a buffer's last unit has arrived, the buffer
-        // goes back to the MMA warp, the next buffer's barriers are tested (not waited for) and, if they have completed, its first
-        // unit is requested, all before the last unit is folded in; so in the steady state neither the hand-over nor a round
-        // trip to tensor or shared memory is paid, and there is one hand-over per 128 codes. 
+        // goes back to the MMA warp, the next buffer is waited for (it is there in the steady state) and its first
+        // unit requested, all before the last unit is folded in; so neither the hand-over nor a round
+        // trip to tensor or shared memory is paid, and there is one hand-over per 128 codes.
         const int q = warp & 3;
         const int half = (warp - 4) >> 2;
         const int lr4 = lane >> 2;        // row inside a group of 8
         const int lc2 = (lane & 3) * 2;   // first of this thread's two columns inside a block of 8
         uint32_t b = 0, bph = 0;          // accumulator tile read next, parity its "full" barrier is waited with
-        uint32_t slot = 0, sph = 0;       // scale slot of the current k-block, parity of its "full" barrier
-        long long w_tfull = 0, w_sc = 0;
+        uint32_t slot = 0;                // scale record of the current k-block
+        long long w_tfull = 0;
         const long long t_epi = clock64();
         const uint32_t taddr0 = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + half * HB;
         // No vote after a wait: the warp is converged there, so the barrier test, the abort flag and the clock are read
@@ -419,6 +408,16 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
         for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
             const int m0 = (tile % num_m_blocks) * BM;
             const int n0 = (tile / num_m_blocks) * BN;
+            if (!SPLITK && m0 + q * 32 >= p.M) {  // a warp without token rows only hands the buffers back
+                for (int i = kb0; i <= kb1; ++i) {
+                    ok = mbar_wait(tfull_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE);
+                    if (!ok) break;
+                    release_tile(b);
+                    if (++b == NBUF) { b = 0; bph ^= 1; }
+                    if (i < kb1 && ++slot == SC_SLOTS) slot = 0;
+                }
+                continue;
+            }
             const int rbase = m0 + q * 32 + lr4;  // this thread's rows: rbase + 8 i, i = 0..3
             const int colbase = n0 + half * HB;
             uint64_t acc2[HB / 2];  // two adjacent columns per 64-bit register: [(block of 8 columns) * 4 + row i]
@@ -447,43 +446,38 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
 
             // first buffer and scales of this output tile (split plan: of this CTA's range, which may be empty, and only the gathering
             // CTA has a rank-r tile)
-            if (!SPLITK || kb1 > kb0) {
-                ok = timed_wait(scfull_bar(slot), sph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_sc);
-                if (ok) request_scales(slot, 0);
-            }
             if (!SPLITK || kb1 > kb0 || lr_here > 0) {
-                ok = ok && timed_wait(tfull_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
+                ok = timed_wait(tfull_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
                 if (!ok) break;
                 if (warp == 4 && lane == 0) TRACE_CLK(p.status, 20);
                 tc_fence_after_sync();
                 request_unit(b, 0, raw[0]);
+                if (!SPLITK || kb1 > kb0) request_scales(slot, 0);  // (they landed with the operands the buffer was made from)
             }
 
             for (int kb = kb0; kb < kb1; ++kb) {
                 if (warp == 4 && lane == 0 && kb * GPK == 8) TRACE_CLK(p.status, 21);
                 // what comes after this buffer: the next k-block's, or the rank-r tile
                 const uint32_t nb = b + 1 == NBUF ? 0 : b + 1, nbph = b + 1 == NBUF ? bph ^ 1 : bph;
-                const uint32_t nslot = slot + 1 == SC_SLOTS ? 0 : slot + 1, nsph = slot + 1 == SC_SLOTS ? sph ^ 1 : sph;
+                const uint32_t nslot = slot + 1 == SC_SLOTS ? 0 : slot + 1;
                 const bool new_scales = kb + 1 < kb1;
                 const bool more = !SPLITK || new_scales || lr_here > 0;  // another buffer follows (always, unless split)
-                const int nu = GPK == 1 || 2 * kb + 1 < p.n_g ? NU : UPG;  // an odd number of groups: the last k-block has one
-                bool ahead = false;
 #pragma unroll
                 for (int u = 0; u < NU; ++u) {
-                    if (u >= nu) break;
                     unit_arrived(raw[u & 1]);
                     if constexpr (GPK == 1) {
 #pragma unroll
                         for (int i = 0; i < 4; ++i) sxv[0][i] = u == 0 ? sxv[1][i] : sxv[0][i];
                     }
-                    if (u + 1 < nu) {
+                    if (u + 1 < NU) {
                         request_unit(b, u + 1, raw[(u + 1) & 1]);
                         request_scales(slot, u + 1);
                     } else {
-                        // the whole buffer is in registers: hand it back to the MMA warp, and look at the next one
+                        // the whole buffer is in registers: hand it back to the MMA warp, and request the next one's first unit
                         release_tile(b);
-                        ahead = u == NU - 1 && more && mbar_test_wait(tfull_bar(nb), nbph) && (!new_scales || mbar_test_wait(scfull_bar(nslot), nsph));
-                        if (ahead) {
+                        if (more) {
+                            ok = timed_wait(tfull_bar(nb), nbph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
+                            if (!ok) break;
                             tc_fence_after_sync();
                             request_unit(nb, 0, raw[0]);  // (NU is even: the last unit sits in raw[1])
                             if (new_scales) request_scales(nslot, 0);
@@ -491,20 +485,10 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                     }
                     fold_unit(u);
                 }
-                // this k-block's scales have all been read (the multiply-adds that consumed them were issued above)
-                mbar_arrive(scempty_bar(slot));
+                if (!ok) break;
                 slot = nslot;
-                sph = nsph;
                 b = nb;
                 bph = nbph;
-                if (!ahead && more) {
-                    if (new_scales) ok = timed_wait(scfull_bar(slot), sph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_sc);
-                    ok = ok && timed_wait(tfull_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_EPILOGUE, w_tfull);
-                    if (!ok) break;
-                    tc_fence_after_sync();
-                    request_unit(b, 0, raw[0]);
-                    if (new_scales) request_scales(slot, 0);
-                }
             }
             if (!ok) break;
             if (warp == 4 && lane == 0) TRACE_CLK(p.status, 22);
@@ -594,13 +578,12 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
         if (warp == 4 && lane == 0) TRACE_CLK(p.status, 24);
         if (warp == 4 && lane == 0) {
             flush_wait(p.status, WS_EPI_TFULL, w_tfull);
-            flush_wait(p.status, WS_EPI_SCALES, w_sc);
             flush_wait(p.status, WS_EPI_TOTAL, clock64() - t_epi);
         }
     }
 
     // ---------------------------------------------------------------- teardown
-    if (warp == 1 && lane == 0 && *abort_flag != 0) umma_drain(bar_base + 8u * (3 * STAGES + 2 * SC_SLOTS + 8));  // a wait gave up: let issued MMAs finish first
+    if (warp == 1 && lane == 0 && *abort_flag != 0) umma_drain(bar_base + 8u * (3 * STAGES + 8));  // a wait gave up: let issued MMAs finish first
     tc_fence_before_sync();
     __syncthreads();
     if constexpr (SPLITK) cluster_sync_all();  // no CTA of the cluster leaves while another may still write into it or signal it
