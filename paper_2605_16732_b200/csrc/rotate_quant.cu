@@ -19,6 +19,11 @@
 // stages, so the ring depth, i.e. the latency of a loaded L2, sets the rate), with the MMAs 0.064 ms (a
 // stage is only refilled once its MMAs have completed, which adds their time to each slot's cycle), with
 // the epilogue 0.069 ms (0.074 ms with four epilogue warps).  All 227 KB of shared memory are in use.
+//
+// Where there are few tiles per SM the producer's and the MMA warp's chains of instructions per stage set the pace: warp numbers known to be uniform,
+// stage, parity and descriptor carried along instead of divided out and rebuilt took two k-blocks of a 64-column tile from 826 to 572 cycles;
+// us alone, before and after: 256 x 1152 7.1 -> 6.4, 200 x 3072 12.5 -> 11.0, 512 x 3072 (asymmetric) 16.0 -> 13.8, 4096 x 1152 13.0 -> 11.2,
+// 4173 x 3072 projection form 24.3 -> 19.8; 4608 x 3072 the same.
 #include "common.h"
 #include "ptx.cuh"
 
@@ -243,14 +248,14 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + STAGES * STAGE_BYTES + 192);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + STAGES * STAGE_BYTES + 196);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // (known to be uniform: roles, addresses and barriers follow from it)
     const int lane = threadIdx.x & 31;
     // Trace build (TRACE_CLK): slot 9 entry, 10 set-up done, 11 previous grid ended, 12 producer has filled the ring once, 13 producer has
     // issued everything, 14 / 15 MMA warp sees the first / ninth stage, 16 MMA warp has committed its last tile, 17 first epilogue
     // warp sees its first accumulator, 18 that warp has finished its last tile.
     if (threadIdx.x == 0) TRACE_CLK(p.status, 9);
 
-    const uint32_t cta_rank = PAIR ? cluster_ctarank() : 0u;
+    const uint32_t cta_rank = PAIR ? blockIdx.x & 1u : 0u;  // (the rank in the cluster)
     constexpr int TILE_ROWS = PAIR ? 2 * BM : BM;  // token rows of a tile (of the pair's tile)
     const int tile_first = PAIR ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
     const int tile_step = PAIR ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
@@ -307,7 +312,11 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // then stay warp-uniform, which shortens the chain of instructions per stage (337 against 475 cycles per stage
         // measured with 18 SMs busy, where that chain paces the kernel).
         {
-            uint32_t it = 0;
+            uint32_t it = 0, s = 0, ph = 0;  // stage and parity carried along, not divided out
+            auto step = [&]() {
+                ++it;
+                if (++s == STAGES) { s = 0; ph ^= 1; }
+            };
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
                 const int mn = PH ? num_mn - 1 - tile : tile % num_mn, sp = tile / num_mn;
@@ -316,9 +325,7 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 if constexpr (PH) {
                     const int nv = num_kb;                            // k-blocks of the projection term
                     const int nx = min(BN, p.n_out - n0) / BK;        // 64-column pieces of x under this tile
-                    for (int i = 0; i < nv + nx; ++i, ++it) {
-                        const int s = it % STAGES;
-                        const uint32_t ph = (it / STAGES) & 1;
+                    for (int i = 0; i < nv + nx; ++i, step()) {
                         if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                         const uint32_t sa = smem_base + s * STAGE_BYTES;
                         if (!elect_one()) continue;
@@ -337,9 +344,7 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 }
                 // a split reduction is dealt out k-block by k-block: range sp takes k-blocks sp, sp + ksplit, ... (measured the
                 // same as contiguous ranges)
-                for (int kb = sp; kb < num_kb; kb += p.ksplit * KSUB, ++it) {
-                    const int s = it % STAGES;
-                    const uint32_t ph = (it / STAGES) & 1;
+                for (int kb = sp; kb < num_kb; kb += p.ksplit * KSUB, step()) {
                     if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                     const uint32_t sa = smem_base + s * STAGE_BYTES;
                     if (!elect_one()) continue;
@@ -388,7 +393,12 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // ------------------------------------------------------------ MMA issuer (whole warp in the loops, one lane issues)
         if (cta_rank == 0) {
             constexpr uint32_t idesc = umma_idesc(1 /*f32*/, 1 /*bf16*/, PAIR ? 2 * BM_MMA : BM_MMA, BN);
-            uint32_t it = 0, tcount = 0;
+            uint32_t it = 0, tcount = 0, s = 0, ph = 0;
+            auto step = [&]() {
+                ++it;
+                if (++s == STAGES) { s = 0; ph ^= 1; }
+            };
+            const uint64_t desc0 = umma_desc_sw128(smem_base);  // (stages differ in the address field of the low word, which cannot overflow)
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step, ++tcount) {
                 const uint32_t acc = tcount % ACC_BUFS;
@@ -400,14 +410,10 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     constexpr uint32_t idesc_g = umma_idesc(1 /*f32*/, 1 /*bf16*/, BM_MMA, G);
                     const int n0 = ((num_mn - 1 - tile) / num_m_blocks) * BN;
                     const int nv = num_kb, nx = min(BN, p.n_out - n0) / BK;
-                    for (int i = 0; i < nv + nx; ++i, ++it) {
-                        const int s = it % STAGES;
-                        const uint32_t ph = (it / STAGES) & 1;
+                    for (int i = 0; i < nv + nx; ++i, step()) {
                         if (!mbar_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                         tc_fence_after_sync();
-                        const uint32_t sa = smem_base + s * STAGE_BYTES;
-                        const uint64_t adesc = umma_desc_sw128(sa);
-                        const uint64_t bdesc = umma_desc_sw128(sa + A_BYTES);
+                        const uint64_t adesc = desc0 + s * (STAGE_BYTES >> 4), bdesc = adesc + (A_BYTES >> 4);
                         if (!elect_one()) continue;
                         if (i < nv) {
 #pragma unroll
@@ -424,14 +430,10 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 }
                 const int sp = tile / num_mn;
                 const int kb_begin = sp;
-                for (int kb = kb_begin; kb < num_kb; kb += p.ksplit * KSUB, ++it) {
-                    const int s = it % STAGES;
-                    const uint32_t ph = (it / STAGES) & 1;
+                for (int kb = kb_begin; kb < num_kb; kb += p.ksplit * KSUB, step()) {
                     if (!mbar_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                     tc_fence_after_sync();
-                    const uint32_t sa = smem_base + s * STAGE_BYTES;
-                    const uint64_t adesc = umma_desc_sw128(sa);
-                    const uint64_t bdesc = umma_desc_sw128(sa + A_BYTES);
+                    const uint64_t adesc = desc0 + s * (STAGE_BYTES >> 4), bdesc = adesc + (A_BYTES >> 4);
                     if (!elect_one()) continue;
                     if (it == 0) TRACE_CLK(p.status, 14);
                     if (it == 8) TRACE_CLK(p.status, 15);
