@@ -167,14 +167,14 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + BAR_OFFSET + 192);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + BAR_OFFSET + 196);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // (known to be uniform)
     const int lane = threadIdx.x & 31;
     // Trace build (TRACE_CLK), stages 6..8 of the block's first tile: slots 9..11 producer has issued the stage, 12..14 first copier warp
     // sees it landed, 15..17 / 18..20 first / second copier warp has committed its scale copies, 21..23 MMA warp sees the scales
     // ready, 24..26 it has committed the stage's MMAs; tiles 0, 1, 2 of the first epilogue warp: accumulator seen / released / outputs
     // handed over in slots 27..29, 1..3, 4..6; slot 30 entry.
     if (threadIdx.x == 0) TRACE_CLK(p.status, 30);
-    const uint32_t cta_rank = PAIR ? cluster_ctarank() : 0u;
+    const uint32_t cta_rank = PAIR ? blockIdx.x & 1u : 0u;  // (the rank in the cluster)
     constexpr int TILE_ROWS = PAIR ? 2 * BM : BM;  // token rows of a tile (of the pair's tile)
     const int tile_first = PAIR ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
     const int tile_step = PAIR ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
@@ -226,7 +226,7 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
         // (the whole warp walks the loops and waits, one elected lane issues: counters, addresses and coordinates stay
         // warp-uniform, which shortens the chain of instructions per stage; the same in the MMA and copier warps)
         {
-            uint32_t it = 0;
+            RingPos<STAGES> at;
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
                 // m_blk: this CTA's block of 128 token rows
@@ -238,9 +238,9 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
                 // pairs: the second CTA's block of rows may lie past M (odd number of row blocks): it has no scale atoms
                 // (its codes are read as zeros, its outputs never stored)
                 const int sfa_here = m0 < p.M ? 1 : 0;
-                for (int kb = 0; kb < p.num_kb; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
+                for (int kb = 0; kb < p.num_kb; ++kb, at.next()) {
+                    const uint32_t s = at.s;
+                    if (!mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                     const uint32_t st = smem_base + s * STAGE_BYTES;
                     if (!elect_one()) continue;
                     mbar_arrive_expect_tx(full_bar(s), A_BYTES + B_BYTES + (sfa_here + nb_here) * SF_BYTES);
@@ -255,12 +255,12 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
                     // the atoms of the tile's 128-column blocks for this k-block are contiguous: one copy
                     bulk_load(st + A_BYTES + B_BYTES + SF_BYTES, p.wsf + wsf_atom_offset(n_blk * NB, kb * 4, p.nkb64p),
                               nb_here * SF_BYTES, full_bar(s));
-                    if (it >= 6 && it <= 8) TRACE_CLK(p.status, 3 + it);
+                    if (at.it >= 6 && at.it <= 8) TRACE_CLK(p.status, 3 + at.it);
                 }
                 if (!ok) break;
-                for (int lr = 0; lr < p.lr_chunks; ++lr, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
+                for (int lr = 0; lr < p.lr_chunks; ++lr, at.next()) {
+                    const uint32_t s = at.s;
+                    if (!mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                     const uint32_t st = smem_base + s * STAGE_BYTES;
                     if (!elect_one()) continue;
                     mbar_arrive_expect_tx(full_bar(s), A_BYTES + B_BYTES);
@@ -272,8 +272,8 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
                 }
             }
             if (!ok && lane == 0) {
-                const uint32_t first = it > STAGES ? it - STAGES : 0;
-                for (uint32_t j = first; j < it; ++j) {
+                const uint32_t first = at.it > STAGES ? at.it - STAGES : 0;
+                for (uint32_t j = first; j < at.it; ++j) {
                     const unsigned long long t0 = globaltimer_ns();
                     while (!mbar_try_wait(full_bar(j % STAGES), (j / STAGES) & 1) && globaltimer_ns() - t0 < 100000000ull) {}
                 }
@@ -284,25 +284,26 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
         if (cta_rank == 0) {
             constexpr uint32_t idesc_nv = nvfp4_idesc(TILE_ROWS, BN);
             constexpr uint32_t idesc_bf = umma_idesc(1 /*f32*/, 1 /*bf16*/, TILE_ROWS, BN);
-            uint32_t it = 0, tcount = 0;
+            RingPos<STAGES> at;
+            uint32_t tcount = 0;
+            const uint64_t desc0 = umma_desc_sw128(smem_base);  // (stages differ in the low word's address field, which cannot overflow)
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step, ++tcount) {
                 const uint32_t acc = tcount % ACC_BUFS;
                 if (!mbar_wait(tempty_bar(acc), ((tcount / ACC_BUFS) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                 tc_fence_after_sync();
                 const uint32_t d = tmem_base + acc * BN;
-                for (int kb = 0; kb < p.num_kb; ++kb, ++it) {
-                    const int s = it % STAGES;
+                for (int kb = 0; kb < p.num_kb; ++kb, at.next()) {
+                    const uint32_t s = at.s;
                     const uint32_t st = smem_base + s * STAGE_BYTES;
                     const uint32_t tsf = tmem_base + TMEM_SF_BASE + s * SF_COLS;
                     // the scale factors of this stage are copied into tensor memory by the copier warps, which have seen the
                     // stage's loads land first (in both CTAs of a pair): their barrier covers the operands as well
-                    if (!mbar_wait(sfready_bar(s), (it / STAGES) & 1, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
+                    if (!mbar_wait(sfready_bar(s), at.ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                     tc_fence_after_sync();
-                    const uint64_t adesc = umma_desc_sw128(st);
-                    const uint64_t bdesc = umma_desc_sw128(st + A_BYTES);
+                    const uint64_t adesc = desc0 + s * (STAGE_BYTES >> 4), bdesc = adesc + (A_BYTES >> 4);
                     if (!elect_one()) continue;
-                    if (it >= 6 && it <= 8) TRACE_CLK(p.status, 15 + it);
+                    if (at.it >= 6 && at.it <= 8) TRACE_CLK(p.status, 15 + at.it);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {  // K = 64 elements = 32 bytes per instruction
                         if constexpr (PAIR)
@@ -312,16 +313,15 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
                     }
                     if constexpr (PAIR) umma_commit_pair(empty_bar(s), 3);  // both CTAs' producers may refill the stage
                     else umma_commit(empty_bar(s));
-                    if (it >= 6 && it <= 8) TRACE_CLK(p.status, 18 + it);
+                    if (at.it >= 6 && at.it <= 8) TRACE_CLK(p.status, 18 + at.it);
                 }
                 if (!ok) break;
-                for (int lr = 0; lr < p.lr_chunks; ++lr, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(sfready_bar(s), (it / STAGES) & 1, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
+                for (int lr = 0; lr < p.lr_chunks; ++lr, at.next()) {
+                    const uint32_t s = at.s;
+                    if (!mbar_wait(sfready_bar(s), at.ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint32_t st = smem_base + s * STAGE_BYTES;
-                    const uint64_t adesc = umma_desc_sw128(st);
-                    const uint64_t bdesc = umma_desc_sw128(st + A_BYTES);
+                    const uint64_t adesc = desc0 + s * (STAGE_BYTES >> 4), bdesc = adesc + (A_BYTES >> 4);
                     if (!elect_one()) continue;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
@@ -344,27 +344,27 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
         // copier thread, itself the bound; 0.093 ms with two).  Each copier hands its half of a stage over through an
         // mbarrier that tcgen05.commit arrives on once the copies have landed in tensor memory.
         {
-            uint32_t it = 0;
+            RingPos<STAGES> at;
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
                 const int items = p.num_kb + p.lr_chunks;
-                for (int i = 0; i < items; ++i, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(full_bar(s), (it / STAGES) & 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
+                for (int i = 0; i < items; ++i, at.next()) {
+                    const uint32_t s = at.s;
+                    if (!mbar_wait(full_bar(s), at.ph, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
                     if constexpr (PAIR) {
                         if (cta_rank != 0) {
                             // this CTA's stage has landed: one word to the leader, whose copiers and MMA thread act for both
                             if (warp == 2 && elect_one()) mbar_arrive_cluster(map_to_cta(peer_bar(s), 0));
                             continue;
                         }
-                        if (!mbar_wait(peer_bar(s), (it / STAGES) & 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
+                        if (!mbar_wait(peer_bar(s), at.ph, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
                     }
                     if (i < p.num_kb) {
                         tc_fence_after_sync();
                         const uint32_t sf = smem_base + s * STAGE_BYTES + A_BYTES + B_BYTES;
                         const uint32_t tsf = tmem_base + TMEM_SF_BASE + s * SF_COLS;
                         if (!elect_one()) continue;
-                        if (warp == 2 && it >= 6 && it <= 8) TRACE_CLK(p.status, 6 + it);
+                        if (warp == 2 && at.it >= 6 && at.it <= 8) TRACE_CLK(p.status, 6 + at.it);
                         if (warp == 2) {
                             // activation scales: the four K = 64 steps of the k-block, 4 columns each
 #pragma unroll
@@ -386,7 +386,7 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
                         }
                         if constexpr (PAIR) umma_commit_pair(sfready_bar(s), 1);  // the leader's barrier only
                         else umma_commit(sfready_bar(s));
-                        if (it >= 6 && it <= 8) TRACE_CLK(p.status, (warp == 2 ? 9 : 12) + it);
+                        if (at.it >= 6 && at.it <= 8) TRACE_CLK(p.status, (warp == 2 ? 9 : 12) + at.it);
                     } else if (elect_one()) {
                         mbar_arrive(sfready_bar(s));  // a rank-r chunk: nothing to copy
                     }

@@ -124,6 +124,20 @@ __device__ __forceinline__ bool elect_one() {
     return pred != 0;
 }
 
+// Place in a ring of STAGES slots: item number, slot and parity of the slot's current phase, carried along.  (Divided out of the item
+// number they lengthen the chain of instructions per stage of the warps that issue loads and MMAs, which sets the pace of small calls.)
+template <int STAGES>
+struct RingPos {
+    uint32_t it = 0, s = 0, ph = 0;
+    __device__ __forceinline__ void next() {
+        ++it;
+        if (++s == STAGES) {
+            s = 0;
+            ph ^= 1;
+        }
+    }
+};
+
 // ---------------------------------------------------------------- proxies / fences
 
 __device__ __forceinline__ void fence_proxy_async_smem() {

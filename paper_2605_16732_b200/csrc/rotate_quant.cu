@@ -312,11 +312,7 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // then stay warp-uniform, which shortens the chain of instructions per stage (337 against 475 cycles per stage
         // measured with 18 SMs busy, where that chain paces the kernel).
         {
-            uint32_t it = 0, s = 0, ph = 0;  // stage and parity carried along, not divided out
-            auto step = [&]() {
-                ++it;
-                if (++s == STAGES) { s = 0; ph ^= 1; }
-            };
+            RingPos<STAGES> at;
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
                 const int mn = PH ? num_mn - 1 - tile : tile % num_mn, sp = tile / num_mn;
@@ -325,7 +321,8 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 if constexpr (PH) {
                     const int nv = num_kb;                            // k-blocks of the projection term
                     const int nx = min(BN, p.n_out - n0) / BK;        // 64-column pieces of x under this tile
-                    for (int i = 0; i < nv + nx; ++i, step()) {
+                    for (int i = 0; i < nv + nx; ++i, at.next()) {
+                        const uint32_t s = at.s, ph = at.ph;
                         if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                         const uint32_t sa = smem_base + s * STAGE_BYTES;
                         if (!elect_one()) continue;
@@ -344,7 +341,8 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 }
                 // a split reduction is dealt out k-block by k-block: range sp takes k-blocks sp, sp + ksplit, ... (measured the
                 // same as contiguous ranges)
-                for (int kb = sp; kb < num_kb; kb += p.ksplit * KSUB, step()) {
+                for (int kb = sp; kb < num_kb; kb += p.ksplit * KSUB, at.next()) {
+                    const uint32_t s = at.s, ph = at.ph;
                     if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                     const uint32_t sa = smem_base + s * STAGE_BYTES;
                     if (!elect_one()) continue;
@@ -355,7 +353,7 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                             tma_load_2d(sa + j * SUB_BYTES, &tmap_x, full_bar(s), (kb + j) * BK, m0);
                             tma_load_2d(sa + j * SUB_BYTES + A_BYTES, &tmap_qt, full_bar(s), (kb + j) * BK, n0);
                         }
-                        if (it == STAGES - 1) TRACE_CLK(p.status, 12);
+                        if (at.it == STAGES - 1) TRACE_CLK(p.status, 12);
                         continue;
                     }
                     if constexpr (PAIR) {
@@ -369,7 +367,7 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         tma_load_2d(sa, &tmap_x, full_bar(s), kb * BK, m0);
                         tma_load_2d(sa + A_BYTES, &tmap_qt, full_bar(s), kb * BK, n0);
                     }
-                    if (it == STAGES - 1) TRACE_CLK(p.status, 12);
+                    if (at.it == STAGES - 1) TRACE_CLK(p.status, 12);
                 }
             }
             if (lane == 0) TRACE_CLK(p.status, 13);
@@ -381,8 +379,8 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 while (globaltimer_ns() - t0 < 1000000ull) {}
             } else if (!ok) {
                 // leave no bulk copy in flight: wait (bounded) for the loads already issued
-                const uint32_t first = it > STAGES ? it - STAGES : 0;
-                for (uint32_t j = first; j < it; ++j) {
+                const uint32_t first = at.it > STAGES ? at.it - STAGES : 0;
+                for (uint32_t j = first; j < at.it; ++j) {
                     const unsigned long long t0 = globaltimer_ns();
                     while (!mbar_try_wait(full_bar(j % STAGES), (j / STAGES) & 1) &&
                            globaltimer_ns() - t0 < 100000000ull) {}
@@ -393,11 +391,8 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // ------------------------------------------------------------ MMA issuer (whole warp in the loops, one lane issues)
         if (cta_rank == 0) {
             constexpr uint32_t idesc = umma_idesc(1 /*f32*/, 1 /*bf16*/, PAIR ? 2 * BM_MMA : BM_MMA, BN);
-            uint32_t it = 0, tcount = 0, s = 0, ph = 0;
-            auto step = [&]() {
-                ++it;
-                if (++s == STAGES) { s = 0; ph ^= 1; }
-            };
+            RingPos<STAGES> at;
+            uint32_t tcount = 0;
             const uint64_t desc0 = umma_desc_sw128(smem_base);  // (stages differ in the address field of the low word, which cannot overflow)
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step, ++tcount) {
@@ -410,7 +405,8 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     constexpr uint32_t idesc_g = umma_idesc(1 /*f32*/, 1 /*bf16*/, BM_MMA, G);
                     const int n0 = ((num_mn - 1 - tile) / num_m_blocks) * BN;
                     const int nv = num_kb, nx = min(BN, p.n_out - n0) / BK;
-                    for (int i = 0; i < nv + nx; ++i, step()) {
+                    for (int i = 0; i < nv + nx; ++i, at.next()) {
+                        const uint32_t s = at.s, ph = at.ph;
                         if (!mbar_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                         tc_fence_after_sync();
                         const uint64_t adesc = desc0 + s * (STAGE_BYTES >> 4), bdesc = adesc + (A_BYTES >> 4);
@@ -430,13 +426,14 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 }
                 const int sp = tile / num_mn;
                 const int kb_begin = sp;
-                for (int kb = kb_begin; kb < num_kb; kb += p.ksplit * KSUB, step()) {
+                for (int kb = kb_begin; kb < num_kb; kb += p.ksplit * KSUB, at.next()) {
+                    const uint32_t s = at.s, ph = at.ph;
                     if (!mbar_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint64_t adesc = desc0 + s * (STAGE_BYTES >> 4), bdesc = adesc + (A_BYTES >> 4);
                     if (!elect_one()) continue;
-                    if (it == 0) TRACE_CLK(p.status, 14);
-                    if (it == 8) TRACE_CLK(p.status, 15);
+                    if (at.it == 0) TRACE_CLK(p.status, 14);
+                    if (at.it == 8) TRACE_CLK(p.status, 15);
                     if constexpr (KSUB > 1) {
                         const int nsub = min(KSUB, num_kb - kb);
                         for (int j = 0; j < nsub; ++j) {

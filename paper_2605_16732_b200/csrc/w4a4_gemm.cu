@@ -133,7 +133,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + BAR_OFFSET + 400);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + BAR_OFFSET + 404);
 
-    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // (known to be uniform)
     const int lane = threadIdx.x & 31;
     // Trace build (TRACE_CLK): slot 9 entry, 10 set-up done, 11 previous grid ended, 12 / 13 producer has issued its first k-block /
     // everything, 14 / 15 first unpack warp sees / has expanded the first stage, 16 / 17 / 18 MMA warp starts the first / fifth / last
@@ -199,15 +199,16 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             // (the whole warp walks the loops and waits, one elected lane issues: counters, addresses and coordinates stay
             // warp-uniform, which shortens the chain of instructions per stage)
             {
-                uint32_t it = 0, slot = 0;
+                RingPos<STAGES> at;
+                uint32_t slot = 0;
                 long long w_empty = 0;
                 bool ok = true;
                 for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
                     const int m0 = tile_row(tile);
                     const int n0 = (tile / num_m_blocks) * BN, w0 = n0 + static_cast<int>(crank) * P::WROWS;
-                    for (int kb = 0; kb < p.num_kb; ++kb, ++it) {
-                        const int s = it % STAGES;
-                        if (!timed_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER, w_empty)) { ok = false; break; }
+                    for (int kb = 0; kb < p.num_kb; ++kb, at.next()) {
+                        const uint32_t s = at.s;
+                        if (!timed_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER, w_empty)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         const int groups = min(GPK, p.n_g - kb * GPK);  // (an odd number of groups: the last k-block has one)
                         if (elect_one()) {
@@ -223,16 +224,16 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                                     const uint32_t sc = sc_base + slot * SC_BYTES;
                                     tma_load_2d(sc, &tmap_wscale, full_bar(s), n0, kb * GPK + gi);
                                     tma_load_2d(sc + SC_SW_BYTES, &tmap_xscale, full_bar(s), m0, kb * GPK + gi);
-                                    if (it == 0) TRACE_CLK(p.status, 12);
+                                    if (at.it == 0) TRACE_CLK(p.status, 12);
                                 }
                                 if (++slot == SC_SLOTS) slot = 0;
                             }
                         }
                     }
                     if (!ok) break;
-                    for (int lr = 0; lr < p.lr_chunks; ++lr, ++it) {
-                        const int s = it % STAGES;
-                        if (!mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
+                    for (int lr = 0; lr < p.lr_chunks; ++lr, at.next()) {
+                        const uint32_t s = at.s;
+                        if (!mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         if (elect_one()) {
                             mbar_arrive_expect_tx(full_bar(s), AC_BYTES + BU_BYTES);
@@ -245,8 +246,8 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 if (lane == 0) TRACE_CLK(p.status, 13);
                 if (lane == 0) flush_wait(p.status, WS_PROD_EMPTY, w_empty);
                 if (!ok && lane == 0) {
-                    const uint32_t first = it > STAGES ? it - STAGES : 0;
-                    for (uint32_t j = first; j < it; ++j) {
+                    const uint32_t first = at.it > STAGES ? at.it - STAGES : 0;
+                    for (uint32_t j = first; j < at.it; ++j) {
                         const unsigned long long t0 = globaltimer_ns();
                         while (!mbar_try_wait(full_bar(j % STAGES), (j / STAGES) & 1) &&
                                globaltimer_ns() - t0 < 100000000ull) {}
@@ -367,16 +368,16 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         } else {
             // -------------------------------------------------------- nibble -> byte unpack (warps 2, 3)
             const int u = threadIdx.x - 64;  // 0..63
-            uint32_t it = 0;
+            RingPos<STAGES> at;
             long long w_full = 0;
             bool ok = true;
             for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
                 const int items = p.num_kb + p.lr_chunks;
-                for (int i = 0; i < items; ++i, ++it) {
-                    const int s = it % STAGES;
-                    ok = timed_wait(full_bar(s), (it / STAGES) & 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK, w_full);
+                for (int i = 0; i < items; ++i, at.next()) {
+                    const uint32_t s = at.s;
+                    ok = timed_wait(full_bar(s), at.ph, abort_flag, p.status, DEV_TIMEOUT_UNPACK, w_full);
                     if (!ok) break;
-                    if (it == 0 && u == 0) TRACE_CLK(p.status, 14);
+                    if (at.it == 0 && u == 0) TRACE_CLK(p.status, 14);
                     if (i < p.num_kb) {
                         // 16-byte piece idx = u + 64 j of the packed tile: row = idx/4 = u/4 + 16 j, piece c = u%4.
                         // The swizzle phase row%8 = (u/4)%8 and the piece do not depend on j, so every address is
@@ -418,7 +419,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     } else {
                         mbar_arrive(unp_bar(s));
                     }
-                    if (it == 0 && u == 0) TRACE_CLK(p.status, 15);
+                    if (at.it == 0 && u == 0) TRACE_CLK(p.status, 15);
                 }
             }
             if (u == 0) flush_wait(p.status, WS_UNPACK_FULL, w_full);

@@ -159,15 +159,16 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
             // (the whole warp walks the loops and waits, one elected lane issues: counters, addresses and coordinates stay
             // warp-uniform, which shortens the chain of instructions per stage)
             {
-                uint32_t it = 0, slot = 0;
+                RingPos<STAGES> at;
+                uint32_t slot = 0;
                 long long w_empty = 0;
                 bool ok = true;
                 for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
                     const int m0 = (tile % num_m_blocks) * BM;
                     const int n0 = (tile / num_m_blocks) * BN;
-                    for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                        const int s = it % STAGES;
-                        if (!timed_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER, w_empty)) { ok = false; break; }
+                    for (int kb = kb0; kb < kb1; ++kb, at.next()) {
+                        const uint32_t s = at.s;
+                        if (!timed_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER, w_empty)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         if (elect_one()) {
                             const uint32_t sc = sc_base + slot * SC_BYTES;
@@ -176,14 +177,14 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                             tma_load_2d(st + A_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), n0);
                             tma_load_2d(sc, &tmap_wscale, full_bar(s), n0, kb * GPK);
                             tma_load_2d(sc + SC_SW_BYTES, &tmap_xscale, full_bar(s), m0, kb * GPK);
-                            if (it == 0) TRACE_CLK(p.status, 12);
+                            if (at.it == 0) TRACE_CLK(p.status, 12);
                         }
                         if (++slot == SC_SLOTS) slot = 0;
                     }
                     if (!ok) break;
-                    for (int lr = 0; lr < lr_here; ++lr, ++it) {
-                        const int s = it % STAGES;
-                        if (!mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
+                    for (int lr = 0; lr < lr_here; ++lr, at.next()) {
+                        const uint32_t s = at.s;
+                        if (!mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         if (elect_one()) {
                             mbar_arrive_expect_tx(full_bar(s), A_BYTES + BU_BYTES);
@@ -195,8 +196,8 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                 if (lane == 0) TRACE_CLK(p.status, 13);
                 if (lane == 0) flush_wait(p.status, WS_PROD_EMPTY, w_empty);
                 if (!ok && lane == 0) {
-                    const uint32_t first = it > STAGES ? it - STAGES : 0;
-                    for (uint32_t j = first; j < it; ++j) {
+                    const uint32_t first = at.it > STAGES ? at.it - STAGES : 0;
+                    for (uint32_t j = first; j < at.it; ++j) {
                         const unsigned long long t0 = globaltimer_ns();
                         while (!mbar_try_wait(full_bar(j % STAGES), (j / STAGES) & 1) &&
                                globaltimer_ns() - t0 < 100000000ull) {}

@@ -89,7 +89,7 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + BAR_OFFSET + 192);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + BAR_OFFSET + 196);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // (known to be uniform)
     const int lane = threadIdx.x & 31;
     // Trace build (TRACE_CLK), stages 10..12 of the block's first tile: slots 9..11 producer has issued the stage, 12..14 first unpack warp
     // sees it landed, 15..17 it has expanded it, 18..20 MMA warp starts on it; tiles 0, 1, 2 of the first epilogue warp: accumulators
@@ -137,21 +137,21 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         // (the whole warp walks the loops and waits, one elected lane issues: counters, addresses and coordinates stay
         // warp-uniform, which shortens the chain of instructions per stage; the same in the MMA warp)
         {
-            uint32_t it = 0;
+            RingPos<STAGES> at;
             bool ok = true;
             for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
                 const int m0 = (tile % num_m_blocks) * BM;
                 const int n0 = (tile / num_m_blocks) * BN;
-                for (int i = 0; i < items; ++i, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
+                for (int i = 0; i < items; ++i, at.next()) {
+                    const uint32_t s = at.s;
+                    if (!mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                     const uint32_t st = smem_base + s * STAGE_BYTES;
                     if (!elect_one()) continue;
                     if (i < p.num_kb) {
                         mbar_arrive_expect_tx(full_bar(s), A_BYTES + BP_BYTES);
                         tma_load_2d(st, &tmap_codes, full_bar(s), i * BKC, m0);
                         tma_load_2d(st + BP_OFFSET, &tmap_wpacked, full_bar(s), i * (BKC / 2), n0);
-                        if (it >= 10 && it <= 12) TRACE_CLK(p.status, it - 1);
+                        if (at.it >= 10 && at.it <= 12) TRACE_CLK(p.status, at.it - 1);
                     } else {
                         mbar_arrive_expect_tx(full_bar(s), A_BYTES + BU_BYTES);
                         tma_load_2d(st, &tmap_xh, full_bar(s), (i - p.num_kb) * 64, m0);
@@ -160,8 +160,8 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 }
             }
             if (!ok && lane == 0) {  // let the copies in flight land before the CTA's shared memory goes away
-                const uint32_t first = it > STAGES ? it - STAGES : 0;
-                for (uint32_t j = first; j < it; ++j) {
+                const uint32_t first = at.it > STAGES ? at.it - STAGES : 0;
+                for (uint32_t j = first; j < at.it; ++j) {
                     const unsigned long long t0 = globaltimer_ns();
                     while (!mbar_try_wait(full_bar(j % STAGES), (j / STAGES) & 1) && globaltimer_ns() - t0 < 100000000ull) {}
                 }
@@ -172,25 +172,25 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         {
             constexpr uint32_t idesc_i8 = umma_idesc(2 /*s32*/, 1 /*s8*/, BM, BN);
             constexpr uint32_t idesc_bf = umma_idesc(1 /*f32*/, 1 /*bf16*/, BM, BN);
-            uint32_t it = 0, tcount = 0;
+            RingPos<STAGES> at;
+            uint32_t tcount = 0;
+            const uint64_t desc0 = umma_desc_sw128(smem_base);  // (stages differ in the low word's address field, which cannot overflow)
             bool ok = true;
             for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x, ++tcount) {
                 // with narrow tiles two accumulator pairs alternate: a tile's epilogue runs under the next tile's MMAs
                 const uint32_t acc = tcount % NACC, tacc = tmem_base + acc * 2 * BN;
                 if (!mbar_wait(tempty_bar(acc), ((tcount / NACC) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                 tc_fence_after_sync();
-                for (int i = 0; i < items; ++i, ++it) {
-                    const int s = it % STAGES;
-                    const uint32_t ph = (it / STAGES) & 1;
+                for (int i = 0; i < items; ++i, at.next()) {
+                    const uint32_t s = at.s, ph = at.ph;
                     // (the unpack warps arrive after they have seen the stage's loads land, and one barrier counts both operands'
                     // bytes: their barrier covers the activation codes as well)
                     if (!mbar_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint32_t st = smem_base + s * STAGE_BYTES;
-                    const uint64_t adesc = umma_desc_sw128(st);
-                    const uint64_t bdesc = umma_desc_sw128(st + A_BYTES);
+                    const uint64_t adesc = desc0 + s * (STAGE_BYTES >> 4), bdesc = adesc + (A_BYTES >> 4);
                     if (!elect_one()) continue;
-                    if (it >= 10 && it <= 12) TRACE_CLK(p.status, it + 8);
+                    if (at.it >= 10 && at.it <= 12) TRACE_CLK(p.status, at.it + 8);
                     if (i < p.num_kb) {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) umma_i8(tacc, adesc + 2 * k, bdesc + 2 * k, idesc_i8, (i | k) != 0);
@@ -207,14 +207,14 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     } else if (warp < 2 + NUM_UNPACK_WARPS) {
         // ------------------------------------------------------------ nibble -> byte unpack (warps 2..5)
         const int u = threadIdx.x - 64;  // 0..127
-        uint32_t it = 0;
+        RingPos<STAGES> at;
         bool ok = true;
         for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
-            for (int i = 0; i < items; ++i, ++it) {
-                const int s = it % STAGES;
+            for (int i = 0; i < items; ++i, at.next()) {
+                const uint32_t s = at.s;
                 // The four unpack warps meet at a hardware barrier below, which has no time limit: they must all go on or
                 // all give up.  Every thread reaches this reducing barrier once per item whatever its wait returned.
-                const bool mine = mbar_wait(full_bar(s), (it / STAGES) & 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK);
+                const bool mine = mbar_wait(full_bar(s), at.ph, abort_flag, p.status, DEV_TIMEOUT_UNPACK);
                 uint32_t any_failed;
                 asm volatile(
                     "{\n\t"
@@ -228,7 +228,7 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     : "memory");
                 ok = any_failed == 0;
                 if (!ok) break;
-                if (u == 0 && it >= 10 && it <= 12) TRACE_CLK(p.status, it + 2);
+                if (u == 0 && at.it >= 10 && at.it <= 12) TRACE_CLK(p.status, at.it + 2);
                 if (i < p.num_kb) {
                     // 16-byte piece idx = u + 128 j of the packed tile: row = idx / 4 = u / 4 + 32 j, piece c = u % 4; the
                     // swizzle phase row % 8 and the piece do not depend on j
@@ -257,7 +257,7 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     }
                     fence_proxy_async_smem();
                 }
-                if (u == 0 && it >= 10 && it <= 12) TRACE_CLK(p.status, it + 5);
+                if (u == 0 && at.it >= 10 && at.it <= 12) TRACE_CLK(p.status, at.it + 5);
                 mbar_arrive(unp_bar(s));  // every lane arrives for itself: a warp barrier followed by one elected lane's arrival costs about a hundred cycles more
             }
         }

@@ -11,6 +11,8 @@
 // weights, expanded weights), the expansion done by three teams of two warps that take k-blocks in turn (one team's turn is
 // mostly waiting).  A k-block takes 650 cycles, of which the MMAs 512.  Second kernel, before -> after: 4608 x 3072 -> 9216 165 ->
 // 100 us (2.6 POP/s), 1024 x 3072 -> 3072 17.7 -> 16.4, 2048 x 1152 -> 4608 16.9 -> 15.4.
+// Ring slots and parities are carried along (a division by the ring depth per item and role cost more than it looks: 4096 x 4608 -> 1152 29.8 -> 22.5 us,
+// 256 x 1152 -> 1152 8.0 -> 6.6).
 // An output tile is two accumulator passes, the int32 one over K and the fp32 one of the rank-r branch, in two tensor-memory
 // buffers; the epilogue warps take the first into registers while the second runs, so the next tile's MMAs start at once.
 #include "common.h"
@@ -87,12 +89,12 @@ w4a8_pair_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + P::BAR_OFFSET + 448);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + P::BAR_OFFSET + 452);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // (the warp known to be uniform)
     // Trace build (TRACE_CLK), k-blocks 18..20 of the block's first tile: slots 9..11 producer has issued the packed weights, 12..14 a
     // team sees them landed, 15..17 it has an operand slot, 18..20 it has expanded them, 21..23 MMA warp sees them, 24..26 it
     // has issued; slot 30 entry, 31 previous grid ended.
     if (threadIdx.x == 0) TRACE_CLK(p.status, 30);
-    const uint32_t cta_rank = cluster_ctarank();
+    const uint32_t cta_rank = blockIdx.x & 1u;  // (the rank in the cluster)
     const int tile_first = static_cast<int>(blockIdx.x >> 1), tile_step = static_cast<int>(gridDim.x >> 1);
     const int num_m_blocks = (p.M + 2 * BM - 1) / (2 * BM), num_n_blocks = (p.N + BN - 1) / BN;
     const int num_tiles = num_m_blocks * num_n_blocks;
@@ -142,7 +144,7 @@ w4a8_pair_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         if (warp == 0) {
             // -------------------------------------------------------- TMA producer (whole warp in the loops, one lane issues)
             // Its chain of instructions per k-block is on the critical path: slots, parities and addresses are carried along.
-            uint32_t sa = 0, pha = 1, sp = 0, php = 1, it = 0;
+            uint32_t sa = 0, pha = 1, sp = 0, php = 1, sw = 0, phw = 1, it = 0;
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
                 const int m0 = (tile % num_m_blocks) * 2 * BM + static_cast<int>(cta_rank) * BM;
@@ -159,8 +161,7 @@ w4a8_pair_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     } else {
                         // the bf16 weights of the rank-r branch go straight into an operand slot; only when their bytes are expected
                         // are the expanding warps let through, whose arrivals complete the slot's phase
-                        const uint32_t sw = it % NW;
-                        if (!mbar_wait(w_empty(sw), ((it / NW) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
+                        if (!mbar_wait(w_empty(sw), phw, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                         if (elect_one()) {
                             if (cta_rank == 0) mbar_expect_tx(w_full(sw), 2 * W_BYTES);
                             tma_load_2d_pair(smem_base + W_OFFSET + sw * W_BYTES, &tmap_wh, map_to_cta(w_full(sw), 0), (i - p.num_kb) * 64, n0);
@@ -174,6 +175,7 @@ w4a8_pair_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     }
                     if (++sa == NA) { sa = 0; pha ^= 1; }
                     if (++sp == NP) { sp = 0; php ^= 1; }
+                    if (++sw == NW) { sw = 0; phw ^= 1; }
                 }
             }
             if (!ok && lane == 0) {  // give the loads in flight, some of which report to the other CTA, a fixed time
@@ -227,18 +229,19 @@ w4a8_pair_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             constexpr int PIECES = ROWS / 16;
             const int team = (warp - 2) >> 1, u = threadIdx.x & 63, part = u & 3, r0 = u >> 2, swz = r0 & 7;
             uint32_t first_it = 0;  // items before this tile
+            uint32_t sp = team % NP, php = 0, sw = team % NW, phw = 1;  // slots and parities of this team's next item (NP, NW >= TEAMS)
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step, first_it += items) {
                 for (int i = (team + TEAMS - static_cast<int>(first_it % TEAMS)) % TEAMS; i < items; i += TEAMS) {
-                    const uint32_t it = first_it + i, sp = it % NP, sw = it % NW;
-                    if (!mbar_wait(p_full(sp), (it / NP) & 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
+                    const uint32_t it = first_it + i;
+                    if (!mbar_wait(p_full(sp), php, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
                     if (i < p.num_kb) {
                         if (u == 0 && it >= 18 && it <= 20) TRACE_CLK(p.status, it - 6);
                         uint4 pk[PIECES];
                         const uint4* src = reinterpret_cast<const uint4*>(smem_gen + P_OFFSET + sp * P_BYTES) + u;
 #pragma unroll
                         for (int j = 0; j < PIECES; ++j) pk[j] = src[64 * j];
-                        if (!mbar_wait(w_empty(sw), ((it / NW) & 1) ^ 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
+                        if (!mbar_wait(w_empty(sw), phw, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
                         if (u == 0 && it >= 18 && it <= 20) TRACE_CLK(p.status, it - 3);
                         uint8_t* dst = smem_gen + W_OFFSET + sw * W_BYTES + r0 * 128;
 #pragma unroll
@@ -261,6 +264,10 @@ w4a8_pair_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         mbar_arrive(p_empty(sp));
                         mbar_arrive_cluster(map_to_cta(w_full(sw), 0));
                     }
+                    sp += TEAMS;
+                    if (sp >= NP) { sp -= NP; php ^= 1; }
+                    sw += TEAMS;
+                    if (sw >= NW) { sw -= NW; phw ^= 1; }
                 }
             }
         }
