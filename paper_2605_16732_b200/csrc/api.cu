@@ -622,7 +622,9 @@ static dirotq_status_t first_kernel(const dirotq_layer_t* layer, const RotateArg
     return launch_rotate_quantize(layer, ra, s);
 }
 
-static dirotq_status_t second_kernel(const dirotq_layer_t* layer, const RotateArgs& ra, int M, void* y, cudaStream_t s) {
+// `behind_first`: this call has just enqueued the layer's first stage on the same stream.  Its kernels write no weights, and it starts the
+// second kernel only when everything before the call has finished, so that kernel need not wait for its weights.
+static dirotq_status_t second_kernel(const dirotq_layer_t* layer, const RotateArgs& ra, int M, void* y, bool behind_first, cudaStream_t s) {
     if (layer->geo.fmt == 3) {
         A8GemmArgs ga;
         ga.M = M; ga.codes = ra.codes; ga.xscale = ra.xscale; ga.xh = ra.xh;
@@ -637,7 +639,7 @@ static dirotq_status_t second_kernel(const dirotq_layer_t* layer, const RotateAr
     }
     GemmArgs ga;
     ga.M = M; ga.codes = ra.codes; ga.xscale = ra.xscale; ga.ldm = ra.ldm; ga.xh = ra.xh;
-    ga.y = static_cast<uint16_t*>(y); ga.partials = nullptr; ga.status = ra.status;
+    ga.y = static_cast<uint16_t*>(y); ga.partials = nullptr; ga.status = ra.status; ga.early_weights = behind_first;
     return launch_w4a4_gemm(layer, ga, s);
 }
 
@@ -679,7 +681,7 @@ dirotq_status_t dirotq_linear(const void* x, int M, const dirotq_layer_t* layer,
     const RotateArgs ra = rotate_args(layer, x, M, ws, nullptr);
     st = first_kernel(layer, ra, M, static_cast<cudaStream_t>(stream));
     if (st != DIROTQ_OK) return st;
-    return second_kernel(layer, ra, M, y, static_cast<cudaStream_t>(stream));
+    return second_kernel(layer, ra, M, y, true, static_cast<cudaStream_t>(stream));
 }
 
 dirotq_status_t dirotq_w4a4_gemm(int M, const dirotq_layer_t* layer, const void* workspace, size_t workspace_bytes,
@@ -689,7 +691,7 @@ dirotq_status_t dirotq_w4a4_gemm(int M, const dirotq_layer_t* layer, const void*
     if (!y || !aligned16(y)) return DIROTQ_ERR_INVALID_ARG;
     char* ws = const_cast<char*>(static_cast<const char*>(workspace));
     const RotateArgs ra = rotate_args(layer, nullptr, M, ws, nullptr);
-    return second_kernel(layer, ra, M, y, static_cast<cudaStream_t>(stream));
+    return second_kernel(layer, ra, M, y, false, static_cast<cudaStream_t>(stream));
 }
 
 dirotq_status_t dirotq_workspace_status(const void* workspace, dirotq_stream_t stream, int* device_code) {

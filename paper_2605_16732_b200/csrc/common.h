@@ -298,6 +298,7 @@ struct GemmArgs {
     uint16_t* y;        // bf16 [M][N]
     int32_t* partials;  // debug: int32 [n_g][M][N]; when set, y is not written
     int* status;
+    bool early_weights = false;  // the previous kernel of the stream is this call's own first stage: weights may be loaded while it runs
 };
 
 // tensor-map factory (api.cu)

@@ -21,6 +21,7 @@ struct GemmKernelParams {
     uint16_t* y;
     int32_t* partials;
     int* status;
+    int early_weights;  // see GemmArgs
 };
 
 // Compile-time loop: f(Int<0>{}), ..., f(Int<N - 1>{}).

@@ -93,7 +93,7 @@ struct Plan {
     static constexpr int SMEM_BYTES = BAR_OFFSET + 512 + 1024;
     static_assert(SMEM_BYTES <= 232448, "shared memory plan too large");
     static_assert(STAGE_BYTES % 1024 == 0 && SC_BYTES % 128 == 0, "tile alignment");
-    static_assert(8 * (3 * STAGES + 11) <= 400, "barriers end below the words at +400");
+    static_assert(8 * (4 * STAGES + 11) <= 400, "barriers end below the words at +400");
 };
 
 template <int G, bool kPartials, int BN, Rows ROWS>
@@ -130,6 +130,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     auto tfull_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + a); };
     auto tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 4 + a); };
     auto peer_tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 9 + a); };  // pairs: in the leader, the other CTA's
+    auto pre_bar = [&](int s) { return bar_base + 8u * (3 * STAGES + 11 + s); };  // see early_weights below
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + BAR_OFFSET + 400);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + BAR_OFFSET + 404);
 
@@ -154,6 +155,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
             // every thread of the two unpack warps arrives for itself; of a pair's four, one lane each, on the leader's barrier
             mbar_init(unp_bar(s), PAIR ? 4 : 64);
             mbar_init(empty_bar(s), 1);
+            mbar_init(pre_bar(s), 1);
         }
         for (int a = 0; a < NBUF; ++a) {
             mbar_init(tfull_bar(a), 1);
@@ -186,10 +188,27 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
     const uint32_t tmem_base = *tmem_slot;
     // everything above touched only this CTA's own shared and tensor memory; what follows reads the first kernel's output
     if (threadIdx.x == 0) TRACE_CLK(p.status, 10);
-    grid_dependency_wait();
-    if (threadIdx.x == 0) TRACE_CLK(p.status, 11);
-    // the next layer's first kernel may be scheduled as this grid's CTAs leave their SMs (it waits for this whole grid)
-    grid_launch_dependents();
+    // Weights and their scales may be loaded, and expanded, while the previous kernel is still running (GemmArgs::early_weights): those of the
+    // first tile's first stages land on barriers of their own, the stage's barrier then counts the activations only.
+    // (Not in pairs, where one barrier tells the leader of both operands.)
+    const int pre = !PAIR && p.early_weights && first_tile() < num_tiles ? min(STAGES, p.num_kb) : 0;
+    if (warp == 0 && pre > 0 && elect_one()) {
+        const int n0 = (first_tile() / num_m_blocks) * BN;
+        for (int j = 0; j < pre; ++j) {
+            const int groups = min(GPK, p.n_g - j * GPK);
+            mbar_arrive_expect_tx(pre_bar(j), BP_BYTES + groups * SC_SW_BYTES);
+            tma_load_2d(smem_base + j * STAGE_BYTES + AC_BYTES + BU_BYTES, &tmap_wpacked, pre_bar(j), j * (BKC / 2), n0);
+            for (int gi = 0; gi < groups; ++gi)
+                tma_load_2d(sc_base + (j * GPK + gi) * SC_BYTES, &tmap_wscale, pre_bar(j), n0, j * GPK + gi);
+        }
+    }
+    __syncwarp();
+    if (PAIR || (warp != 2 && warp != 3)) {  // (the unpack warps read nothing but what lands on barriers)
+        grid_dependency_wait();
+        if (threadIdx.x == 0) TRACE_CLK(p.status, 11);
+        // the next layer's first kernel may be scheduled as this grid's CTAs leave their SMs (it waits for this whole grid)
+        grid_launch_dependents();
+    }
 
     if (warp < 4) {
         reg_dealloc<P::AUX_REGS>();
@@ -211,18 +230,19 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         if (!timed_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER, w_empty)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         const int groups = min(GPK, p.n_g - kb * GPK);  // (an odd number of groups: the last k-block has one)
+                        const bool weights = at.it >= static_cast<uint32_t>(pre);
                         if (elect_one()) {
-                            mbar_arrive_expect_tx(full_bar(s), AC_BYTES + BP_BYTES + groups * SC_BYTES);
+                            mbar_arrive_expect_tx(full_bar(s), AC_BYTES + (weights ? BP_BYTES : 0) + groups * (weights ? SC_BYTES : SC_BYTES - SC_SW_BYTES));
                             tma_load_2d(st, &tmap_codes, full_bar(s), kb * BKC, m0);
                             if (ROWS == TALL) tma_load_2d(st + A_BYTES, &tmap_codes, full_bar(s), kb * BKC, m0 + BM);
-                            tma_load_2d(st + AC_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), w0);
+                            if (weights) tma_load_2d(st + AC_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), w0);
                         }
 #pragma unroll
                         for (int gi = 0; gi < GPK; ++gi) {
                             if (gi < groups) {
                                 if (elect_one()) {
                                     const uint32_t sc = sc_base + slot * SC_BYTES;
-                                    tma_load_2d(sc, &tmap_wscale, full_bar(s), n0, kb * GPK + gi);
+                                    if (weights) tma_load_2d(sc, &tmap_wscale, full_bar(s), n0, kb * GPK + gi);
                                     tma_load_2d(sc + SC_SW_BYTES, &tmap_xscale, full_bar(s), m0, kb * GPK + gi);
                                     if (at.it == 0) TRACE_CLK(p.status, 12);
                                 }
@@ -288,6 +308,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 };
                 uint32_t s = 0, ph = 0;        // stage of the operand ring and its parity
                 uint32_t b = 0, bph = 1;       // accumulator tile and the parity its "empty" barrier is waited with
+                int pre_left = pre;
                 long long w_ops = 0, w_tempty = 0;
                 const long long t_kernel = clock64();
                 bool ok = true;
@@ -297,6 +318,10 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         // the unpack warps arrive after they have seen the stage's loads land (one barrier for both operands), so
                         // their barrier covers the activation codes as well
                         if (!timed_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_ops)) { ok = false; break; }
+                        if (!PAIR && pre_left > 0) {  // (these were expanded before their activations had been asked for)
+                            --pre_left;
+                            if (!mbar_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
+                        }
                         if (lane == 0) { if (kb == 0) TRACE_CLK(p.status, 16); if (kb == 4) TRACE_CLK(p.status, 17); if (kb == p.num_kb - 1) TRACE_CLK(p.status, 18); }
                         tc_fence_after_sync();
                         const uint32_t a_lo = desc_lo0 + s * (STAGE_BYTES >> 4), b_lo = a_lo + (AC_BYTES >> 4);
@@ -375,7 +400,10 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 const int items = p.num_kb + p.lr_chunks;
                 for (int i = 0; i < items; ++i, at.next()) {
                     const uint32_t s = at.s;
-                    ok = timed_wait(full_bar(s), at.ph, abort_flag, p.status, DEV_TIMEOUT_UNPACK, w_full);
+                    // A barrier is waited on by its phase's parity, and of a stage expanded early this warp has not seen the activations land: they have when
+                    // the stage's MMAs are done.  (Not a wait for the landing itself: the barrier may be two phases on by now.)
+                    if (at.it - STAGES < static_cast<uint32_t>(pre) && !mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
+                    ok = timed_wait(at.it < static_cast<uint32_t>(pre) ? pre_bar(s) : full_bar(s), at.ph, abort_flag, p.status, DEV_TIMEOUT_UNPACK, w_full);
                     if (!ok) break;
                     if (at.it == 0 && u == 0) TRACE_CLK(p.status, 14);
                     if (i < p.num_kb) {
@@ -422,6 +450,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     if (at.it == 0 && u == 0) TRACE_CLK(p.status, 15);
                 }
             }
+            grid_dependency_wait();
             if (u == 0) flush_wait(p.status, WS_UNPACK_FULL, w_full);
         }
     } else {
@@ -677,7 +706,7 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
     p.num_kb = (g.K_lp + BKC - 1) / BKC;
     p.lr_chunks = g.r_pad / 64;
     p.bias = reinterpret_cast<const float*>(L->blob + L->lay.off_bias);
-    p.y = a.y; p.partials = a.partials; p.status = a.status;
+    p.y = a.y; p.partials = a.partials; p.status = a.status; p.early_weights = a.early_weights;
 
     constexpr int CTAS = PAIR ? 2 : 1;
     const int num_tiles = ((a.M + P::TILE_ROWS - 1) / P::TILE_ROWS) * ((g.N + BN - 1) / BN), slots = sm_count(L->device) / CTAS;

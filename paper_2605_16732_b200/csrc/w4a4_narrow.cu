@@ -48,7 +48,7 @@ struct Plan {
     static constexpr int RED_OFFSET = BAR_OFFSET + 512;  // split plan: the other CTAs' partial tiles land here (last CTA)
     static constexpr int SMEM_BYTES = BAR_OFFSET + 512 + 1024 + (SPLITK ? (SPLIT_MAX - 1) * RED_BYTES : 0);
     static_assert(SMEM_BYTES <= 232448 && STAGE_BYTES % 1024 == 0 && SC_BYTES % 128 == 0, "shared memory plan");
-    static_assert(8 * (3 * STAGES + 11) <= 400, "barriers end below the words at +400");
+    static_assert(8 * (4 * STAGES + 11) <= 400, "barriers end below the words at +400");
     // A k-block's scales land with its operands, on the same barrier, in a ring of their own that has no "empty" barriers: the producer
     // loads k-block j when the MMAs of j - STAGES are done, those had waited until the epilogue was through with the buffer four before.
     static_assert(SC_SLOTS >= STAGES + 5, "scale records");
@@ -81,6 +81,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
     auto empty_bar = [&](int s) { return bar_base + 8u * (2 * STAGES + s); };
     auto tfull_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + a); };
     auto tempty_bar = [&](int a) { return bar_base + 8u * (3 * STAGES + 4 + a); };
+    auto pre_bar = [&](int s) { return bar_base + 8u * (3 * STAGES + 11 + s); };  // see early_weights below
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + BAR_OFFSET + 400);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + BAR_OFFSET + 404);
 
@@ -115,6 +116,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
             mbar_init(full_bar(s), 1);
             mbar_init(unp_bar(s), 32);  // every thread of the unpack warp whose turn it is arrives for itself
             mbar_init(empty_bar(s), 1);
+            mbar_init(pre_bar(s), 1);
         }
         for (int a = 0; a < NBUF; ++a) {
             mbar_init(tfull_bar(a), 1);
@@ -146,10 +148,24 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
     const uint32_t tmem_base = *tmem_slot;
     // everything above touched only this CTA's own shared and tensor memory; what follows reads the first kernel's output
     if (threadIdx.x == 0) TRACE_CLK(p.status, 10);
-    grid_dependency_wait();
-    if (threadIdx.x == 0) TRACE_CLK(p.status, 11);
-    // the next layer's first kernel may be scheduled as this grid's CTAs leave their SMs (it waits for this whole grid)
-    grid_launch_dependents();
+    // Weights and their scales may be loaded, and expanded, while the previous kernel is still running (GemmArgs::early_weights): those of the
+    // first tile's first stages land on barriers of their own, the stage's barrier then counts the activations only.
+    const int pre = p.early_weights && first_tile() < num_tiles ? min(STAGES, kb1 - kb0) : 0;
+    if (warp == 0 && pre > 0 && elect_one()) {
+        const int n0 = (first_tile() / num_m_blocks) * BN;
+        for (int j = 0; j < pre; ++j) {
+            mbar_arrive_expect_tx(pre_bar(j), BP_BYTES + GPK * BN * 4);
+            tma_load_2d(smem_base + j * STAGE_BYTES + A_BYTES + BU_BYTES, &tmap_wpacked, pre_bar(j), (kb0 + j) * (BKC / 2), n0);
+            tma_load_2d(sc_base + j * SC_BYTES, &tmap_wscale, pre_bar(j), n0, (kb0 + j) * GPK);
+        }
+    }
+    __syncwarp();
+    if (warp != 2 && warp != 3) {  // (the unpack warps read nothing but what lands on barriers)
+        grid_dependency_wait();
+        if (threadIdx.x == 0) TRACE_CLK(p.status, 11);
+        // the next layer's first kernel may be scheduled as this grid's CTAs leave their SMs (it waits for this whole grid)
+        grid_launch_dependents();
+    }
 
     if (warp < 4) {
         reg_dealloc<AUX_REGS>();
@@ -172,10 +188,13 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         if (elect_one()) {
                             const uint32_t sc = sc_base + slot * SC_BYTES;
-                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + BP_BYTES + GPK * (BN + BM) * 4);
+                            const bool weights = at.it >= static_cast<uint32_t>(pre);
+                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + GPK * BM * 4 + (weights ? BP_BYTES + GPK * BN * 4 : 0));
                             tma_load_2d(st, &tmap_codes, full_bar(s), kb * BKC, m0);
-                            tma_load_2d(st + A_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), n0);
-                            tma_load_2d(sc, &tmap_wscale, full_bar(s), n0, kb * GPK);
+                            if (weights) {
+                                tma_load_2d(st + A_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), n0);
+                                tma_load_2d(sc, &tmap_wscale, full_bar(s), n0, kb * GPK);
+                            }
                             tma_load_2d(sc + SC_SW_BYTES, &tmap_xscale, full_bar(s), m0, kb * GPK);
                             if (at.it == 0) TRACE_CLK(p.status, 12);
                         }
@@ -220,6 +239,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                 auto desc = [&](uint32_t lo) { return (static_cast<uint64_t>(desc_hi) << 32) | lo; };
                 uint32_t s = 0, ph = 0;        // stage of the operand ring and its parity
                 uint32_t b = 0, bph = 1;       // accumulator tile and the parity its "empty" barrier is waited with
+                int pre_left = pre;
                 long long w_ops = 0, w_tempty = 0;
                 const long long t_kernel = clock64();
                 bool ok = true;
@@ -228,6 +248,10 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                         // the unpack warps arrive after they have seen the stage's loads land (one barrier for both operands), so
                         // their barrier covers the activation codes as well
                         if (!timed_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_ops)) { ok = false; break; }
+                        if (pre_left > 0) {  // (these were expanded before their activations had been asked for)
+                            --pre_left;
+                            if (!mbar_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
+                        }
                         if (lane == 0) { if (kb == kb0) TRACE_CLK(p.status, 16); if (kb == 4) TRACE_CLK(p.status, 17); if (kb == kb1 - 1) TRACE_CLK(p.status, 18); }
                         if (!timed_wait(tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_tempty)) { ok = false; break; }
                         tc_fence_after_sync();
@@ -287,7 +311,11 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
             for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
                 const int items = (kb1 - kb0) + lr_here;
                 for (int i = static_cast<int>((warp - 2 + first_it) & 1); i < items; i += 2) {
-                    ok = timed_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_UNPACK, w_full);
+                    // A barrier is waited on by its phase's parity, and of a stage expanded early this warp has not seen the activations land: they have when
+                    // the stage's MMAs are done.  (Not a wait for the landing itself: the barrier may be two phases on by now.)
+                    const uint32_t it = first_it + i;
+                    if (it - STAGES < static_cast<uint32_t>(pre) && !mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
+                    ok = timed_wait(it < static_cast<uint32_t>(pre) ? pre_bar(s) : full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_UNPACK, w_full);
                     if (!ok) break;
                     if (first_it == 0 && i == 0 && u == 0) TRACE_CLK(p.status, 14);
                     if (i < kb1 - kb0) {
@@ -332,6 +360,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                 }
                 first_it += items;
             }
+            grid_dependency_wait();
             if (warp == 2 && u == 0) flush_wait(p.status, WS_UNPACK_FULL, w_full);
         }
     } else {
@@ -615,7 +644,7 @@ dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, boo
     p.num_kb = (g.K_lp + BKC - 1) / BKC;
     p.lr_chunks = g.r_pad / 64;
     p.bias = reinterpret_cast<const float*>(L->blob + L->lay.off_bias);
-    p.y = a.y; p.partials = a.partials; p.status = a.status;
+    p.y = a.y; p.partials = a.partials; p.status = a.status; p.early_weights = a.early_weights;
 
     const int num_tiles = ((a.M + BM - 1) / BM) * ((g.N + BN - 1) / BN), sms = sm_count(L->device), which = g.G == 64 ? 0 : 1;
     using KernelFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
