@@ -80,6 +80,7 @@ struct NvKernelParams {
     const float* out_scale;  // 2^(ex+ew)
     uint16_t* y;
     int* status;
+    int x_rows;  // rows of the activation tiles' boxes (box_rows)
 };
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
@@ -243,7 +244,7 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
                     if (!mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                     const uint32_t st = smem_base + s * STAGE_BYTES;
                     if (!elect_one()) continue;
-                    mbar_arrive_expect_tx(full_bar(s), A_BYTES + B_BYTES + (sfa_here + nb_here) * SF_BYTES);
+                    mbar_arrive_expect_tx(full_bar(s), p.x_rows * 128 + B_BYTES + (sfa_here + nb_here) * SF_BYTES);
                     tma_load_2d(st, &tmap_codes, full_bar(s), kb * 128, m0);             // byte coordinates
 #pragma unroll
                     for (int b = 0; b < NB_DATA; ++b)  // rows past N are filled with zeros (and still counted)
@@ -263,7 +264,7 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_c
                     if (!mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                     const uint32_t st = smem_base + s * STAGE_BYTES;
                     if (!elect_one()) continue;
-                    mbar_arrive_expect_tx(full_bar(s), A_BYTES + B_BYTES);
+                    mbar_arrive_expect_tx(full_bar(s), p.x_rows * 128 + B_BYTES);
                     tma_load_2d(st, &tmap_xh, full_bar(s), lr * 64, m0);
 #pragma unroll
                     for (int b = 0; b < NB_DATA; ++b)
@@ -536,10 +537,10 @@ static dirotq_status_t launch_nvfp4_gemm_bn(const dirotq_layer* L, const Nvfp4Ge
     CUtensorMap tmap_codes, tmap_xh;
     dirotq_status_t st;
     st = encode_tmap_2d(&tmap_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.codes, (uint64_t)g.K4 / 2, (uint64_t)a.M,
-                        (uint64_t)g.K4 / 2, 128, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+                        (uint64_t)g.K4 / 2, 128, PAIR ? BM : box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
     st = encode_tmap_2d(&tmap_xh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.xh, (uint64_t)g.r_pad, (uint64_t)a.M,
-                        (uint64_t)g.r_pad * 2, 64, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+                        (uint64_t)g.r_pad * 2, 64, PAIR ? BM : box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
     NvKernelParams p;
     p.M = a.M; p.N = g.N;
@@ -551,6 +552,7 @@ static dirotq_status_t launch_nvfp4_gemm_bn(const dirotq_layer* L, const Nvfp4Ge
     p.bias = reinterpret_cast<const float*>(L->blob + L->lay.off_bias);
     p.out_scale = reinterpret_cast<const float*>(L->blob + L->lay.off_meta);
     p.y = a.y; p.status = a.status;
+    p.x_rows = PAIR ? BM : box_rows(a.M);
     const int sms = sm_count(L->device);
     static SmemOptIn<1> opt_in;  // one per instantiation of this launcher
     if (!opt_in.ensure(nvfp4_gemm_kernel<BN, PAIR>, 0, L->device, Plan<BN, PAIR>::SMEM_BYTES)) return DIROTQ_ERR_CUDA;

@@ -51,6 +51,7 @@ static_assert(SMEM_BYTES <= 232448, "shared memory plan");
 
 struct RotKernelParams {
     int M, K, K_l, K_lp, r, r_pad, r_pad0, ldm, n_g;
+    int x_rows = 128;      // rows of the activation tile's box (box_rows)
     int n_out, k_red;      // output columns and reduction length of the GEMM (both K for the rotation x Q)
     int8_t* codes;
     float* xscale;
@@ -327,12 +328,12 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         const uint32_t sa = smem_base + s * STAGE_BYTES;
                         if (!elect_one()) continue;
                         if (i < nv) {
-                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + BN * BK * 2);
+                            mbar_arrive_expect_tx(full_bar(s), (p.x_rows + BN) * BK * 2);
                             tma_load_2d(sa, &tmap_x, full_bar(s), i * BK, m0);
                             tma_load_2d(sa + A_BYTES, &tmap_qt, full_bar(s), i * BK, n0);
                         } else {
                             const int j = i - nv;
-                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + G * BK * 2);
+                            mbar_arrive_expect_tx(full_bar(s), (p.x_rows + G) * BK * 2);
                             tma_load_2d(sa, &tmap_x2, full_bar(s), n0 + j * BK, m0);
                             tma_load_2d(sa + A_BYTES, &tmap_had, full_bar(s), (j % (G / BK)) * BK, 0);
                         }
@@ -348,7 +349,7 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     if (!elect_one()) continue;
                     if constexpr (KSUB > 1) {
                         const int nsub = min(KSUB, num_kb - kb);  // k-blocks in this stage
-                        mbar_arrive_expect_tx(full_bar(s), nsub * SUB_BYTES);
+                        mbar_arrive_expect_tx(full_bar(s), nsub * (p.x_rows + BN) * BK * 2);
                         for (int j = 0; j < nsub; ++j) {
                             tma_load_2d(sa + j * SUB_BYTES, &tmap_x, full_bar(s), (kb + j) * BK, m0);
                             tma_load_2d(sa + j * SUB_BYTES + A_BYTES, &tmap_qt, full_bar(s), (kb + j) * BK, n0);
@@ -363,7 +364,7 @@ rotate_quant_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         tma_load_2d_pair(sa, &tmap_x, full_leader, kb * BK, m0);
                         tma_load_2d_pair(sa + A_BYTES, &tmap_qt, full_leader, kb * BK, n0 + static_cast<int>(cta_rank) * B_ROWS);
                     } else {
-                        mbar_arrive_expect_tx(full_bar(s), A_BYTES + BN * BK * 2);
+                        mbar_arrive_expect_tx(full_bar(s), (BM == 256 ? A_BYTES : p.x_rows * BK * 2) + BN * BK * 2);
                         tma_load_2d(sa, &tmap_x, full_bar(s), kb * BK, m0);
                         tma_load_2d(sa + A_BYTES, &tmap_qt, full_bar(s), kb * BK, n0);
                     }
@@ -862,7 +863,7 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
     const Geometry& g = L->geo;
     RotKernelParams p;
     p.n_out = g.K; p.k_red = g.K;
-    p.M = a.M; p.K = g.K; p.K_l = g.K_l; p.K_lp = g.K_lp; p.r = g.r; p.r_pad = g.r_pad; p.r_pad0 = g.r_pad0; p.ldm = a.ldm; p.n_g = g.n_g;
+    p.M = a.M; p.x_rows = box_rows(a.M); p.K = g.K; p.K_l = g.K_l; p.K_lp = g.K_lp; p.r = g.r; p.r_pad = g.r_pad; p.r_pad0 = g.r_pad0; p.ldm = a.ldm; p.n_g = g.n_g;
     p.codes = a.codes; p.xscale = a.xscale; p.xh = a.xh; p.xrot = a.xrot; p.status = a.status;
     p.xsf = a.xsf; p.K4 = g.K4; p.nkb64p = g.nkb64p; p.ex = L->act_scale_log2;
     p.xtilde = a.xtilde;
@@ -939,7 +940,7 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
     if (plan == 5) {
         CUtensorMap tmap_x5;
         dirotq_status_t st5 = encode_tmap_2d(&tmap_x5, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)g.K, (uint64_t)a.M,
-                                             (uint64_t)g.K * 2, BK, 128, CU_TENSOR_MAP_SWIZZLE_128B);
+                                             (uint64_t)g.K * 2, BK, box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_128B);
         if (st5 != DIROTQ_OK) return st5;
         const long tiles5 = mb128 * ((g.K + 63) / 64);
         const int vi5 = g.fmt == 1 ? 1 : g.fmt == 2 ? 2 : g.fmt == 3 ? 3 : 0;
@@ -959,7 +960,7 @@ dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& 
     const int bm = plan == 3 ? 256 : 128, bn = plan == 1 ? 128 : 256;
     CUtensorMap tmap_x;
     dirotq_status_t st = encode_tmap_2d(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)g.K, (uint64_t)a.M,
-                                        (uint64_t)g.K * 2, BK, bm, CU_TENSOR_MAP_SWIZZLE_128B);
+                                        (uint64_t)g.K * 2, BK, bm == 128 ? box_rows(a.M) : bm, CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
     const long num_tiles = ((a.M + bm - 1) / bm) * ((g.K + bn - 1) / bn);
     const int grid = num_tiles < sms ? static_cast<int>(num_tiles) : sms;
@@ -994,11 +995,12 @@ dirotq_status_t launch_project_quantize(const dirotq_layer* L, const RotateArgs&
     RotKernelParams p;
     p.M = a.M; p.K = g.K; p.K_lp = g.K_lp; p.r_pad = g.r_pad; p.r_pad0 = g.r_pad0; p.ldm = a.ldm; p.n_g = g.n_g;
     p.codes = a.codes; p.xscale = a.xscale; p.xh = a.xh; p.xrot = nullptr; p.status = a.status;
+    p.x_rows = box_rows(a.M);
     p.xsf = nullptr; p.K4 = 0; p.nkb64p = 0; p.ex = 0; p.xtilde = nullptr;
     dirotq_status_t st;
     CUtensorMap tmap_x;
     st = encode_tmap_2d(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)g.K, (uint64_t)a.M, (uint64_t)g.K * 2, BK,
-                        128, CU_TENSOR_MAP_SWIZZLE_128B);
+                        box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
     {
         // step 1: all r_pad output columns are "high" (K_l = 0): the epilogue only rounds them to bf16 into xh
@@ -1035,7 +1037,7 @@ dirotq_status_t launch_project_quantize(const dirotq_layer* L, const RotateArgs&
         // kernel's PH note); every output column is low-precision (K_l = K)
         CUtensorMap tmap_xh;
         st = encode_tmap_2d(&tmap_xh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.xh, (uint64_t)g.r_pad, (uint64_t)a.M,
-                            (uint64_t)g.r_pad * 2, BK, 128, CU_TENSOR_MAP_SWIZZLE_128B);
+                            (uint64_t)g.r_pad * 2, BK, box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_128B);
         if (st != DIROTQ_OK) return st;
         RotKernelParams p2 = p;
         p2.n_out = g.K; p2.k_red = g.r_pad; p2.K_l = g.K; p2.r = g.r;

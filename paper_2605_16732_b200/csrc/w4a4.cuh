@@ -22,6 +22,7 @@ struct GemmKernelParams {
     int32_t* partials;
     int* status;
     int early_weights;  // see GemmArgs
+    int x_rows;         // rows of the activation tiles' boxes (box_rows)
 };
 
 // Compile-time loop: f(Int<0>{}), ..., f(Int<N - 1>{}).

@@ -232,7 +232,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         const int groups = min(GPK, p.n_g - kb * GPK);  // (an odd number of groups: the last k-block has one)
                         const bool weights = at.it >= static_cast<uint32_t>(pre);
                         if (elect_one()) {
-                            mbar_arrive_expect_tx(full_bar(s), AC_BYTES + (weights ? BP_BYTES : 0) + groups * (weights ? SC_BYTES : SC_BYTES - SC_SW_BYTES));
+                            mbar_arrive_expect_tx(full_bar(s), (ROWS == ONE ? p.x_rows * BKC : AC_BYTES) + (weights ? BP_BYTES : 0) + groups * (weights ? SC_BYTES : SC_BYTES - SC_SW_BYTES));
                             tma_load_2d(st, &tmap_codes, full_bar(s), kb * BKC, m0);
                             if (ROWS == TALL) tma_load_2d(st + A_BYTES, &tmap_codes, full_bar(s), kb * BKC, m0 + BM);
                             if (weights) tma_load_2d(st + AC_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), w0);
@@ -256,7 +256,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         if (!mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         if (elect_one()) {
-                            mbar_arrive_expect_tx(full_bar(s), AC_BYTES + BU_BYTES);
+                            mbar_arrive_expect_tx(full_bar(s), (ROWS == ONE ? p.x_rows * BKC : AC_BYTES) + BU_BYTES);
                             tma_load_2d(st, &tmap_xh, full_bar(s), lr * 64, m0);
                             if (ROWS == TALL) tma_load_2d(st + A_BYTES, &tmap_xh, full_bar(s), lr * 64, m0 + BM);
                             tma_load_2d(st + AC_BYTES, &tmap_wh, full_bar(s), lr * 64, w0);
@@ -692,13 +692,13 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
     CUtensorMap tmap_codes, tmap_xscale, tmap_xh;
     dirotq_status_t st;
     st = encode_tmap_2d(&tmap_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.codes, (uint64_t)g.K_lp, (uint64_t)a.M,
-                        (uint64_t)g.K_lp, BKC, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+                        (uint64_t)g.K_lp, BKC, ROWS == ONE ? box_rows(a.M) : BM, CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
     st = encode_tmap_2d(&tmap_xscale, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.xscale, (uint64_t)a.ldm, (uint64_t)g.n_g,
                         (uint64_t)a.ldm * 4, P::CTA_ROWS, 1, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st != DIROTQ_OK) return st;
     st = encode_tmap_2d(&tmap_xh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.xh, (uint64_t)g.r_pad, (uint64_t)a.M,
-                        (uint64_t)g.r_pad * 2, 64, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+                        (uint64_t)g.r_pad * 2, 64, ROWS == ONE ? box_rows(a.M) : BM, CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
 
     GemmKernelParams p;
@@ -706,7 +706,7 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
     p.num_kb = (g.K_lp + BKC - 1) / BKC;
     p.lr_chunks = g.r_pad / 64;
     p.bias = reinterpret_cast<const float*>(L->blob + L->lay.off_bias);
-    p.y = a.y; p.partials = a.partials; p.status = a.status; p.early_weights = a.early_weights;
+    p.y = a.y; p.partials = a.partials; p.status = a.status; p.early_weights = a.early_weights; p.x_rows = ROWS == ONE ? box_rows(a.M) : BM;
 
     constexpr int CTAS = PAIR ? 2 : 1;
     const int num_tiles = ((a.M + P::TILE_ROWS - 1) / P::TILE_ROWS) * ((g.N + BN - 1) / BN), slots = sm_count(L->device) / CTAS;

@@ -189,7 +189,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                         if (elect_one()) {
                             const uint32_t sc = sc_base + slot * SC_BYTES;
                             const bool weights = at.it >= static_cast<uint32_t>(pre);
-                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + GPK * BM * 4 + (weights ? BP_BYTES + GPK * BN * 4 : 0));
+                            mbar_arrive_expect_tx(full_bar(s), p.x_rows * BKC + GPK * BM * 4 + (weights ? BP_BYTES + GPK * BN * 4 : 0));
                             tma_load_2d(st, &tmap_codes, full_bar(s), kb * BKC, m0);
                             if (weights) {
                                 tma_load_2d(st + A_BYTES + BU_BYTES, &tmap_wpacked, full_bar(s), kb * (BKC / 2), n0);
@@ -206,7 +206,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                         if (!mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
                         const uint32_t st = smem_base + s * STAGE_BYTES;
                         if (elect_one()) {
-                            mbar_arrive_expect_tx(full_bar(s), A_BYTES + BU_BYTES);
+                            mbar_arrive_expect_tx(full_bar(s), p.x_rows * BKC + BU_BYTES);
                             tma_load_2d(st, &tmap_xh, full_bar(s), lr * 64, m0);
                             tma_load_2d(st + A_BYTES, &tmap_wh, full_bar(s), lr * 64, n0);
                         }
@@ -630,13 +630,13 @@ dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, boo
     CUtensorMap tmap_codes, tmap_xscale, tmap_xh;
     dirotq_status_t st;
     st = encode_tmap_2d(&tmap_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.codes, (uint64_t)g.K_lp, (uint64_t)a.M,
-                        (uint64_t)g.K_lp, BKC, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+                        (uint64_t)g.K_lp, BKC, box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
     st = encode_tmap_2d(&tmap_xscale, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.xscale, (uint64_t)a.ldm, (uint64_t)g.n_g,
                         (uint64_t)a.ldm * 4, BM, BKC / g.G, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (st != DIROTQ_OK) return st;
     st = encode_tmap_2d(&tmap_xh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.xh, (uint64_t)g.r_pad, (uint64_t)a.M,
-                        (uint64_t)g.r_pad * 2, 64, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+                        (uint64_t)g.r_pad * 2, 64, box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
 
     GemmKernelParams p;
@@ -644,7 +644,7 @@ dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, boo
     p.num_kb = (g.K_lp + BKC - 1) / BKC;
     p.lr_chunks = g.r_pad / 64;
     p.bias = reinterpret_cast<const float*>(L->blob + L->lay.off_bias);
-    p.y = a.y; p.partials = a.partials; p.status = a.status; p.early_weights = a.early_weights;
+    p.y = a.y; p.partials = a.partials; p.status = a.status; p.early_weights = a.early_weights; p.x_rows = box_rows(a.M);
 
     const int num_tiles = ((a.M + BM - 1) / BM) * ((g.N + BN - 1) / BN), sms = sm_count(L->device), which = g.G == 64 ? 0 : 1;
     using KernelFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,

@@ -56,6 +56,7 @@ struct A8KernelParams {
     uint16_t* y;
     int32_t* partials;
     int* status;
+    int x_rows;  // rows of the activation tiles' boxes (box_rows)
 };
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
@@ -148,12 +149,12 @@ w4a8_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                     const uint32_t st = smem_base + s * STAGE_BYTES;
                     if (!elect_one()) continue;
                     if (i < p.num_kb) {
-                        mbar_arrive_expect_tx(full_bar(s), A_BYTES + BP_BYTES);
+                        mbar_arrive_expect_tx(full_bar(s), p.x_rows * BKC + BP_BYTES);
                         tma_load_2d(st, &tmap_codes, full_bar(s), i * BKC, m0);
                         tma_load_2d(st + BP_OFFSET, &tmap_wpacked, full_bar(s), i * (BKC / 2), n0);
                         if (at.it >= 10 && at.it <= 12) TRACE_CLK(p.status, at.it - 1);
                     } else {
-                        mbar_arrive_expect_tx(full_bar(s), A_BYTES + BU_BYTES);
+                        mbar_arrive_expect_tx(full_bar(s), p.x_rows * BKC + BU_BYTES);
                         tma_load_2d(st, &tmap_xh, full_bar(s), (i - p.num_kb) * 64, m0);
                         tma_load_2d(st + A_BYTES, &tmap_wh, full_bar(s), (i - p.num_kb) * 64, n0);
                     }
@@ -402,10 +403,10 @@ static dirotq_status_t launch_single(const dirotq_layer* L, const A8GemmArgs& a,
     CUtensorMap tmap_codes, tmap_xh;
     dirotq_status_t st;
     st = encode_tmap_2d(&tmap_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.codes, (uint64_t)g.K_lp, (uint64_t)a.M,
-                        (uint64_t)g.K_lp, BKC, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+                        (uint64_t)g.K_lp, BKC, box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
     st = encode_tmap_2d(&tmap_xh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.xh, (uint64_t)g.r_pad, (uint64_t)a.M,
-                        (uint64_t)g.r_pad * 2, 64, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+                        (uint64_t)g.r_pad * 2, 64, box_rows(a.M), CU_TENSOR_MAP_SWIZZLE_128B);
     if (st != DIROTQ_OK) return st;
     A8KernelParams p;
     p.M = a.M; p.N = g.N;
@@ -415,6 +416,7 @@ static dirotq_status_t launch_single(const dirotq_layer* L, const A8GemmArgs& a,
     p.wscale = reinterpret_cast<const float*>(L->blob + L->lay.off_wscale);
     p.bias = reinterpret_cast<const float*>(L->blob + L->lay.off_bias);
     p.y = a.y; p.partials = a.partials; p.status = a.status;
+    p.x_rows = box_rows(a.M);
     const int num_tiles = ((a.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
     const int grid = num_tiles < sm_count(L->device) ? num_tiles : sm_count(L->device);
     const bool dbg = a.partials != nullptr;
