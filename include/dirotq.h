@@ -177,7 +177,8 @@ DIROTQ_API dirotq_status_t dirotq_int_gemm_debug(const int8_t* act_codes, int M,
 /* Tuning knob of the second kernels (all four formats): output columns per tile.
  * 0 (default): chosen per call from M, N and the number of SMs, the shortest schedule of the plans below, 66 apart (NVFP4: 256
  * columns unless 128-column tiles, at 0.6 of a wide one, shorten the schedule);
- * 128 or 256: forced; 64: the grouped INT4 kernel's plan for few token rows, forced, one CTA per tile; 66: the same
+ * 128 or 256: forced; 64: the grouped INT4 kernel's plan for few token rows, forced, one CTA per tile (32: the same with half the
+ * columns, groups of 64 only, else 64 is taken); 66: the same
  * tiles with the K-groups of a tile cut over a cluster of up to four CTAs (partial tiles added in one of them through
  * distributed shared memory) wherever every tile's cluster is resident at once and every CTA keeps two k-blocks; never
  * chosen automatically, because its outputs differ from the other plans' in fp32 summation order (a bf16 step on a few

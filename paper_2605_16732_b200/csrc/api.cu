@@ -176,6 +176,7 @@ static dirotq_status_t encode_tmaps_rows(dirotq_layer* L, int N, int group, int 
 
 static dirotq_status_t encode_tmaps_192(dirotq_layer* L, int N, int group) {
     dirotq_status_t st64 = encode_tmaps_rows(L, N, group, 64, &L->tmap_wpacked64, &L->tmap_wscale64, &L->tmap_wh64);
+    if (st64 == DIROTQ_OK) st64 = encode_tmaps_rows(L, N, group, 32, &L->tmap_wpacked32, &L->tmap_wscale32, &L->tmap_wh32);
     if (st64 != DIROTQ_OK) return st64;
     const Geometry& g = L->geo;
     const BlobLayout& lay = L->lay;
@@ -656,8 +657,8 @@ dirotq_status_t dirotq_set_dependent_launch(int enabled) {
 }
 
 dirotq_status_t dirotq_set_gemm_tile(int columns) {
-    // 64, 66, 130 and 192: plans of the grouped INT4 second kernel only
-    const bool int4_only = columns == 64 || columns == 66 || columns == 130 || columns == 192;  // 66: 64 columns with the reduction split over a cluster
+    // 32, 64, 66, 130 and 192: plans of the grouped INT4 second kernel only
+    const bool int4_only = columns == 32 || columns == 64 || columns == 66 || columns == 130 || columns == 192;  // 66: 64 columns with the reduction split over a cluster
     dirotq_status_t st = set_w4a4_tile_columns(columns);
     if (st == DIROTQ_OK) st = set_nvfp4_tile_columns(int4_only ? 0 : columns);
     return st != DIROTQ_OK ? st : set_w4a8_tile_columns(int4_only ? 0 : columns);

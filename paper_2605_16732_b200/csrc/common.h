@@ -254,6 +254,7 @@ struct dirotq_layer {
     CUtensorMap tmap_wpacked128, tmap_wscale128, tmap_wh128;  // the same three with 128-row boxes (narrow W4A4 tiles)
     CUtensorMap tmap_wpacked192, tmap_wscale192, tmap_wh192;  // ... and with 192-row boxes (grouped INT4 formats)
     CUtensorMap tmap_wpacked64, tmap_wscale64, tmap_wh64;     // ... and with 64-row boxes (calls with few token rows)
+    CUtensorMap tmap_wpacked32, tmap_wscale32, tmap_wh32;     // ... and with 32-row boxes (the same, groups of 64)
     CUtensorMap tmap_qt64;     // the rotation with box 64 x 64 (calls with few token rows, groups of 64)
     int act_scale_log2;        // NVFP4 variant: exponent of the activations' per-tensor power-of-two scale
 };
@@ -318,7 +319,7 @@ dirotq_status_t check_call(const dirotq_layer_t* layer, int M, const void* works
 
 // launchers (each returns after enqueueing on `stream`)
 dirotq_status_t launch_rotate_quantize(const dirotq_layer* L, const RotateArgs& a, cudaStream_t stream);
-dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, bool may_split, cudaStream_t stream);  // (not for partials)
+dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, int columns, bool may_split, cudaStream_t stream);  // (not for partials)
 dirotq_status_t launch_w4a4_gemm(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream);
 dirotq_status_t set_w4a4_tile_columns(int columns);
 // Launches `kern`; with `dependent` (and unless switched off process-wide) as a programmatic dependent launch: the

@@ -29,7 +29,7 @@
 // bf16 rank-r branch is issued as one more "group" (kind::f16 into the same ping-pong tile) and added
 // unscaled.
 //
-// Tiles of 256, 192 or 128 columns here; w4a4_narrow.cu has the same computation in 64-column tiles.
+// Tiles of 256, 192 or 128 columns here; w4a4_narrow.cu has the same computation in 64- and 32-column tiles.
 //
 // What bounds it: the issue slots of the schedulers.  The rescale's packed multiply and multiply-add hold a scheduler's issue port for two
 // cycles each and nothing issues beside them: of the 1125 cycles a K-group of a 128 x 256 tile took, 660 were these, and everything else that
@@ -739,7 +739,7 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
 static std::atomic<int> g_tile_columns{0};  // 0: chosen per call; 64 / 128 / 192 / 256: forced; 66: 64 columns, split plan where it applies
 
 dirotq_status_t set_w4a4_tile_columns(int columns) {
-    if (columns != 0 && columns != 64 && columns != 66 && columns != 128 && columns != 192 && columns != 256 && columns != 512 && columns != 130) return DIROTQ_ERR_INVALID_ARG;
+    if (columns != 0 && columns != 32 && columns != 64 && columns != 66 && columns != 128 && columns != 192 && columns != 256 && columns != 512 && columns != 130) return DIROTQ_ERR_INVALID_ARG;
     g_tile_columns.store(columns);
     return DIROTQ_OK;
 }
@@ -752,12 +752,13 @@ dirotq_status_t launch_w4a4_gemm(const dirotq_layer* L, const GemmArgs& a, cudaS
     const int forced = g_tile_columns.load(), sms = sm_count(L->device);
     const bool g64 = L->geo.G == 64;
     struct Candidate { int knob, rows, columns, ctas; double cost64, cost128; };
-    static constexpr Candidate kPlans[] = {{64, 128, 64, 1, 0.295, 0.38}, {128, 128, 128, 1, 0.615, 0.73}, {192, 128, 192, 1, 0.846, 0.957},
+    static constexpr Candidate kPlans[] = {{32, 128, 32, 1, 0.25, 0.0}, {64, 128, 64, 1, 0.295, 0.38}, {128, 128, 128, 1, 0.615, 0.73}, {192, 128, 192, 1, 0.846, 0.957},
                                            {130, 256, 128, 1, 1.02, 1.03}, {256, 128, 256, 1, 1.068, 1.21}, {512, 256, 256, 2, 1.0, 1.0}};
     int plan = forced;
     double best = 0.0;
     for (const Candidate& c : kPlans) {
         if (forced) break;
+        if (c.knob == 32 && (!g64 || ((a.M + 127) / 128) * ((L->geo.N + 31) / 32) > sms / 2)) continue;  // (see w4a4_narrow.cu)
         const long tiles = static_cast<long>((a.M + c.rows - 1) / c.rows) * ((L->geo.N + c.columns - 1) / c.columns), slots = sms / c.ctas;
         const double t = static_cast<double>((tiles + slots - 1) / slots) * (g64 ? c.cost64 : c.cost128) + (c.ctas == 2 ? 100.0 / L->geo.K_lp : 0.0);
         if (plan == 0 || t < best) {
@@ -765,7 +766,7 @@ dirotq_status_t launch_w4a4_gemm(const dirotq_layer* L, const GemmArgs& a, cudaS
             best = t;
         }
     }
-    if (a.partials == nullptr && (plan == 64 || plan == 66)) return launch_w4a4_narrow(L, a, plan == 66, stream);
+    if (a.partials == nullptr && plan <= 66) return launch_w4a4_narrow(L, a, plan == 32 && g64 ? 32 : 64, plan == 66, stream);
     if (plan == 512 && a.partials == nullptr) return launch_w4a4_gemm_bn<256, PAIRED>(L, a, stream);
     if (plan == 130 && a.partials == nullptr) return launch_w4a4_gemm_bn<128, TALL>(L, a, stream);
     if (plan == 192) return launch_w4a4_gemm_bn<192>(L, a, stream);

@@ -1,5 +1,5 @@
 // Second kernel of the grouped INT4 formats for calls with few token rows: w4a4_gemm.cu's computation (same formats, same exact group
-// sums, same order of additions, same bits) in tiles of 128 rows x 64 columns.
+// sums, same order of additions, same bits) in tiles of 128 rows x 64 columns, or 32 with groups of 64.
 //
 // With few tiles a tile's k-blocks are a chain of hand-overs between the tensor core and the epilogue, so the call takes as
 // long as the chain: more, narrower tiles on more SMs, and a short chain.  A tensor-memory buffer holds the accumulator tiles
@@ -10,6 +10,9 @@
 // the next buffer's first unit requested at one of two places, and addresses that were not known to be uniform, and 1060 with one hand-over
 // per group: us alone, 256 x 1152 -> 1152 7.0 -> 6.0, 16 x 12288 -> 3072 41.0 -> 29.8, 64 x 3072 -> 9216 13.3 -> 10.4.  Tried: a whole buffer
 // per tensor-memory wait 0 to 6 % slower, three expanding warps in a block of 16 warps 4 to 13 %.
+// 32-column tiles halve the expansion and the epilogue of a k-block and leave the MMA warp's chain: second kernel 256 x 1152 -> 1152 6.2 -> 5.7 us, 16 x 3072 ->
+// 3072 9.4 -> 8.4, 16 x 12288 -> 3072 28.5 -> 24.5.  Only where they keep at most half of the SMs busy: 512 x 1152 -> 1152, 144 tiles, gains 0.4 us alone and loses
+// as much behind the rotation, whose 72 CTAs leave it no room to start early.
 //
 // Roles (384 threads = 3 warpgroups):
 //   warpgroup 0: warp 0 TMA producer, warp 1 MMA issuer + TMEM owner, warps 2-3 nibble -> byte unpack (k-blocks in turn)
@@ -26,20 +29,19 @@
 namespace dirotq {
 namespace {
 
-constexpr int BN = 64;
 constexpr int SPLIT_MAX = 4;          // CTAs per cluster of the split plan
 constexpr int NUM_EPI_WARPS = 8, NUM_THREADS = 384;
 constexpr int EPI_REGS = 224, AUX_REGS = 56;  // setmaxnreg budgets: 256 x EPI + 128 x AUX <= 384 x 168
 constexpr int RED_BYTES = 128 * 64 * 4;  // one CTA's partial tile: 128 rows x 64 columns fp32
 constexpr int SC_SLOTS = 11;          // scale records, one per k-block
-constexpr int BU_BYTES = BN * BKC;         // unpacked weight codes / bf16 W~_h chunk
-constexpr int BP_BYTES = BN * BKC / 2;     // packed weight codes (TMA staging)
-constexpr int STAGE_BYTES = A_BYTES + BU_BYTES + BP_BYTES;  // 28 KB
-constexpr int SC_SW_BYTES = 2 * BN * 4;    // up to two groups per k-block
-constexpr int SC_SX_BYTES = 2 * BM * 4;    // activation scales of up to two groups
-constexpr int SC_BYTES = SC_SW_BYTES + SC_SX_BYTES;
-template <bool SPLITK>
+template <bool SPLITK, int BN>
 struct Plan {
+    static constexpr int BU_BYTES = BN * BKC;         // unpacked weight codes / bf16 W~_h chunk
+    static constexpr int BP_BYTES = BN * BKC / 2;     // packed weight codes (TMA staging)
+    static constexpr int STAGE_BYTES = A_BYTES + BU_BYTES + BP_BYTES;  // 28 KB, or 22
+    static constexpr int SC_SW_BYTES = 2 * BN * 4;    // up to two groups per k-block
+    static constexpr int SC_SX_BYTES = 2 * BM * 4;    // activation scales of up to two groups
+    static constexpr int SC_BYTES = SC_SW_BYTES + SC_SX_BYTES;
     static constexpr int STAGES = SPLITK ? 4 : 6;
     // (Even: then an unpack warp, which takes every second k-block, has itself seen the previous one of a stage land, and cannot take that
     // one's missing phase for its own: a barrier is waited on by parity.)
@@ -54,14 +56,16 @@ struct Plan {
     static_assert(SC_SLOTS >= STAGES + 5, "scale records");
 };
 
-template <int G, bool SPLITK>
+template <int G, bool SPLITK, int BN>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_constant__ CUtensorMap tmap_wpacked,
                  const __grid_constant__ CUtensorMap tmap_wscale, const __grid_constant__ CUtensorMap tmap_xscale,
                  const __grid_constant__ CUtensorMap tmap_xh, const __grid_constant__ CUtensorMap tmap_wh,
                  const GemmKernelParams p) {
-    using P = Plan<SPLITK>;
-    constexpr int STAGES = P::STAGES, BAR_OFFSET = P::BAR_OFFSET;
+    using P = Plan<SPLITK, BN>;
+    static_assert(BN == 64 || (BN == 32 && G == 64 && !SPLITK), "32-column tiles: groups of 64, not split");
+    constexpr int STAGES = P::STAGES, BAR_OFFSET = P::BAR_OFFSET, STAGE_BYTES = P::STAGE_BYTES, BU_BYTES = P::BU_BYTES, BP_BYTES = P::BP_BYTES;
+    constexpr int SC_SW_BYTES = P::SC_SW_BYTES, SC_BYTES = P::SC_BYTES;
     constexpr int HB = BN / 2;         // columns per epilogue warp: the warpgroup selects the half of the tile
     constexpr int GPK = BKC / G;       // groups per k-block: 2 (G = 64) or 1 (G = 128)
     constexpr int MMA_PER_G = G / 32;  // 8-bit MMA instructions (K = 32) per group
@@ -330,7 +334,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                         // The loads of a batch are issued before any of its stores: the compiler cannot prove that the
                         // staging buffer and the operand tile do not overlap, so a load written after a store would wait
                         // for it and the whole unpack would run as one dependent chain.
-                        constexpr int PIECES = (BN * 4) / 32, BATCH = 8;
+                        constexpr int PIECES = (BN * 4) / 32, BATCH = PIECES < 8 ? PIECES : 8;
 #pragma unroll
                         for (int jb = 0; jb < PIECES; jb += BATCH) {
                             uint4 pk[BATCH];
@@ -567,7 +571,22 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                         acc2[j] = add_f32x2(acc2[j], ld_shared_u64(red_base + r * RED_BYTES + j * (NUM_EPI_WARPS * 256u) + et * 8u));
                 }
             }
-            {
+            if constexpr (HB < 32) {
+                // two blocks of 8 columns: four bytes of each per lane
+#pragma unroll
+                for (int t = 0; t < HB / 8; ++t) {
+                    const int col = colbase + t * 8 + lc2;
+                    const float2 bv = col < p.N ? __ldg(reinterpret_cast<const float2*>(p.bias + col)) : make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float y_lo, y_hi;
+                        unpack_f32x2(acc2[t * 4 + i], y_lo, y_hi);
+                        const int row = rbase + 8 * i;
+                        if (row < p.M && col < p.N)
+                            *reinterpret_cast<uint32_t*>(p.y + static_cast<size_t>(row) * p.N + col) = pack_bf16x2(y_lo + bv.x, y_hi + bv.y);
+                    }
+                }
+            } else {
                 // A lane holds 2 of the 8 columns of every block; four blocks are transposed inside the quad of lanes
                 // (two exchange steps) so that each lane ends up with all 8 columns = 16 bytes of one block and the
                 // warp writes 64 contiguous bytes per row.
@@ -625,7 +644,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
 
 }  // namespace
 
-dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, bool may_split, cudaStream_t stream) {
+dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, int columns, bool may_split, cudaStream_t stream) {
     const Geometry& g = L->geo;
     CUtensorMap tmap_codes, tmap_xscale, tmap_xh;
     dirotq_status_t st;
@@ -646,7 +665,7 @@ dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, boo
     p.bias = reinterpret_cast<const float*>(L->blob + L->lay.off_bias);
     p.y = a.y; p.partials = a.partials; p.status = a.status; p.early_weights = a.early_weights; p.x_rows = box_rows(a.M);
 
-    const int num_tiles = ((a.M + BM - 1) / BM) * ((g.N + BN - 1) / BN), sms = sm_count(L->device), which = g.G == 64 ? 0 : 1;
+    const int num_tiles = ((a.M + BM - 1) / BM) * ((g.N + columns - 1) / columns), sms = sm_count(L->device), which = g.G == 64 ? 0 : 1;
     using KernelFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                               const CUtensorMap, const CUtensorMap, const GemmKernelParams);
     if (may_split) {
@@ -654,8 +673,8 @@ dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, boo
         // k-blocks and whose clusters, one per tile, are all resident at once (asked of the runtime once per device and size).
         // Only on request (knob value 66): the partial tiles are added in another order than one CTA adds the groups, and by
         // default a token's output bits do not depend on how many other tokens the call has.
-        const KernelFn kern = g.G == 64 ? w4a4_narrow_kernel<64, true> : w4a4_narrow_kernel<128, true>;
-        constexpr int smem = Plan<true>::SMEM_BYTES;
+        const KernelFn kern = g.G == 64 ? w4a4_narrow_kernel<64, true, 64> : w4a4_narrow_kernel<128, true, 64>;
+        constexpr int smem = Plan<true, 64>::SMEM_BYTES;
         static SmemOptIn<2> opt_in;
         static std::atomic<int> resident[64][SPLIT_MAX + 1];  // 0: not asked yet; else clusters resident at once + 1
         if (!opt_in.ensure(kern, which, L->device, smem)) return DIROTQ_ERR_CUDA;
@@ -673,12 +692,14 @@ dirotq_status_t launch_w4a4_narrow(const dirotq_layer* L, const GemmArgs& a, boo
             return err == cudaSuccess ? DIROTQ_OK : DIROTQ_ERR_CUDA;
         }
     }
-    const KernelFn kern = g.G == 64 ? w4a4_narrow_kernel<64, false> : w4a4_narrow_kernel<128, false>;
-    constexpr int smem = Plan<false>::SMEM_BYTES;
-    static SmemOptIn<2> opt_in;
-    if (!opt_in.ensure(kern, which, L->device, smem)) return DIROTQ_ERR_CUDA;
+    const bool half = columns == 32;
+    const KernelFn kern = half ? w4a4_narrow_kernel<64, false, 32> : g.G == 64 ? w4a4_narrow_kernel<64, false, 64> : w4a4_narrow_kernel<128, false, 64>;
+    const int smem = half ? Plan<false, 32>::SMEM_BYTES : Plan<false, 64>::SMEM_BYTES;
+    static SmemOptIn<3> opt_in;
+    if (!opt_in.ensure(kern, half ? 2 : which, L->device, smem)) return DIROTQ_ERR_CUDA;
     const cudaError_t err = launch_kernel(kern, num_tiles < sms ? num_tiles : sms, NUM_THREADS, smem, stream, true, tmap_codes,
-                                          L->tmap_wpacked64, L->tmap_wscale64, tmap_xscale, tmap_xh, L->tmap_wh64, p);
+                                          half ? L->tmap_wpacked32 : L->tmap_wpacked64, half ? L->tmap_wscale32 : L->tmap_wscale64, tmap_xscale, tmap_xh,
+                                          half ? L->tmap_wh32 : L->tmap_wh64, p);
     return err == cudaSuccess ? DIROTQ_OK : DIROTQ_ERR_CUDA;
 }
 

@@ -23,7 +23,7 @@ def _layer(fmt, W, Q, r):
     return dq.dirotq_prepare_layer_ph(W, Uh, 64) if fmt == "int4_ph" else dq.dirotq_prepare_layer_nvfp4_ph(W, Uh, -6)
 
 
-@pytest.mark.parametrize("plan", [0, 128, 192, 256])
+@pytest.mark.parametrize("plan", [0, 64, 128, 192, 256])
 @pytest.mark.parametrize("fmt", ["int4", "int4_g128", "int4_asym", "w4a8", "nvfp4", "int4_ph", "nvfp4_ph"])
 def test_same_bits_as_in_a_full_row_block(fmt, plan):
     K, N, r = 768, 400, 32

@@ -21,7 +21,7 @@ def plan(request):
 
 
 # second row block without rows; ragged columns; second half of the columns without any; an odd number of groups (K - r = 560 and 480)
-@pytest.mark.parametrize("plan", PLANS, indirect=True)
+@pytest.mark.parametrize("plan", [*PLANS, 32], indirect=True)  # (32: 32-column tiles, ragged here too)
 @pytest.mark.parametrize("M, K, N, r, G", [(1, 512, 96, 16, 64), (129, 576, 160, 16, 64), (257, 512, 400, 32, 128), (300, 640, 272, 128, 64)])
 def test_parity_at_tile_edges(plan, M, K, N, r, G):
     spec = synth.LayerSpec(K=K, N=N, r=r, G=G, model=synth.PIXART, seed=71, calib_tokens=512)
@@ -45,7 +45,7 @@ def test_same_bits_as_other_tiles(G, r):
     ws = dq.alloc_workspace(layer, M)
     outs = []
     try:
-        for columns in (256, 0, 128, 192, *PLANS):
+        for columns in (256, 0, 32, 64, 128, 192, *PLANS):
             dq.dirotq_set_gemm_tile(columns)
             outs.append(torch.empty(M, N, dtype=torch.bfloat16, device="cuda"))
             dq.dirotq_linear(x, layer, outs[-1], ws)
