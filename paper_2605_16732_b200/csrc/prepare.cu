@@ -137,40 +137,59 @@ __host__ __device__ __forceinline__ int packed_byte_index(int k) {  // byte of c
     return (k >> 5) * 16 + (w >> 3) * 4 + (w & 3);
 }
 
-// One thread per (group, output column): Eq. 1 with z = 0, s = bf16(max|w|/7), ties to even.
-__global__ void quantize_weights_kernel(const double* Wt, uint8_t* wpacked, float* wscale, uint16_t* wh, Geometry g) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+// Eq. 1 with z = 0, s = bf16(max|w|/7), ties to even.  A block takes a group of G rows by 32 output columns, a thread eight rows of one
+// column, read once and held in registers; the words go through shared memory so that a warp writes whole sectors of four rows.
+// One thread per group and column instead read its G values twice, one latency after another: 24.3 us, now 14.2, at
+// 1152 -> 4608 (42 MB of doubles, 6.5 us at the copy rate).
+template <int G>
+__global__ void __launch_bounds__(4 * G) quantize_weights_kernel(const double* Wt, uint8_t* wpacked, float* wscale, uint16_t* wh, Geometry g) {
+    constexpr int WORDS = G / 8;
+    __shared__ double amax[WORDS][32];
+    __shared__ uint32_t words[32][WORDS + 1];
+    __shared__ int sums[WORDS][32];
+    const int x = threadIdx.x, y = threadIdx.y, n0 = blockIdx.x * 32, n = n0 + x;
     const int grp = blockIdx.y;
-    if (n >= g.N) return;
-    const int j0 = grp * g.G;
-    const int len = min(g.G, g.K_l - j0);
+    const int j0 = grp * G;
+    const int len = n < g.N ? min(G, g.K_l - j0) : 0;
     const double* col = Wt + static_cast<size_t>(g.r + j0) * g.N + n;
-    double a = 0.0;
-    for (int j = 0; j < len; ++j) a = fmax(a, fabs(col[static_cast<size_t>(j) * g.N]));
+    double v[8], a = 0.0;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) v[t] = 8 * y + t < len ? col[static_cast<size_t>(8 * y + t) * g.N] : 0.0;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) a = fmax(a, fabs(v[t]));
+    amax[y][x] = a;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < WORDS; ++i) a = fmax(a, amax[i][x]);
     const uint16_t sb = (a == 0.0) ? 0 : f64_to_bf16(a / 7.0);
     const double s = bf16_to_f64(sb);
-    wscale[wscale_index(g.N, grp, n)] = static_cast<float>(s) * kWScaleFold;  // a power of two times a bf16 value: exact
-    uint8_t* row = wpacked + static_cast<size_t>(n) * (g.K_lp / 2);
+    uint32_t word = 0;
     int csum = 0;
-    for (int jb = 0; jb < g.G; jb += 8) {
-        // codes j0+jb .. j0+jb+7 share four bytes
-        uint32_t word = 0;
+    if (s != 0.0) {
+        // v / s rounds as v (1 / s) does unless that is within a few units in the last place of a half (or is not a number)
+        const double inv = 1.0 / s;
+#pragma unroll
         for (int t = 0; t < 8; ++t) {
-            const int j = jb + t;
-            int q = 0;
-            if (j < len && s != 0.0) {
-                double qq = rint(col[static_cast<size_t>(j) * g.N] / s);
-                qq = fmin(7.0, fmax(-7.0, qq));
-                q = static_cast<int>(qq);
-            }
+            const double p = v[t] * inv;
+            int q;
+            if (fabs(p - rint(p)) < 0.499999) q = max(-7, min(7, __double2int_rn(p)));
+            else q = static_cast<int>(fmin(7.0, fmax(-7.0, rint(v[t] / s))));
             csum += q;
             word |= signmag_nibble_bits(t, q);
         }
-        *reinterpret_cast<uint32_t*>(row + packed_byte_index(j0 + jb)) = word;
     }
+    words[x][y] = word;
+    sums[y][x] = csum;
+    __syncthreads();
+    const int flat = y * 32 + x, row = flat / WORDS, w = flat % WORDS;
+    if (n0 + row < g.N)  // the words of 64 codes are 32 bytes side by side
+        *reinterpret_cast<uint32_t*>(wpacked + static_cast<size_t>(n0 + row) * (g.K_lp / 2) + packed_byte_index(j0 + 8 * w)) = words[row][w];
+    if (y != 0 || n >= g.N) return;
+    wscale[wscale_index(g.N, grp, n)] = static_cast<float>(s) * kWScaleFold;  // a power of two times a bf16 value: exact
     if (g.fmt == 2) {
         // zero-point term of asymmetric activations: d = s_w * sum(q_w) (at most 17 significant bits), stored as three
         // bf16 pieces that add up to it exactly, in the extra columns of the rank-r weight operand
+        for (int i = 1; i < WORDS; ++i) csum += sums[i][x];
         double rem = s * static_cast<double>(csum);
         uint16_t* ext = wh + static_cast<size_t>(n) * g.r_pad + g.r_pad0;
         for (int piece = 0; piece < 3; ++piece) {
@@ -179,6 +198,15 @@ __global__ void quantize_weights_kernel(const double* Wt, uint8_t* wpacked, floa
             rem -= bf16_to_f64(pb);
         }
     }
+}
+void launch_quantize_weights(const dirotq_layer* L, const double* Wt, cudaStream_t stream) {
+    const Geometry& g = L->geo;
+    uint8_t* wpacked = reinterpret_cast<uint8_t*>(L->blob + L->lay.off_wpacked);
+    float* wscale = reinterpret_cast<float*>(L->blob + L->lay.off_wscale);
+    uint16_t* wh = reinterpret_cast<uint16_t*>(L->blob + L->lay.off_wh);
+    const dim3 grid((g.N + 31) / 32, g.n_g), block(32, g.G / 8);
+    if (g.G == 64) quantize_weights_kernel<64><<<grid, block, 0, stream>>>(Wt, wpacked, wscale, wh, g);
+    else quantize_weights_kernel<128><<<grid, block, 0, stream>>>(Wt, wpacked, wscale, wh, g);
 }
 
 // Residual weights rounded by the caller (GPTQ or any other offline rounding): codes [K_l][N] int8 and bf16 scales
@@ -634,9 +662,7 @@ dirotq_status_t launch_prepare(const dirotq_layer* L, const void* W, int w_dtype
             wcodes, static_cast<const uint16_t*>(wscales), reinterpret_cast<uint8_t*>(blob + L->lay.off_wpacked),
             reinterpret_cast<float*>(blob + L->lay.off_wscale), reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
     else
-        quantize_weights_kernel<<<dim3((g.N + 127) / 128, g.n_g), 128, 0, stream>>>(
-            scratch, reinterpret_cast<uint8_t*>(blob + L->lay.off_wpacked),
-            reinterpret_cast<float*>(blob + L->lay.off_wscale), reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
+        launch_quantize_weights(L, scratch, stream);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     if (!g.no_rot) {
         rotation_kernel<<<dim3((g.K + 31) / 32, (g.K + 31) / 32), dim3(32, 8), 0, stream>>>(
@@ -782,9 +808,7 @@ dirotq_status_t launch_prepare_ph(const dirotq_layer* L, const void* W, int w_dt
     // scratch now holds [r + K][N]: the same shape the INT4 pipeline quantizes (rows < r in 16 bits, the rest in groups)
     high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
-    quantize_weights_kernel<<<dim3((g.N + 127) / 128, g.n_g), 128, 0, stream>>>(
-        scratch, reinterpret_cast<uint8_t*>(blob + L->lay.off_wpacked), reinterpret_cast<float*>(blob + L->lay.off_wscale),
-        reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
+    launch_quantize_weights(L, scratch, stream);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     bias_kernel<<<(g.N + 255) / 256, 256, 0, stream>>>(static_cast<const uint16_t*>(bias),
                                                        reinterpret_cast<float*>(blob + L->lay.off_bias), g.N);
