@@ -73,12 +73,12 @@ def main():
     if args.what == "small_m":
         c = suite.Case(256, 1152, 1152, 32, 64, synth.PIXART)
         dq.dirotq_set_rotation_tile(5)
-        dq.dirotq_set_gemm_tile(64)
+        dq.dirotq_set_gemm_tile(32)
         us = c.graph_ms(lambda: dq.dirotq_rotate_quantize(c.x, c.layer, c.ws)) * 1e3
         _show("rotate_quant_kernel", f"128 x 64 tiles, {us:.2f} us per call in graph replay", c.ws)
         c.ws[:256].zero_()
         us = c.graph_ms(lambda: dq.dirotq_w4a4_gemm(c.M, c.layer, c.ws, c.y)) * 1e3
-        _show("w4a4_narrow_kernel", f"128 x 64 tiles, {us:.2f} us per call in graph replay", c.ws)
+        _show("w4a4_narrow_kernel", f"128 x 32 tiles, {us:.2f} us per call in graph replay", c.ws)
     else:
         suite.FMT, kernel, tile = WIDE[args.what]
         c = suite.Case(4608, 3072, 9216, 32, 64, synth.FLUX)
