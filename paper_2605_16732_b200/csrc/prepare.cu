@@ -139,6 +139,7 @@ __host__ __device__ __forceinline__ int packed_byte_index(int k) {  // byte of c
 
 // Eq. 1 with z = 0, s = bf16(max|w|/7), ties to even.  A block takes a group of G rows by 32 output columns, a thread eight rows of one
 // column, read once and held in registers; the words go through shared memory so that a warp writes whole sectors of four rows.
+// Every code of the layer is written (K_lp = n_g G), zeros behind a ragged last group: nothing has to be cleared before.
 // One thread per group and column instead read its G values twice, one latency after another: 24.3 us, now 14.2, at
 // 1152 -> 4608 (42 MB of doubles, 6.5 us at the copy rate).
 template <int G>
@@ -245,10 +246,12 @@ __global__ void pack_codes_kernel(const int8_t* codes, const uint16_t* scales, u
 }
 
 // wh[n][i] = bf16(Wt[i][n]) for i < r, zero up to r_pad: eight rows i per thread, one 16-byte store (one thread per column, all
-// rows in sequence, took 25 us for 32 rows of 4608 columns).
-__global__ void high_rows_kernel(const double* Wt, uint16_t* wh, Geometry g) {
+// rows in sequence, took 25 us for 32 rows of 4608 columns).  The blocks of the first eight rows also widen the bias: a launch of its own
+// for it, and a fill of the codes that the quantizer then wrote, were 6 of 498 us at 1152 -> 4608.
+__global__ void high_rows_kernel(const double* Wt, uint16_t* wh, const uint16_t* bias, float* bias_out, Geometry g) {
     const int n = blockIdx.x * blockDim.x + threadIdx.x, i0 = blockIdx.y * 8;
     if (n >= g.N) return;
+    if (i0 == 0) bias_out[n] = bias ? __uint_as_float(static_cast<uint32_t>(bias[n]) << 16) : 0.f;
     uint32_t w[4] = {};
 #pragma unroll
     for (int u = 0; u < 8; ++u)
@@ -651,11 +654,10 @@ dirotq_status_t launch_prepare(const dirotq_layer* L, const void* W, int w_dtype
     const Geometry& g = L->geo;
     char* blob = L->blob;
     if (!launch_fold(Q, q_dtype, W, w_dtype, w_layout, scratch, g.K, g.N, stream)) return DIROTQ_ERR_CUDA;
-    // zero the packed codes first: slots of a ragged last group stay zero
-    if (cudaMemsetAsync(blob + L->lay.off_wpacked, 0, static_cast<size_t>(g.N) * (g.K_lp / 2), stream) != cudaSuccess)
-        return DIROTQ_ERR_CUDA;
     // the rank-r rows first (zero padded to r_pad), then the quantizer, which for fmt 2 fills its extra columns
-    high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
+    high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(
+        scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), static_cast<const uint16_t*>(bias),
+        reinterpret_cast<float*>(blob + L->lay.off_bias), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     if (wcodes)
         pack_codes_kernel<<<dim3((g.N + 127) / 128, g.n_g), 128, 0, stream>>>(
@@ -669,17 +671,13 @@ dirotq_status_t launch_prepare(const dirotq_layer* L, const void* W, int w_dtype
             Q, q_dtype, reinterpret_cast<uint16_t*>(blob + L->lay.off_qt), g);
         if (!launch_ok()) return DIROTQ_ERR_CUDA;
     }
-    bias_kernel<<<(g.N + 255) / 256, 256, 0, stream>>>(static_cast<const uint16_t*>(bias),
-                                                       reinterpret_cast<float*>(blob + L->lay.off_bias), g.N);
-    return launch_ok() ? DIROTQ_OK : DIROTQ_ERR_CUDA;
+    return DIROTQ_OK;
 }
 
 // Replaces the residual codes and scales of a prepared grouped-INT4 layer (codes int8 [K_l][N], bf16 scales [n_g][N], device).
 dirotq_status_t launch_pack_codes(const dirotq_layer* L, const int8_t* wcodes, const uint16_t* wscales, cudaStream_t stream) {
     const Geometry& g = L->geo;
     char* blob = L->blob;
-    if (cudaMemsetAsync(blob + L->lay.off_wpacked, 0, static_cast<size_t>(g.N) * (g.K_lp / 2), stream) != cudaSuccess)
-        return DIROTQ_ERR_CUDA;
     pack_codes_kernel<<<dim3((g.N + 127) / 128, g.n_g), 128, 0, stream>>>(
         wcodes, wscales, reinterpret_cast<uint8_t*>(blob + L->lay.off_wpacked), reinterpret_cast<float*>(blob + L->lay.off_wscale),
         reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
@@ -803,15 +801,12 @@ dirotq_status_t launch_prepare_ph(const dirotq_layer* L, const void* W, int w_dt
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     ph_fold_low_kernel<<<dim3((g.N + 127) / 128, g.K), 128, 0, stream>>>(W, w_dtype, w_layout, scratch, g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
-    if (cudaMemsetAsync(blob + L->lay.off_wpacked, 0, static_cast<size_t>(g.N) * (g.K_lp / 2), stream) != cudaSuccess)
-        return DIROTQ_ERR_CUDA;
     // scratch now holds [r + K][N]: the same shape the INT4 pipeline quantizes (rows < r in 16 bits, the rest in groups)
-    high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
+    high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(
+        scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), static_cast<const uint16_t*>(bias),
+        reinterpret_cast<float*>(blob + L->lay.off_bias), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     launch_quantize_weights(L, scratch, stream);
-    if (!launch_ok()) return DIROTQ_ERR_CUDA;
-    bias_kernel<<<(g.N + 255) / 256, 256, 0, stream>>>(static_cast<const uint16_t*>(bias),
-                                                       reinterpret_cast<float*>(blob + L->lay.off_bias), g.N);
     return launch_ok() ? DIROTQ_OK : DIROTQ_ERR_CUDA;
 }
 
@@ -855,16 +850,15 @@ dirotq_status_t launch_prepare_w4a8(const dirotq_layer* L, const void* W, int w_
     const Geometry& g = L->geo;
     char* blob = L->blob;
     if (!launch_fold(Q, q_dtype, W, w_dtype, w_layout, scratch, g.K, g.N, stream)) return DIROTQ_ERR_CUDA;
-    high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), g);
+    high_rows_kernel<<<dim3((g.N + 127) / 128, g.r_pad / 8), 128, 0, stream>>>(
+        scratch, reinterpret_cast<uint16_t*>(blob + L->lay.off_wh), static_cast<const uint16_t*>(bias),
+        reinterpret_cast<float*>(blob + L->lay.off_bias), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     w4a8_quantize_weights_kernel<<<(g.N + 31) / 32, dim3(32, 16), 0, stream>>>(
         scratch, reinterpret_cast<uint8_t*>(blob + L->lay.off_wpacked), reinterpret_cast<float*>(blob + L->lay.off_wscale), g);
     if (!launch_ok()) return DIROTQ_ERR_CUDA;
     rotation_kernel<<<dim3((g.K + 31) / 32, (g.K + 31) / 32), dim3(32, 8), 0, stream>>>(
         Q, q_dtype, reinterpret_cast<uint16_t*>(blob + L->lay.off_qt), g);
-    if (!launch_ok()) return DIROTQ_ERR_CUDA;
-    bias_kernel<<<(g.N + 255) / 256, 256, 0, stream>>>(static_cast<const uint16_t*>(bias),
-                                                       reinterpret_cast<float*>(blob + L->lay.off_bias), g.N);
     return launch_ok() ? DIROTQ_OK : DIROTQ_ERR_CUDA;
 }
 
