@@ -203,7 +203,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
         }
     }
     __syncwarp();
-    if (PAIR || (warp != 2 && warp != 3)) {  // (the unpack warps read nothing but what lands on barriers)
+    if (pre == 0 || (warp != 2 && warp != 3)) {  // (otherwise the unpack warps wait when they are through with the early weights)
         grid_dependency_wait();
         if (threadIdx.x == 0) TRACE_CLK(p.status, 11);
         // the next layer's first kernel may be scheduled as this grid's CTAs leave their SMs (it waits for this whole grid)
@@ -320,7 +320,7 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                         if (!timed_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_ops)) { ok = false; break; }
                         if (!PAIR && pre_left > 0) {  // (these were expanded before their activations had been asked for)
                             --pre_left;
-                            if (!mbar_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
+                            if (!timed_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_ops)) { ok = false; break; }
                         }
                         if (lane == 0) { if (kb == 0) TRACE_CLK(p.status, 16); if (kb == 4) TRACE_CLK(p.status, 17); if (kb == p.num_kb - 1) TRACE_CLK(p.status, 18); }
                         tc_fence_after_sync();
@@ -400,6 +400,8 @@ w4a4_gemm_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_co
                 const int items = p.num_kb + p.lr_chunks;
                 for (int i = 0; i < items; ++i, at.next()) {
                     const uint32_t s = at.s;
+                    // (before the first wait on what the previous kernel leaves: how long that one runs is no part of a bounded wait, nor of w_full)
+                    if (!PAIR && at.it == static_cast<uint32_t>(pre)) grid_dependency_wait();
                     // A barrier is waited on by its phase's parity, and of a stage expanded early this warp has not seen the activations land: they have when
                     // the stage's MMAs are done.  (Not a wait for the landing itself: the barrier may be two phases on by now.)
                     if (at.it - STAGES < static_cast<uint32_t>(pre) && !mbar_wait(empty_bar(s), at.ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }

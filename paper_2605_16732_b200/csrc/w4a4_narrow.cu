@@ -164,7 +164,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
         }
     }
     __syncwarp();
-    if (warp != 2 && warp != 3) {  // (the unpack warps read nothing but what lands on barriers)
+    if (pre == 0 || (warp != 2 && warp != 3)) {  // (otherwise the unpack warps wait when they are through with the early weights)
         grid_dependency_wait();
         if (threadIdx.x == 0) TRACE_CLK(p.status, 11);
         // the next layer's first kernel may be scheduled as this grid's CTAs leave their SMs (it waits for this whole grid)
@@ -254,7 +254,7 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
                         if (!timed_wait(unp_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_ops)) { ok = false; break; }
                         if (pre_left > 0) {  // (these were expanded before their activations had been asked for)
                             --pre_left;
-                            if (!mbar_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA)) { ok = false; break; }
+                            if (!timed_wait(full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_ops)) { ok = false; break; }
                         }
                         if (lane == 0) { if (kb == kb0) TRACE_CLK(p.status, 16); if (kb == 4) TRACE_CLK(p.status, 17); if (kb == kb1 - 1) TRACE_CLK(p.status, 18); }
                         if (!timed_wait(tempty_bar(b), bph, abort_flag, p.status, DEV_TIMEOUT_MMA, w_tempty)) { ok = false; break; }
@@ -315,9 +315,12 @@ w4a4_narrow_kernel(const __grid_constant__ CUtensorMap tmap_codes, const __grid_
             for (int tile = first_tile(); ok && tile < num_tiles; tile += tile_stride()) {
                 const int items = (kb1 - kb0) + lr_here;
                 for (int i = static_cast<int>((warp - 2 + first_it) & 1); i < items; i += 2) {
+                    const uint32_t it = first_it + i;
+                    // (before this warp's first wait on what the previous kernel leaves: how long that one runs is no part of a bounded wait, nor of
+                    // w_full; a warp's items are two apart)
+                    if (it - static_cast<uint32_t>(pre) < 2u) grid_dependency_wait();
                     // A barrier is waited on by its phase's parity, and of a stage expanded early this warp has not seen the activations land: they have when
                     // the stage's MMAs are done.  (Not a wait for the landing itself: the barrier may be two phases on by now.)
-                    const uint32_t it = first_it + i;
                     if (it - STAGES < static_cast<uint32_t>(pre) && !mbar_wait(empty_bar(s), ph ^ 1, abort_flag, p.status, DEV_TIMEOUT_UNPACK)) { ok = false; break; }
                     ok = timed_wait(it < static_cast<uint32_t>(pre) ? pre_bar(s) : full_bar(s), ph, abort_flag, p.status, DEV_TIMEOUT_UNPACK, w_full);
                     if (!ok) break;
