@@ -275,7 +275,9 @@ WAIT_COUNTER_NAMES = ("producer_wait_stage", "mma_wait_operands", "mma_wait_accu
 
 
 def dirotq_workspace_wait_counters(workspace: torch.Tensor, stream=None) -> dict:
-    """Per-role blocked-cycle counters of the W4A4 kernel (summed over CTAs and calls since the workspace was zeroed)."""
+    """Per-role blocked-cycle counters of the W4A4 kernel (summed over CTAs and calls since the workspace was zeroed).  Every wait is counted by the
+    diagnostic build; the default build leaves out what the hardware's suspension of a thread covers.  epilogue_wait_scales is always 0: scales
+    land with the operands."""
     out = (ctypes.c_ulonglong * 8)()
     _check(lib().dirotq_workspace_wait_counters(workspace.data_ptr(), _stream(stream), out),
            "dirotq_workspace_wait_counters")

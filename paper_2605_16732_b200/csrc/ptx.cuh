@@ -32,11 +32,13 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 // Diagnostic build (-DDIROTQ_TRACE, optionally -DDIROTQ_TRACE_BLOCK=n): block n (0) stamps the SM clock at marked points of each role into the 8-byte slots
 // 9..31 of the workspace's status block, for reading a small call's critical path off the device.
 #ifdef DIROTQ_TRACE
+constexpr bool kTraceBuild = true;
 #ifndef DIROTQ_TRACE_BLOCK
 #define DIROTQ_TRACE_BLOCK 0
 #endif
 #define TRACE_CLK(status, slot) do { if (blockIdx.x == DIROTQ_TRACE_BLOCK) reinterpret_cast<volatile unsigned long long*>(status)[slot] = clock64(); } while (0)
 #else
+constexpr bool kTraceBuild = false;
 #define TRACE_CLK(status, slot) do {} while (0)
 #endif
 

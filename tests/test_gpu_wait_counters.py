@@ -1,4 +1,9 @@
 """What the wait counters of the INT4 second kernels contain: a role's waits in its own kernel, not what was left of the kernel before it."""
+import json
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -46,3 +51,24 @@ def test_waits_leave_the_previous_kernel_out(plan, parts):
     assert c["unpack_wait_tma"] <= 1.25 * c["mma_role_total"], c
     assert c["epilogue_wait_accumulator"] <= c["epilogue_total"] <= 1.25 * c["mma_role_total"], c
     assert c["mma_wait_operands"] + c["mma_wait_accumulator"] <= c["mma_role_total"], c
+
+
+PROGRAM = """
+import json
+from paper_2605_16732_b200 import binding as dq, build
+dq.use_library(build.build_trace())
+from test_gpu_wait_counters import _counters
+print(json.dumps([_counters(plan, False) for plan in (32, 64, 128, 130, 192, 256)]))
+"""
+
+
+def test_the_diagnostic_build_counts_every_wait():
+    here = os.path.dirname(os.path.abspath(__file__))
+    r = subprocess.run([sys.executable, "-c", PROGRAM], capture_output=True, text=True, timeout=300, cwd=os.path.dirname(here),
+                       env=dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(here), here])))
+    assert r.returncode == 0, r.stderr[-2000:]
+    for c in json.loads(r.stdout):
+        # a kernel's first activations are waited for by everyone; nothing waits for scales by themselves
+        assert min(c["mma_wait_operands"], c["unpack_wait_tma"], c["epilogue_wait_accumulator"]) > 0 and c["epilogue_wait_scales"] == 0, c
+        assert c["unpack_wait_tma"] <= 1.25 * c["mma_role_total"] and c["epilogue_wait_accumulator"] <= c["epilogue_total"], c
+        assert c["mma_wait_operands"] + c["mma_wait_accumulator"] <= c["mma_role_total"], c
