@@ -188,9 +188,9 @@ DIROTQ_API dirotq_status_t dirotq_int_gemm_debug(const int8_t* act_codes, int M,
  * distributed shared memory) wherever every tile's cluster is resident at once and every CTA keeps two k-blocks; never
  * chosen automatically, because its outputs differ from the other plans' in fp32 summation order (a bf16 step on a few
  * values), and with 0 a token's output bits do not depend on how many tokens a call has; 130: the grouped INT4 kernel with 256 token
- * rows x 128 columns per CTA; 192: the grouped INT4 kernel's plan
- * with three epilogue warpgroups (64 columns per thread); 512: the grouped INT4 and NVFP4 kernels in pairs of CTAs (clusters of two,
- * tcgen05.mma.cta_group::2, 256 token rows x 256 columns per pair, each CTA loading its own rows and one half of the weight tile), forced;
+ * rows x 128 columns per CTA, 258: in pairs of CTAs (clusters of two, tcgen05.mma.cta_group::2, 256 token rows x 256 columns per pair,
+ * each CTA loading its own rows and one half of the weight tile); 192: the grouped INT4 kernel's plan
+ * with three epilogue warpgroups (64 columns per thread); 512: the NVFP4 kernel in pairs of CTAs (as 258), forced;
  * 0 takes it where its schedule is the shortest (every FLUX
  * shape at M = 4608); for W4A8 128 is single CTAs, 256 and 512 are CTA pairs with 128 and 256 columns.  A value that names a plan of
  * one kernel leaves the other formats' kernels choosing for themselves.  Process-wide; results do not depend on it, 66

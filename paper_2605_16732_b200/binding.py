@@ -530,8 +530,9 @@ def dirotq_layer_export_v(layer: Layer, stream=None) -> torch.Tensor:
 
 def dirotq_set_gemm_tile(columns: int) -> None:
     """Tile plan of the second kernels (process-wide): 0 automatic; 128 or 256 columns per tile; 32, 64, 66 (the reduction split over a
-    cluster), 130 (256 token rows x 128 columns) and 192: plans of the INT4 kernels only; 512: CTA pairs with 256 columns (for W4A8 128 is
-    single CTAs, 256 CTA pairs with 128 columns)."""
+    cluster), 130 (256 token rows x 128 columns), 192 and 258 (CTA pairs with 256 columns): plans of the INT4 kernels only; 512: CTA pairs with
+    256 columns, NVFP4 and W4A8 (for which 128 is single CTAs, 256 CTA pairs with 128 columns).  A value that names no plan of a format's kernel
+    leaves that kernel choosing for itself."""
     _check(lib().dirotq_set_gemm_tile(int(columns)), "dirotq_set_gemm_tile")
 
 

@@ -1,5 +1,6 @@
 // C ABI of libdirotq: argument validation, tensor-map construction, launch sequencing.
 #include "common.h"
+#include "w4a4_plan.h"
 
 #include <algorithm>
 
@@ -657,8 +658,7 @@ dirotq_status_t dirotq_set_dependent_launch(int enabled) {
 }
 
 dirotq_status_t dirotq_set_gemm_tile(int columns) {
-    // 32, 64, 66, 130 and 192: plans of the grouped INT4 second kernel only
-    const bool int4_only = columns == 32 || columns == 64 || columns == 66 || columns == 130 || columns == 192;  // 66: 64 columns with the reduction split over a cluster
+    const bool int4_only = w4a4_plan_exists(columns) && columns != 128 && columns != 256;  // (the other kernels then choose for themselves)
     dirotq_status_t st = set_w4a4_tile_columns(columns);
     if (st == DIROTQ_OK) st = set_nvfp4_tile_columns(int4_only ? 0 : columns);
     return st != DIROTQ_OK ? st : set_w4a8_tile_columns(int4_only ? 0 : columns);

@@ -50,6 +50,7 @@
 //   warpgroups 1-2: epilogue; warp%4 selects the TMEM lane quadrant (token rows), the warpgroup
 //                   selects the half of the tile's columns.
 #include "w4a4.cuh"
+#include "w4a4_plan.h"
 
 #include <atomic>
 
@@ -738,38 +739,20 @@ static dirotq_status_t launch_w4a4_gemm_bn(const dirotq_layer* L, const GemmArgs
 
 }  // namespace
 
-static std::atomic<int> g_tile_columns{0};  // 0: chosen per call; 64 / 128 / 192 / 256: forced; 66: 64 columns, split plan where it applies
+static std::atomic<int> g_forced_plan{0};  // 0: chosen per call
 
 dirotq_status_t set_w4a4_tile_columns(int columns) {
-    if (columns != 0 && columns != 32 && columns != 64 && columns != 66 && columns != 128 && columns != 192 && columns != 256 && columns != 512 && columns != 130) return DIROTQ_ERR_INVALID_ARG;
-    g_tile_columns.store(columns);
+    const int plan = w4a4_forced_plan(columns);
+    if (plan < 0) return DIROTQ_ERR_INVALID_ARG;
+    g_forced_plan.store(plan);
     return DIROTQ_OK;
 }
 
 dirotq_status_t launch_w4a4_gemm(const dirotq_layer* L, const GemmArgs& a, cudaStream_t stream) {
-    // The plan with the shortest schedule: turns of the SMs (or of the pairs of SMs) x what one tile of the plan costs.  Costs relative to a pair's tile,
-    // from 4608 x 3072 -> 9216 (a turn of pairs: 26.2 us with groups of 64, 17.0 with groups of 128), whose clusters cost a call 0.9 us more.  Over 110
-    // shapes of 16 to 17816 rows, 512 to 11776 coefficients and 512 to 12240 columns what is chosen is within 3 % of the fastest plan, in the mean
-    // within 0.5 % (one call of 7 us: 5 %).
-    const int forced = g_tile_columns.load(), sms = sm_count(L->device);
-    const bool g64 = L->geo.G == 64;
-    struct Candidate { int knob, rows, columns, ctas; double cost64, cost128; };
-    static constexpr Candidate kPlans[] = {{32, 128, 32, 1, 0.25, 0.0}, {64, 128, 64, 1, 0.295, 0.38}, {128, 128, 128, 1, 0.615, 0.73}, {192, 128, 192, 1, 0.846, 0.957},
-                                           {130, 256, 128, 1, 1.02, 1.03}, {256, 128, 256, 1, 1.068, 1.21}, {512, 256, 256, 2, 1.0, 1.0}};
-    int plan = forced;
-    double best = 0.0;
-    for (const Candidate& c : kPlans) {
-        if (forced) break;
-        if (c.knob == 32 && (!g64 || ((a.M + 127) / 128) * ((L->geo.N + 31) / 32) > sms / 2)) continue;  // (see w4a4_narrow.cu)
-        const long tiles = static_cast<long>((a.M + c.rows - 1) / c.rows) * ((L->geo.N + c.columns - 1) / c.columns), slots = sms / c.ctas;
-        const double t = static_cast<double>((tiles + slots - 1) / slots) * (g64 ? c.cost64 : c.cost128) + (c.ctas == 2 ? 100.0 / L->geo.K_lp : 0.0);
-        if (plan == 0 || t < best) {
-            plan = c.knob;
-            best = t;
-        }
-    }
-    if (a.partials == nullptr && plan <= 66) return launch_w4a4_narrow(L, a, plan == 32 && g64 ? 32 : 64, plan == 66, stream);
-    if (plan == 512 && a.partials == nullptr) return launch_w4a4_gemm_bn<256, PAIRED>(L, a, stream);
+    const int forced = g_forced_plan.load();
+    const int plan = forced ? forced : choose_w4a4_plan(a.M, L->geo.N, L->geo.K_lp, L->geo.G, sm_count(L->device));
+    if (a.partials == nullptr && plan <= 66) return launch_w4a4_narrow(L, a, plan == 32 && L->geo.G == 64 ? 32 : 64, plan == 66, stream);
+    if (plan == 258 && a.partials == nullptr) return launch_w4a4_gemm_bn<256, PAIRED>(L, a, stream);
     if (plan == 130 && a.partials == nullptr) return launch_w4a4_gemm_bn<128, TALL>(L, a, stream);
     if (plan == 192) return launch_w4a4_gemm_bn<192>(L, a, stream);
     return plan >= 256 ? launch_w4a4_gemm_bn<256>(L, a, stream) : launch_w4a4_gemm_bn<128>(L, a, stream);

@@ -8,7 +8,7 @@ from paper_2605_16732_b200 import binding as dq
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("plan", [32, 64, 66, 128, 130, 192, 256, 512])
+@pytest.mark.parametrize("plan", [32, 64, 66, 128, 130, 192, 256, 258, 512])
 @pytest.mark.parametrize("M, K, N, r, G", [(5, 256, 48, 16, 64), (130, 512, 400, 32, 64), (300, 768, 272, 64, 64), (257, 1024, 320, 128, 128), (1500, 1664, 2832, 32, 64)])
 def test_linear_equals_its_two_parts(plan, M, K, N, r, G):
     g = torch.Generator(device="cuda").manual_seed(K + plan)
