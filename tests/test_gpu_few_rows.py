@@ -44,3 +44,13 @@ def test_same_bits_as_in_a_full_row_block(fmt, plan):
         dq.dirotq_set_gemm_tile(0)
     assert dq.dirotq_workspace_status(ws) == 0
     layer.close()
+
+
+@pytest.mark.parametrize("plan", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("fmt", ["int4", "int4_g128", "int4_asym", "w4a8", "nvfp4"])  # (the projection form's first stage has one plan)
+def test_same_bits_under_every_rotation_plan(fmt, plan):
+    dq.dirotq_set_rotation_tile(plan)
+    try:
+        test_same_bits_as_in_a_full_row_block(fmt, 0)
+    finally:
+        dq.dirotq_set_rotation_tile(0)
