@@ -157,8 +157,8 @@ dirotq_status_t dirotq_workspace_bytes(const dirotq_layer_t* layer, int M, size_
     return DIROTQ_OK;
 }
 
-// Weight-side tensor maps with 192-row boxes (the 192-column tile plan of the grouped INT4 second kernel) and with 64-row
-// boxes (its plan for calls with few token rows).
+// Weight-side tensor maps of the grouped INT4 second kernel with boxes of 64 and 32 rows (its plans for calls with few token rows, whose
+// scale boxes hold all groups of a k-block) and, below, of 192 rows (its 192-column plan).
 static dirotq_status_t encode_tmaps_rows(dirotq_layer* L, int N, int group, int rows, CUtensorMap* wpacked, CUtensorMap* wscale,
                                          CUtensorMap* wh) {
     const Geometry& g = L->geo;

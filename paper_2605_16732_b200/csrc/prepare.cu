@@ -1,7 +1,7 @@
 // Offline part (paper Eq. 5, right factor): fold the rotation into the weight, split at row r,
 // quantize the low rows to INT4 per (group, output column) with round-to-nearest, pack, and lay
-// everything out the way the two online kernels read it.  Plain CUDA cores, fp64: this runs once
-// per layer and is not on the timed path.
+// everything out the way the two online kernels read it.  fp64 throughout (the fold on the double-precision
+// matrix instruction): this runs once per layer, when it is loaded.
 //
 // Packed weight-code layout, row n of u8 [N][K_lp/2] (K-major): codes are taken 32 at a time
 // (16 bytes, four 32-bit words); word j of such a piece holds codes 8*j .. 8*j + 7.  In the grouped INT4
@@ -50,7 +50,7 @@ __device__ __forceinline__ double load_w(const void* W, int w_dtype, int w_layou
 // Bound by fp64 arithmetic: 28 TFLOP/s at 3072^3.  Eight 8-byte loads per lane feed 16 instructions of 256 multiply-adds; with
 // scalar multiply-adds (8 x 4 per thread) their register operands held the pipe at 55 %.  The next tile's loads are in flight
 // under the arithmetic and are held in their own type (converted at once, every tile waited for them).  Preparation and export,
-// 1152 -> 4608: 1595 us with a scalar 4 x 4 per thread, 682 with 8 x 4, 508 now.
+// 1152 -> 4608: 1595 us with a scalar 4 x 4 per thread, 682 with 8 x 4, 508 with this (490 since the kernels behind it were trimmed).
 constexpr int FOLD_I = 64, FOLD_N = 64, FOLD_THREADS = 128;
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return static_cast<double>(v); }

@@ -66,7 +66,7 @@ namespace {
 //   128: two warpgroups, 64 columns per thread, four accumulator tiles; for layers whose wider tiles would leave SMs idle.
 // and of how many token rows:
 //   ONE:  128.
-//   PAIR: 128 in each of two CTAs that share every MMA (tcgen05.mma.cta_group::2, 256 columns): each loads its own activation codes and loads and
+//   PAIRED: 128 in each of two CTAs that share every MMA (tcgen05.mma.cta_group::2, 256 columns): each loads its own activation codes and loads and
 //         expands half of the tile's weights.
 //   TALL: 256 in one CTA, a warpgroup for each half (128 columns): a warp's share is that of the 256-column tile, the weights to expand are half.
 enum Rows : int { ONE, PAIRED, TALL };
@@ -88,7 +88,7 @@ struct Plan {
     static constexpr int AC_BYTES = CTA_ROWS * BKC;   // activation codes / bf16 x~_h chunk
     static constexpr int BU_BYTES = WROWS * BKC;      // unpacked weight codes / bf16 W~_h chunk (32 KB at BN = 256)
     static constexpr int BP_BYTES = WROWS * BKC / 2;  // packed weight codes (TMA staging)
-    static constexpr int STAGE_BYTES = AC_BYTES + BU_BYTES + BP_BYTES;  // 64 KB / 40 KB
+    static constexpr int STAGE_BYTES = AC_BYTES + BU_BYTES + BP_BYTES;  // KB: 256 columns 64, 192 52, 128 40; tall 56, a pair's CTA 40
     static constexpr int SC_SW_BYTES = BN * 4, SC_BYTES = SC_SW_BYTES + CTA_ROWS * 4;  // weight scales, activation scales
     static constexpr int BAR_OFFSET = STAGES * STAGE_BYTES + SC_SLOTS * SC_BYTES;
     static constexpr int SMEM_BYTES = BAR_OFFSET + 512 + 1024;
